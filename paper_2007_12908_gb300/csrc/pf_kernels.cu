@@ -1,5 +1,5 @@
 // Element kernels (energy, quartic energy difference, gradient, Hessian-vector
-// product), fracture rasterisation and grid transfers for sm_103a.
+// product) and fracture rasterisation for sm_103a.
 //
 // Element loops are owner-computes: a CTA owns a tile of nodes, evaluates
 // every element touching them (one halo layer on the low side) and sums the
@@ -1532,148 +1532,6 @@ cudaError_t rasterize(const Geom& g, int kind, int n, const double* rows_dev, do
   long long nb = (g.N + 255) / 256;
   if (nb > 4096) nb = 4096;
   k_raster<<<int(nb), 256, 0, st>>>(g, kind, n, rows_dev, band, c_plane, c_prev);
-  return cudaGetLastError();
-}
-
-// ------------------------------------------------------------ transfers
-// Q1 prolongation: a fine node on an even index coincides with a coarse
-// node; on an odd index it averages its two coarse neighbours (per axis).
-template <class T>
-__global__ void k_prolong(Geom gc, Geom gf, int nf, const T* __restrict__ in, T* __restrict__ out,
-                          const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  const long long total = gf.N * nf;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int f = int(t / gf.N);
-    const long long i = t - f * gf.N;
-    const int ix = int(i % gf.n[0]);
-    const long long r = i / gf.n[0];
-    const int iy = int(r % gf.n[1]);
-    const int iz = int(r / gf.n[1]);
-    int c0[3] = {ix >> 1, iy >> 1, iz >> 1};
-    int odd[3] = {ix & 1, iy & 1, iz & 1};
-    const T* src = in + f * gc.N;
-    T acc = T(0);
-    for (int dz = 0; dz <= odd[2]; ++dz)
-      for (int dy = 0; dy <= odd[1]; ++dy)
-        for (int dx = 0; dx <= odd[0]; ++dx) {
-          T wgt = T(1);
-          if (odd[0]) wgt *= T(0.5);
-          if (odd[1]) wgt *= T(0.5);
-          if (odd[2]) wgt *= T(0.5);
-          const long long j = (c0[0] + dx) + gc.n[0] * ((c0[1] + dy) + (long long)gc.n[1] * (c0[2] + dz));
-          acc += wgt * src[j];
-        }
-    out[t] = acc;
-  }
-}
-
-// Restriction R = I^T: a coarse node collects the fine nodes within one fine
-// spacing, weight 1 on the coincident node and 1/2 per odd offset and axis.
-// With normalise, the sum is divided by the sum of the weights (P).
-template <class T>
-__global__ void k_restrict(Geom gc, Geom gf, int nf, const T* __restrict__ in,
-                           T* __restrict__ out, bool normalise, const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  const long long total = gc.N * nf;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int f = int(t / gc.N);
-    const long long j = t - f * gc.N;
-    const int jx = int(j % gc.n[0]);
-    const long long r = j / gc.n[0];
-    const int jy = int(r % gc.n[1]);
-    const int jz = int(r / gc.n[1]);
-    const T* src = in + f * gf.N;
-    T acc = T(0), wsum = T(0);
-    const int zlo = gf.dim == 3 ? -1 : 0, zhi = gf.dim == 3 ? 1 : 0;
-    for (int dz = zlo; dz <= zhi; ++dz) {
-      const int iz = 2 * jz + dz;
-      if (iz < 0 || iz >= gf.n[2]) continue;
-      for (int dy = -1; dy <= 1; ++dy) {
-        const int iy = 2 * jy + dy;
-        if (iy < 0 || iy >= gf.n[1]) continue;
-        for (int dx = -1; dx <= 1; ++dx) {
-          const int ix = 2 * jx + dx;
-          if (ix < 0 || ix >= gf.n[0]) continue;
-          T wgt = T(1);
-          if (dx) wgt *= T(0.5);
-          if (dy) wgt *= T(0.5);
-          if (dz) wgt *= T(0.5);
-          acc += wgt * src[ix + gf.n[0] * (iy + (long long)gf.n[1] * iz)];
-          wsum += wgt;
-        }
-      }
-    }
-    out[t] = normalise ? acc / wsum : acc;
-  }
-}
-
-__global__ void k_bounds(Geom gc, Geom gf, int nf, const double* __restrict__ lo_f,
-                         const double* __restrict__ hi_f, double* __restrict__ lo_c,
-                         double* __restrict__ hi_c) {
-  const long long total = gc.N * nf;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int f = int(t / gc.N);
-    const long long j = t - f * gc.N;
-    const int jx = int(j % gc.n[0]);
-    const long long r = j / gc.n[0];
-    const int jy = int(r % gc.n[1]);
-    const int jz = int(r / gc.n[1]);
-    double lo = -INFINITY, hi = INFINITY;
-    const int zlo = gf.dim == 3 ? -1 : 0, zhi = gf.dim == 3 ? 1 : 0;
-    for (int dz = zlo; dz <= zhi; ++dz) {
-      const int iz = 2 * jz + dz;
-      if (iz < 0 || iz >= gf.n[2]) continue;
-      for (int dy = -1; dy <= 1; ++dy) {
-        const int iy = 2 * jy + dy;
-        if (iy < 0 || iy >= gf.n[1]) continue;
-        for (int dx = -1; dx <= 1; ++dx) {
-          const int ix = 2 * jx + dx;
-          if (ix < 0 || ix >= gf.n[0]) continue;
-          const long long i = f * gf.N + ix + gf.n[0] * (iy + (long long)gf.n[1] * iz);
-          lo = fmax(lo, lo_f[i]);
-          hi = fmin(hi, hi_f[i]);
-        }
-      }
-    }
-    lo_c[t] = lo;
-    hi_c[t] = hi;
-  }
-}
-
-static int grid_for(long long n) {
-  long long b = (n + 255) / 256;
-  if (b > 8192) b = 8192;
-  if (b < 1) b = 1;
-  return int(b);
-}
-
-cudaError_t xfer_prolong(const Geom& gc, const Geom& gf, int nf, const void* in, void* out,
-                         int prec, cudaStream_t st, const int* skip) {
-  const int nb = grid_for(gf.N * nf);
-  if (prec)
-    k_prolong<float><<<nb, 256, 0, st>>>(gc, gf, nf, static_cast<const float*>(in), static_cast<float*>(out), skip);
-  else
-    k_prolong<double><<<nb, 256, 0, st>>>(gc, gf, nf, static_cast<const double*>(in), static_cast<double*>(out), skip);
-  return cudaGetLastError();
-}
-
-cudaError_t xfer_restrict(const Geom& gc, const Geom& gf, int nf, const void* in, void* out,
-                          int prec, bool normalise, cudaStream_t st, const int* skip) {
-  const int nb = grid_for(gc.N * nf);
-  if (prec)
-    k_restrict<float><<<nb, 256, 0, st>>>(gc, gf, nf, static_cast<const float*>(in), static_cast<float*>(out), normalise, skip);
-  else
-    k_restrict<double><<<nb, 256, 0, st>>>(gc, gf, nf, static_cast<const double*>(in), static_cast<double*>(out), normalise, skip);
-  return cudaGetLastError();
-}
-
-cudaError_t xfer_bounds(const Geom& gc, const Geom& gf, int nf, const double* lo_f,
-                        const double* hi_f, double* lo_c, double* hi_c, cudaStream_t st) {
-  k_bounds<<<grid_for(gc.N * nf), 256, 0, st>>>(gc, gf, nf, lo_f, hi_f, lo_c, hi_c);
   return cudaGetLastError();
 }
 
