@@ -1003,125 +1003,9 @@ cudaError_t elem_energy_df(const Geom& g, const Mat<double>& m, const double* x,
 // The lagged FP64 Hessian stored as a (3^d)-point block stencil: for node i,
 // offset o (component k of the offset = o_k - 1 in {-1, 0, 1}) and fields
 // f, g, the entry S[((o * F + f) * F + g) * N + i] couples dof (f, i) with
-// dof (g, i + offset).  Assembled from the stored Gauss-point coefficients
-// (A, M, B) of the up to 2^d elements around each node; each thread owns
-// one node's row, so the sums need no atomics.
-template <int D>
-__device__ __forceinline__ void shape_tables(int a, int q, double& na, double (&da)[D]) {
-  double n1[D];
-#pragma unroll
-  for (int k = 0; k < D; ++k) n1[k] = (((q >> k) & 1) == ((a >> k) & 1)) ? PF_XI1 : PF_XI0;
-  na = 1.0;
-#pragma unroll
-  for (int k = 0; k < D; ++k) na *= n1[k];
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    double t = ((a >> k) & 1) ? 1.0 : -1.0;  // raw derivative of the 1D factor
-#pragma unroll
-    for (int j = 0; j < D; ++j)
-      if (j != k) t *= n1[j];
-    da[k] = t;
-  }
-}
-
-// One thread per (node i, stencil offset o): the 4x4 (3x3 in 2D) block of
-// the lagged Hessian coupling node i with node i + o, summed over the corner
-// pairs (a, b = a + o) of the elements that contain both and over their
-// Gauss points.  Every entry of S is written once (no atomics, no clearing);
-// per pair the Gauss-point sum is formed first, then added to the block.
-template <int D>
-__global__ void __launch_bounds__(128) k_assemble(Geom g, Mat<double> m,
-                                                  const double* __restrict__ coef,
-                                                  double* __restrict__ S) {
-  constexpr int F = D + 1, NC = 1 << D, NCF = NCoef<D>::value, NO = D == 3 ? 27 : 9;
-  const double kc = m.w * m.Gc * m.ls * m.inv_h * m.inv_h;
-  const long long total = NO * g.N;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int o = int(t / g.N);
-    const long long i = t - (long long)o * g.N;
-    const int ix = int(i % g.n[0]);
-    const long long r = i / g.n[0];
-    const int iy = int(r % g.n[1]);
-    const int iz = int(r / g.n[1]);
-    const int ic[3] = {ix, iy, iz};
-    int dof[3] = {0, 0, 0};  // o = sum_k (d_k + 1) 3^k
-    {
-      int oo = o;
-#pragma unroll
-      for (int k = 0; k < D; ++k) {
-        dof[k] = oo % 3 - 1;
-        oo /= 3;
-      }
-    }
-    double tot[F][F];
-#pragma unroll
-    for (int f = 0; f < F; ++f)
-#pragma unroll
-      for (int h = 0; h < F; ++h) tot[f][h] = 0.0;
-    for (int a = 0; a < NC; ++a) {  // node i is corner a of element i - corner(a)
-      int ec[3] = {0, 0, 0}, b = 0;
-      bool ok = true;
-#pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const int ak = (a >> k) & 1, bk = ak + dof[k];
-        ec[k] = ic[k] - ak;
-        ok = ok && ec[k] >= 0 && ec[k] < g.ne[k] && bk >= 0 && bk <= 1;
-        b |= (bk & 1) << k;
-      }
-      if (!ok) continue;
-      const long long e = ec[0] + (long long)g.ne[0] * (ec[1] + (long long)g.ne[1] * ec[2]);
-      double blk[F][F];
-#pragma unroll
-      for (int f = 0; f < F; ++f)
-#pragma unroll
-        for (int h = 0; h < F; ++h) blk[f][h] = 0.0;
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {
-        double na, nb, da[D], db[D];
-        shape_tables<D>(a, q, na, da);
-        shape_tables<D>(b, q, nb, db);
-        const double A = coef[(q * NCF + 0) * g.NE + e];
-        const double M = coef[(q * NCF + 1) * g.NE + e];
-        double B[D][D];
-#pragma unroll
-        for (int ii = 0; ii < D; ++ii)
-#pragma unroll
-          for (int kk = 0; kk < D; ++kk) B[ii][kk] = coef[(q * NCF + 2 + sym_index<D>(ii, kk)) * g.NE + e];
-        double dd = 0.0;
-#pragma unroll
-        for (int k = 0; k < D; ++k) dd += da[k] * db[k];
-#pragma unroll
-        for (int ii = 0; ii < D; ++ii) {
-#pragma unroll
-          for (int jj = 0; jj < D; ++jj) {
-            double v = m.lam * da[ii] * db[jj] + m.mu * da[jj] * db[ii];
-            if (ii == jj) v += m.mu * dd;
-            blk[ii][jj] += A * v;
-          }
-          double bu = 0.0, bc = 0.0;
-#pragma unroll
-          for (int k = 0; k < D; ++k) {
-            bu += B[ii][k] * da[k];
-            bc += B[ii][k] * db[k];
-          }
-          blk[ii][D] += bu * nb;  // u_i(a) - c(b)
-          blk[D][ii] += na * bc;  // c(a) - u_i(b)
-        }
-        blk[D][D] += M * na * nb + kc * dd;
-      }
-#pragma unroll
-      for (int f = 0; f < F; ++f)
-#pragma unroll
-        for (int h = 0; h < F; ++h) tot[f][h] += blk[f][h];
-    }
-#pragma unroll
-    for (int f = 0; f < F; ++f)
-#pragma unroll
-      for (int h = 0; h < F; ++h) S[((long long)(o * F + f) * F + h) * g.N + i] = tot[f][h];
-  }
-}
-
+// dof (g, i + offset).  Assembled in pf_assemble.cu from the stored
+// Gauss-point coefficients (A, M, B) of the up to 2^d elements around each
+// node.
 template <int D>
 __global__ void __launch_bounds__(256) k_stencil_apply(Geom g, const double* __restrict__ S,
                                                        const double* __restrict__ v,
@@ -1300,15 +1184,6 @@ cudaError_t scaled_rowsum(const Geom& g, const double* S, double* out, cudaStrea
   const int nb = int(std::min<long long>((g.N + 127) / 128, 16LL * 1216));
   if (g.dim == 3) k_scaled_rowsum<3><<<nb, 128, 0, st>>>(g, S, out);
   else k_scaled_rowsum<2><<<nb, 128, 0, st>>>(g, S, out);
-  return cudaGetLastError();
-}
-
-cudaError_t stencil_assemble(const Geom& g, const Mat<double>& m, const double* coef, double* S,
-                             cudaStream_t st) {
-  const long long total = (g.dim == 3 ? 27LL : 9LL) * g.N;
-  const int nb = int(std::min<long long>((total + 127) / 128, 16LL * 1216));
-  if (g.dim == 3) k_assemble<3><<<nb, 128, 0, st>>>(g, m, coef, S);
-  else k_assemble<2><<<nb, 128, 0, st>>>(g, m, coef, S);
   return cudaGetLastError();
 }
 
