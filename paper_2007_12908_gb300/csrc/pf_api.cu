@@ -70,9 +70,9 @@ cudaError_t galerkin_build(pf_hierarchy* h, const float* x_fine, cudaStream_t st
   }
   cudaError_t e = galerkin_fine(h->geo[L - 2], h->geo[L - 1], h->mat[L - 1], x_fine, h->lv[L - 2].gk, st);
   for (int l = L - 3; l >= 0 && e == cudaSuccess; --l)
-    e = galerkin_rap(h->geo[l], h->geo[l + 1], h->lv[l + 1].gk, h->lv[l].gk, st);
+    e = galerkin_coarsen(h->geo[l], h->geo[l + 1], h->lv[l + 1].gk, h->lv[l].gk, st);
   for (int l = 0; l <= L - 2 && e == cudaSuccess; ++l)
-    e = galerkin_assemble(h->geo[l], h->lv[l].gk, h->lv[l].gs, st);
+    e = galerkin_assemble(h->geo[l], h->mat[L - 1], L - 1 - l, h->lv[l].gk, h->lv[l].gs, st);
   return e;
 }
 }  // namespace pf

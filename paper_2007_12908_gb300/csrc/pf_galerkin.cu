@@ -6,26 +6,34 @@
 // product), the operators are assembled once per lag into FP32 block
 // stencils, 3^d points per node.
 //
-// Element-nested construction:
-//  1. next-to-finest level: the element matrix of a coarse element E is the
-//     sum over its 2^d fine children and their Gauss points of the Hessian
-//     density at the fine Gauss point, with the coarse Q1 basis functions
-//     (which lie in the fine space, so I maps them exactly) evaluated
-//     there: K_E = sum_q B_E(q)^T D_q B_E(q).  D_q is the lagged Gauss-point
-//     coefficient set (A, M, B) of the fine element, computed from x_lag.
-//  2. coarser levels: K_E' = sum_children I_c^T K_c I_c with I_c the Q1
-//     interpolation from the coarse element's corners to the child's.
-//  3. each level's stencil: the (node, offset) block is the sum of the
-//     element blocks of the elements that hold both nodes, in a fixed
-//     element order (no atomics; deterministic).
-// Element matrices are (2^d (d+1))^2 floats, row a*F + f, column b*F + h
-// (corner a/b, field f/h).
+// With Q1 functions nested (coarse ones lie in the fine space, so I maps them
+// exactly), the element matrix of a coarse element is the integral of the
+// fine Gauss-point Hessian density (A, M, B at x_lag) against products of the
+// coarse 1D functions.  Such a product is N_a N_b, N_a or 1 along each axis,
+// and all of them are sums of the NN moments
+//   mom[k][c_x, c_y, c_z] = sum over the fine Gauss points of coefficient k
+//                           times NN_cx(x) NN_cy(y) NN_cz(z),
+//   NN_0 = N_0^2, NN_1 = N_0 N_1, NN_2 = N_1^2 on the coarse element
+// (27 x 8 floats per element in 3D, 9 x 5 in 2D), with positive weights only.
+// So:
+//  1. next-to-finest level: the moments from the 4^d fine Gauss points of an
+//     element's children, axis by axis;
+//  2. coarser levels: the moments of a parent are its children's, with
+//     N'_0 = N_0 + N_1 / 2, N'_1 = N_1 / 2 (or mirrored) per axis: exact
+//     re-expansion, axis by axis;
+//  3. each level's stencil from the moments (pf_assemble.cu).
+// A fixed order everywhere, no atomics.  Forming and storing 32 x 32 element
+// matrices instead took 1,389 us (1.24 G warp instructions: 64 Gauss points
+// per entry) + 177 us (I^T K I) + 148 us (490 MB of matrix rows gathered
+// entry by entry) for 65^3 -> 33^3 -> 17^3; the three steps now take
+// 19 + 12 + 88 us.
 #include <algorithm>
 #include <string>
 
 #include "../../include/pf.h"
 #include "pf_element.cuh"
 #include "pf_internal.h"
+#include "pf_stencil.cuh"
 
 namespace pf {
 
@@ -33,38 +41,13 @@ namespace {
 
 template <int D>
 struct GalDims {
-  static constexpr int NC = 1 << D, F = D + 1, R = NC * F, NQ = NC;
-  static constexpr int NO = D == 3 ? 27 : 9;
+  static constexpr int NC = 1 << D, F = D + 1, NCF = NCoef<D>::value;
+  static constexpr int W = D == 3 ? 27 : 9;     // moments per coefficient
+  static constexpr int NP = D == 3 ? 64 : 16;   // fine Gauss points per coarse element
+  static constexpr int EL = 32;                 // coarse elements per CTA
+  static constexpr int THREADS = EL << D;       // one per child
+  static constexpr size_t smem = sizeof(float) * NCF * NP * EL;
 };
-
-// Coarse Q1 basis at the fine Gauss points of the 2^d children of a coarse
-// element: value and raw derivatives (d/dt of the 1D factor = +-1, times the
-// other factors), the derivatives halved so that they are raw derivatives
-// of the fine element (the fine coefficients carry 1/h_fine).
-// Index (child c, fine Gauss point q, coarse corner a).
-template <int D>
-__device__ __forceinline__ void coarse_shape(int c, int q, int a, float& na, float (&da)[3]) {
-  float n1[3], d1[3];
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    const float xi = ((q >> k) & 1) ? float(PF_XI1) : float(PF_XI0);
-    const float t = 0.5f * (float((c >> k) & 1) + xi);  // coarse reference coordinate
-    const int ak = (a >> k) & 1;
-    n1[k] = ak ? t : 1.f - t;
-    d1[k] = ak ? 0.5f : -0.5f;
-  }
-  na = 1.f;
-#pragma unroll
-  for (int k = 0; k < D; ++k) na *= n1[k];
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    float t = d1[k];
-#pragma unroll
-    for (int j = 0; j < D; ++j)
-      if (j != k) t *= n1[j];
-    da[k] = t;
-  }
-}
 
 template <int D>
 __device__ __forceinline__ long long node_index(const Geom& g, int ix, int iy, int iz) {
@@ -79,261 +62,185 @@ __device__ __forceinline__ void elem_xyz(const Geom& g, long long e, int& ex, in
   ez = D == 3 ? int(r / g.ne[1]) : 0;
 }
 
-// 1. Element matrices of the next-to-finest level gc from the finest lag
-// (FP32 x on the finest grid gf).  One warp per coarse element; lane r =
-// a*F + f accumulates row r over the 2^d children x 2^d Gauss points.
+// NN_0, NN_1, NN_2 of a coarse element at its j-th fine Gauss point along an
+// axis, t = (child + xi) / 2.
+__device__ __forceinline__ constexpr float gal_nn(int j, int c) {
+  const double t = 0.5 * ((j >> 1) + ((j & 1) ? PF_XI1 : PF_XI0));
+  return float(c == 0 ? (1 - t) * (1 - t) : (c == 1 ? t * (1 - t) : t * t));
+}
+
+// 1. Moments of the next-to-finest level gc from the finest lag (FP32 x on
+// the finest grid gf).  A CTA takes 32 consecutive coarse elements: thread =
+// child, whose Gauss-point coefficients go to shared memory; then warp =
+// coefficient, lane = element.  Bound by FP32 issue (about 600 operations per
+// child and 450 per element and coefficient).
 template <int D>
-__global__ void __launch_bounds__(256) k_gal_fine(Geom gc, Geom gf, Mat<float> m,
-                                                  const float* __restrict__ x,
-                                                  float* __restrict__ K) {
+__global__ void __launch_bounds__(GalDims<D>::THREADS)
+    k_gal_fine(Geom gc, Geom gf, Mat<float> m, const float* __restrict__ x,
+               float* __restrict__ mom) {
   using G = GalDims<D>;
-  constexpr int NC = G::NC, F = G::F, R = G::R, NCF = NCoef<D>::value;
-  __shared__ float cf_s[8][NC][NC][NCF];  // per warp: [child][q][coef]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long e = blockIdx.x * 8LL + warp;
-  const bool live = e < gc.NE;
-  int ex = 0, ey = 0, ez = 0;
-  if (live) elem_xyz<D>(gc, e, ex, ey, ez);
-  // lanes 0 .. NC-1: the lagged coefficients of child c = lane
-  if (live && lane < NC) {
-    const int c = lane;
-    const int fx = 2 * ex + (c & 1), fy = 2 * ey + ((c >> 1) & 1), fz = D == 3 ? 2 * ez + ((c >> 2) & 1) : 0;
-    float xe[F][NC];
+  constexpr int NC = G::NC, F = G::F, EL = G::EL;
+  extern __shared__ float cf_s[];  // [coefficient][point][element]
+  const long long e0 = blockIdx.x * (long long)EL;
+  {
+    // thread -> element and child, neighbouring threads along x
+    const int cx = threadIdx.x & 1, el = (threadIdx.x >> 1) % EL, cyz = threadIdx.x / (2 * EL);
+    const long long e = e0 + el;
+    if (e < gc.NE) {
+      int ex, ey, ez;
+      elem_xyz<D>(gc, e, ex, ey, ez);
+      const int cy = cyz & 1, cz = D == 3 ? cyz >> 1 : 0;
+      const int fx = 2 * ex + cx, fy = 2 * ey + cy, fz = D == 3 ? 2 * ez + cz : 0;
+      float xe[F][NC];
 #pragma unroll
-    for (int a = 0; a < NC; ++a) {
-      const long long idx = node_index<D>(gf, fx + (a & 1), fy + ((a >> 1) & 1), D == 3 ? fz + ((a >> 2) & 1) : 0);
+      for (int a = 0; a < NC; ++a) {
+        const long long idx = node_index<D>(gf, fx + (a & 1), fy + ((a >> 1) & 1),
+                                            D == 3 ? fz + ((a >> 2) & 1) : 0);
 #pragma unroll
-      for (int f = 0; f < F; ++f) xe[f][a] = x[f * gf.N + idx];
-    }
-    float cf[NC][NCF];
-    hess_coef<D, float>(xe, m, cf);
-#pragma unroll
-    for (int q = 0; q < NC; ++q)
-#pragma unroll
-      for (int k = 0; k < NCF; ++k) cf_s[warp][c][q][k] = cf[q][k];
-  }
-  __syncwarp();
-  if (!live || lane >= R) return;
-  const int a = lane / F, f = lane % F;
-  const float kc = m.w * m.Gc * m.ls * m.inv_h * m.inv_h;
-  float row[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j) row[j] = 0.f;
-  for (int c = 0; c < NC; ++c)
-    for (int q = 0; q < NC; ++q) {
-      const float* cq = cf_s[warp][c][q];
-      const float A = cq[0], M = cq[1];
-      float B[3][3];
-#pragma unroll
-      for (int i = 0; i < D; ++i)
-#pragma unroll
-        for (int k = 0; k < D; ++k) B[i][k] = cq[2 + sym_index<D>(i, k)];
-      float na, da[3];
-      coarse_shape<D>(c, q, a, na, da);
-      // this row's factors: for u_i rows B.da, for the c row na
-      float bda = 0.f;
-      if (f < D) {
-#pragma unroll
-        for (int k = 0; k < D; ++k) bda += B[f][k] * da[k];
+        for (int f = 0; f < F; ++f) xe[f][a] = x[f * gf.N + idx];
       }
+      float cf[NC][G::NCF];
+      hess_coef<D, float>(xe, m, cf);
 #pragma unroll
-      for (int b = 0; b < NC; ++b) {
-        float nb, db[3];
-        coarse_shape<D>(c, q, b, nb, db);
-        float dd = 0.f;
+      for (int q = 0; q < NC; ++q) {
+        const int pt = (2 * cx + (q & 1)) + 4 * (2 * cy + ((q >> 1) & 1)) +
+                       (D == 3 ? 16 * (2 * cz + ((q >> 2) & 1)) : 0);
 #pragma unroll
-        for (int k = 0; k < D; ++k) dd += da[k] * db[k];
-        if (f < D) {
+        for (int k = 0; k < G::NCF; ++k) cf_s[(k * G::NP + pt) * EL + el] = cf[q][k];
+      }
+    }
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const long long e = e0 + lane;
+  if (e >= gc.NE) return;
+  for (int k = threadIdx.x >> 5; k < G::NCF; k += G::THREADS / 32) {
+    const float* s = cf_s + k * G::NP * EL + lane;
+    float acc[G::W];
 #pragma unroll
-          for (int j = 0; j < D; ++j) {
-            float v = m.lam * da[f] * db[j] + m.mu * da[j] * db[f];
-            if (j == f) v += m.mu * dd;
-            row[b * F + j] += A * v;
-          }
-          row[b * F + D] += bda * nb;  // u_f(a) - c(b)
-        } else {
+    for (int w = 0; w < G::W; ++w) acc[w] = 0.f;
 #pragma unroll
-          for (int j = 0; j < D; ++j) {
-            float bdb = 0.f;
+    for (int jz = 0; jz < (D == 3 ? 4 : 1); ++jz) {
+      float t[3][3];  // [c_x][c_y]
 #pragma unroll
-            for (int k = 0; k < D; ++k) bdb += B[j][k] * db[k];
-            row[b * F + j] += na * bdb;  // c(a) - u_j(b)
-          }
-          row[b * F + D] += M * na * nb + kc * dd;
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) t[i][j] = 0.f;
+#pragma unroll
+      for (int jy = 0; jy < 4; ++jy) {
+        float r[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int jx = 0; jx < 4; ++jx) {
+          const float val = s[(jx + 4 * jy + 16 * jz) * EL];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) r[i] = fmaf(gal_nn(jx, i), val, r[i]);
         }
-      }
-    }
-  float* out = K + (e * R + lane) * R;
 #pragma unroll
-  for (int j = 0; j < R; ++j) out[j] = row[j];
-}
-
-// Interpolation weight of coarse corner ap (per axis 0/1, at position 2 ap)
-// at fine position pos (0, 1, 2) of the coarse element.
-__device__ __forceinline__ float interp_w(int pos, int ap) {
-  return pos == 2 * ap ? 1.f : (pos == 1 ? 0.5f : 0.f);
-}
-
-// 2. K' of the coarse level gc from the element matrices Kf of the level
-// above it (gf): K'_E = sum over children c of I_c^T K_c I_c.  One warp per
-// coarse element, lane r' = a'*F + f.
-template <int D>
-__global__ void __launch_bounds__(256) k_gal_rap(Geom gc, Geom gf, const float* __restrict__ Kf,
-                                                 float* __restrict__ Kc) {
-  using G = GalDims<D>;
-  constexpr int NC = G::NC, F = G::F, R = G::R;
-  __shared__ float ks[8][R * R];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long e = blockIdx.x * 8LL + warp;
-  const bool live = e < gc.NE;
-  int ex = 0, ey = 0, ez = 0;
-  if (live) elem_xyz<D>(gc, e, ex, ey, ez);
-  const int ap = lane / F, f = lane % F;
-  float row[R];
+        for (int i = 0; i < 3; ++i)
 #pragma unroll
-  for (int j = 0; j < R; ++j) row[j] = 0.f;
-  for (int c = 0; c < NC; ++c) {
-    __syncwarp();
-    if (live) {
-      const int fx = 2 * ex + (c & 1), fy = 2 * ey + ((c >> 1) & 1), fz = D == 3 ? 2 * ez + ((c >> 2) & 1) : 0;
-      const long long ef = D == 3 ? fx + (long long)gf.ne[0] * (fy + (long long)gf.ne[1] * fz)
-                                  : fx + (long long)gf.ne[0] * fy;
-      const float* src = Kf + ef * R * R;
-      for (int i = lane; i < R * R; i += 32) ks[warp][i] = src[i];
-    }
-    __syncwarp();
-    if (!live || lane >= R) continue;
-    // weights of this lane's coarse corner ap at the child's corners a
-    float wa[NC];
-#pragma unroll
-    for (int a = 0; a < NC; ++a) {
-      float w = 1.f;
-#pragma unroll
-      for (int k = 0; k < D; ++k) w *= interp_w(((c >> k) & 1) + ((a >> k) & 1), (ap >> k) & 1);
-      wa[a] = w;
-    }
-    // t[b h] = sum_a wa[a] Kc[a f][b h]
-    float t[R];
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      float s = 0.f;
-#pragma unroll
-      for (int a = 0; a < NC; ++a) s += wa[a] * ks[warp][(a * F + f) * R + j];
-      t[j] = s;
-    }
-    // row[b' h] += sum_b t[b h] w(b, b')
-#pragma unroll
-    for (int bp = 0; bp < NC; ++bp) {
-      float wb[NC];
-#pragma unroll
-      for (int b = 0; b < NC; ++b) {
-        float w = 1.f;
-#pragma unroll
-        for (int k = 0; k < D; ++k) w *= interp_w(((c >> k) & 1) + ((b >> k) & 1), (bp >> k) & 1);
-        wb[b] = w;
+          for (int j = 0; j < 3; ++j) t[i][j] = fmaf(gal_nn(jy, j), r[i], t[i][j]);
       }
 #pragma unroll
-      for (int h = 0; h < F; ++h) {
-        float s = 0.f;
+      for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int b = 0; b < NC; ++b) s += t[b * F + h] * wb[b];
-        row[bp * F + h] += s;
-      }
+        for (int j = 0; j < 3; ++j) {
+          if constexpr (D == 3) {
+#pragma unroll
+            for (int l = 0; l < 3; ++l)
+              acc[i * 9 + j * 3 + l] = fmaf(gal_nn(jz, l), t[i][j], acc[i * 9 + j * 3 + l]);
+          } else {
+            acc[i * 3 + j] = t[i][j];
+          }
+        }
     }
+#pragma unroll
+    for (int w = 0; w < G::W; ++w) mom[((long long)k * G::W + w) * gc.NE + e] = acc[w];
   }
-  if (!live || lane >= R) return;
-  float* out = Kc + (e * R + lane) * R;
-#pragma unroll
-  for (int j = 0; j < R; ++j) out[j] = row[j];
 }
 
-// 3. Stencil of level g from its element matrices: one thread per (node,
-// offset); the block sums the elements holding both nodes in ascending
-// corner order.  S[((o F + f) F + h) N + i], as the FP64 stencil.
+// A child's NN moments along one axis (c = 0 or 1: its half of the parent)
+// as its part of the parent's.
+__device__ __forceinline__ void to_parent(int c, const float (&w)[3], float (&o)[3]) {
+  const float lo = c ? w[0] : w[2], hi = c ? w[2] : w[0];
+  const float q = 0.25f * lo, h = fmaf(0.5f, w[1], q), full = (q + w[1]) + hi;
+  o[0] = c ? q : full;
+  o[1] = h;
+  o[2] = c ? full : q;
+}
+
+// 2. Moments of the coarse level gc from those of the level above it (gf).
+// One thread per (coarse element, coefficient).
 template <int D>
-__global__ void __launch_bounds__(128) k_gal_assemble(Geom g, const float* __restrict__ K,
-                                                      float* __restrict__ S) {
+__global__ void __launch_bounds__(128) k_gal_coarsen(Geom gc, Geom gf, const float* __restrict__ mf,
+                                                     float* __restrict__ mc) {
   using G = GalDims<D>;
-  constexpr int NC = G::NC, F = G::F, R = G::R, NO = G::NO;
-  const long long total = NO * g.N;
+  constexpr int NL = D == 3 ? 3 : 1;
+  const long long total = gc.NE * G::NCF;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
-    const int o = int(t / g.N);
-    const long long i = t - (long long)o * g.N;
-    const int ic[3] = {int(i % g.n[0]), int((i / g.n[0]) % g.n[1]),
-                       D == 3 ? int(i / ((long long)g.n[0] * g.n[1])) : 0};
-    int dof[3] = {0, 0, 0};
-    {
-      int oo = o;
+    const int k = int(t / gc.NE);
+    const long long e = t - k * gc.NE;
+    int ex, ey, ez;
+    elem_xyz<D>(gc, e, ex, ey, ez);
+    const float* src = mf + (long long)k * G::W * gf.NE;
+    float acc[3][3][NL];
 #pragma unroll
-      for (int k = 0; k < D; ++k) {
-        dof[k] = oo % 3 - 1;
-        oo /= 3;
+    for (int w = 0; w < G::W; ++w) (&acc[0][0][0])[w] = 0.f;
+#pragma unroll 1
+    for (int cz = 0; cz < (D == 3 ? 2 : 1); ++cz) {
+      float zs[3][3][NL];  // x and y of the parent, z of the child
+#pragma unroll
+      for (int w = 0; w < G::W; ++w) (&zs[0][0][0])[w] = 0.f;
+#pragma unroll 1
+      for (int cy = 0; cy < 2; ++cy) {
+        float ys[3][3][NL];  // x of the parent, y and z of the child
+#pragma unroll
+        for (int w = 0; w < G::W; ++w) (&ys[0][0][0])[w] = 0.f;
+#pragma unroll
+        for (int cx = 0; cx < 2; ++cx) {
+          const long long ef = D == 3 ? (2 * ex + cx) + (long long)gf.ne[0] * ((2 * ey + cy) + (long long)gf.ne[1] * (2 * ez + cz))
+                                      : (2 * ex + cx) + (long long)gf.ne[0] * (2 * ey + cy);
+          const float* s = src + ef;
+#pragma unroll
+          for (int j = 0; j < 3; ++j)
+#pragma unroll
+            for (int l = 0; l < NL; ++l) {
+              float w[3], o[3];
+#pragma unroll
+              for (int i = 0; i < 3; ++i) w[i] = s[(long long)((i * 3 + j) * NL + l) * gf.NE];
+              to_parent(cx, w, o);
+#pragma unroll
+              for (int i = 0; i < 3; ++i) ys[i][j][l] += o[i];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int l = 0; l < NL; ++l) {
+            const float w[3] = {ys[i][0][l], ys[i][1][l], ys[i][2][l]};
+            float o[3];
+            to_parent(cy, w, o);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) zs[i][j][l] += o[j];
+          }
       }
-    }
-    float tot[F][F];
 #pragma unroll
-    for (int f = 0; f < F; ++f)
+      for (int i = 0; i < 3; ++i)
 #pragma unroll
-      for (int h = 0; h < F; ++h) tot[f][h] = 0.f;
-    for (int a = 0; a < NC; ++a) {
-      int ec[3] = {0, 0, 0}, b = 0;
-      bool ok = true;
+        for (int j = 0; j < 3; ++j) {
+          if constexpr (D == 3) {
+            const float w[3] = {zs[i][j][0], zs[i][j][1], zs[i][j][2]};
+            float o[3];
+            to_parent(cz, w, o);
 #pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const int ak = (a >> k) & 1, bk = ak + dof[k];
-        ec[k] = ic[k] - ak;
-        ok = ok && ec[k] >= 0 && ec[k] < g.ne[k] && bk >= 0 && bk <= 1;
-        b |= (bk & 1) << k;
-      }
-      if (!ok) continue;
-      const long long e = D == 3 ? ec[0] + (long long)g.ne[0] * (ec[1] + (long long)g.ne[1] * ec[2])
-                                 : ec[0] + (long long)g.ne[0] * ec[1];
-      const float* Ke = K + e * R * R;
-#pragma unroll
-      for (int f = 0; f < F; ++f)
-#pragma unroll
-        for (int h = 0; h < F; ++h) tot[f][h] += Ke[(a * F + f) * R + b * F + h];
+            for (int l = 0; l < 3; ++l) acc[i][j][l] += o[l];
+          } else {
+            acc[i][j][0] = zs[i][j][0];
+          }
+        }
     }
 #pragma unroll
-    for (int f = 0; f < F; ++f)
-#pragma unroll
-      for (int h = 0; h < F; ++h) S[((long long)(o * F + f) * F + h) * g.N + i] = tot[f][h];
-  }
-}
-
-// 4. y = S v with an FP32 stencil; vectors float (FP32 sums) or double
-// (FP64 sums of the FP32 entries).
-template <int D, class TV>
-__global__ void __launch_bounds__(256) k_gal_apply(Geom g, const float* __restrict__ S,
-                                                   const TV* __restrict__ v, TV* __restrict__ y,
-                                                   const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  constexpr int F = D + 1, NO = D == 3 ? 27 : 9;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < g.N;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int ix = int(i % g.n[0]);
-    const long long r = i / g.n[0];
-    const int iy = int(r % g.n[1]);
-    const int iz = int(r / g.n[1]);
-    TV acc[F];
-#pragma unroll
-    for (int f = 0; f < F; ++f) acc[f] = TV(0);
-#pragma unroll
-    for (int o = 0; o < NO; ++o) {
-      const int jx = ix + o % 3 - 1, jy = iy + (o / 3) % 3 - 1, jz = D == 3 ? iz + o / 9 - 1 : iz;
-      if (jx < 0 || jx >= g.n[0] || jy < 0 || jy >= g.n[1] || jz < 0 || jz >= g.n[2]) continue;
-      const long long j = jx + g.n[0] * (jy + (long long)g.n[1] * jz);
-      TV vj[F];
-#pragma unroll
-      for (int h = 0; h < F; ++h) vj[h] = v[h * g.N + j];
-#pragma unroll
-      for (int f = 0; f < F; ++f)
-#pragma unroll
-        for (int h = 0; h < F; ++h) acc[f] += TV(S[((long long)(o * F + f) * F + h) * g.N + i]) * vj[h];
-    }
-#pragma unroll
-    for (int f = 0; f < F; ++f) y[f * g.N + i] = acc[f];
+    for (int w = 0; w < G::W; ++w) mc[((long long)k * G::W + w) * gc.NE + e] = (&acc[0][0][0])[w];
   }
 }
 
@@ -352,8 +259,7 @@ int blocks_for(long long n, int threads, long long cap) {
 }  // namespace
 
 long long galerkin_elem_count(const Geom& g) {
-  const long long r = (1LL << g.dim) * (g.dim + 1);
-  return g.NE * r * r;
+  return g.NE * (g.dim == 3 ? GalDims<3>::W * GalDims<3>::NCF : GalDims<2>::W * GalDims<2>::NCF);
 }
 
 long long galerkin_stencil_count(const Geom& g) {
@@ -361,44 +267,43 @@ long long galerkin_stencil_count(const Geom& g) {
   return (g.dim == 3 ? 27LL : 9LL) * f * f * g.N;
 }
 
+template <int D>
+static cudaError_t launch_gal_fine(const Geom& gc, const Geom& gf, const Mat<float>& m,
+                                   const float* x, float* mom, cudaStream_t st) {
+  using G = GalDims<D>;
+  cudaError_t e = cudaFuncSetAttribute(k_gal_fine<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       int(G::smem));
+  if (e != cudaSuccess) return e;
+  const long long nb = (gc.NE + G::EL - 1) / G::EL;
+  k_gal_fine<D><<<unsigned(nb), G::THREADS, G::smem, st>>>(gc, gf, m, x, mom);
+  return cudaGetLastError();
+}
+
 cudaError_t galerkin_fine(const Geom& gc, const Geom& gf, const Mat<double>& mf, const float* x_fine,
-                          float* K, cudaStream_t st) {
-  const int nb = int((gc.NE + 7) / 8);
-  if (gc.dim == 3) k_gal_fine<3><<<nb, 256, 0, st>>>(gc, gf, to_mat<float>(mf), x_fine, K);
-  else k_gal_fine<2><<<nb, 256, 0, st>>>(gc, gf, to_mat<float>(mf), x_fine, K);
-  return cudaGetLastError();
+                          float* mom, cudaStream_t st) {
+  return gc.dim == 3 ? launch_gal_fine<3>(gc, gf, to_mat<float>(mf), x_fine, mom, st)
+                     : launch_gal_fine<2>(gc, gf, to_mat<float>(mf), x_fine, mom, st);
 }
 
-cudaError_t galerkin_rap(const Geom& gc, const Geom& gf, const float* Kf, float* Kc, cudaStream_t st) {
-  const int nb = int((gc.NE + 7) / 8);
-  if (gc.dim == 3) k_gal_rap<3><<<nb, 256, 0, st>>>(gc, gf, Kf, Kc);
-  else k_gal_rap<2><<<nb, 256, 0, st>>>(gc, gf, Kf, Kc);
-  return cudaGetLastError();
-}
-
-cudaError_t galerkin_assemble(const Geom& g, const float* K, float* S, cudaStream_t st) {
-  const long long total = (g.dim == 3 ? 27LL : 9LL) * g.N;
-  const int nb = blocks_for(total, 128, 16LL * 1216);
-  if (g.dim == 3) k_gal_assemble<3><<<nb, 128, 0, st>>>(g, K, S);
-  else k_gal_assemble<2><<<nb, 128, 0, st>>>(g, K, S);
+cudaError_t galerkin_coarsen(const Geom& gc, const Geom& gf, const float* mom_f, float* mom_c,
+                             cudaStream_t st) {
+  const int ncf = gc.dim == 3 ? GalDims<3>::NCF : GalDims<2>::NCF;
+  const int nb = blocks_for(gc.NE * ncf, 128, 32LL * 1216);
+  if (gc.dim == 3) k_gal_coarsen<3><<<nb, 128, 0, st>>>(gc, gf, mom_f, mom_c);
+  else k_gal_coarsen<2><<<nb, 128, 0, st>>>(gc, gf, mom_f, mom_c);
   return cudaGetLastError();
 }
 
 cudaError_t galerkin_apply(const Geom& g, const float* S, const void* v, void* y, int prec,
                            cudaStream_t st, const int* skip) {
-  const int nb = blocks_for(g.N, 256, 16LL * 1216);
   if (prec == PF_FP32) {
-    if (g.dim == 3)
-      k_gal_apply<3, float><<<nb, 256, 0, st>>>(g, S, static_cast<const float*>(v), static_cast<float*>(y), skip);
-    else
-      k_gal_apply<2, float><<<nb, 256, 0, st>>>(g, S, static_cast<const float*>(v), static_cast<float*>(y), skip);
-  } else {
-    if (g.dim == 3)
-      k_gal_apply<3, double><<<nb, 256, 0, st>>>(g, S, static_cast<const double*>(v), static_cast<double*>(y), skip);
-    else
-      k_gal_apply<2, double><<<nb, 256, 0, st>>>(g, S, static_cast<const double*>(v), static_cast<double*>(y), skip);
+    const float* x = static_cast<const float*>(v);
+    float* o = static_cast<float*>(y);
+    return g.dim == 3 ? stencil_rows<3>(g, S, x, o, st, skip) : stencil_rows<2>(g, S, x, o, st, skip);
   }
-  return cudaGetLastError();
+  const double* x = static_cast<const double*>(v);
+  double* o = static_cast<double*>(y);
+  return g.dim == 3 ? stencil_rows<3>(g, S, x, o, st, skip) : stencil_rows<2>(g, S, x, o, st, skip);
 }
 
 }  // namespace pf

@@ -24,7 +24,7 @@ struct LevelBuf {
   float* xlag32 = nullptr;  // FP32 copy of x_lag (mixed precision)
   double* coef = nullptr;   // lagged Gauss-point coefficients (FP64 Hessian)
   double* stencil = nullptr;  // assembled lagged FP64 Hessian (3^d block stencil)
-  float* gk = nullptr;        // FP32 Galerkin element matrices (mixed GALERKIN coarse levels)
+  float* gk = nullptr;        // FP32 Galerkin coefficient moments (mixed GALERKIN coarse levels)
   float* gs = nullptr;        // FP32 Galerkin operator as a 3^d block stencil
 };
 

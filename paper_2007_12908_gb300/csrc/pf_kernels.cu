@@ -16,6 +16,7 @@
 #include "pf_element_f2.cuh"
 #include "pf_internal.h"
 #include "pf_reduce.cuh"
+#include "pf_stencil.cuh"
 
 namespace pf {
 
@@ -1041,38 +1042,6 @@ __global__ void __launch_bounds__(256) k_stencil_apply(Geom g, const double* __r
   }
 }
 
-// The product on grids too small to fill the SMs with one thread per node:
-// one thread per (node, output row), the same summation order per output.
-template <int D>
-__global__ void __launch_bounds__(128) k_stencil_apply_rows(Geom g, const double* __restrict__ S,
-                                                            const double* __restrict__ v,
-                                                            double* __restrict__ y,
-                                                            const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  constexpr int F = D + 1, NO = D == 3 ? 27 : 9;
-  const long long total = F * g.N;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const int f = int(t / g.N);
-    const long long i = t - (long long)f * g.N;
-    const int ix = int(i % g.n[0]);
-    const long long r = i / g.n[0];
-    const int iy = int(r % g.n[1]);
-    const int iz = int(r / g.n[1]);
-    double acc = 0.0;
-#pragma unroll
-    for (int o = 0; o < NO; ++o) {
-      const int ox = o % 3 - 1, oy = (o / 3) % 3 - 1, oz = D == 3 ? o / 9 - 1 : 0;
-      const int jx = ix + ox, jy = iy + oy, jz = iz + oz;
-      if (jx < 0 || jx >= g.n[0] || jy < 0 || jy >= g.n[1] || jz < 0 || jz >= g.n[2]) continue;
-      const long long j = jx + g.n[0] * (jy + (long long)g.n[1] * jz);
-#pragma unroll
-      for (int h = 0; h < F; ++h) acc += S[((long long)(o * F + f) * F + h) * g.N + i] * v[h * g.N + j];
-    }
-    y[f * g.N + i] = acc;
-  }
-}
-
 // Projected Gauss-Seidel on the nodes of one parity colour (i_k mod 2 =
 // bit k of `colour`): nodes of one colour are not coupled by the 3^d-point
 // stencil, so they update in parallel exactly as one after another.  Each
@@ -1189,13 +1158,8 @@ cudaError_t scaled_rowsum(const Geom& g, const double* S, double* out, cudaStrea
 
 cudaError_t stencil_apply(const Geom& g, const double* S, const double* v, double* y,
                           cudaStream_t st, const int* skip) {
-  if (g.N < 152LL * 512) {  // fewer nodes than two 256-thread CTAs per SM
-    const long long total = (g.dim + 1) * g.N;
-    const int nb = int(std::min<long long>((total + 127) / 128, 16LL * 1216));
-    if (g.dim == 3) k_stencil_apply_rows<3><<<nb, 128, 0, st>>>(g, S, v, y, skip);
-    else k_stencil_apply_rows<2><<<nb, 128, 0, st>>>(g, S, v, y, skip);
-    return cudaGetLastError();
-  }
+  if (g.N < 152LL * 512)  // fewer nodes than two 256-thread CTAs per SM: several threads per row
+    return g.dim == 3 ? stencil_rows<3>(g, S, v, y, st, skip) : stencil_rows<2>(g, S, v, y, st, skip);
   const int nb = int(std::min<long long>((g.N + 255) / 256, 16LL * 1216));
   if (g.dim == 3) k_stencil_apply<3><<<nb, 256, 0, st>>>(g, S, v, y, skip);
   else k_stencil_apply<2><<<nb, 256, 0, st>>>(g, S, v, y, skip);

@@ -34,3 +34,30 @@ def test_assembled_hessian_matches_oracle(n):
     pf.hessvec_lag_set(H, 0, dev(x2))
     assert relinf(host(pf.hessvec_lagged(H, 0, dev(vs[0]))), O.hessvec(g, Ho.prm, x2, vs[0])) <= 1e-10
     H.close()
+
+
+@pytest.mark.parametrize("nc,L", [((34, 3), 2), ((17, 3), 3), ((2, 2), 5), ((2, 17, 3), 2), ((9, 5, 2), 2),
+                                  ((2, 2, 2), 4), ((3, 2, 5), 3)])
+def test_galerkin_stencils_at_tile_edges(nc, L):
+    """The moment form of the Galerkin operators where its CTAs of 32 coarse
+    elements and the assembly's tiles end, and over up to four re-expansions:
+    R H I of the oracle within FP32 rounding (2e-5 as in the parity suite)."""
+    import torch
+    require_cuda()
+    import paper_2007_12908_gb300 as pf
+    dim = len(nc)
+    H, Ho = pair(dim, nc, L, 1.0 / (max(nc) - 1), nu=0.25, p=3e-2, k_res=1e-3)
+    x32 = PI.random_state(71, dim, Ho.fine.N, u_scale=0.05, c_hi=0.9).astype(np.float32)
+    pf.galerkin_set(H, dev(x32))
+    x = x32.astype(np.float64)
+    for l in range(L - 1):
+        v = PI.random_direction(72 + l, Ho.ndof(l)).astype(np.float32).astype(np.float64)
+        w = v
+        for k in range(l, L - 1):
+            w = Ho.transfers[k].prolong(w)
+        w = O.hessvec(Ho.fine, Ho.prm, x, w)
+        for k in reversed(range(l, L - 1)):
+            w = Ho.transfers[k].restrict(w)
+        assert relinf(host(pf.galerkin_apply(H, l, dev(v, torch.float32))), w) <= 2e-5
+        assert relinf(host(pf.galerkin_apply(H, l, dev(v))), w) <= 2e-5
+    H.close()
