@@ -4,16 +4,31 @@
 // weights and Adam moments.  Every convolution (forward, data gradient,
 // weight gradient) is an implicit GEMM on the tensor cores with BF16
 // operands and FP32 accumulation; the data-gradient and weight-gradient
-// operand dL/d(out) (FP32) is staged as a BF16 pair hi + lo and multiplied
+// operand dL/d(out) (FP32) is split into a BF16 pair hi + lo and multiplied
 // twice, keeping about 16 significant bits of the gradient.
 //
-// Convolutions read their input through a fused transform: the first
-// operand may be pooled (it lives at twice the resolution) or upsampled (it
-// lives at half the resolution), and a second operand (the encoder skip) is
-// concatenated after it, so neither the pooled, the upsampled nor the
-// concatenated tensor is ever stored.
+// Layout.  Activations are channel-innermost ([y][x][channel], channels
+// padded to 16 with zeros), so that 16 channels of a pixel are two 16-byte
+// cp.async pieces and an ldmatrix row is 8 channels of any pixel: a tap is a
+// shift of row addresses.  With channel planes every operand word was two
+// scalar loads with the pooling, upsampling or concatenation worked out per
+// value, and the tensor pipe was 4-9 % busy; now it is 40-60 % busy on the
+// large layers (of what mma.sync can issue).  Forward and backward:
+//   1032^2  1.92 -> 0.44 ms and  9.19 -> 1.61 ms
+//    136^2   604 ->   66 us and  1183 ->  271 us (latency of 16 and 45
+//                                                launches in sequence)
+// The input transforms need no passes of their own:
+//  - the second convolution of an encoder level also writes the 2x2 average
+//    the next level reads (a thread holds both rows of a pixel pair);
+//  - nearest upsampling and the skip concatenation are source addresses.
+// The backward pass stores no FP32 gradient but those of the skips: a data
+// gradient's epilogue applies the adjoint of the input transform in FP32
+// (with the skip's gradient where there is one), masks by the ReLU of the
+// layer below, adds that layer's bias gradient and writes the hi + lo pair
+// the next two products read.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -29,44 +44,44 @@ using namespace pf;
 
 namespace {
 
-enum { IN_PLAIN = 0, IN_POOL = 1, IN_UP = 2 };
+typedef __nv_bfloat16 bf16;
+typedef __nv_bfloat162 bf162;
 
-struct ConvIn {
-  const __nv_bfloat16* a;  // first operand (ca channels)
-  int ca, mode;            // mode: IN_PLAIN / IN_POOL / IN_UP
-  const __nv_bfloat16* b;  // concatenated operand (cb channels, same resolution), or null
+// Input of a convolution on an H x W grid: channels [0, ca) from a (at half
+// the resolution with up), then [ca, ca + cb) from b; both padded to 16.
+struct ConvSrc {
+  const bf16* a;
+  int ca, up;
+  const bf16* b;
   int cb;
 };
 
-// value of input channel c at (y, x) of the conv's H x W grid (0 outside)
-__device__ __forceinline__ float conv_in(const ConvIn& in, int c, int y, int x, int H, int W) {
-  if (y < 0 || y >= H || x < 0 || x >= W) return 0.f;
-  if (c < in.ca) {
-    if (in.mode == IN_PLAIN) return __bfloat162float(in.a[((long long)c * H + y) * W + x]);
-    if (in.mode == IN_POOL) {
-      const int W2 = 2 * W;
-      const __nv_bfloat16* p = in.a + ((long long)c * 2 * H + 2 * y) * W2 + 2 * x;
-      return 0.25f * (__bfloat162float(p[0]) + __bfloat162float(p[1]) + __bfloat162float(p[W2]) +
-                      __bfloat162float(p[W2 + 1]));
-    }
-    const int Hh = H / 2, Wh = W / 2;
-    return __bfloat162float(in.a[((long long)c * Hh + (y >> 1)) * Wh + (x >> 1)]);
-  }
-  return __bfloat162float(in.b[((long long)(c - in.ca) * H + y) * W + x]);
+// ---------------------------------------------------------------- primitives
+__device__ __forceinline__ unsigned smem_addr(const void* p) {
+  return unsigned(__cvta_generic_to_shared(p));
 }
-
-// ---------------------------------------------------------------- tensor cores
-// The convolutions are implicit GEMMs on the tensor cores: BF16 operands,
-// FP32 accumulation, mma.sync.m16n8k16 (one warp-wide 16x8x16 product per
-// instruction).
-//
-// Forward:  out[co](p)  = sum_{ci, tap} w[co][ci][tap] in[ci](p + off(tap))
-//           (M = co, N = pixels, K = ci for each tap)
-// Data gradient: din[ci](p) = sum_{co, tap} w[co][ci][KK-1-tap] dpre[co](p + off(tap))
-//           (the same form with the weights transposed and flipped)
-// Weight gradient: dw[co][ci][tap] = sum_p dpre[co](p) in[ci](p + off(tap))
-//           (M = co, N = ci, K = pixels)
-
+// 16 bytes to shared memory, zeros where !in
+__device__ __forceinline__ void cp16(unsigned dst, const void* src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0));
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N));
+}
+__device__ __forceinline__ void ldm4(unsigned (&r)[4], unsigned a) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+__device__ __forceinline__ void ldm4t(unsigned (&r)[4], unsigned a) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+}
+__device__ __forceinline__ void ldm2t(unsigned (&r)[2], unsigned a) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r[0]), "=r"(r[1]) : "r"(a));
+}
+// one warp-wide 16 x 8 x 16 product
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], unsigned b0,
                                          unsigned b1) {
   asm volatile(
@@ -76,389 +91,617 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const unsigned*>(&v);
+// Byte offset of 16-byte piece c of row p in a tile of rows of CH channels;
+// the pieces are permuted so that eight consecutive rows' pieces c fall in
+// distinct banks.
+template <int CH>
+__device__ __forceinline__ int swz(int p, int c) {
+  static_assert(CH == 16 || CH == 32, "rows of 16 or 32 channels");
+  return CH == 16 ? p * 32 + ((c ^ ((p >> 2) & 1)) << 4) : p * 64 + ((c ^ ((p >> 1) & 3)) << 4);
 }
 
-// 16 channels of one pixel (or one GEMM row) are 8 32-bit words; words 4..7
-// of rows whose bit 2 is set are swapped with words 0..3, so that the eight
-// rows a fragment load touches fall in distinct banks.
-__device__ __forceinline__ int swz(int row, int word) { return row * 8 + (word ^ (((row >> 2) & 1) << 2)); }
+// v = hi + lo, both BF16 (about 16 significant bits)
+__device__ __forceinline__ void split2(float v0, float v1, bf162& hi, bf162& lo) {
+  hi = __floats2bfloat162_rn(v0, v1);
+  lo = __floats2bfloat162_rn(v0 - __low2float(hi), v1 - __high2float(hi));
+}
 
-// Operand sources of the forward / data-gradient kernel.
-struct MmaIn {
-  ConvIn conv;                     // forward: the fused input transform
-  const float* dout;               // data gradient: dL/d(out) (FP32) ...
-  const __nv_bfloat16* out;        // ... masked by out > 0 when relu
-  int relu;
+// ---------------------------------------------------------------- convolution
+// Forward:  out[p][co]  = sum_{ci, tap} in[p + off(tap)][ci] w[co][ci][tap]
+// Data gradient: din[p][ci] = sum_{co, tap} dpre[p + off(tap)][co] w[co][ci][KK-1-tap]
+// Both are M = pixels, N = output channels, K = input channels of each tap.
+// A CTA takes 16 x 8 pixels and NB output channels; a warp takes XT = 1 or 2
+// M tiles of 2 x 8 pixels (side by side in two pixel rows) and all NB
+// channels, so there are 8 or 4 warps.  Input
+// channels come in chunks of 16, staged with their weights by cp.async in a
+// ring of ST stages; per chunk the taps run in order, so an output's sum is
+// over (chunk, tap) in a fixed order whatever NB is.
+enum { EPI_FWD = 0, EPI_HEAD = 1, EPI_PLAIN = 2, EPI_POOL = 3, EPI_UP = 4 };
+
+struct EpiArgs {
+  const float* bias;   // EPI_FWD, EPI_HEAD
+  int co;              // real output channels (EPI_FWD, EPI_HEAD)
+  int cp;              // padded channels of the tensor written
+  bf16* out;           // EPI_FWD: activation
+  bf16* pool;          // EPI_FWD: its 2 x 2 average, or null
+  float* y;            // EPI_HEAD: planes
+  // gradient of the layer below (activation act, cp channels): hi + lo pair
+  const bf16* act;
+  bf16 *hi, *lo;
+  const float* skip_in;  // EPI_POOL: gradient through the skip, FP32, on act's grid
+  float* skip_out;       // EPI_UP: gradient of the concatenated skip (cb channels)
+  int ca, cb;            // EPI_UP: channels of the upsampled operand and of the skip
+  float* part_b;         // bias gradient of the layer below: [tile][cp]
 };
 
-template <bool DGRAD>
-__device__ __forceinline__ float mma_in_value(const MmaIn& s, int c, int Kc, int y, int x, int H,
-                                              int W) {
-  if (c >= Kc) return 0.f;
-  if constexpr (!DGRAD) {
-    return conv_in(s.conv, c, y, x, H, W);
-  } else {
-    if (y < 0 || y >= H || x < 0 || x >= W) return 0.f;
-    const long long o = ((long long)c * H + y) * W + x;
-    float v = s.dout[o];
-    if (s.relu && !(__bfloat162float(s.out[o]) > 0.f)) v = 0.f;
-    return v;
-  }
-}
+constexpr int TW = 16, TH = 8;  // pixels of a CTA
 
-// grid: (W/16, H/16, ceil(M/MB)); 256 threads = 8 warps, warp w owns pixel
-// rows 2w, 2w+1 of the 16 x 16 tile (four 8-pixel n-tiles) and all MB rows.
-// Forward (DGRAD = false): M = CO rows co, Kc = CI, A[co][ci] =
-// w[co][ci][tap]; epilogue bias + ReLU, BF16 and/or FP32 output.
-// Data gradient: M = CI rows ci, Kc = CO, A[ci][co] = w[co][ci][KK-1-tap];
-// FP32 output, no bias.
-// The data gradient's operand dpre is FP32: it is staged as a BF16 pair
-// hi + lo (hi = bf16(v), lo = bf16(v - hi), about 16 significant bits) and
-// multiplied twice, so that the gradient keeps more than BF16 precision
-// through the layers; activations and weights are BF16 already.
-template <int K, int MB, bool DGRAD>
-__global__ void __launch_bounds__(256) k_conv_mma(MmaIn src, int H, int W, int M, int Kc, int CIw,
-                                                  const __nv_bfloat16* __restrict__ w,
-                                                  const float* __restrict__ bias, int relu,
-                                                  __nv_bfloat16* __restrict__ out_bf,
-                                                  float* __restrict__ out_f) {
-  constexpr int R = K / 2, T = 16 + 2 * R, KK = K * K, MT = MB / 16, NS = DGRAD ? 2 : 1;
-  __shared__ unsigned s_in[NS][T * T * 8];  // [pixel][16 channels] BF16 pairs, swizzled
-  __shared__ unsigned s_w[KK * MB * 8];     // [tap][row][16 channels]
+template <int K, int NB, int NS>
+struct ConvSmem {
+  static constexpr int R = K / 2, XW = TW + 2 * R, XH = TH + 2 * R, NP = XW * XH, KK = K * K;
+  static constexpr int px = NS * NP * 32, stage = px + KK * NB * 32;
+  // stages: up to eight within 84 KB; a launch takes no more than it has chunks
+  static constexpr int FIT = 84 * 1024 / stage, ST = FIT > 8 ? 8 : FIT;
+  static constexpr int bytes = ST * stage;
+};
+
+template <int K, int NB, int XT, int EPI>
+__global__ void __launch_bounds__(256 / XT)
+    k_conv(ConvSrc s, const bf16* __restrict__ s_lo, const bf16* __restrict__ w, int H, int W, int KC,
+           EpiArgs e) {
+  constexpr bool GRAD = EPI >= EPI_PLAIN;
+  constexpr int NS = GRAD ? 2 : 1;
+  using S = ConvSmem<K, NB, NS>;
+  constexpr int R = S::R, XW = S::XW, NP = S::NP, KK = S::KK, ST = S::ST, NT = NB / 8;
+  constexpr int THREADS = 256 / XT, WARPS = 8 / XT;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const unsigned sm = smem_addr(smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rows = 2 * (XT == 2 ? warp : warp >> 1), xw = XT == 2 ? 0 : (warp & 1) * 8;  // the warp's pixels
   const int g = lane >> 2, t4 = lane & 3;
-  const int x0 = blockIdx.x * 16, y0 = blockIdx.y * 16, m0 = blockIdx.z * MB;
-  float acc[MT][4][4];
+  const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TH, n0 = blockIdx.z * NB;
+
+  auto load_weights = [&](int kc, int buf) {
+    // [group of 16 outputs][chunk][tap][16 outputs][16 inputs]
+    const unsigned d = sm + buf * S::stage + S::px;
+    for (int i = threadIdx.x; i < KK * NB * 2; i += THREADS) {
+      const int h = i & 1, n = (i >> 1) & 15, r = i >> 5, tap = r % KK, cg = r / KK;
+      const long long o = ((((long long)(n0 / 16 + cg) * KC + kc) * KK + tap) * 16 + n) * 16 + h * 8;
+      cp16(d + swz<16>(tap * NB + cg * 16 + n, h), w + o, true);
+    }
+  };
+  auto load_pixels = [&](int kc, int buf) {
+    const unsigned d = sm + buf * S::stage;
+    const int c0 = kc * 16;
+    const bool from_a = GRAD || c0 < s.ca;
+    const bf16* src = from_a ? s.a : s.b;
+    const int cs = from_a ? s.ca : s.cb, co = from_a ? c0 : c0 - s.ca;
+    const int sh = from_a && s.up ? 1 : 0, ws = W >> sh;
+    for (int i = threadIdx.x; i < NP * 2; i += THREADS) {
+      const int p = i >> 1, h = i & 1;
+      const int yy = y0 - R + p / XW, xx = x0 - R + p % XW;
+      const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
+      const long long o = in ? ((long long)(yy >> sh) * ws + (xx >> sh)) * cs + co + h * 8 : 0;
+      cp16(d + swz<16>(p, h), src + o, in);
+      if constexpr (NS == 2) cp16(d + NP * 32 + swz<16>(p, h), s_lo + o, in);
+    }
+  };
+
+  float acc[XT][NT][4];
 #pragma unroll
-  for (int a = 0; a < MT; ++a)
+  for (int a = 0; a < XT; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
+    for (int b = 0; b < NT; ++b)
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-  for (int k0 = 0; k0 < Kc; k0 += 16) {
-    for (int i = threadIdx.x; i < T * T * 8; i += 256) {
-      const int q = i % (T * T), j = i / (T * T);
-      const int yy = y0 - R + q / T, xx = x0 - R + q % T;
-      const float v0 = mma_in_value<DGRAD>(src, k0 + 2 * j, Kc, yy, xx, H, W);
-      const float v1 = mma_in_value<DGRAD>(src, k0 + 2 * j + 1, Kc, yy, xx, H, W);
-      s_in[0][swz(q, j)] = pack_bf16(v0, v1);
-      if constexpr (DGRAD)
-        s_in[1][swz(q, j)] = pack_bf16(v0 - __bfloat162float(__float2bfloat16(v0)),
-                                       v1 - __bfloat162float(__float2bfloat16(v1)));
-    }
-    for (int i = threadIdx.x; i < KK * MB * 8; i += 256) {
-      const int j = i & 7, row = (i >> 3) % MB, tap = i / (8 * MB);
-      const int m = m0 + row;
-      float v[2];
+
+  // the weights do not depend on the launch before (only on one further back):
+  // fetch the first of them while it finishes, then let the next launch start
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int kc = k0 + 2 * j + h;
-        v[h] = 0.f;
-        if (m < M && kc < Kc) {
-          // forward: w[m][kc][tap]; data gradient: w[kc][m][KK-1-tap]
-          const long long o = DGRAD ? ((long long)kc * CIw + m) * KK + (KK - 1 - tap)
-                                    : ((long long)m * CIw + kc) * KK + tap;
-          v[h] = __bfloat162float(w[o]);
-        }
-      }
-      s_w[tap * MB * 8 + swz(row, j)] = pack_bf16(v[0], v[1]);
-    }
+  for (int st = 0; st < ST - 1; ++st)
+    if (st < KC) load_weights(st, st);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+#pragma unroll
+  for (int st = 0; st < ST - 1; ++st) {
+    if (st < KC) load_pixels(st, st);
+    cp_commit();
+  }
+  // ldmatrix rows of this lane: A row (pixel) and half, B row (channel) and half
+  const int a_q = (rows + ((lane >> 3) & 1)) * XW + xw + (lane & 7), a_h = lane >> 4;
+  const int b_n = (lane & 7) + 8 * (lane >> 4), b_h = (lane >> 3) & 1;
+  for (int kc = 0; kc < KC; ++kc) {
+    cp_wait<ST - 2>();
     __syncthreads();
+    if (kc + ST - 1 < KC) {
+      load_weights(kc + ST - 1, (kc + ST - 1) % ST);
+      load_pixels(kc + ST - 1, (kc + ST - 1) % ST);
+    }
+    cp_commit();
+    const unsigned px = sm + (kc % ST) * S::stage, wt = px + S::px;
 #pragma unroll
     for (int tap = 0; tap < KK; ++tap) {
       const int ky = tap / K, kx = tap % K;
+      unsigned a[NS][XT][4], b[NT / 2][4];
 #pragma unroll
-      for (int part = 0; part < NS; ++part) {
-        unsigned bfr[4][2];
+      for (int part = 0; part < NS; ++part)
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-          const int py = 2 * warp + (nt >> 1), px = (nt & 1) * 8 + g;
-          const int q = (py + ky) * T + px + kx;
-          bfr[nt][0] = s_in[part][swz(q, t4)];
-          bfr[nt][1] = s_in[part][swz(q, t4 + 4)];
-        }
+        for (int xt = 0; xt < XT; ++xt)
+          ldm4(a[part][xt], px + part * NP * 32 + swz<16>(a_q + ky * XW + kx + xt * 8, a_h));
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-          const unsigned* sw = s_w + tap * MB * 8;
-          const int r0 = mt * 16 + g, r1 = r0 + 8;
-          const unsigned a[4] = {sw[swz(r0, t4)], sw[swz(r1, t4)], sw[swz(r0, t4 + 4)],
-                                 sw[swz(r1, t4 + 4)]};
+      for (int j = 0; j < NT / 2; ++j) ldm4(b[j], wt + swz<16>(tap * NB + j * 16 + b_n, b_h));
 #pragma unroll
-          for (int nt = 0; nt < 4; ++nt) mma_bf16(acc[mt][nt], a, bfr[nt][0], bfr[nt][1]);
-        }
-      }
+      for (int part = 0; part < NS; ++part)
+#pragma unroll
+        for (int xt = 0; xt < XT; ++xt)
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt)
+            mma_bf16(acc[xt][nt], a[part][xt], b[nt / 2][(nt & 1) * 2], b[nt / 2][(nt & 1) * 2 + 1]);
     }
-    __syncthreads();
   }
-  // epilogue: c0 (row g, pixel 2t), c1 (row g, 2t+1), c2 (row g+8, 2t), c3 (row g+8, 2t+1)
+  cp_wait<0>();
+
+  // epilogue: lane (g, t4) holds pixels (y, x), (y + 1, x) of channels ch, ch + 1
+  const int y = y0 + rows;
+  float bsum[NT][2];
 #pragma unroll
-  for (int mt = 0; mt < MT; ++mt)
+  for (int nt = 0; nt < NT; ++nt) bsum[nt][0] = bsum[nt][1] = 0.f;
+  // gradient of the layer below at pixel o (of its grid): mask, split, bias
+  auto grad_out = [&](long long o, int ch, float v0, float v1, float (&bs)[2]) {
+    const long long k = o * e.cp + ch;
+    const bf162 a = *reinterpret_cast<const bf162*>(e.act + k);
+    v0 = __low2float(a) > 0.f ? v0 : 0.f;
+    v1 = __high2float(a) > 0.f ? v1 : 0.f;
+    bf162 hi, lo;
+    split2(v0, v1, hi, lo);
+    *reinterpret_cast<bf162*>(e.hi + k) = hi;
+    *reinterpret_cast<bf162*>(e.lo + k) = lo;
+    bs[0] += v0;
+    bs[1] += v1;
+  };
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      const int y = y0 + 2 * warp + (nt >> 1);
-      const int xb = x0 + (nt & 1) * 8 + 2 * t4;
+  for (int xt = 0; xt < XT; ++xt) {
+    const int x = x0 + xw + xt * 8 + g;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int m = m0 + mt * 16 + g + 8 * h;
-        if (m >= M || y >= H) continue;
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int x = xb + e;
-          if (x >= W) continue;
-          float v = acc[mt][nt][2 * h + e];
-          if (!DGRAD) {
-            v += bias[m];
-            if (relu) v = fmaxf(v, 0.f);
+    for (int nt = 0; nt < NT; ++nt) {
+      const int ch = n0 + nt * 8 + 2 * t4;
+      float(&c)[4] = acc[xt][nt];
+      const bool in0 = x < W && y < H, in1 = x < W && y + 1 < H;
+      if constexpr (EPI == EPI_FWD || EPI == EPI_HEAD) {
+        const float b0 = ch < e.co ? e.bias[ch] : 0.f, b1 = ch + 1 < e.co ? e.bias[ch + 1] : 0.f;
+        if constexpr (EPI == EPI_HEAD) {
+          const long long HW = (long long)H * W, o = (long long)y * W + x;
+          if (ch < e.co) {
+            if (in0) e.y[ch * HW + o] = c[0] + b0;
+            if (in1) e.y[ch * HW + o + W] = c[2] + b0;
           }
-          const long long o = ((long long)m * H + y) * W + x;
-          if (out_bf) out_bf[o] = __float2bfloat16(v);
-          if (out_f) out_f[o] = v;
+          if (ch + 1 < e.co) {
+            if (in0) e.y[(ch + 1) * HW + o] = c[1] + b1;
+            if (in1) e.y[(ch + 1) * HW + o + W] = c[3] + b1;
+          }
+        } else {
+          const bf162 r0 = __floats2bfloat162_rn(fmaxf(c[0] + b0, 0.f), fmaxf(c[1] + b1, 0.f));
+          const bf162 r1 = __floats2bfloat162_rn(fmaxf(c[2] + b0, 0.f), fmaxf(c[3] + b1, 0.f));
+          bf16* o = e.out + ((long long)y * W + x) * e.cp + ch;
+          if (ch < e.cp) {
+            if (in0) *reinterpret_cast<bf162*>(o) = r0;
+            if (in1) *reinterpret_cast<bf162*>(o + (long long)W * e.cp) = r1;
+          }
+          if (e.pool) {
+            // the average of the stored (rounded) values, ((00 + 01) + 10) + 11
+            const float p0 = __low2float(r0), p1 = __high2float(r0);
+            const float q0 = __low2float(r1), q1 = __high2float(r1);
+            const float pr0 = __shfl_xor_sync(0xffffffffu, p0, 4), pr1 = __shfl_xor_sync(0xffffffffu, p1, 4);
+            const float qr0 = __shfl_xor_sync(0xffffffffu, q0, 4), qr1 = __shfl_xor_sync(0xffffffffu, q1, 4);
+            if (!(g & 1) && in1 && ch < e.cp)
+              *reinterpret_cast<bf162*>(e.pool + ((long long)(y >> 1) * (W >> 1) + (x >> 1)) * e.cp + ch) =
+                  __floats2bfloat162_rn(0.25f * (p0 + pr0 + q0 + qr0), 0.25f * (p1 + pr1 + q1 + qr1));
+          }
+        }
+      } else if constexpr (EPI == EPI_PLAIN) {
+        if (ch < e.cp) {
+          if (in0) grad_out((long long)y * W + x, ch, c[0], c[1], bsum[nt]);
+          if (in1) grad_out((long long)(y + 1) * W + x, ch, c[2], c[3], bsum[nt]);
+        }
+      } else if constexpr (EPI == EPI_POOL) {
+        // each coarse value goes to its 2 x 2 pixels with weight 1/4
+        if (ch < e.cp) {
+          const int W2 = 2 * W;
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            if (!(r ? in1 : in0)) continue;
+            const float v0 = 0.25f * c[2 * r], v1 = 0.25f * c[2 * r + 1];
+#pragma unroll
+            for (int d = 0; d < 4; ++d) {
+              const long long o = (long long)(2 * (y + r) + (d >> 1)) * W2 + 2 * x + (d & 1);
+              const float2 sk = *reinterpret_cast<const float2*>(e.skip_in + o * e.cp + ch);
+              grad_out(o, ch, sk.x + v0, sk.y + v1, bsum[nt]);
+            }
+          }
+        }
+      } else {
+        if (n0 + nt * 8 < e.ca) {
+          // the upsampled operand: sums of 2 x 2 pixels, ((00 + 01) + 10) + 11
+          const float r0 = __shfl_xor_sync(0xffffffffu, c[0], 4), r1 = __shfl_xor_sync(0xffffffffu, c[1], 4);
+          const float r2 = __shfl_xor_sync(0xffffffffu, c[2], 4), r3 = __shfl_xor_sync(0xffffffffu, c[3], 4);
+          if (!(g & 1) && in1)
+            grad_out((long long)(y >> 1) * (W >> 1) + (x >> 1), ch, c[0] + r0 + c[2] + r2,
+                     c[1] + r1 + c[3] + r3, bsum[nt]);
+        } else if (ch < e.ca + e.cb) {
+          float* o = e.skip_out + ((long long)y * W + x) * e.cb + ch - e.ca;
+          if (in0) *reinterpret_cast<float2*>(o) = make_float2(c[0], c[1]);
+          if (in1) *reinterpret_cast<float2*>(o + (long long)W * e.cb) = make_float2(c[2], c[3]);
         }
       }
     }
+  }
+  if constexpr (GRAD) {
+    // bias gradient of the layer below: lanes of a channel, then warps
+    __syncthreads();
+    float* sb = reinterpret_cast<float*>(smem);  // [warp][NB]
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        float v = bsum[nt][k];
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 16);
+        if (g == 0) sb[warp * NB + nt * 8 + 2 * t4 + k] = v;
+      }
+    __syncthreads();
+    const int ch = n0 + threadIdx.x;
+    if (threadIdx.x < NB && ch < e.cp) {
+      float t = 0.f;
+#pragma unroll
+      for (int r = 0; r < WARPS; ++r) t += sb[r * NB + threadIdx.x];
+      e.part_b[((long long)blockIdx.y * gridDim.x + blockIdx.x) * e.cp + ch] = t;
+    }
+  }
 }
 
-// Weight gradient partials on the tensor cores.  grid: (ceil(CI/NB),
-// ceil(CO/MB), P); the 16 x 16 pixel tiles of the layer (tx per row, T in
-// all, row-major) are cut into P contiguous chunks, chunk p taking tiles
-// [p T / P, (p+1) T / P) in order.
-// The CTA stages, per 16 x 16 pixel tile, dpre for its MB output channels
-// (A rows; K = the 16 pixels of a tile row) and the fused input for its NB
-// input channels (three copies shifted by kx, so that every pixel pair a
-// fragment reads is 4-byte aligned).  Per-channel strides are padded by 4
-// words so the eight rows of a fragment fall in distinct banks.  Warp w
-// accumulates the (m-tile, n-tile, tap) products w, w+8, ...; the bias
-// gradient sums the FP32 dpre of each channel (warp w: channels w, w+8, ...)
-// lane-wise and by a fixed shuffle tree.  Every sum runs over the pixels in
-// a fixed order, so the partials are deterministic.
+// Opt-in to dynamic shared memory above 48 KB, once per kernel, device and
+// thread.
+template <class F>
+cudaError_t opt_in(F kernel, int bytes, int& done_dev) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || done_dev == dev) return e;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done_dev = dev;
+  return e;
+}
+
+template <int K, int NB, int XT, int EPI>
+cudaError_t launch_conv_nb(const ConvSrc& s, const bf16* lo, const bf16* w, int H, int W, int N, int KC,
+                           const EpiArgs& e, cudaStream_t st) {
+  using S = ConvSmem<K, NB, (EPI >= EPI_PLAIN ? 2 : 1)>;
+  static thread_local int done = -1;
+  cudaError_t rc = opt_in(k_conv<K, NB, XT, EPI>, S::bytes, done);
+  if (rc != cudaSuccess) return rc;
+  // programmatic dependent launch: the CTAs start while the launch before
+  // drains and wait for it where they first read what it wrote
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((W + TW - 1) / TW, (H + TH - 1) / TH, N / NB);
+  cfg.blockDim = dim3(256 / XT);
+  cfg.dynamicSmemBytes = size_t(std::min(S::ST, KC)) * S::stage;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_conv<K, NB, XT, EPI>, s, lo, w, H, W, KC, e);
+}
+
+// N output channels (a multiple of 16) in blocks of 64, 32 or 16: the largest
+// that divides N and leaves two CTAs per SM.  A block of 64 reuses a pixel
+// fragment eight times where 16 reuses it twice, but the deep levels have few
+// pixel tiles (at 136^2 and 17 x 17 pixels: 6) and there the parallelism wins;
+// a launch below two CTAs per SM also halves each warp's share (8 warps with
+// one M tile: its length is then set by one warp's instruction latencies).
+template <int K, int EPI>
+cudaError_t launch_conv(const ConvSrc& s, const bf16* lo, const bf16* w, int H, int W, int N, int KC,
+                        const EpiArgs& e, int sms, cudaStream_t st) {
+  const long long tiles = (long long)((W + TW - 1) / TW) * ((H + TH - 1) / TH);
+  const auto full = [&](int nb) { return N % nb == 0 && tiles * (N / nb) >= 2LL * sms; };
+  if (full(64)) return launch_conv_nb<K, 64, 2, EPI>(s, lo, w, H, W, N, KC, e, st);
+  if (full(32)) return launch_conv_nb<K, 32, 2, EPI>(s, lo, w, H, W, N, KC, e, st);
+  if (full(16)) return launch_conv_nb<K, 16, 2, EPI>(s, lo, w, H, W, N, KC, e, st);
+  return launch_conv_nb<K, 16, 1, EPI>(s, lo, w, H, W, N, KC, e, st);
+}
+
+// ---------------------------------------------------------------- weight gradient
+// dw[co][ci][tap] = sum_p dpre[p][co] in[p + off(tap)][ci]: M = co, N = ci,
+// K = pixels, 16 of a tile row at a time.  Both operands are channel-innermost
+// tiles, so their fragments are transposing ldmatrix reads.  A CTA of 8 warps
+// takes MB x NB channels and a contiguous chunk of the layer's 16 x 16 pixel
+// tiles (staged in two alternating buffers by cp.async); a warp takes one
+// 16 x 8 block of (co, ci) with all its taps, marching down rows with the
+// input fragments of three rows in registers: a row's six loads (2 of dpre,
+// 3 of the input) feed 18 products.  Where MB x NB has fewer than 8 blocks
+// the warps share the rows and their sums are added at the end.
 template <int K, int MB, int NB>
 struct WgradSmem {
-  static constexpr int R = K / 2, YT = 16 + 2 * R;
-  static constexpr int SD = 16 * 8 + 4, SX = YT * 8 + 4;
-  static constexpr size_t bytes = sizeof(unsigned) * (2 * size_t(MB) * SD + size_t(K) * NB * SX);
+  static constexpr int R = K / 2, XW = 16 + 2 * R, NX = XW * XW, KK = K * K;
+  static constexpr int BLK = (MB / 16) * (NB / 8), KG = 8 / BLK, ROWS = 16 / KG;
+  static constexpr int d_part = 256 * MB * 2, x_off = 2 * d_part, stage = x_off + NX * NB * 2;
+  static constexpr int red = 8 * KK * 4 * 32 * 4;
+  static constexpr int bytes = 2 * stage > red ? 2 * stage : red;
 };
 
 template <int K, int MB, int NB>
-__global__ void __launch_bounds__(256) k_conv_wgrad_mma(const float* __restrict__ dout,
-                                                        const __nv_bfloat16* __restrict__ out,
-                                                        int relu, ConvIn in, int H, int W, int CO,
-                                                        int P, float* __restrict__ part,
-                                                        float* __restrict__ part_b) {
+__global__ void __launch_bounds__(256, 2)
+    k_wgrad(const bf16* __restrict__ dh, const bf16* __restrict__ dl, int coP, ConvSrc in, int ca,
+            int cb, int H, int W, int CO, int P, float* __restrict__ part) {
   using S = WgradSmem<K, MB, NB>;
-  constexpr int R = S::R, YT = S::YT, SD = S::SD, SX = S::SX, KK = K * K;
-  constexpr int MT = MB / 16, NT = NB / 8;
-  constexpr int COMBOS = MT * NT * KK, PER = (COMBOS + 7) / 8, BPW = MB / 8;
-  extern __shared__ unsigned smem_u[];
-  unsigned* s_d = smem_u;             // [2][MB][SD] (hi, lo): row r, pixel pair wd at r * 8 + wd
-  unsigned* s_x = s_d + 2 * MB * SD;  // [K][NB][SX]: row r, pixel pair wd at r * 8 + wd
-  const int CI = in.ca + in.cb;
+  constexpr int R = S::R, XW = S::XW, KK = S::KK, KG = S::KG, ROWS = S::ROWS;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const unsigned sm = smem_addr(smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int g = lane >> 2, t4 = lane & 3;
+  const int blk = warp % S::BLK, kg = warp / S::BLK;
+  const int mt = blk % (MB / 16), nt = blk / (MB / 16);
   const int n0 = blockIdx.x * NB, m0 = blockIdx.y * MB, p = blockIdx.z;
   const int tx = (W + 15) / 16;
   const long long T = (long long)tx * ((H + 15) / 16);
   const long long t_lo = p * T / P, t_hi = (p + 1) * T / P;
-  float acc[PER][4];
-#pragma unroll
-  for (int i = 0; i < PER; ++i)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
-  float accb[BPW];
-#pragma unroll
-  for (int j = 0; j < BPW; ++j) accb[j] = 0.f;
-  auto dpre = [&](int c, int yy, int xx) -> float {
-    if (m0 + c >= CO || yy >= H || xx >= W) return 0.f;
-    const long long o = ((long long)(m0 + c) * H + yy) * W + xx;
-    const float d = dout[o];
-    return (relu && !(__bfloat162float(out[o]) > 0.f)) ? 0.f : d;
-  };
-  for (long long ti = t_lo; ti < t_hi; ++ti) {
+
+  auto load = [&](long long ti, int buf) {
+    const unsigned d = sm + buf * S::stage;
     const int yb = int(ti / tx) * 16, xb = int(ti % tx) * 16;
-    {
-      for (int i = threadIdx.x; i < MB * 16 * 8; i += 256) {
-        const int wd = i & 7, r = (i >> 3) & 15, c = i >> 7;
-        const float v0 = dpre(c, yb + r, xb + 2 * wd), v1 = dpre(c, yb + r, xb + 2 * wd + 1);
-        s_d[c * SD + r * 8 + wd] = pack_bf16(v0, v1);
-        s_d[(MB + c) * SD + r * 8 + wd] = pack_bf16(v0 - __bfloat162float(__float2bfloat16(v0)),
-                                                   v1 - __bfloat162float(__float2bfloat16(v1)));
-      }
-      for (int i = threadIdx.x; i < K * NB * YT * 8; i += 256) {
-        const int wd = i & 7, r = (i >> 3) % YT, c = (i / (8 * YT)) % NB, kx = i / (8 * YT * NB);
-        const int yy = yb - R + r, xx = xb - R + kx + 2 * wd;
-        const float lo = (n0 + c < CI) ? conv_in(in, n0 + c, yy, xx, H, W) : 0.f;
-        const float hi = (n0 + c < CI) ? conv_in(in, n0 + c, yy, xx + 1, H, W) : 0.f;
-        s_x[(kx * NB + c) * SX + r * 8 + wd] = pack_bf16(lo, hi);
-      }
-      // bias (blocks of the first input-channel block only): FP32 sums of
-      // dpre, lane-wise over the tile then a fixed tree
-      if (blockIdx.x == 0)
-#pragma unroll
-      for (int j = 0; j < BPW; ++j) {
-        const int c = warp + 8 * j;
-        float s = 0.f;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int px = lane + 32 * k;
-          s += dpre(c, yb + px / 16, xb + px % 16);
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        accb[j] += s;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int i = 0; i < PER; ++i) {
-        const int combo = warp + 8 * i;
-        if (combo < COMBOS) {
-          const int mt = combo % MT, nt = (combo / MT) % NT, tap = combo / (MT * NT);
-          const int ky = tap / K, kx = tap % K;
-          const unsigned* xb0 = s_x + (kx * NB + nt * 8 + g) * SX + ky * 8;
-#pragma unroll
-          for (int part = 0; part < 2; ++part) {  // dpre = hi + lo
-            const unsigned* da0 = s_d + (part * MB + mt * 16 + g) * SD;
-            const unsigned* da1 = da0 + 8 * SD;
-#pragma unroll 4
-            for (int r = 0; r < 16; ++r) {
-              const unsigned a[4] = {da0[r * 8 + t4], da1[r * 8 + t4], da0[r * 8 + t4 + 4],
-                                     da1[r * 8 + t4 + 4]};
-              mma_bf16(acc[i], a, xb0[r * 8 + t4], xb0[r * 8 + t4 + 4]);
-            }
-          }
-        }
-      }
-      __syncthreads();
+    for (int i = threadIdx.x; i < 256 * (MB / 8); i += 256) {
+      const int c = i % (MB / 8), q = i / (MB / 8);
+      const int yy = yb + q / 16, xx = xb + q % 16, ch = m0 + c * 8;
+      const bool ok = yy < H && xx < W && ch < coP;
+      const long long o = ok ? ((long long)yy * W + xx) * coP + ch : 0;
+      cp16(d + swz<MB>(q, c), dh + o, ok);
+      cp16(d + S::d_part + swz<MB>(q, c), dl + o, ok);
     }
+    for (int i = threadIdx.x; i < S::NX * (NB / 8); i += 256) {
+      const int c = i % (NB / 8), q = i / (NB / 8);
+      const int yy = yb - R + q / XW, xx = xb - R + q % XW, ch = n0 + c * 8;
+      const bool a = ch < in.ca;
+      const bool ok = yy >= 0 && yy < H && xx >= 0 && xx < W && ch < in.ca + in.cb;
+      const int sh = a && in.up ? 1 : 0;
+      const long long o = ok ? ((long long)(yy >> sh) * (W >> sh) + (xx >> sh)) * (a ? in.ca : in.cb) +
+                                   (a ? ch : ch - in.ca)
+                             : 0;
+      cp16(d + S::x_off + swz<NB>(q, c), (a || !ok ? in.a : in.b) + o, ok);
+    }
+  };
+
+  float acc[KK][4];
+#pragma unroll
+  for (int k = 0; k < KK; ++k)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[k][c] = 0.f;
+  // transposed ldmatrix rows of this lane
+  const int d_q = (lane >> 4) * 8 + (lane & 7), d_c = mt * 2 + ((lane >> 3) & 1);
+  const int x_q = ((lane >> 3) & 1) * 8 + (lane & 7);
+  if (t_lo < t_hi) load(t_lo, 0);
+  cp_commit();
+  for (long long ti = t_lo; ti < t_hi; ++ti) {
+    const int buf = int((ti - t_lo) & 1);
+    if (ti + 1 < t_hi) load(ti + 1, buf ^ 1);
+    cp_commit();
+    cp_wait<1>();
+    __syncthreads();
+    const unsigned d = sm + buf * S::stage, x = d + S::x_off;
+    const int r0 = kg * ROWS;
+    unsigned bf[K][K][2];  // [input row mod K][kx]
+#pragma unroll
+    for (int r = 0; r < K - 1; ++r)
+#pragma unroll
+      for (int kx = 0; kx < K; ++kx) ldm2t(bf[r][kx], x + swz<NB>((r0 + r) * XW + kx + x_q, nt));
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      unsigned ah[4], al[4];
+      ldm4t(ah, d + swz<MB>((r0 + r) * 16 + d_q, d_c));
+      ldm4t(al, d + S::d_part + swz<MB>((r0 + r) * 16 + d_q, d_c));
+#pragma unroll
+      for (int kx = 0; kx < K; ++kx)
+        ldm2t(bf[(r + K - 1) % K][kx], x + swz<NB>((r0 + r + K - 1) * XW + kx + x_q, nt));
+#pragma unroll
+      for (int tap = 0; tap < KK; ++tap) {
+        const unsigned(&b)[2] = bf[(r + tap / K) % K][tap % K];
+        mma_bf16(acc[tap], ah, b[0], b[1]);
+        mma_bf16(acc[tap], al, b[0], b[1]);
+      }
+    }
+    __syncthreads();
   }
-  // c0 (m = g, n = 2t), c1 (g, 2t+1), c2 (g+8, 2t), c3 (g+8, 2t+1)
+  cp_wait<0>();
+  if constexpr (KG > 1) {
+    float* red = reinterpret_cast<float*>(smem);  // [warp][tap][4][lane]
+    __syncthreads();
+    if (kg > 0)
 #pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    const int combo = warp + 8 * i;
-    if (combo >= COMBOS) continue;
-    const int mt = combo % MT, nt = (combo / MT) % NT, tap = combo / (MT * NT);
+      for (int k = 0; k < KK; ++k)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int co = m0 + mt * 16 + g + 8 * (e >> 1), ci = n0 + nt * 8 + 2 * t4 + (e & 1);
-      if (co < CO && ci < CI) part[(((long long)p * CO + co) * CI + ci) * KK + tap] = acc[i][e];
-    }
+        for (int c = 0; c < 4; ++c) red[((warp * KK + k) * 4 + c) * 32 + lane] = acc[k][c];
+    __syncthreads();
+    if (kg > 0) return;
+#pragma unroll
+    for (int o = 1; o < KG; ++o)
+#pragma unroll
+      for (int k = 0; k < KK; ++k)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[k][c] += red[(((warp + o * S::BLK) * KK + k) * 4 + c) * 32 + lane];
   }
-  if (blockIdx.x == 0 && lane == 0)
+  const int g = lane >> 2, t4 = lane & 3, CI = ca + cb;
 #pragma unroll
-    for (int j = 0; j < BPW; ++j) {
-      const int c = warp + 8 * j;
-      if (m0 + c < CO) part_b[(long long)p * CO + m0 + c] = accb[j];
-    }
+  for (int c = 0; c < 4; ++c) {
+    const int co = m0 + mt * 16 + g + 8 * (c >> 1), cp = n0 + nt * 8 + 2 * t4 + (c & 1);
+    // padded input channel -> real one
+    const int ci = cp < in.ca ? (cp < ca ? cp : -1) : (cp - in.ca < cb ? ca + cp - in.ca : -1);
+    if (co < CO && ci >= 0)
+#pragma unroll
+      for (int k = 0; k < KK; ++k) part[(((long long)p * CO + co) * CI + ci) * KK + k] = acc[k][c];
+  }
 }
 
-
-// Forward (DGRAD = false) or data-gradient convolution on the tensor cores;
-// MB (GEMM rows per CTA) follows the row count M.
-template <int K, bool DGRAD>
-void launch_conv_mma(const MmaIn& src, int H, int W, int M, int Kc, int CIw,
-                     const __nv_bfloat16* w, const float* bias, int relu, __nv_bfloat16* ob,
-                     float* of, cudaStream_t st) {
-  const int MB = M <= 16 ? 16 : (M <= 32 ? 32 : 64);
-  const dim3 grid((W + 15) / 16, (H + 15) / 16, (M + MB - 1) / MB);
-  if (MB == 16)
-    k_conv_mma<K, 16, DGRAD><<<grid, 256, 0, st>>>(src, H, W, M, Kc, CIw, w, bias, relu, ob, of);
-  else if (MB == 32)
-    k_conv_mma<K, 32, DGRAD><<<grid, 256, 0, st>>>(src, H, W, M, Kc, CIw, w, bias, relu, ob, of);
-  else
-    k_conv_mma<K, 64, DGRAD><<<grid, 256, 0, st>>>(src, H, W, M, Kc, CIw, w, bias, relu, ob, of);
-}
-
-constexpr int WG_MB = 32, WG_NB = 16;
+// Channel blocks of a weight gradient: 32 where the layer has more than 16.
+int wg_block(int cp) { return cp > 16 ? 32 : 16; }
 
 // Pixel-tile chunks of a weight-gradient launch: enough for two CTAs per SM
 // over the (input block, output block) grid, at most one chunk per tile.
-int wgrad_chunks(int H, int W, int CI, int CO, int sms) {
+int wgrad_chunks(int H, int W, int ciP, int coP, int sms) {
   const long long T = (long long)((W + 15) / 16) * ((H + 15) / 16);
-  const long long base = (long long)((CI + WG_NB - 1) / WG_NB) * ((CO + WG_MB - 1) / WG_MB);
+  const int mb = wg_block(coP), nb = wg_block(ciP);
+  const long long base = (long long)((ciP + nb - 1) / nb) * ((coP + mb - 1) / mb);
   const long long want = (2LL * sms + base - 1) / base;
   return int(std::max<long long>(1, std::min(T, want)));
 }
 
-template <int K>
-cudaError_t launch_wgrad_mma(const float* dout, const __nv_bfloat16* out, int relu, const ConvIn& in,
-                             int H, int W, int CO, int P, float* part, float* part_b, cudaStream_t st) {
-  const int CI = in.ca + in.cb;
-  const dim3 grid((CI + WG_NB - 1) / WG_NB, (CO + WG_MB - 1) / WG_MB, P);
-  const size_t bytes = WgradSmem<K, WG_MB, WG_NB>::bytes;
-  static_assert(WgradSmem<3, WG_MB, WG_NB>::bytes <= 100 * 1024, "wgrad shared memory above 100 KB");
-  static thread_local int dev_done = -1;  // opt-in above 48 KB, once per device and thread
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev_done != dev) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv_wgrad_mma<K, WG_MB, WG_NB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-    if (e != cudaSuccess) return e;
-    dev_done = dev;
-  }
-  k_conv_wgrad_mma<K, WG_MB, WG_NB><<<grid, 256, bytes, st>>>(dout, out, relu, in, H, W, CO, P,
-                                                             part, part_b);
+template <int K, int MB, int NB>
+cudaError_t launch_wgrad_b(const bf16* dh, const bf16* dl, int coP, const ConvSrc& in, int ca, int cb,
+                           int H, int W, int CO, int P, float* part, cudaStream_t st) {
+  using S = WgradSmem<K, MB, NB>;
+  static thread_local int done = -1;
+  cudaError_t rc = opt_in(k_wgrad<K, MB, NB>, S::bytes, done);
+  if (rc != cudaSuccess) return rc;
+  const dim3 grid((in.ca + in.cb + NB - 1) / NB, (coP + MB - 1) / MB, P);
+  k_wgrad<K, MB, NB><<<grid, 256, S::bytes, st>>>(dh, dl, coP, in, ca, cb, H, W, CO, P, part);
   return cudaGetLastError();
 }
 
-// grad += sum_p part[p] in order p = 0 .. P-1 (deterministic)
-__global__ void k_sum_parts(const float* __restrict__ part, int P, long long n,
-                            float* __restrict__ grad) {
+template <int K>
+cudaError_t launch_wgrad(const bf16* dh, const bf16* dl, int coP, const ConvSrc& in, int ca, int cb,
+                         int H, int W, int CO, int P, float* part, cudaStream_t st) {
+  const bool m32 = wg_block(coP) == 32, n32 = wg_block(in.ca + in.cb) == 32;
+  if (m32 && n32) return launch_wgrad_b<K, 32, 32>(dh, dl, coP, in, ca, cb, H, W, CO, P, part, st);
+  if (m32) return launch_wgrad_b<K, 32, 16>(dh, dl, coP, in, ca, cb, H, W, CO, P, part, st);
+  if (n32) return launch_wgrad_b<K, 16, 32>(dh, dl, coP, in, ca, cb, H, W, CO, P, part, st);
+  return launch_wgrad_b<K, 16, 16>(dh, dl, coP, in, ca, cb, H, W, CO, P, part, st);
+}
+
+// grad += sum_p part[p] for a layer's weights (n values, P partials) and
+// biases (nb of the ldb columns, Pb partials).  A warp covers `cols`
+// neighbouring values and 32 / cols partials at a time: few values with many
+// partials (16 biases, 2,178 tiles at 528 x 520: 44 us with one value per
+// lane) take narrow blocks.  Added in a fixed order: every (256 / cols)-th
+// partial per thread, then a tree over the threads of a value.
+__device__ __forceinline__ void sum_columns(const float* __restrict__ src, int P, long long n,
+                                            long long ld, int cols, long long block,
+                                            float* __restrict__ grad) {
+  __shared__ float sh[256];
+  const int col = threadIdx.x % cols, row = threadIdx.x / cols, rows = 256 / cols;
+  const long long i = block * cols + col;
+  float s = 0.f;
+  if (i < n)
+#pragma unroll 4
+    for (int p = row; p < P; p += rows) s += src[p * ld + i];
+  sh[threadIdx.x] = s;
+  __syncthreads();
+  for (int o = rows / 2; o > 0; o >>= 1) {
+    if (row < o) sh[threadIdx.x] += sh[threadIdx.x + o * cols];
+    __syncthreads();
+  }
+  if (row == 0 && i < n) grad[i] += sh[col];
+}
+constexpr int kBiasCols = 2;
+__global__ void __launch_bounds__(256)
+    k_sum_parts(const float* __restrict__ part, int P, long long n, int cols, float* __restrict__ grad,
+                const float* __restrict__ part_b, int Pb, int nb, int ldb, float* __restrict__ grad_b) {
+  const long long wb = (n + cols - 1) / cols;
+  if (blockIdx.x < wb) sum_columns(part, P, n, n, cols, blockIdx.x, grad);
+  else sum_columns(part_b, Pb, nb, ldb, kBiasCols, blockIdx.x - wb, grad_b);
+}
+
+// x (planes) to the channel-innermost BF16 input, padded channels 0; eight
+// channels of a pixel per store
+__global__ void __launch_bounds__(256) k_input(const float* __restrict__ x, int C, int CP, long long HW,
+                                               bf16* __restrict__ o) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HW;
+       i += (long long)gridDim.x * blockDim.x)
+    for (int c = 0; c < CP; c += 8) {
+      bf162 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        v[k] = __floats2bfloat162_rn(c + 2 * k < C ? x[(c + 2 * k) * HW + i] : 0.f,
+                                     c + 2 * k + 1 < C ? x[(c + 2 * k + 1) * HW + i] : 0.f);
+      *reinterpret_cast<uint4*>(o + i * CP + c) = *reinterpret_cast<const uint4*>(v);
+    }
+}
+
+// dL/dy (planes) to the head's hi + lo pair, and its bias gradient partials
+__global__ void __launch_bounds__(256) k_head_grad(const float* __restrict__ dy, int C, int CP,
+                                                   long long HW, bf16* __restrict__ hi,
+                                                   bf16* __restrict__ lo, float* __restrict__ part_b) {
+  __shared__ float sh[8][8];
+  for (int c = 0; c < CP; c += 8) {
+    float s[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] = 0.f;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HW;
+         i += (long long)gridDim.x * blockDim.x) {
+      bf162 h[4], l[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float v0 = c + 2 * k < C ? dy[(c + 2 * k) * HW + i] : 0.f;
+        const float v1 = c + 2 * k + 1 < C ? dy[(c + 2 * k + 1) * HW + i] : 0.f;
+        split2(v0, v1, h[k], l[k]);
+        s[2 * k] += v0;
+        s[2 * k + 1] += v1;
+      }
+      *reinterpret_cast<uint4*>(hi + i * CP + c) = *reinterpret_cast<const uint4*>(h);
+      *reinterpret_cast<uint4*>(lo + i * CP + c) = *reinterpret_cast<const uint4*>(l);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) sh[threadIdx.x >> 5][k] = s[k];
+    __syncthreads();
+    if (threadIdx.x < 8) {
+      float t = 0.f;
+      for (int r = 0; r < 8; ++r) t += sh[r][threadIdx.x];
+      part_b[(long long)blockIdx.x * CP + c + threadIdx.x] = t;
+    }
+  }
+}
+
+// The BF16 weights of every layer in the order the convolutions stage them:
+// forward [16 co][chunk of 16 ci][tap][co][ci], data gradient
+// [16 ci][chunk of 16 co][flipped tap][ci][co]; padded channels 0.
+struct PackLayer {
+  long long off_w, off_f, off_d;  // FP32 weights, packed forward, packed gradient
+  int co, ca, cb, coP, caP, cbP, kk;
+};
+constexpr int kMaxLayers = 15;
+struct PackTable {
+  PackLayer l[kMaxLayers];
+  int n;
+};
+__global__ void __launch_bounds__(256) k_pack(PackTable t, const float* __restrict__ w,
+                                              bf16* __restrict__ wf, bf16* __restrict__ wd) {
+  const PackLayer L = t.l[blockIdx.y];
+  const int ciP = L.caP + L.cbP, ci = L.ca + L.cb;
+  const long long n = (long long)L.coP * ciP * L.kk;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int p = 0; p < P; ++p) s += part[p * n + i];
-    grad[i] += s;
+    const int k = int(i & 15), r = int((i >> 4) & 15);
+    long long q = i >> 8;
+    const int tap = int(q % L.kk);
+    q /= L.kk;
+    auto value = [&](int co, int cp, int tp) {
+      const int c = cp < L.caP ? (cp < L.ca ? cp : -1) : (cp - L.caP < L.cb ? L.ca + cp - L.caP : -1);
+      return co < L.co && c >= 0 ? w[L.off_w + ((long long)co * ci + c) * L.kk + tp] : 0.f;
+    };
+    const int kf = int(q % (ciP / 16)), gf = int(q / (ciP / 16));
+    wf[L.off_f + i] = __float2bfloat16(value(gf * 16 + r, kf * 16 + k, tap));
+    const int kd = int(q % (L.coP / 16)), gd = int(q / (L.coP / 16));
+    wd[L.off_d + i] = __float2bfloat16(value(kd * 16 + k, gd * 16 + r, L.kk - 1 - tap));
   }
 }
 
-// Adjoint of the fused input transform: scatter dIn (conv grid H x W, CI
-// channels) into the FP32 gradients of the two operands (accumulating).
-__global__ void k_in_adjoint(const float* __restrict__ din, int H, int W, int ca, int mode,
-                             int cb, float* __restrict__ ga, float* __restrict__ gb) {
-  const long long total_a = (mode == IN_POOL ? 4LL : (mode == IN_UP ? 0 : 1)) * ca * H * W;
-  // plain / pool: one thread per element of the operand's own grid
-  if (mode == IN_PLAIN || mode == IN_POOL) {
-    const int Hs = mode == IN_POOL ? 2 * H : H, Ws = mode == IN_POOL ? 2 * W : W;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total_a;
-         i += (long long)gridDim.x * blockDim.x) {
-      const int c = int(i / ((long long)Hs * Ws));
-      const long long r = i % ((long long)Hs * Ws);
-      const int y = int(r / Ws), x = int(r % Ws);
-      const float g = mode == IN_POOL ? 0.25f * din[((long long)c * H + y / 2) * W + x / 2]
-                                      : din[((long long)c * H + y) * W + x];
-      ga[i] += g;
-    }
-  } else {
-    const int Hh = H / 2, Wh = W / 2;
-    const long long n = (long long)ca * Hh * Wh;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-      const int c = int(i / ((long long)Hh * Wh));
-      const long long r = i % ((long long)Hh * Wh);
-      const int y = int(r / Wh), x = int(r % Wh);
-      const float* p = din + ((long long)c * H + 2 * y) * W + 2 * x;
-      ga[i] += p[0] + p[1] + p[W] + p[W + 1];
-    }
-  }
-  if (gb) {
-    const long long nb = (long long)cb * H * W;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nb;
-         i += (long long)gridDim.x * blockDim.x)
-      gb[i] += din[(long long)ca * H * W + i];
-  }
-}
-
-__global__ void k_to_bf16(const float* __restrict__ a, __nv_bfloat16* __restrict__ b, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    b[i] = __float2bfloat16(a[i]);
-}
-
-// Adam (Kingma & Ba) on the FP32 master weights; refreshes the BF16 copy.
+// Adam (Kingma & Ba) on the FP32 master weights.
 __global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ g, __nv_bfloat16* __restrict__ wb, long long n,
-                       float lr, float b1, float b2, float eps, float c1, float c2, float scale) {
+                       float* __restrict__ g, long long n, float lr, float b1, float b2, float eps,
+                       float c1, float c2, float scale) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i] * scale;
@@ -466,24 +709,30 @@ __global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __re
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    w[i] = wi;
-    if (wb) wb[i] = __float2bfloat16(wi);
+    w[i] = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    g[i] = 0.f;
   }
 }
 
-// masked MSE: loss partials per block, dy = (y - t) mask / n
+// masked MSE: loss partials per block, dy = (y - t) mask / n.  One FP64
+// conversion and FMA per value: dy's quotient is formed in FP32 with 1/n as
+// inv + inv_lo and the product's rounding error (26 -> 7 us at 528 x 520;
+// with FP64 products and back-conversions that pipe was 81 % busy).
 __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, const float* __restrict__ t,
                                              const float* __restrict__ mask, int C, long long HW,
-                                             double inv_n, float* __restrict__ dy,
+                                             float inv, float inv_lo, float* __restrict__ dy,
                                              double* __restrict__ part) {
   double acc = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < C * HW;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HW;
        i += (long long)gridDim.x * blockDim.x) {
-    const float mk = mask ? mask[i % HW] : 1.f;
-    const float d = (y[i] - t[i]) * mk;
-    dy[i] = float(d * inv_n);
-    acc += 0.5 * double(d) * double(d) * inv_n;
+    const float mk = mask ? mask[i] : 1.f;
+    for (int c = 0; c < C; ++c) {
+      const long long j = c * HW + i;
+      const float d = (y[j] - t[j]) * mk;
+      const float q = d * inv, r = fmaf(d, inv_lo, fmaf(d, inv, -q));
+      dy[j] = isfinite(r) ? q + r : q;
+      acc += double(d) * double(d);
+    }
   }
   __shared__ double sh[256];
   sh[threadIdx.x] = acc;
@@ -495,9 +744,11 @@ __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, const 
   if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
+constexpr int kMaxGrid = 1216;  // eight 256-thread blocks per SM
+
 int grid1(long long n) {
   long long b = (n + 255) / 256;
-  if (b > 8192) b = 8192;
+  if (b > kMaxGrid) b = kMaxGrid;
   return int(b < 1 ? 1 : b);
 }
 
@@ -507,43 +758,42 @@ int grid1(long long n) {
 struct ConvLayer {
   int co, ci, k;
   long long off_w, off_b;  // offsets into the parameter vector
-  bool relu;
+  int ca, cb;              // input channels: first operand, concatenated skip
+  int coP, caP, cbP;       // padded to 16
+  long long off_f, off_d;  // packed weights, forward and data gradient
 };
 
 struct pf_unet {
   int H = 0, W = 0, nin = 0, nout = 0, L = 4;
-  int sms = 1;  // SMs of the device (the weight-gradient chunking)
+  int sms = 1;  // SMs of the device (tile and chunk choices)
   int ch[4] = {16, 32, 64, 128};
   cudaStream_t st = nullptr;
   std::vector<ConvLayer> layers;  // enc0a, enc0b, ..., enc3b, dec2a, dec2b, dec1a, ..., head
   long long nparam = 0;
   float *w32 = nullptr, *m = nullptr, *v = nullptr, *g = nullptr;
-  __nv_bfloat16* wbf = nullptr;
+  bf16 *wf = nullptr, *wd = nullptr;  // packed BF16 weights
+  PackTable pack{};
   int adam_t = 0;
-  // activations (BF16): input, and the output of every 3x3 layer
-  __nv_bfloat16* xin = nullptr;
-  std::vector<__nv_bfloat16*> act;  // one per layer (head excluded)
-  std::vector<float*> gact;         // FP32 gradient of each activation
-  float* gin = nullptr;             // gradient of the input (unused but kept for adjoint writes)
-  float* dscratch = nullptr;        // dIn of one conv (largest layer)
-  float* wpart = nullptr;           // weight-gradient partials
-  long long wpart_n = 0;
+  bf16* xin = nullptr;                 // input, channel-innermost
+  std::vector<bf16*> act;              // output of every 3x3 layer
+  bf16* pool[3] = {nullptr, nullptr, nullptr};   // 2x2 average of encoder level k
+  float* skip[3] = {nullptr, nullptr, nullptr};  // gradient of encoder level k through its skip
+  std::vector<bf16*> dh, dl;           // dL/d(pre-activation) of every layer, hi and lo
+  float* wpart = nullptr;              // weight-gradient partials
+  std::vector<float*> bpart;           // bias-gradient partials of every layer
+  // the backward pass's second stream: weight gradients beside the chain of
+  // data gradients
+  cudaStream_t side = nullptr;
+  std::vector<cudaEvent_t> ev;         // layer l's gradient is written; last: the side stream is done
   double* lpart = nullptr;
   double* h_loss = nullptr;
-  std::vector<void*> allocs;
+  void* slab = nullptr;  // device memory of everything above
 };
 
 namespace {
 
-pf_status ualloc(pf_unet* u, void** p, size_t bytes) {
-  if (cudaMalloc(p, bytes) != cudaSuccess) {
-    set_error("unet: cudaMalloc failed");
-    return PF_ENOMEM;
-  }
-  u->allocs.push_back(*p);
-  cudaMemsetAsync(*p, 0, bytes, u->st);
-  return PF_OK;
-}
+int pad16(int c) { return (c + 15) / 16 * 16; }
+long long conv_tiles(int H, int W) { return (long long)((W + TW - 1) / TW) * ((H + TH - 1) / TH); }
 
 // resolution of layer l's output: level of the layer
 int layer_level(const pf_unet* u, int l) {
@@ -552,29 +802,33 @@ int layer_level(const pf_unet* u, int l) {
   if (d >= 2 * (u->L - 1)) return 0;
   return u->L - 2 - d / 2;
 }
+bool is_head(const pf_unet* u, int l) { return l == int(u->layers.size()) - 1; }
+bool reads_pool(const pf_unet* u, int l) { return l > 0 && l < 2 * u->L && l % 2 == 0; }
+// first convolution of a decoder level: [up(below), skip of level k]
+bool reads_up(const pf_unet* u, int l) { return l >= 2 * u->L && !is_head(u, l) && (l - 2 * u->L) % 2 == 0; }
 
-ConvIn layer_input(const pf_unet* u, int l) {
-  ConvIn in{};
-  const int L = u->L;
+ConvSrc layer_input(const pf_unet* u, int l) {
+  ConvSrc in{};
+  const ConvLayer& c = u->layers[l];
+  in.ca = c.caP;
+  in.cb = c.cbP;
   if (l == 0) {
-    in.a = u->xin; in.ca = u->nin; in.mode = IN_PLAIN;
-  } else if (l < 2 * L) {
-    in.a = u->act[l - 1];
-    in.ca = u->layers[l - 1].co;
-    in.mode = (l % 2 == 0) ? IN_POOL : IN_PLAIN;
+    in.a = u->xin;
+  } else if (reads_pool(u, l)) {
+    in.a = u->pool[l / 2 - 1];
   } else {
-    const int d = l - 2 * L;
-    if (d >= 2 * (L - 1)) {  // head
-      in.a = u->act[l - 1]; in.ca = u->layers[l - 1].co; in.mode = IN_PLAIN;
-    } else if (d % 2 == 0) {  // first conv of a decoder level: [up(below), skip]
-      const int k = L - 2 - d / 2;
-      in.a = u->act[l - 1]; in.ca = u->layers[l - 1].co; in.mode = IN_UP;
-      in.b = u->act[2 * k + 1]; in.cb = u->ch[k];
-    } else {
-      in.a = u->act[l - 1]; in.ca = u->layers[l - 1].co; in.mode = IN_PLAIN;
+    in.a = u->act[l - 1];
+    if (reads_up(u, l)) {
+      in.up = 1;
+      in.b = u->act[2 * layer_level(u, l) + 1];
     }
   }
   return in;
+}
+
+cudaError_t pack_weights(pf_unet* u) {
+  k_pack<<<dim3(256, u->pack.n), 256, 0, u->st>>>(u->pack, u->w32, u->wf, u->wd);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -585,7 +839,12 @@ pf_status pf_unet_destroy(pf_unet* u) {
   if (!u) return PF_OK;
   if (u->st) cudaStreamSynchronize(u->st);
   else cudaDeviceSynchronize();
-  for (void* p : u->allocs) cudaFree(p);
+  if (u->side) {
+    cudaStreamSynchronize(u->side);
+    cudaStreamDestroy(u->side);
+  }
+  for (cudaEvent_t e : u->ev) cudaEventDestroy(e);
+  if (u->slab) cudaFree(u->slab);
   if (u->h_loss) cudaFreeHost(u->h_loss);
   delete u;
   return PF_OK;
@@ -618,62 +877,95 @@ pf_status pf_unet_create(int height, int width, int n_in, int n_out, const int c
   }
   for (int k = 0; k < 4; ++k) u->ch[k] = channels[k];
   u->st = static_cast<cudaStream_t>(stream);
-  long long off = 0;
-  auto add = [&](int co, int ci, int k, bool relu) {
-    ConvLayer c{co, ci, k, off, off + (long long)co * ci * k * k, relu};
-    off += (long long)co * ci * k * k + co;
+  long long off = 0, off_p = 0;
+  auto add = [&](int co, int ca, int cb, int k) {
+    ConvLayer c{};
+    c.co = co; c.ci = ca + cb; c.k = k; c.ca = ca; c.cb = cb;
+    c.coP = pad16(co); c.caP = pad16(ca); c.cbP = pad16(cb);
+    c.off_w = off;
+    c.off_b = off + (long long)co * c.ci * k * k;
+    off = c.off_b + co;
+    c.off_f = c.off_d = off_p;
+    off_p += (long long)c.coP * (c.caP + c.cbP) * k * k;
     u->layers.push_back(c);
   };
   int cprev = n_in;
   for (int k = 0; k < 4; ++k) {
-    add(u->ch[k], cprev, 3, true);
-    add(u->ch[k], u->ch[k], 3, true);
+    add(u->ch[k], cprev, 0, 3);
+    add(u->ch[k], u->ch[k], 0, 3);
     cprev = u->ch[k];
   }
   for (int k = 2; k >= 0; --k) {
-    add(u->ch[k], u->ch[k + 1] + u->ch[k], 3, true);
-    add(u->ch[k], u->ch[k], 3, true);
+    add(u->ch[k], u->ch[k + 1], u->ch[k], 3);
+    add(u->ch[k], u->ch[k], 0, 3);
   }
-  add(n_out, u->ch[0], 1, false);
+  add(n_out, u->ch[0], 0, 1);
   u->nparam = off;
-  pf_status rc;
+  for (const ConvLayer& c : u->layers)
+    u->pack.l[u->pack.n++] = PackLayer{c.off_w, c.off_f, c.off_d, c.co, c.ca, c.cb, c.coP, c.caP, c.cbP, c.k * c.k};
   const long long HW = (long long)height * width;
-  if ((rc = ualloc(u, (void**)&u->w32, sizeof(float) * off)) ||
-      (rc = ualloc(u, (void**)&u->m, sizeof(float) * off)) ||
-      (rc = ualloc(u, (void**)&u->v, sizeof(float) * off)) ||
-      (rc = ualloc(u, (void**)&u->g, sizeof(float) * off)) ||
-      (rc = ualloc(u, (void**)&u->wbf, sizeof(__nv_bfloat16) * off)) ||
-      (rc = ualloc(u, (void**)&u->xin, sizeof(__nv_bfloat16) * n_in * HW)) ||
-      (rc = ualloc(u, (void**)&u->lpart, sizeof(double) * 8192))) {
-    pf_unet_destroy(u);
-    return rc;
-  }
-  long long max_din = 0, max_part = 0;
+  std::vector<std::pair<void**, size_t>> need;
+  auto want = [&](void* p, size_t bytes) { need.push_back({static_cast<void**>(p), bytes}); };
+  want(&u->w32, sizeof(float) * off);
+  want(&u->m, sizeof(float) * off);
+  want(&u->v, sizeof(float) * off);
+  want(&u->g, sizeof(float) * off);
+  want(&u->wf, sizeof(bf16) * off_p);
+  want(&u->wd, sizeof(bf16) * off_p);
+  want(&u->xin, sizeof(bf16) * pad16(n_in) * HW);
+  want(&u->lpart, sizeof(double) * kMaxGrid);
   const int nl = int(u->layers.size());
   u->act.assign(nl - 1, nullptr);
-  u->gact.assign(nl - 1, nullptr);
+  u->dh.assign(nl, nullptr);
+  u->dl.assign(nl, nullptr);
+  u->bpart.assign(nl, nullptr);
+  long long max_part = 0;
   for (int l = 0; l < nl; ++l) {
     const int lev = layer_level(u, l);
+    const int Hl = height >> lev, Wl = width >> lev;
     const long long hw = HW >> (2 * lev);
     const ConvLayer& c = u->layers[l];
-    if (l < nl - 1) {
-      if ((rc = ualloc(u, (void**)&u->act[l], sizeof(__nv_bfloat16) * c.co * hw)) ||
-          (rc = ualloc(u, (void**)&u->gact[l], sizeof(float) * c.co * hw))) {
-        pf_unet_destroy(u);
-        return rc;
-      }
-    }
-    max_din = std::max(max_din, (long long)c.ci * hw);
-    const int P = wgrad_chunks(height >> lev, width >> lev, c.ci, c.co, u->sms);
-    max_part = std::max(max_part, (long long)P * ((long long)c.co * c.ci * c.k * c.k + c.co));
+    if (l < nl - 1) want(&u->act[l], sizeof(bf16) * c.coP * hw);
+    want(&u->dh[l], sizeof(bf16) * c.coP * hw);
+    want(&u->dl[l], sizeof(bf16) * c.coP * hw);
+    const int P = wgrad_chunks(Hl, Wl, c.caP + c.cbP, c.coP, u->sms);
+    max_part = std::max(max_part, (long long)P * c.co * c.ci * c.k * c.k);
+    // bias partials: one row per tile of the data gradient of the layer above
+    const int la = l < nl - 1 ? layer_level(u, l + 1) : 0;
+    const long long rows = l < nl - 1 ? conv_tiles(height >> la, width >> la) : kMaxGrid;
+    want(&u->bpart[l], sizeof(float) * rows * c.coP);
   }
-  if ((rc = ualloc(u, (void**)&u->dscratch, sizeof(float) * max_din)) ||
-      (rc = ualloc(u, (void**)&u->wpart, sizeof(float) * max_part)) ||
-      (rc = ualloc(u, (void**)&u->gin, sizeof(float) * n_in * HW))) {
+  for (int k = 0; k < 3; ++k) {
+    want(&u->pool[k], sizeof(bf16) * pad16(u->ch[k]) * (HW >> (2 * k + 2)));
+    want(&u->skip[k], sizeof(float) * pad16(u->ch[k]) * (HW >> (2 * k)));
+  }
+  want(&u->wpart, sizeof(float) * max_part);
+  // one allocation for all of them, each on a 256-byte boundary
+  size_t total = 0;
+  for (auto& n : need) total += (n.second + 255) / 256 * 256;
+  if (cudaMalloc((void**)&u->slab, total) != cudaSuccess) {
     pf_unet_destroy(u);
-    return rc;
+    set_error("unet: cudaMalloc failed");
+    return PF_ENOMEM;
   }
-  if (cudaMallocHost((void**)&u->h_loss, sizeof(double) * 8192) != cudaSuccess) {
+  cudaMemsetAsync(u->slab, 0, total, u->st);
+  total = 0;
+  for (auto& n : need) {
+    *n.first = static_cast<char*>(u->slab) + total;
+    total += (n.second + 255) / 256 * 256;
+  }
+  bool ok = cudaStreamCreateWithFlags(&u->side, cudaStreamNonBlocking) == cudaSuccess;
+  for (int l = 0; l <= nl && ok; ++l) {
+    cudaEvent_t e = nullptr;
+    ok = cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    if (ok) u->ev.push_back(e);
+  }
+  if (!ok) {
+    pf_unet_destroy(u);
+    set_error("unet_create: stream or event creation failed");
+    return PF_ECUDA;
+  }
+  if (cudaMallocHost((void**)&u->h_loss, sizeof(double) * kMaxGrid) != cudaSuccess) {
     pf_unet_destroy(u);
     set_error("unet_create: cudaMallocHost failed");
     return PF_ENOMEM;
@@ -703,12 +995,12 @@ pf_status pf_unet_set_params(pf_unet* u, const float* params) {
   }
   cudaError_t e = cudaMemcpyAsync(u->w32, params, sizeof(float) * u->nparam, cudaMemcpyHostToDevice, u->st);
   if (e == cudaSuccess) {
-    k_to_bf16<<<grid1(u->nparam), 256, 0, u->st>>>(u->w32, u->wbf, u->nparam);
+    e = pack_weights(u);
     cudaMemsetAsync(u->m, 0, sizeof(float) * u->nparam, u->st);
     cudaMemsetAsync(u->v, 0, sizeof(float) * u->nparam, u->st);
     cudaMemsetAsync(u->g, 0, sizeof(float) * u->nparam, u->st);
     u->adam_t = 0;
-    e = cudaStreamSynchronize(u->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(u->st);
   }
   if (e != cudaSuccess) {
     set_error(std::string("unet_set_params: ") + cudaGetErrorString(e));
@@ -740,23 +1032,27 @@ pf_status pf_unet_forward(pf_unet* u, const float* x, float* y) {
     return PF_EINVAL;
   }
   const long long HW = (long long)u->H * u->W;
-  k_to_bf16<<<grid1(u->nin * HW), 256, 0, u->st>>>(x, u->xin, u->nin * HW);
+  k_input<<<grid1(HW), 256, 0, u->st>>>(x, u->nin, pad16(u->nin), HW, u->xin);
+  cudaError_t e = cudaGetLastError();
   const int nl = int(u->layers.size());
-  for (int l = 0; l < nl; ++l) {
+  for (int l = 0; l < nl && e == cudaSuccess; ++l) {
     const ConvLayer& c = u->layers[l];
     const int lev = layer_level(u, l);
-    const int H = u->H >> lev, W = u->W >> lev;
-    const ConvIn in = layer_input(u, l);
-    const __nv_bfloat16* w = u->wbf + c.off_w;
-    const float* b = u->w32 + c.off_b;
-    MmaIn src{};
-    src.conv = in;
-    if (c.k == 3)
-      launch_conv_mma<3, false>(src, H, W, c.co, c.ci, c.ci, w, b, 1, u->act[l], nullptr, u->st);
-    else
-      launch_conv_mma<1, false>(src, H, W, c.co, c.ci, c.ci, w, b, 0, nullptr, y, u->st);
+    const int H = u->H >> lev, W = u->W >> lev, KC = (c.caP + c.cbP) / 16;
+    const ConvSrc in = layer_input(u, l);
+    EpiArgs a{};
+    a.bias = u->w32 + c.off_b;
+    a.co = c.co;
+    a.cp = c.coP;
+    if (is_head(u, l)) {
+      a.y = y;
+      e = launch_conv<1, EPI_HEAD>(in, nullptr, u->wf + c.off_f, H, W, c.coP, KC, a, u->sms, u->st);
+    } else {
+      a.out = u->act[l];
+      if (l < 2 * u->L && l % 2 == 1 && lev < u->L - 1) a.pool = u->pool[lev];
+      e = launch_conv<3, EPI_FWD>(in, nullptr, u->wf + c.off_f, H, W, c.coP, KC, a, u->sms, u->st);
+    }
   }
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error(std::string("unet_forward: ") + cudaGetErrorString(e));
     return PF_ECUDA;
@@ -773,51 +1069,63 @@ pf_status pf_unet_backward(pf_unet* u, const float* dy) {
   }
   const int nl = int(u->layers.size());
   const long long HW = (long long)u->H * u->W;
-  for (int l = 0; l < nl - 1; ++l) {
-    const int lev = layer_level(u, l);
-    cudaMemsetAsync(u->gact[l], 0, sizeof(float) * u->layers[l].co * (HW >> (2 * lev)), u->st);
-  }
-  for (int l = nl - 1; l >= 0; --l) {
+  int Pb = grid1(HW);  // bias partials of layer l
+  k_head_grad<<<Pb, 256, 0, u->st>>>(dy, u->nout, u->layers[nl - 1].coP, HW, u->dh[nl - 1], u->dl[nl - 1],
+                                     u->bpart[nl - 1]);
+  cudaError_t e = cudaGetLastError();
+  for (int l = nl - 1; l >= 0 && e == cudaSuccess; --l) {
     const ConvLayer& c = u->layers[l];
     const int lev = layer_level(u, l);
     const int H = u->H >> lev, W = u->W >> lev;
-    const ConvIn in = layer_input(u, l);
-    const float* dout = (l == nl - 1) ? dy : u->gact[l];
-    const __nv_bfloat16* out = (l == nl - 1) ? nullptr : u->act[l];
-    const int relu = c.relu ? 1 : 0;
-    // weight and bias gradients
-    const int P = wgrad_chunks(H, W, c.ci, c.co, u->sms);
+    const ConvSrc in = layer_input(u, l);
+    const bf16 *dh = u->dh[l], *dl = u->dl[l];
+    // weight and bias gradients, on the side stream once this layer's
+    // gradient is written (the deep levels' launches leave most SMs idle)
+    if ((e = cudaEventRecord(u->ev[l], u->st)) != cudaSuccess) break;
+    if ((e = cudaStreamWaitEvent(u->side, u->ev[l], 0)) != cudaSuccess) break;
+    const int P = wgrad_chunks(H, W, c.caP + c.cbP, c.coP, u->sms);
     const long long nw = (long long)c.co * c.ci * c.k * c.k;
-    float* part_b = u->wpart + (long long)P * nw;
-    if (c.k == 3)
-      launch_wgrad_mma<3>(dout, out, relu, in, H, W, c.co, P, u->wpart, part_b, u->st);
-    else
-      launch_wgrad_mma<1>(dout, out, relu, in, H, W, c.co, P, u->wpart, part_b, u->st);
-    k_sum_parts<<<grid1(nw), 256, 0, u->st>>>(u->wpart, P, nw, u->g + c.off_w);
-    k_sum_parts<<<grid1(c.co), 256, 0, u->st>>>(part_b, P, c.co, u->g + c.off_b);
-    if (l == 0) continue;  // no gradient needed for the input features
-    // data gradient on the conv grid, then the adjoint of the input transform
-    const __nv_bfloat16* w = u->wbf + c.off_w;
-    MmaIn src{};
-    src.dout = dout;
-    src.out = out;
-    src.relu = relu;
-    if (c.k == 3)
-      launch_conv_mma<3, true>(src, H, W, c.ci, c.co, c.ci, w, nullptr, 0, nullptr, u->dscratch, u->st);
-    else
-      launch_conv_mma<1, true>(src, H, W, c.ci, c.co, c.ci, w, nullptr, 0, nullptr, u->dscratch, u->st);
-    // operand a is the output of layer l-1; operand b (decoder) a skip
-    float* ga = u->gact[l - 1];
-    float* gb = nullptr;
-    if (in.cb > 0) {
-      const int d = l - 2 * u->L;
-      const int k = u->L - 2 - d / 2;
-      gb = u->gact[2 * k + 1];
+    e = c.k == 3 ? launch_wgrad<3>(dh, dl, c.coP, in, c.ca, c.cb, H, W, c.co, P, u->wpart, u->side)
+                 : launch_wgrad<1>(dh, dl, c.coP, in, c.ca, c.cb, H, W, c.co, P, u->wpart, u->side);
+    if (e != cudaSuccess) break;
+    const int cols = P >= 64 ? 8 : 32;
+    k_sum_parts<<<unsigned((nw + cols - 1) / cols + (c.co + kBiasCols - 1) / kBiasCols), 256, 0, u->side>>>(
+        u->wpart, P, nw, cols, u->g + c.off_w, u->bpart[l], Pb, c.co, c.coP, u->g + c.off_b);
+    e = cudaGetLastError();
+    if (l == 0 || e != cudaSuccess) continue;  // no gradient needed for the input features
+    // data gradient, down to dL/d(pre-activation) of layer l - 1
+    const ConvLayer& b = u->layers[l - 1];
+    ConvSrc s{};
+    s.a = dh;
+    s.ca = c.coP;
+    EpiArgs a{};
+    a.cp = b.coP;
+    a.act = u->act[l - 1];
+    a.hi = u->dh[l - 1];
+    a.lo = u->dl[l - 1];
+    a.part_b = u->bpart[l - 1];
+    const bf16* w = u->wd + c.off_d;
+    const int KC = c.coP / 16, N = c.caP + c.cbP;
+    if (reads_up(u, l)) {
+      a.ca = c.caP;
+      a.cb = c.cbP;
+      a.skip_out = u->skip[lev];
+      e = launch_conv<3, EPI_UP>(s, dl, w, H, W, N, KC, a, u->sms, u->st);
+    } else if (reads_pool(u, l)) {
+      a.skip_in = u->skip[lev - 1];
+      e = launch_conv<3, EPI_POOL>(s, dl, w, H, W, N, KC, a, u->sms, u->st);
+    } else if (is_head(u, l)) {
+      e = launch_conv<1, EPI_PLAIN>(s, dl, w, H, W, N, KC, a, u->sms, u->st);
+    } else {
+      e = launch_conv<3, EPI_PLAIN>(s, dl, w, H, W, N, KC, a, u->sms, u->st);
     }
-    k_in_adjoint<<<grid1((long long)c.ci * H * W * 4), 256, 0, u->st>>>(u->dscratch, H, W, in.ca, in.mode,
-                                                                         in.cb, ga, gb);
+    Pb = int(conv_tiles(H, W));
   }
-  cudaError_t e = cudaGetLastError();
+  // the caller's stream goes on once every gradient is added (also after a
+  // failed launch: what was started must not outlive the call's order)
+  const cudaError_t ej = cudaEventRecord(u->ev[nl], u->side);
+  const cudaError_t ew = cudaStreamWaitEvent(u->st, u->ev[nl], 0);
+  if (e == cudaSuccess) e = ej != cudaSuccess ? ej : ew;
   if (e != cudaSuccess) {
     set_error(std::string("unet_backward: ") + cudaGetErrorString(e));
     return PF_ECUDA;
@@ -832,10 +1140,10 @@ pf_status pf_unet_adam(pf_unet* u, float lr, float beta1, float beta2, float eps
   }
   u->adam_t += 1;
   const float c1 = 1.f - std::pow(beta1, float(u->adam_t)), c2 = 1.f - std::pow(beta2, float(u->adam_t));
-  k_adam<<<grid1(u->nparam), 256, 0, u->st>>>(u->w32, u->m, u->v, u->g, u->wbf, u->nparam, lr, beta1,
-                                               beta2, eps, c1, c2, grad_scale);
-  cudaMemsetAsync(u->g, 0, sizeof(float) * u->nparam, u->st);
+  k_adam<<<grid1(u->nparam), 256, 0, u->st>>>(u->w32, u->m, u->v, u->g, u->nparam, lr, beta1, beta2,
+                                               eps, c1, c2, grad_scale);
   cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = pack_weights(u);
   if (e != cudaSuccess) {
     set_error(std::string("unet_adam: ") + cudaGetErrorString(e));
     return PF_ECUDA;
@@ -851,8 +1159,10 @@ pf_status pf_unet_mse(pf_unet* u, const float* y, const float* t, const float* m
   }
   const long long HW = (long long)u->H * u->W;
   const double n = double(u->nout) * (mask ? n_valid : double(HW));
-  const int nb = std::min(grid1(u->nout * HW), 8192);
-  k_mse<<<nb, 256, 0, u->st>>>(y, t, mask, u->nout, HW, 1.0 / n, dy, u->lpart);
+  const int nb = grid1(HW);
+  const double inv = 1.0 / n;
+  k_mse<<<nb, 256, 0, u->st>>>(y, t, mask, u->nout, HW, float(inv), float(inv - double(float(inv))), dy,
+                               u->lpart);
   cudaError_t e = cudaMemcpyAsync(u->h_loss, u->lpart, sizeof(double) * nb, cudaMemcpyDeviceToHost, u->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(u->st);
   if (e != cudaSuccess) {
@@ -861,7 +1171,7 @@ pf_status pf_unet_mse(pf_unet* u, const float* y, const float* t, const float* m
   }
   double s = 0;
   for (int i = 0; i < nb; ++i) s += u->h_loss[i];
-  *loss = s;
+  *loss = 0.5 * s * inv;
   return PF_OK;
 }
 
