@@ -23,6 +23,7 @@ struct Mat {
   T lam, mu, Gc, ls, k, p;  // Lame, toughness, length scale, residual, pressure
   T inv_h;                  // 1/h
   T w;                      // Gauss weight times det J = h^d / 2^d
+  T gcl;                    // Gc / ls
 };
 
 // ---------------------------------------------------------------- 3D passes
@@ -248,38 +249,220 @@ __device__ __forceinline__ constexpr int sym_index(int i, int k) {
 // Every op takes the element's nodal values xe[f][a] (f = field plane,
 // a = corner) and, for hessvec / energy_diff, a second vector ve[f][a].
 
-// Energy of one element: sum_q w [g psi + Gc/2 (c^2/ls + ls |grad c|^2) + p g tr]
-template <int D, class T>
+// ---------------------------------------------------------------- monomials
+// An element field as c + x X + y Y + ... in its reference coordinates: 12
+// (4 in 2D) differences, after which values and derivatives at the Gauss
+// points are nested FMAs that share their inner terms (at fixed z, the
+// x-derivative is a + y b and the y-derivative a2 + x b with the same b).
+// Energy, gradient and Hessian coefficients are written this way because
+// FP64 and double-float instructions are what bounds them (in 3D 2 lanes of
+// FP64 per SM and clock; some 13 instructions per double-float operation).
+
+// a b + c
+template <class T>
+__device__ __forceinline__ T madd(T a, T b, T c) { return a * b + c; }
+// 2 x
+template <class T>
+__device__ __forceinline__ T twice(T x) { return x + x; }
+
+template <class T>
+struct Mono3 {
+  T c, x, y, z, xy, xz, yz, xyz;
+  __device__ __forceinline__ void set(const T f[8]) {
+    c = f[0];
+    x = f[1] - f[0];
+    y = f[2] - f[0];
+    z = f[4] - f[0];
+    const T x10 = f[3] - f[2], x01 = f[5] - f[4], x11 = f[7] - f[6], y01 = f[6] - f[4];
+    xy = x10 - x;
+    xz = x01 - x;
+    yz = y01 - y;
+    xyz = (x11 - x01) - xy;
+  }
+  // z-derivative at Gauss point (qx, qy), independent of z
+  __device__ __forceinline__ void dz(T (&o)[2][2]) const {
+#pragma unroll
+    for (int qy = 0; qy < 2; ++qy) {
+      const T t = qy ? T(PF_XI1) : T(PF_XI0), a = madd(t, yz, z), b = madd(t, xyz, xz);
+      o[0][qy] = madd(T(PF_XI0), b, a);
+      o[1][qy] = madd(T(PF_XI1), b, a);
+    }
+  }
+  // at height zq: x-derivative by qy, y-derivative by qx
+  __device__ __forceinline__ void dxy(T zq, T (&gx)[2], T (&gy)[2]) const {
+    const T a = madd(zq, xz, x), a2 = madd(zq, yz, y), b = madd(zq, xyz, xy);
+    gx[0] = madd(T(PF_XI0), b, a);
+    gx[1] = madd(T(PF_XI1), b, a);
+    gy[0] = madd(T(PF_XI0), b, a2);
+    gy[1] = madd(T(PF_XI1), b, a2);
+  }
+  // the same and the values v[qx][qy]
+  __device__ __forceinline__ void all(T zq, T (&v)[2][2], T (&gx)[2], T (&gy)[2]) const {
+    const T v0 = madd(zq, z, c), a = madd(zq, xz, x);
+    dxy(zq, gx, gy);
+#pragma unroll
+    for (int qx = 0; qx < 2; ++qx) {
+      const T s = madd(qx ? T(PF_XI1) : T(PF_XI0), a, v0);
+      v[qx][0] = madd(T(PF_XI0), gy[qx], s);
+      v[qx][1] = madd(T(PF_XI1), gy[qx], s);
+    }
+  }
+};
+
+template <class T>
+struct Mono2 {
+  T c, x, y, xy;
+  __device__ __forceinline__ void set(const T f[4]) {
+    c = f[0];
+    x = f[1] - f[0];
+    y = f[2] - f[0];
+    xy = (f[3] - f[2]) - x;
+  }
+  __device__ __forceinline__ void dxy(T (&gx)[2], T (&gy)[2]) const {
+    gx[0] = madd(T(PF_XI0), xy, x);
+    gx[1] = madd(T(PF_XI1), xy, x);
+    gy[0] = madd(T(PF_XI0), xy, y);
+    gy[1] = madd(T(PF_XI1), xy, y);
+  }
+  __device__ __forceinline__ void all(T (&v)[2][2], T (&gx)[2], T (&gy)[2]) const {
+    dxy(gx, gy);
+#pragma unroll
+    for (int qx = 0; qx < 2; ++qx) {
+      const T s = madd(qx ? T(PF_XI1) : T(PF_XI0), x, c);
+      v[qx][0] = madd(T(PF_XI0), gy[qx], s);
+      v[qx][1] = madd(T(PF_XI1), gy[qx], s);
+    }
+  }
+};
+
+// Energy of one element: sum_q w [g psi + Gc/2 (c^2/ls + ls |grad c|^2) + p g tr].
+// With raw differences and 1/h folded into the constants, psi + p tr is a
+// quadratic in the nine derivatives; the squares of the x-derivatives depend
+// on (qy, qz) only, those of the y- and z-derivatives likewise, so a Gauss
+// point adds three such sums and the six cross products (364 instead of 612
+// FP64 instructions per 3D element, 93 instead of 152 in 2D).  ROLL keeps the
+// two z layers of Gauss points a loop (see the double-float kernels).
+template <int D, class T, bool ROLL = false>
 __device__ __forceinline__ T elem_energy(const T (*xe)[1 << D], const Mat<T>& m) {
-  constexpr int NQ = 1 << D;
-  T gu[D][D][NQ], cv[NQ], gc[D][NQ], dummy[NQ];
+  const T x0 = T(PF_XI0), x1 = T(PF_XI1);
+  const T omk = T(1) - m.k, ih2 = m.inv_h * m.inv_h;
+  const T cl = m.lam * ih2, cm = m.mu * ih2, hcm = T(0.5) * cm, clm = madd(T(0.5), cl, cm);
+  const T cp = m.p * m.inv_h;
+  T acc = T(0), c2 = T(0), gr = T(0);
+  if constexpr (D == 3) {
+    Mono3<T> u[3], c;
 #pragma unroll
-  for (int i = 0; i < D; ++i) interp<D, T>(xe[i], dummy, gu[i]);
-  interp<D, T>(xe[D], cv, gc);
-  T e = T(0);
-  const T ils = T(1) / m.ls;  // one division per element, not one per Gauss point
+    for (int i = 0; i < 3; ++i) u[i].set(xe[i]);
+    c.set(xe[3]);
+    T uz[3][2][2], C[2][2];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    T G[D][D];
+    for (int i = 0; i < 3; ++i) u[i].dz(uz[i]);
+    {
+      T cz[2][2];
+      c.dz(cz);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const T t = cz[k & 1][k >> 1];
+        gr = madd(t, t, gr);
+        const T zx = uz[0][k & 1][k >> 1], zy = uz[1][k & 1][k >> 1], zz = uz[2][k & 1][k >> 1];
+        C[k & 1][k >> 1] = madd(zz, madd(clm, zz, cp), hcm * madd(zx, zx, zy * zy));
+      }
+    }
+#pragma unroll (ROLL ? 1 : 2)
+    for (int qz = 0; qz < 2; ++qz) {
+      const T zq = qz ? x1 : x0;
+      T ux[3][2], uy[3][2], v[2][2], cx[2], cy[2], A[2], B[2];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) u[i].dxy(zq, ux[i], uy[i]);
+      c.all(zq, v, cx, cy);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        gr = madd(cx[k], cx[k], madd(cy[k], cy[k], gr));
+        A[k] = madd(ux[0][k], madd(clm, ux[0][k], cp), hcm * madd(ux[1][k], ux[1][k], ux[2][k] * ux[2][k]));
+        B[k] = madd(uy[1][k], madd(clm, uy[1][k], cp), hcm * madd(uy[0][k], uy[0][k], uy[2][k] * uy[2][k]));
+        // cross-term factors
+        ux[0][k] = cl * ux[0][k];
+        ux[1][k] = cm * ux[1][k];
+        ux[2][k] = cm * ux[2][k];
+        uy[2][k] = cm * uy[2][k];
+      }
+#pragma unroll
+      for (int qx = 0; qx < 2; ++qx) {
+        const T ly = cl * uy[1][qx];
+#pragma unroll
+        for (int qy = 0; qy < 2; ++qy) {
+          T W = (A[qy] + B[qx]) + C[qx][qy];
+          W = madd(ux[0][qy], uy[1][qx] + uz[2][qx][qy], W);
+          W = madd(ly, uz[2][qx][qy], W);
+          W = madd(ux[1][qy], uy[0][qx], W);
+          W = madd(ux[2][qy], uz[0][qx][qy], W);
+          W = madd(uy[2][qx], uz[1][qx][qy], W);
+          const T cq = v[qx][qy], o = T(1) - cq;
+          acc = madd(madd(omk * o, o, m.k), W, acc);
+          c2 = madd(cq, cq, c2);
+        }
+      }
+    }
+  } else {
+    Mono2<T> u[2], c;
+    u[0].set(xe[0]);
+    u[1].set(xe[1]);
+    c.set(xe[2]);
+    T ux[2][2], uy[2][2], v[2][2], cx[2], cy[2], A[2], B[2];
+    u[0].dxy(ux[0], uy[0]);
+    u[1].dxy(ux[1], uy[1]);
+    c.all(v, cx, cy);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      gr = madd(cx[k], cx[k], madd(cy[k], cy[k], gr));
+      A[k] = madd(ux[0][k], madd(clm, ux[0][k], cp), hcm * (ux[1][k] * ux[1][k]));
+      B[k] = madd(uy[1][k], madd(clm, uy[1][k], cp), hcm * (uy[0][k] * uy[0][k]));
+      ux[0][k] = cl * ux[0][k];
+      ux[1][k] = cm * ux[1][k];
+    }
+#pragma unroll
+    for (int qx = 0; qx < 2; ++qx)
+#pragma unroll
+      for (int qy = 0; qy < 2; ++qy) {
+        T W = A[qy] + B[qx];
+        W = madd(ux[0][qy], uy[1][qx], W);
+        W = madd(ux[1][qy], uy[0][qx], W);
+        const T cq = v[qx][qy], o = T(1) - cq;
+        acc = madd(madd(omk * o, o, m.k), W, acc);
+        c2 = madd(cq, cq, c2);
+      }
+  }
+  // each derivative of c was squared once for its two Gauss points
+  return m.w * madd(T(0.5) * m.gcl, c2, madd(m.Gc * m.ls * ih2, gr, acc));
+}
+
+// What the gradient and the Hessian coefficients share at one Gauss point,
+// from the raw differences G[i][k] of the displacement: t_i = (sigma + p I)_ii
+// and t_ik = sigma_ik (physical), and W = (2 h) (psi + p tr).
+template <int D, class T>
+struct Point {
+  T t[D], ts[D == 3 ? 3 : 1], W;
+  __device__ __forceinline__ void set(const T (&G)[D][D], T lh, T mh, T mh2, T p) {
+    T tr = G[0][0] + G[1][1];
+    if constexpr (D == 3) tr = tr + G[D - 1][D - 1];
+    const T dia = madd(lh, tr, p);
+    W = p * tr;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      t[i] = madd(mh2, G[i][i], dia);
+      W = madd(t[i], G[i][i], W);
+    }
 #pragma unroll
     for (int i = 0; i < D; ++i)
 #pragma unroll
-      for (int k = 0; k < D; ++k) G[i][k] = gu[i][k][q] * m.inv_h;
-    Strain<D, T> s;
-    s.set(G);
-    const T psi = T(0.5) * m.lam * s.tr * s.tr + m.mu * s.ddot(s);
-    const T omc = T(1) - cv[q];
-    const T g = (T(1) - m.k) * omc * omc + m.k;
-    T gc2 = T(0);
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-      const T t = gc[k][q] * m.inv_h;
-      gc2 += t * t;
-    }
-    e += g * psi + T(0.5) * m.Gc * (cv[q] * cv[q] * ils + m.ls * gc2) + m.p * g * s.tr;
+      for (int k = i + 1; k < D; ++k) {
+        const int j = sym_index<D>(i, k) - D;
+        const T s = G[i][k] + G[k][i];
+        ts[j] = mh * s;
+        W = madd(ts[j], s, W);
+      }
   }
-  return m.w * e;
-}
+};
 
 // Strain invariants of a displacement gradient G (physical units):
 // tr = div u, ee = eps : eps, and the symmetric off-diagonal sums
@@ -325,7 +508,7 @@ __device__ __forceinline__ void elem_energy_diff(const T (*xe)[1 << D], const T 
   const T omk = T(1) - m.k;
   const T ih2 = m.inv_h * m.inv_h;
   const T hl = T(0.5) * m.lam * ih2, lam2 = m.lam * ih2, mu2 = m.mu * ih2, ph = m.p * m.inv_h;
-  const T gls = m.Gc * m.ls * ih2, hgls = T(0.5) * gls, gcl = m.Gc / m.ls, hgcl = T(0.5) * gcl;
+  const T gls = m.Gc * m.ls * ih2, hgls = T(0.5) * gls, gcl = m.gcl, hgcl = T(0.5) * gcl;
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
     T G[D][D], Gs[D][D];
@@ -368,52 +551,184 @@ __device__ __forceinline__ void elem_energy_diff(const T (*xe)[1 << D], const T 
 }
 
 // Gradient: u-rows  int g (sigma + p I) : grad phi,
-//           c-row   int [g'(psi + p tr) + Gc c/ls] phi + Gc ls grad c . grad phi
-template <int D, class T>
+//           c-row   int [g'(psi + p tr) + Gc c/ls] phi + Gc ls grad c . grad phi.
+// The test functions' sums go axis by axis: an x-derivative row is summed
+// over qx, weighted by N_ay, then by N_az, and enters the corners ax = 0, 1
+// with opposite signs; the others likewise.
+
+// N_0 and N_1 weighted sums of the two Gauss values along an axis
+template <class T>
+__device__ __forceinline__ void n_sums(T v0, T v1, T& n0, T& n1) {
+  const T x0 = T(PF_XI0), x1 = T(PF_XI1);
+  n0 = madd(x1, v0, x0 * v1);
+  n1 = madd(x0, v0, x1 * v1);
+}
+
+// Sums of one field's derivative rows over a z layer of Gauss points.
+template <class T>
+struct Rows3 {
+  T tx[2][2], ty[2][2], zs[2][2];  // [ay][az], [ax][az], [qx][qy]
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tx[i & 1][i >> 1] = ty[i & 1][i >> 1] = zs[i & 1][i >> 1] = T(0);
+  }
+  // sx by qy (summed over qx), sy by qx (summed over qy), weights of az
+  __device__ __forceinline__ void add_xy(T sx0, T sx1, T sy0, T sy1, T w0, T w1) {
+    T a, b;
+    n_sums(sx0, sx1, a, b);
+    tx[0][0] = madd(w0, a, tx[0][0]);
+    tx[0][1] = madd(w1, a, tx[0][1]);
+    tx[1][0] = madd(w0, b, tx[1][0]);
+    tx[1][1] = madd(w1, b, tx[1][1]);
+    n_sums(sy0, sy1, a, b);
+    ty[0][0] = madd(w0, a, ty[0][0]);
+    ty[0][1] = madd(w1, a, ty[0][1]);
+    ty[1][0] = madd(w0, b, ty[1][0]);
+    ty[1][1] = madd(w1, b, ty[1][1]);
+  }
+  __device__ __forceinline__ void corners(T* r) {
+    T tz[2][2];
+    {
+      T n[2][2];
+      n_sums(zs[0][0], zs[1][0], n[0][0], n[1][0]);
+      n_sums(zs[0][1], zs[1][1], n[0][1], n[1][1]);
+      n_sums(n[0][0], n[0][1], tz[0][0], tz[0][1]);
+      n_sums(n[1][0], n[1][1], tz[1][0], tz[1][1]);
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const int ax = a & 1, ay = (a >> 1) & 1, az = a >> 2;
+      T v = ax ? tx[ay][az] : -tx[ay][az];
+      v = ay ? v + ty[ax][az] : v - ty[ax][az];
+      r[a] = az ? v + tz[ax][ay] : v - tz[ax][ay];
+    }
+  }
+};
+
+template <int D, class T, bool ROLL = false>
 __device__ __forceinline__ void elem_gradient(const T (*xe)[1 << D], const Mat<T>& m,
                                               T (*out)[1 << D]) {
-  constexpr int NQ = 1 << D;
-  T gu[D][D][NQ], cv[NQ], gc[D][NQ], dummy[NQ];
+  const T x0 = T(PF_XI0), x1 = T(PF_XI1);
+  const T wh = m.w * m.inv_h, wo = wh * (T(1) - m.k), wk = wh * m.k, wc = m.w * m.gcl;
+  const T lh = m.lam * m.inv_h, mh = m.mu * m.inv_h, mh2 = twice(mh);
+  const T kc2 = twice(wh * m.Gc * m.ls * m.inv_h);  // a derivative of c stands for two Gauss points
+  if constexpr (D == 3) {
+    Mono3<T> u[3], c;
 #pragma unroll
-  for (int i = 0; i < D; ++i) interp<D, T>(xe[i], dummy, gu[i]);
-  interp<D, T>(xe[D], cv, gc);
-  T su[D][D][NQ], s0[NQ], sc[D][NQ];
-  const T omk = T(1) - m.k;
-  const T kc = m.w * m.Gc * m.ls * m.inv_h * m.inv_h;
-  const T gcl = m.Gc / m.ls;  // one division per element, not one per Gauss point
+    for (int i = 0; i < 3; ++i) u[i].set(xe[i]);
+    c.set(xe[3]);
+    T uz[3][2][2];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    T G[D][D];
+    for (int i = 0; i < 3; ++i) u[i].dz(uz[i]);
+    Rows3<T> r[3], rc;
+    T s[2][2][2];  // value row of c: [ax][ay][az]
 #pragma unroll
-    for (int i = 0; i < D; ++i)
+    for (int i = 0; i < 3; ++i) r[i].zero();
+    rc.zero();
 #pragma unroll
-      for (int k = 0; k < D; ++k) G[i][k] = gu[i][k][q] * m.inv_h;
-    StrainSym<D, T> e;
-    e.set(G);
-    const T psi = T(0.5) * m.lam * e.tr * e.tr + m.mu * e.ee;
-    const T omc = T(1) - cv[q];
-    const T g = omk * omc * omc + m.k;
-    const T dg = T(-2) * omk * omc;
-    // weight and 1/h of the test gradient folded into the coefficient
-    const T wg = m.w * m.inv_h * g;
-    const T dia = m.lam * e.tr + m.p, wgm = wg * m.mu;
+    for (int i = 0; i < 8; ++i) s[i & 1][(i >> 1) & 1][i >> 2] = T(0);
+#pragma unroll (ROLL ? 1 : 2)
+    for (int qz = 0; qz < 2; ++qz) {
+      const T zq = qz ? x1 : x0, w0 = qz ? x0 : x1, w1 = zq;
+      T ux[3][2], uy[3][2], v[2][2], s0[2][2];
+      T sx[3][2], sy[3][2];  // by qy, by qx
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-      su[i][i][q] = wg * (dia + T(2) * m.mu * G[i][i]);
+      for (int i = 0; i < 3; ++i) u[i].dxy(zq, ux[i], uy[i]);
+      {
+        T cx[2], cy[2];
+        c.all(zq, v, cx, cy);
+        rc.add_xy(cx[0], cx[1], cy[0], cy[1], w0, w1);
+      }
 #pragma unroll
-      for (int k = i + 1; k < D; ++k) {
-        const T v = wgm * e.off[sym_index<D>(i, k) - D];
-        su[i][k][q] = v;
-        su[k][i][q] = v;
+      for (int qx = 0; qx < 2; ++qx)
+#pragma unroll
+        for (int qy = 0; qy < 2; ++qy) {
+          T G[3][3];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            G[i][0] = ux[i][qy];
+            G[i][1] = uy[i][qx];
+            G[i][2] = uz[i][qx][qy];
+          }
+          Point<3, T> P;
+          P.set(G, lh, mh, mh2, m.p);
+          const T o = T(1) - v[qx][qy], q1 = wo * o, g = madd(q1, o, wk);
+          s0[qx][qy] = madd(-q1, P.W, wc * v[qx][qy]);
+          const T S01 = g * P.ts[0], S02 = g * P.ts[1], S12 = g * P.ts[2];
+          const T S[3][3] = {{g * P.t[0], S01, S02}, {S01, g * P.t[1], S12}, {S02, S12, g * P.t[2]}};
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            sx[i][qy] = qx ? sx[i][qy] + S[i][0] : S[i][0];
+            sy[i][qx] = qy ? sy[i][qx] + S[i][1] : S[i][1];
+            r[i].zs[qx][qy] = r[i].zs[qx][qy] + S[i][2];
+          }
+        }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) r[i].add_xy(sx[i][0], sx[i][1], sy[i][0], sy[i][1], w0, w1);
+      T n[2][2], nn[2][2];
+      n_sums(s0[0][0], s0[1][0], n[0][0], n[1][0]);
+      n_sums(s0[0][1], s0[1][1], n[0][1], n[1][1]);
+      n_sums(n[0][0], n[0][1], nn[0][0], nn[0][1]);
+      n_sums(n[1][0], n[1][1], nn[1][0], nn[1][1]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        s[i & 1][i >> 1][0] = madd(w0, nn[i & 1][i >> 1], s[i & 1][i >> 1][0]);
+        s[i & 1][i >> 1][1] = madd(w1, nn[i & 1][i >> 1], s[i & 1][i >> 1][1]);
       }
     }
-    s0[q] = m.w * (dg * (psi + m.p * e.tr) + gcl * cv[q]);
 #pragma unroll
-    for (int k = 0; k < D; ++k) sc[k][q] = kc * gc[k][q];
+    for (int i = 0; i < 3; ++i) r[i].corners(out[i]);
+    c.dz(rc.zs);
+    T rr[8];
+    rc.corners(rr);
+#pragma unroll
+    for (int a = 0; a < 8; ++a) out[3][a] = madd(kc2, rr[a], s[a & 1][(a >> 1) & 1][a >> 2]);
+  } else {
+    Mono2<T> u[2], c;
+    u[0].set(xe[0]);
+    u[1].set(xe[1]);
+    c.set(xe[2]);
+    T ux[2][2], uy[2][2], v[2][2], cx[2], cy[2], s0[2][2], sx[2][2], sy[2][2];
+    u[0].dxy(ux[0], uy[0]);
+    u[1].dxy(ux[1], uy[1]);
+    c.all(v, cx, cy);
+#pragma unroll
+    for (int qx = 0; qx < 2; ++qx)
+#pragma unroll
+      for (int qy = 0; qy < 2; ++qy) {
+        const T G[2][2] = {{ux[0][qy], uy[0][qx]}, {ux[1][qy], uy[1][qx]}};
+        Point<2, T> P;
+        P.set(G, lh, mh, mh2, m.p);
+        const T o = T(1) - v[qx][qy], q1 = wo * o, g = madd(q1, o, wk);
+        s0[qx][qy] = madd(-q1, P.W, wc * v[qx][qy]);
+        const T S01 = g * P.ts[0];
+        const T S[2][2] = {{g * P.t[0], S01}, {S01, g * P.t[1]}};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          sx[i][qy] = qx ? sx[i][qy] + S[i][0] : S[i][0];
+          sy[i][qx] = qy ? sy[i][qx] + S[i][1] : S[i][1];
+        }
+      }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      T a, b, e, f;
+      n_sums(i < 2 ? sx[i & 1][0] : cx[0], i < 2 ? sx[i & 1][1] : cx[1], a, b);  // by ay
+      n_sums(i < 2 ? sy[i & 1][0] : cy[0], i < 2 ? sy[i & 1][1] : cy[1], e, f);  // by ax
+      const T d[4] = {-a - e, a - f, e - b, b + f};
+      if (i < 2) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out[i][k] = d[k];
+      } else {
+        T n[2][2], nn[2][2];
+        n_sums(s0[0][0], s0[1][0], n[0][0], n[1][0]);
+        n_sums(s0[0][1], s0[1][1], n[0][1], n[1][1]);
+        n_sums(n[0][0], n[0][1], nn[0][0], nn[0][1]);
+        n_sums(n[1][0], n[1][1], nn[1][0], nn[1][1]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out[2][k] = madd(kc2, d[k], nn[k & 1][k >> 1]);
+      }
+    }
   }
-#pragma unroll
-  for (int i = 0; i < D; ++i) test<D, T>(nullptr, su[i], out[i]);
-  test<D, T>(s0, sc, out[D]);
 }
 
 // Gradient difference grad E_e(x + s) - grad E_e(x), written so that every
@@ -442,7 +757,7 @@ __device__ __forceinline__ void elem_gradient_diff(const T (*xe)[1 << D], const 
     interp<D, T>(se[D], scv, gsc);
     const T omk = T(1) - m.k;
     const T kc = m.w * m.Gc * m.ls * m.inv_h * m.inv_h;
-    const T gcl = m.Gc / m.ls;
+    const T gcl = m.gcl;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       T G[D][D], Gs[D][D];
@@ -507,45 +822,65 @@ __device__ __forceinline__ void elem_gradient_diff(const T (*xe)[1 << D], const 
 template <int D, class T>
 __device__ __forceinline__ void hess_coef(const T (*xe)[1 << D], const Mat<T>& m,
                                           T (*cf)[NCoef<D>::value]) {
-  constexpr int NQ = 1 << D;
-  T gu[D][D][NQ], cv[NQ], gdummy[D][NQ], dummy[NQ];
-#pragma unroll
-  for (int i = 0; i < D; ++i) interp<D, T>(xe[i], dummy, gu[i]);
-  interp<D, T>(xe[D], cv, gdummy);
-  const T omk = T(1) - m.k;
-  const T wh2 = m.w * m.inv_h * m.inv_h, wh = m.w * m.inv_h;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    T G[D][D];
-#pragma unroll
-    for (int i = 0; i < D; ++i)
-#pragma unroll
-      for (int k = 0; k < D; ++k) G[i][k] = gu[i][k][q] * m.inv_h;
-    T tr = T(0);
-#pragma unroll
-    for (int i = 0; i < D; ++i) tr += G[i][i];
-    T ee = T(0);  // eps : eps
+  const T omk = T(1) - m.k, wh = m.w * m.inv_h, wo = wh * omk, nwo2 = -twice(wo);
+  const T a1 = wo * m.inv_h, a0 = wh * m.inv_h * m.k, wc = m.w * m.gcl;
+  const T lh = m.lam * m.inv_h, mh = m.mu * m.inv_h, mh2 = twice(mh);
+  auto point = [&](const T (&G)[D][D], T cq, T (&o)[NCoef<D>::value]) {
+    Point<D, T> P;
+    P.set(G, lh, mh, mh2, m.p);
+    const T omc = T(1) - cq, dgw = nwo2 * omc;
+    o[0] = madd(a1 * omc, omc, a0);
+    o[1] = madd(wo, P.W, wc);
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-      ee += G[i][i] * G[i][i];
+      o[2 + i] = dgw * P.t[i];
 #pragma unroll
-      for (int k = i + 1; k < D; ++k) {
-        const T e = T(0.5) * (G[i][k] + G[k][i]);
-        ee += T(2) * e * e;
+      for (int k = i + 1; k < D; ++k)
+        o[2 + sym_index<D>(i, k)] = dgw * P.ts[sym_index<D>(i, k) - D];
+    }
+  };
+  if constexpr (D == 3) {
+    Mono3<T> u[3], c;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) u[i].set(xe[i]);
+    c.set(xe[3]);
+    T uz[3][2][2];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) u[i].dz(uz[i]);
+#pragma unroll
+    for (int qz = 0; qz < 2; ++qz) {
+      const T zq = qz ? T(PF_XI1) : T(PF_XI0);
+      T ux[3][2], uy[3][2], v[2][2], cx[2], cy[2];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) u[i].dxy(zq, ux[i], uy[i]);
+      c.all(zq, v, cx, cy);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int qx = q & 1, qy = q >> 1;
+        T G[3][3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          G[i][0] = ux[i][qy];
+          G[i][1] = uy[i][qx];
+          G[i][2] = uz[i][qx][qy];
+        }
+        point(G, v[qx][qy], cf[q + 4 * qz]);
       }
     }
-    const T psi = T(0.5) * m.lam * tr * tr + m.mu * ee;
-    const T omc = T(1) - cv[q];
-    const T g = omk * omc * omc + m.k;
-    const T dgw = T(-2) * omk * omc * wh;
-    cf[q][0] = wh2 * g;
-    cf[q][1] = m.w * (T(2) * omk * (psi + m.p * tr) + m.Gc / m.ls);
-    const T diag = m.lam * tr + m.p;
+  } else {
+    Mono2<T> u[2], c;
+    u[0].set(xe[0]);
+    u[1].set(xe[1]);
+    c.set(xe[2]);
+    T ux[2][2], uy[2][2], v[2][2], cx[2], cy[2];
+    u[0].dxy(ux[0], uy[0]);
+    u[1].dxy(ux[1], uy[1]);
+    c.all(v, cx, cy);
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-      cf[q][2 + i] = dgw * (diag + T(2) * m.mu * G[i][i]);
-#pragma unroll
-      for (int k = i + 1; k < D; ++k) cf[q][2 + sym_index<D>(i, k)] = dgw * m.mu * (G[i][k] + G[k][i]);
+    for (int q = 0; q < 4; ++q) {
+      const int qx = q & 1, qy = q >> 1;
+      const T G[2][2] = {{ux[0][qy], uy[0][qx]}, {ux[1][qy], uy[1][qx]}};
+      point(G, v[qx][qy], cf[q]);
     }
   }
 }
@@ -627,7 +962,7 @@ __device__ __forceinline__ void elem_hessdiag(const T (*xe)[1 << D], const Mat<T
     const T psi = T(0.5) * m.lam * e.tr * e.tr + m.mu * e.ddot(e);
     const T omk = T(1) - m.k, omc = T(1) - cv[q];
     gq[q] = m.w * (omk * omc * omc + m.k);
-    mq[q] = m.w * (T(2) * omk * (psi + m.p * e.tr) + m.Gc / m.ls);
+    mq[q] = m.w * (T(2) * omk * (psi + m.p * e.tr) + m.gcl);
   }
   const T h2 = m.inv_h * m.inv_h;
 #pragma unroll

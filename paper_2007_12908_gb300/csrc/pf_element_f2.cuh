@@ -156,7 +156,7 @@ __device__ __forceinline__ void coef(const float (*xe)[8], const Mat<float>& m, 
     const float2 g = fma2(mul2(bc(omk), omc), omc, bc(m.k));
     const float2 dgw = mul2(bc(-2.f * omk * wh), omc);
     cf[pp].A = mul2(bc(wh2), g);
-    cf[pp].M = mul2(bc(m.w), fma2(bc(2.f * omk), fma2(bc(m.p), tr, psi), bc(m.Gc / m.ls)));
+    cf[pp].M = mul2(bc(m.w), fma2(bc(2.f * omk), fma2(bc(m.p), tr, psi), bc(m.gcl)));
     const float2 diag = fma2(bc(m.lam), tr, bc(m.p));
     const float2 tmu = bc(2.f * m.mu);
     cf[pp].B[0] = mul2(dgw, fma2(tmu, G[0][0], diag));

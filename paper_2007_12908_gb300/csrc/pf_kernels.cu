@@ -47,6 +47,7 @@ Mat<double> make_mat(const Geom& g, double E, double nu, double Gc, double ls, d
   m.p = p;
   m.inv_h = 1.0 / g.h;
   m.w = std::pow(g.h, g.dim) / double(1 << g.dim);
+  m.gcl = Gc / ls;
   return m;
 }
 
@@ -54,7 +55,7 @@ template <class T>
 static Mat<T> cast_mat(const Mat<double>& m) {
   Mat<T> r;
   r.lam = T(m.lam); r.mu = T(m.mu); r.Gc = T(m.Gc); r.ls = T(m.ls); r.k = T(m.k);
-  r.p = T(m.p); r.inv_h = T(m.inv_h); r.w = T(m.w);
+  r.p = T(m.p); r.inv_h = T(m.inv_h); r.w = T(m.w); r.gcl = T(m.gcl);
   return r;
 }
 
@@ -92,6 +93,16 @@ __device__ __forceinline__ void elem_coords(const Geom& g, long long e, int& ex,
     ey = int(r);
     ez = 0;
   }
+}
+
+// Threads per block of the one-element-per-thread FP64 passes: an FP64
+// instruction holds its SM's pipe for 16 cycles per warp, so a grid of few
+// elements is spread over as many SMs as it has warps (69 x 45 nodes in
+// blocks of 256: 12 SMs at work, 18 us for the energy).
+static int fp64_threads(const Geom& g, int most) {
+  int t = most;
+  while (t > 32 && g.NE < 2LL * 152 * t) t /= 2;
+  return t;
 }
 
 // ------------------------------------------------------------ energy
@@ -772,11 +783,12 @@ cudaError_t elem_hessvec(const Geom& g, const Mat<double>& m, const void* x, con
 
 cudaError_t elem_hess_coef(const Geom& g, const Mat<double>& m, const double* x, double* coef,
                            cudaStream_t st) {
-  const int nb = int(std::min<long long>((g.NE + 255) / 256, 8LL * 1216));
+  const int nt = fp64_threads(g, 256);
+  const int nb = int(std::min<long long>((g.NE + nt - 1) / nt, 8LL * 1216));
   if (g.dim == 3)
-    k_hess_coef<3, double><<<nb, 256, 0, st>>>(g, cast_mat<double>(m), x, coef);
+    k_hess_coef<3, double><<<nb, nt, 0, st>>>(g, cast_mat<double>(m), x, coef);
   else
-    k_hess_coef<2, double><<<nb, 256, 0, st>>>(g, cast_mat<double>(m), x, coef);
+    k_hess_coef<2, double><<<nb, nt, 0, st>>>(g, cast_mat<double>(m), x, coef);
   return cudaGetLastError();
 }
 
@@ -838,14 +850,16 @@ __global__ void __launch_bounds__(256) k_grad_gather(Geom g, const double* __res
 
 cudaError_t elem_gradient_fp64(const Geom& g, const Mat<double>& m, const double* x, double* y,
                                double* scratch, cudaStream_t st) {
-  const int nb = int(std::min<long long>((g.NE + 127) / 128, 32LL * 1216));
-  const int nn = int(std::min<long long>((g.N + 255) / 256, 16LL * 1216));
+  const int nt = fp64_threads(g, 128);
+  const int nb = int(std::min<long long>((g.NE + nt - 1) / nt, 32LL * 1216));
+  const int gt = fp64_threads(g, 256);
+  const int nn = int(std::min<long long>((g.N + gt - 1) / gt, 16LL * 1216));
   if (g.dim == 3) {
-    k_grad_elem<3><<<nb, 128, 0, st>>>(g, m, x, scratch);
-    k_grad_gather<3><<<nn, 256, 0, st>>>(g, scratch, y);
+    k_grad_elem<3><<<nb, nt, 0, st>>>(g, m, x, scratch);
+    k_grad_gather<3><<<nn, gt, 0, st>>>(g, scratch, y);
   } else {
-    k_grad_elem<2><<<nb, 128, 0, st>>>(g, m, x, scratch);
-    k_grad_gather<2><<<nn, 256, 0, st>>>(g, scratch, y);
+    k_grad_elem<2><<<nb, nt, 0, st>>>(g, m, x, scratch);
+    k_grad_gather<2><<<nn, gt, 0, st>>>(g, scratch, y);
   }
   return cudaGetLastError();
 }
@@ -855,10 +869,16 @@ cudaError_t elem_gradient_fp64(const Geom& g, const Mat<double>& m, const double
 // FP32 pipes: x is split once per call into (hi, lo) planes, the element
 // algebra is the FP64 code instantiated with df, and nodal sums and totals
 // are formed in df (gradient) or FP64 (energy totals across threads).
+// A double-float operation is 7 to 15 instructions, so an element's code is
+// what bounds these passes: the fully unrolled gradient (11,400 instructions,
+// 183 KB) was fetched from L2 by every warp and issued 31 % of the time.  The
+// two z layers of Gauss points are a loop now (9,400 instructions executed,
+// well under the instruction cache's size in memory): issue 70 %, 828 ->
+// 305 us on 97 x 105 x 89 nodes; the energy 268 -> 167 us.
 __global__ void k_to_df(long long n, const double* __restrict__ x, float2* __restrict__ xd) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    const df v = df_from(x[i]);
+    const df v = df_split(x[i]);
     xd[i] = make_float2(v.hi, v.lo);
   }
 }
@@ -888,7 +908,7 @@ __global__ void __launch_bounds__(128) k_grad_elem_df(Geom g, Mat<df> m,
     elem_coords<D>(g, e, ex, ey, ez);
     df xe[F][NC], out[F][NC];
     gather_df<D>(g, xd, ex, ey, ez, xe);
-    elem_gradient<D, df>(xe, m, out);
+    elem_gradient<D, df, true>(xe, m, out);
 #pragma unroll
     for (int f = 0; f < F; ++f)
 #pragma unroll
@@ -942,7 +962,7 @@ __global__ void __launch_bounds__(256) k_energy_df(Geom g, Mat<df> m, const floa
     elem_coords<D>(g, e, ex, ey, ez);
     df xe[D + 1][1 << D];
     gather_df<D>(g, xd, ex, ey, ez, xe);
-    part = add_accurate(part, elem_energy<D, df>(xe, m));
+    part = add_accurate(part, elem_energy<D, df, true>(xe, m));
   }
   double acc[1] = {df_to_double(part)};
   grid_finish<1, OpSum>(acc, partials, counter, out);
@@ -971,14 +991,15 @@ cudaError_t elem_gradient_df(const Geom& g, const Mat<double>& m, const double* 
   float2* contrib = reinterpret_cast<float2*>(scratch) + off;
   const long long n = (long long)(g.dim + 1) * g.N;
   const int nv = int(std::min<long long>((n + 255) / 256, 16LL * 1216));
-  const int nb = int(std::min<long long>((g.NE + 127) / 128, 32LL * 1216));
+  const int nt = fp64_threads(g, 128);
+  const int nb = int(std::min<long long>((g.NE + nt - 1) / nt, 32LL * 1216));
   const int nn = int(std::min<long long>((g.N + 255) / 256, 16LL * 1216));
   k_to_df<<<nv, 256, 0, st>>>(n, x, xd);
   if (g.dim == 3) {
-    k_grad_elem_df<3><<<nb, 128, 0, st>>>(g, cast_mat<df>(m), xd, contrib);
+    k_grad_elem_df<3><<<nb, nt, 0, st>>>(g, cast_mat<df>(m), xd, contrib);
     k_grad_gather_df<3><<<nn, 256, 0, st>>>(g, contrib, y);
   } else {
-    k_grad_elem_df<2><<<nb, 128, 0, st>>>(g, cast_mat<df>(m), xd, contrib);
+    k_grad_elem_df<2><<<nb, nt, 0, st>>>(g, cast_mat<df>(m), xd, contrib);
     k_grad_gather_df<2><<<nn, 256, 0, st>>>(g, contrib, y);
   }
   return cudaGetLastError();
@@ -991,12 +1012,12 @@ cudaError_t elem_energy_df(const Geom& g, const Mat<double>& m, const double* x,
   float2* xd = reinterpret_cast<float2*>(scratch);
   const long long n = (long long)(g.dim + 1) * g.N;
   const int nv = int(std::min<long long>((n + 255) / 256, 16LL * 1216));
-  const int nb = reduce_grid(g.NE, 256);
+  const int nt = fp64_threads(g, 256), nb = reduce_grid(g.NE, nt);
   k_to_df<<<nv, 256, 0, st>>>(n, x, xd);
   if (g.dim == 3)
-    k_energy_df<3><<<nb, 256, 0, st>>>(g, cast_mat<df>(m), xd, s.partials, s.counter, out);
+    k_energy_df<3><<<nb, nt, 0, st>>>(g, cast_mat<df>(m), xd, s.partials, s.counter, out);
   else
-    k_energy_df<2><<<nb, 256, 0, st>>>(g, cast_mat<df>(m), xd, s.partials, s.counter, out);
+    k_energy_df<2><<<nb, nt, 0, st>>>(g, cast_mat<df>(m), xd, s.partials, s.counter, out);
   return cudaGetLastError();
 }
 
@@ -1185,8 +1206,8 @@ cudaError_t elem_hessvec_mixed(const Geom& g, const Mat<double>& m, const float*
 template <int D, class T>
 static cudaError_t launch_energy(const Geom& g, const Mat<double>& m, const void* x,
                                  const Scratch& s, double* out, cudaStream_t st) {
-  const int nb = reduce_grid(g.NE, 256);
-  k_energy<D, T><<<nb, 256, 0, st>>>(g, m, static_cast<const T*>(x), s.partials, s.counter, out);
+  const int nt = fp64_threads(g, 256);
+  k_energy<D, T><<<reduce_grid(g.NE, nt), nt, 0, st>>>(g, m, static_cast<const T*>(x), s.partials, s.counter, out);
   return cudaGetLastError();
 }
 
@@ -1223,8 +1244,8 @@ template <int D, class T>
 static cudaError_t launch_energy_diff(const Geom& g, const Mat<double>& m, const void* x,
                                       const void* sv, const Scratch& s, double* out,
                                       cudaStream_t st) {
-  const int nb = reduce_grid(g.NE, 256);
-  k_energy_diff<D, T><<<nb, 256, 0, st>>>(g, m, static_cast<const T*>(x),
+  const int nt = fp64_threads(g, 256);
+  k_energy_diff<D, T><<<reduce_grid(g.NE, nt), nt, 0, st>>>(g, m, static_cast<const T*>(x),
                                            static_cast<const T*>(sv), s.partials, s.counter, out);
   return cudaGetLastError();
 }
