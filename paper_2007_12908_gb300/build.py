@@ -13,7 +13,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libpf.so")
 SOURCES = ["pf_kernels.cu", "pf_solver.cu", "pf_api.cu", "pf_noalloc.cu", "pf_unet.cu", "pf_learned.cu",
            "pf_state.cu", "pf_galerkin.cu", "pf_batch.cu", "pf_transfer.cu",
-           "pf_assemble.cu"]
+           "pf_assemble.cu", "pf_subproblem.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "--extended-lambda", "-Xcompiler", "-fPIC",
          "-I", os.path.join(ROOT, "include")]

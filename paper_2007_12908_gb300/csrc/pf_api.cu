@@ -190,6 +190,9 @@ pf_status pf_mesh_hierarchy_create(const pf_mesh_desc* d, pf_hierarchy** out) {
   const int F = d->dim + 1;
   long long part = 0;
   for (const Geom& g : h->geo) part = std::max(part, etile_part_count(g));
+  long long sub_rows = 0;  // rows of the largest level whose subproblem is one launch
+  for (const Geom& g : h->geo)
+    if (subproblem_small(g)) sub_rows = std::max(sub_rows, F * g.N);
   {
     // Everything the hierarchy will hold, checked against the device's free
     // memory before the first allocation: a hierarchy that cannot fit is
@@ -207,6 +210,9 @@ pf_status pf_mesh_hierarchy_create(const pf_mesh_desc* d, pf_hierarchy** out) {
     add(double(sizeof(CgCtrl)));
     add(16.0 * part);
     add(4.0);
+    add(8.0 * kSubPartials);
+    add(256.0);
+    add(8.0 * 5 * sub_rows);
     for (int l = 0; l < h->L; ++l) {
       const double n = double(F) * double(h->geo[l].N);
       for (int v = 0; v < 24; ++v) add(8.0 * (n + 4));
@@ -246,12 +252,21 @@ pf_status pf_mesh_hierarchy_create(const pf_mesh_desc* d, pf_hierarchy** out) {
     pf_mesh_hierarchy_destroy(h);
     return rc;
   }
+  if ((rc = alloc(h, (void**)&h->sub_partials, sizeof(double) * kSubPartials)) ||
+      (rc = alloc(h, (void**)&h->sub_bar, 256)) ||
+      (sub_rows > 0 && (rc = alloc(h, &h->sub_work, sizeof(double) * 5 * sub_rows)))) {
+    pf_mesh_hierarchy_destroy(h);
+    return rc;
+  }
+  h->sub_ctl = reinterpret_cast<SubCtrl*>(h->sub_bar + 32);
+  cudaMemsetAsync(h->sub_bar, 0, 256, h->st);
   if (cudaMallocHost((void**)&h->h_res, sizeof(double) * kMaxSlots) != cudaSuccess ||
-      cudaMallocHost((void**)&h->h_ctrl, sizeof(CgCtrl)) != cudaSuccess) {
+      cudaMallocHost((void**)&h->h_ctrl, sizeof(CgCtrl) + sizeof(SubCtrl)) != cudaSuccess) {
     pf_mesh_hierarchy_destroy(h);
     set_error("cudaMallocHost failed");
     return PF_ENOMEM;
   }
+  h->h_sub_ctl = reinterpret_cast<SubCtrl*>(h->h_ctrl + 1);
   cudaMemsetAsync(h->scratch.counter, 0, sizeof(unsigned), h->st);
   cudaMemsetAsync(h->p_dev, 0, sizeof(float), h->st);  // the material starts at p = 0
   cudaMemsetAsync(h->c_prev, 0, sizeof(double) * h->geo.back().N, h->st);

@@ -47,6 +47,13 @@ struct pf_hierarchy {
   double* c_prev_save = nullptr;  // c_prev at the start of a load step (restored on failure)
   pf::CgCtrl* ctrl = nullptr;    // device CG control block
   pf::CgCtrl* h_ctrl = nullptr;  // pinned host mirror
+  // one-launch subproblems of small levels (pf_subproblem.cu)
+  double* sub_partials = nullptr;
+  void* sub_work = nullptr;          // 5 vectors of the largest small level
+  unsigned* sub_bar = nullptr;       // barrier words, then a SubCtrl
+  pf::SubCtrl* sub_ctl = nullptr;
+  pf::SubCtrl* h_sub_ctl = nullptr;  // pinned host mirror
+  bool sub_ok = true;                // false once a wait ran out or the launch was refused
   void* etile_part = nullptr;  // node sums of the element-owned FP32 Hessian tiles (3D)
   float* p_dev = nullptr;      // the pressure in FP32 on the device (kept by pf_pressure_set)
   // executable graphs of the FP32 CG loop per level (built by the solver)

@@ -203,6 +203,34 @@ cudaError_t galerkin_apply(const Geom& g, const float* S, const void* v, void* y
 cudaError_t hess2_march(const Geom& g, const Mat<double>& m, const float* x, const float* v,
                         float* y, const int* skip, cudaStream_t st);
 
+// The trust-region subproblem of a small level in one cooperative launch
+// (pf_subproblem.cu): min gr.s + s.H s / 2 over lo <= s <= hi with H a stencil
+// (FP64, or FP32 with FP32 arithmetic), the step to s.  Fields of SubCtrl are
+// written when it is done; failed: a wait ran out and s is not written.
+struct SubCtrl {
+  int failed;     // cleared by the caller
+  unsigned base;  // arrivals at the barrier when the last launch had ended
+  int used, restarts, hv_cauchy, hv_search;
+};
+struct SubIn {
+  const void* stencil;
+  bool fp32;
+  const double *gr, *lo, *hi;
+  const void* mi;     // Jacobi inverse in the stencil's precision, or null
+  double* s;
+  void* work;         // 5 level vectors in the stencil's precision
+  double* partials;   // kSubPartials doubles
+  unsigned* bar;      // zero, as ctl, before the first launch
+  SubCtrl* ctl;
+  double delta, cauchy_c;
+  int backtracks, cg_max, max_restarts;
+};
+constexpr int kSubPartials = 2 * 4 * 1216;
+// Whether the level is small enough; cudaErrorNotSupported from the launch
+// where it is not, or where the device cannot hold the CTAs at once.
+bool subproblem_small(const Geom& g);
+cudaError_t subproblem_coop(const Geom& g, const SubIn& in, cudaStream_t st);
+
 // Fracture band rasterisation into the c plane (FP64) of x and c_prev.
 // rows: device array of precomputed shape rows of kRasterRow doubles (see
 // pf_fractures_set); kind 0 line (2D), 1 disc, 2 rectangle (3D).

@@ -1117,6 +1117,7 @@ struct Solver {
       paper_subproblem(l, cg_max);
       return;
     }
+    if (one_launch(l, delta, cg_max)) return;
     if (!sub32(l)) {
       subproblem_t<double>(l, delta, cg_max,
                            {B.g, B.lo, B.hi, B.minv, B.s, B.Hs, B.r, B.p, B.q, B.w, B.Hw, B.t3,
@@ -1154,6 +1155,65 @@ struct Solver {
     const float* s32 = v.s;
     double* s = B.s;
     map(n, [=] __device__(long long i) { s[i] = double(s32[i]); });
+  }
+
+  // The subproblem of a small level whose model Hessian is a stored stencil
+  // (the FP64 one, or the mixed mode's Galerkin operator) in one cooperative
+  // launch; false where it does not apply (the caller solves it otherwise).
+  bool one_launch(int l, double delta, int cg_max) {
+    if (!H->sub_ok || !subproblem_small(H->geo[l])) return false;
+    LevelBuf& B = H->lv[l];
+    SubIn in{};
+    if (gstored(l)) {
+      in.stencil = B.gs;
+      in.fp32 = true;
+    } else if (!mixed && !galerkin(l)) {
+      in.stencil = B.stencil;
+    } else {
+      return false;
+    }
+    in.gr = B.g;
+    in.lo = B.lo;
+    in.hi = B.hi;
+    in.mi = P.precondition ? B.minv : nullptr;
+    in.s = B.s;
+    in.work = H->sub_work;
+    in.partials = H->sub_partials;
+    in.bar = H->sub_bar;
+    in.ctl = H->sub_ctl;
+    in.delta = delta;
+    in.cauchy_c = P.cauchy_c;
+    in.backtracks = P.cauchy_backtracks;
+    in.cg_max = cg_max;
+    in.max_restarts = P.max_restarts;
+    const cudaError_t e = subproblem_coop(H->geo[l], in, st);
+    if (e == cudaErrorNotSupported) return false;  // this level's CTAs do not all fit
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+      cudaGetLastError();
+      H->sub_ok = false;
+      return false;
+    }
+    ck(e, "subproblem");
+    S.launches += 1;
+    ck(cudaMemcpyAsync(H->h_sub_ctl, H->sub_ctl, sizeof(SubCtrl), cudaMemcpyDeviceToHost, st), "sub_ctl");
+    ck(cudaStreamSynchronize(st), "sync");
+    const SubCtrl c = *H->h_sub_ctl;
+    if (c.failed) {
+      // a wait ran out (the CTAs were not all resident): clear the barrier and
+      // leave this hierarchy's subproblems to separate launches
+      ck(cudaMemsetAsync(H->sub_bar, 0, 256, st), "sub_bar");
+      H->sub_ok = false;
+      return false;
+    }
+    S.cg += c.used;
+    S.cg_level[std::min(l, 7)] += c.used;
+    S.hv_cauchy += c.hv_cauchy;
+    S.hv_search += c.hv_search;
+    S.cg_restarts += c.restarts;
+    const long long products = (long long)c.used + c.hv_cauchy + c.hv_search;
+    S.hessvecs += products;
+    S.fe_hessvec += double(products) * hlag_units(l);
+    return true;
   }
 
   template <class V>
