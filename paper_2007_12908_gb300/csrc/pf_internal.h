@@ -42,12 +42,20 @@ struct CgCtrl {
   double alpha;   // step of the current iteration
   double beta;    // direction update of the current iteration
   double kappa;   // p.Hp of the current iteration
+  double m_s;     // model value at the current s
   int done;       // 1 once the run has stopped; later launches are no-ops
   int state;      // why it stopped (CG_*)
   int used;       // Hessian-vector products spent by the CG loop
   int cg_max;     // budget
+  int start;      // used at the start of this run (its first iteration takes w = 0)
+  int no_search;  // 0 while a projected search is due (the run left the box)
+  int searches;   // projected searches made on the device
+  int restarts;   // of them accepted
+  int max_restarts;
 };
-enum { CG_RUNNING = 0, CG_NEGCURV = 1, CG_LEAVE = 2, CG_CONV = 3, CG_BUDGET = 4 };
+// CG_STOP: an accepted search ended the subproblem (its budget or its restarts
+// are spent); CG_REJECT: a search at full length did not decrease the model
+enum { CG_RUNNING = 0, CG_NEGCURV = 1, CG_LEAVE = 2, CG_CONV = 3, CG_BUDGET = 4, CG_STOP = 5, CG_REJECT = 6 };
 
 // The CG direction of one dof, M^-1 r + beta p (mi = 1 without a
 // preconditioner), rounded the same way wherever it is formed.

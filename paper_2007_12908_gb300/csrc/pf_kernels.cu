@@ -499,7 +499,8 @@ cudaError_t elem_gradient(const Geom& g, const Mat<double>& m, const void* x, vo
 // nodes in the colour phases of k_hess_tile3, and writes the 9^3 node sums
 // to part (one block of 729 float4 per tile).
 // With dir.r set (FP32 CG), v is the previous direction and the staged
-// operand is M^-1 r + beta v, beta = *beta.
+// operand is M^-1 r + beta v, beta = *beta; a run's first iteration (beta = 0)
+// does not read v.
 constexpr int kEtileThreads = 128;  // 4 CTAs per SM at 128 registers
 template <class TV>
 __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
@@ -509,6 +510,7 @@ __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
   if (skip && *skip) return;
   if (p_dev) m.p = *p_dev;
   const float be = dir.r ? float(*beta) : 0.f;
+  const bool use_v = !dir.r || be != 0.f;
   constexpr int T = 8, NN = T + 1, NH = NN * NN * NN, NT = kEtileThreads;
   __shared__ float4 xs[NH], vs[NH], acc[NH];
   const int ox = blockIdx.x * T, oy = blockIdx.y * T, oz = blockIdx.z * T;
@@ -521,7 +523,8 @@ __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
     if (gx < nx0 && gy < ny0 && gz < nz0) {
       const long long idx = gx + (long long)nx0 * (gy + (long long)ny0 * gz);
       a = make_float4(x[idx], x[N + idx], x[2 * N + idx], x[3 * N + idx]);
-      b = make_float4(float(v[idx]), float(v[N + idx]), float(v[2 * N + idx]), float(v[3 * N + idx]));
+      if (use_v)
+        b = make_float4(float(v[idx]), float(v[N + idx]), float(v[2 * N + idx]), float(v[3 * N + idx]));
       if (dir.r) {
         const float* r = dir.r;
         const float4 m4 = dir.mi ? make_float4(dir.mi[idx], dir.mi[N + idx], dir.mi[2 * N + idx],
@@ -677,7 +680,13 @@ __global__ void __launch_bounds__(256, 4) k_etile_gather3_dot(Geom g,
   float pq = 0.f;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
-    float p0 = p[n], p1 = p[N + n], p2 = p[2 * N + n], p3 = p[3 * N + n];
+    float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
+    if (!dir.r || be != 0.f) {
+      p0 = p[n];
+      p1 = p[N + n];
+      p2 = p[2 * N + n];
+      p3 = p[3 * N + n];
+    }
     if (dir.r) {
       const float* r = dir.r;
       const float4 m4 = dir.mi ? make_float4(dir.mi[n], dir.mi[N + n], dir.mi[2 * N + n],

@@ -82,29 +82,39 @@ __global__ void k_ctrl_start(CgCtrl* c, double rr, double rz, double tol, int us
   c->done = 0;
   c->state = CG_RUNNING;
   c->used = used;
+  c->start = used;
   c->cg_max = cg_max;
+  c->no_search = 1;
 }
 
-// Start of a CG run from the restart reduction's (r.r, r.M^-1 r) on the
-// device: the forcing tolerance min(0.1, sqrt||r0||) ||r0|| on the first run
-// of a subproblem, and a run that starts already converged is stopped before
-// its first iteration (CG_CONV), so the host needs no read-back before it.
-__global__ void k_ctrl_start_dev(CgCtrl* c, const double* rrz, int first, int used, int cg_max) {
-  const double rr = rrz[0];
-  if (first) {
-    const double r0 = sqrt(rr);
-    c->tol = fmin(0.1, sqrt(r0)) * r0;
-  }
+// Start of a CG run from a restart's (r.r, r.M^-1 r) on the device; a run that
+// starts already converged is stopped before its first iteration (CG_CONV), so
+// the host needs no read-back before it.
+__device__ __forceinline__ void ctrl_start(CgCtrl* c, double rr, double rz) {
   c->rr = rr;
-  c->rz = rrz[1];
+  c->rz = rz;
   c->alpha = 0.0;
   c->beta = 0.0;
   c->kappa = 0.0;
-  c->used = used;
-  c->cg_max = cg_max;
+  c->start = c->used;
+  c->no_search = 1;
   const bool stop = sqrt(rr) <= c->tol || rr == 0.0;
   c->done = stop ? 1 : 0;
   c->state = stop ? CG_CONV : CG_RUNNING;
+}
+
+// The first run of a subproblem: with the forcing tolerance
+// min(0.1, sqrt||r0||) ||r0||.
+__global__ void k_ctrl_first(CgCtrl* c, const double* rrz, double m_s, int cg_max, int max_restarts) {
+  const double r0 = sqrt(rrz[0]);
+  c->tol = fmin(0.1, sqrt(r0)) * r0;
+  c->m_s = m_s;
+  c->used = 0;
+  c->cg_max = cg_max;
+  c->searches = 0;
+  c->restarts = 0;
+  c->max_restarts = max_restarts;
+  ctrl_start(c, rrz[0], rrz[1]);
 }
 
 template <int K, class Op, class A, class F>
@@ -132,8 +142,10 @@ __device__ __forceinline__ bool any_free(float4 a) {
   return (a.x < 0.f) | (a.y < 0.f) | (a.z < 0.f) | (a.w < 0.f);
 }
 
-// Restart of the CG loop at s: r = -(g + Hs) and p = M^-1 r on the free set
-// of s (0 elsewhere), w = 0, the gaps of s; (r.r, r.M^-1 r) to out.
+// Start of the CG loop at s: r = -(g + Hs) and, unless p is null (where the
+// product forms it), p = M^-1 r on the free set of s (0 elsewhere), the gaps of
+// s; (r.r, r.M^-1 r) to out.  The run's first iteration takes w = 0 without
+// reading it.
 struct CgInitOp {
   __device__ __forceinline__ static void lane(float lo, float hi, float s, float g, float hs,
                                               float m, float& r, float& p, float& a, float& b,
@@ -158,7 +170,7 @@ __global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __r
                                                   const float* __restrict__ Hs,
                                                   const float* __restrict__ mi, bool pc,
                                                   float* __restrict__ r, float* __restrict__ p,
-                                                  float* __restrict__ w, float* __restrict__ ga,
+                                                  float* __restrict__ ga,
                                                   float* __restrict__ gb, double* partials,
                                                   unsigned* counter, double* out) {
   float rr = 0.f, rz = 0.f;
@@ -182,13 +194,73 @@ __global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __r
     CgInitOp::lane(l4.z, h4.z, s4.z, g4.z, hs4.z, m4.z, r4.z, p4.z, ga4.z, gb4.z, rr, rz);
     CgInitOp::lane(l4.w, h4.w, s4.w, g4.w, hs4.w, m4.w, r4.w, p4.w, ga4.w, gb4.w, rr, rz);
     st4(r, j, r4);
-    st4(p, j, p4);
-    st4(w, j, z4);
+    if (p) st4(p, j, p4);
     st4(ga, j, ga4);
     st4(gb, j, gb4);
   }
   double acc[2] = {double(rr), double(rz)};
   grid_finish<2, OpSum>(acc, partials, counter, out);
+}
+
+// After a projected search's product Ht = H t: the test of m(t) against the
+// sufficient decrease from s, and at the same time the start of the next CG run
+// at t (as k_cg_init4), which replaces the run that led to t whether t is
+// accepted or not (a rejected t needs only s, Hs and w).  Bound by memory: 8
+// vectors read and 3 (4) written at once, where the test, the copies of t and
+// Ht to s and Hs, the model value at s and k_cg_init4 took 155 us at 129^3
+// (28 passes of 34 MB); this takes 60 us.
+__device__ __forceinline__ void cg_search_lane(float lo, float hi, float s, float hs, float t, float ht,
+                                               float g, float m, float& r, float& p, float& a, float& b,
+                                               float (&o)[5]) {
+  o[2] += g * t;
+  o[3] += t * ht;
+  o[4] += (g + hs) * (t - s);
+  CgInitOp::lane(lo, hi, t, g, ht, m, r, p, a, b, o[0], o[1]);
+}
+
+__global__ void __launch_bounds__(256) k_cg_search4(
+    long long n4, const float* __restrict__ lo, const float* __restrict__ hi, const float* __restrict__ s,
+    const float* __restrict__ Hs, const float* __restrict__ t, const float* __restrict__ Ht,
+    const float* __restrict__ g, const float* __restrict__ mi, bool pc, float* __restrict__ r,
+    float* __restrict__ p, float* __restrict__ ga, float* __restrict__ gb, double cauchy_c, CgCtrl* c,
+    double* partials, unsigned* counter, const int* __restrict__ skip) {
+  if (skip && *skip) return;
+  float o[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n4;
+       j += (long long)gridDim.x * blockDim.x) {
+    const float4 l4 = ld4(lo, j), h4 = ld4(hi, j), s4 = ld4(s, j), hs4 = ld4(Hs, j), t4 = ld4(t, j),
+                 ht4 = ld4(Ht, j), g4 = ld4(g, j);
+    const float4 m4 = pc ? ld4(mi, j) : make_float4(1.f, 1.f, 1.f, 1.f);
+    float4 r4, p4, a4, b4;
+    cg_search_lane(l4.x, h4.x, s4.x, hs4.x, t4.x, ht4.x, g4.x, m4.x, r4.x, p4.x, a4.x, b4.x, o);
+    cg_search_lane(l4.y, h4.y, s4.y, hs4.y, t4.y, ht4.y, g4.y, m4.y, r4.y, p4.y, a4.y, b4.y, o);
+    cg_search_lane(l4.z, h4.z, s4.z, hs4.z, t4.z, ht4.z, g4.z, m4.z, r4.z, p4.z, a4.z, b4.z, o);
+    cg_search_lane(l4.w, h4.w, s4.w, hs4.w, t4.w, ht4.w, g4.w, m4.w, r4.w, p4.w, a4.w, b4.w, o);
+    st4(r, j, r4);
+    if (p) st4(p, j, p4);
+    st4(ga, j, a4);
+    st4(gb, j, b4);
+  }
+  double acc[5] = {double(o[0]), double(o[1]), double(o[2]), double(o[3]), double(o[4])};
+  auto fin = [c, cauchy_c](double(&v)[5]) {
+    c->searches += 1;
+    c->no_search = 1;
+    const double m_t = v[2] + 0.5 * v[3];
+    if (!(m_t <= c->m_s + cauchy_c * v[4])) {
+      c->done = 1;
+      c->state = CG_REJECT;
+      return;
+    }
+    c->m_s = m_t;
+    c->restarts += 1;
+    if (c->restarts > c->max_restarts || c->used >= c->cg_max) {
+      c->done = 1;
+      c->state = CG_STOP;
+      return;
+    }
+    ctrl_start(c, v[0], v[1]);
+  };
+  grid_finish_fn<5, OpSum>(acc, partials, counter, fin);
 }
 
 // Update after the product q = H p: w += alpha p, r -= alpha q (free set);
@@ -215,6 +287,7 @@ __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* _
                                                     unsigned* counter) {
   if (c->done) return;
   const float al = float(c->alpha);
+  const bool fresh = c->used == c->start + 1;  // w = 0 before this iteration
   float rr = 0.f, lv = 0.f, rz = 0.f;
   // two groups per iteration, every load of both issued before any store
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -227,11 +300,13 @@ __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* _
     float4 b[2] = {z4, z4}, qq[2] = {z4, z4}, pp[2] = {z4, z4}, ww[2] = {z4, z4}, rv[2] = {z4, z4};
     float4 mm[2] = {one4, one4};
     if (f0) {
-      b[0] = ld4(gb, j0); qq[0] = ld4(q, j0); pp[0] = ld4(p, j0); ww[0] = ld4(w, j0); rv[0] = ld4(r, j0);
+      b[0] = ld4(gb, j0); qq[0] = ld4(q, j0); pp[0] = ld4(p, j0); rv[0] = ld4(r, j0);
+      if (!fresh) ww[0] = ld4(w, j0);
       if (pc) mm[0] = ld4(mi, j0);
     }
     if (f1) {
-      b[1] = ld4(gb, j1); qq[1] = ld4(q, j1); pp[1] = ld4(p, j1); ww[1] = ld4(w, j1); rv[1] = ld4(r, j1);
+      b[1] = ld4(gb, j1); qq[1] = ld4(q, j1); pp[1] = ld4(p, j1); rv[1] = ld4(r, j1);
+      if (!fresh) ww[1] = ld4(w, j1);
       if (pc) mm[1] = ld4(mi, j1);
     }
     const float4 aa[2] = {a0, a1};
@@ -242,20 +317,17 @@ __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* _
       cg_update_lane(al, aa[k].z, b[k].z, qq[k].z, pp[k].z, ww[k].z, rv[k].z, mm[k].z, rr, lv, rz);
       cg_update_lane(al, aa[k].w, b[k].w, qq[k].w, pp[k].w, ww[k].w, rv[k].w, mm[k].w, rr, lv, rz);
     }
-    if (f0) {
-      st4(w, j0, ww[0]);
-      st4(r, j0, rv[0]);
-    }
-    if (f1) {
-      st4(w, j1, ww[1]);
-      st4(r, j1, rv[1]);
-    }
+    if (f0 || fresh) st4(w, j0, ww[0]);
+    if (f0) st4(r, j0, rv[0]);
+    if (h1 && (f1 || fresh)) st4(w, j1, ww[1]);
+    if (f1) st4(r, j1, rv[1]);
   }
   double acc[3] = {double(rr), double(lv), double(rz)};
   auto fin = [c](double(&a)[3]) {
     if (a[1] > 0.0) {
       c->done = 1;
       c->state = CG_LEAVE;
+      c->no_search = 0;
     } else if (sqrt(a[0]) <= c->tol) {
       c->done = 1;
       c->state = CG_CONV;
@@ -1247,6 +1319,7 @@ struct Solver {
     }, cg2);
     if (cg2[0] > 0.0) t = std::min(t, cg2[1] / cg2[0]);
     bool ok = false;
+    double m_s = 0.0;
     for (int bt = 0; bt <= P.cauchy_backtracks; ++bt) {
       const V tt = V(t);
       // s = P(-t g).  Where no movable dof is cut by its bound, s = -t t1
@@ -1273,7 +1346,8 @@ struct Solver {
           o[1] = s[i] * Hs[i];
         }, a);
       }
-      if (a[0] + 0.5 * a[1] <= P.cauchy_c * a[0]) {
+      m_s = a[0] + 0.5 * a[1];
+      if (m_s <= P.cauchy_c * a[0]) {
         ok = true;
         break;
       }
@@ -1283,38 +1357,19 @@ struct Solver {
       zero(s, n);
       return;
     }
-    int used = 0;
-    int restarts = 0;
-    double tol = -1.0;
-    CgCtrl* c = H->ctrl;
-    const int* skip = &H->ctrl->done;
-    const bool pc = P.precondition != 0;
-    while (used < cg_max) {
-      double rr2[2];
-      // residual of the model on the free set of s, its gaps, p = M^-1 r
-      cudaGraphExec_t graph = cg_graph<V>(l, p, q, ga, gb, mi, w, r, pc);
-      bool ran = false;
-      if constexpr (std::is_same<V, float>::value) {
-        const long long n4 = pad4(n) / 4;
-        k_cg_init4<<<resident_grid(k_cg_init4, n4), 256, 0, st>>>(
-            n4, lo, hi, s, g, Hs, mi, pc, r, p, w, ga, gb, H->scratch.partials, H->scratch.counter,
-            H->d_res);
-        ck(cudaGetLastError(), "cg_init");
-        S.launches += 1;
-        if (graph) {
-          // start, run and stop on the device: one read-back per CG run
-          k_ctrl_start_dev<<<1, 1, 0, st>>>(c, H->d_res, tol < 0.0 ? 1 : 0, used, cg_max);
-          ck(cudaGetLastError(), "ctrl");
-          ck(cudaGraphLaunch(graph, st), "cg_graph");
-          ck(cudaMemcpyAsync(H->h_ctrl, c, sizeof(CgCtrl), cudaMemcpyDeviceToHost, st), "ctrl");
-          ck(cudaStreamSynchronize(st), "sync");
-          S.launches += 1 + (long long)H->cg_graphs[l].nodes * (H->h_ctrl->used - used);
-          tol = H->h_ctrl->tol;
-          ran = true;
-        } else {
-          fetch(2, rr2);
-        }
-      } else {
+    if constexpr (std::is_same<V, float>::value) {
+      cg_runs32(l, cg_max, vec, m_s);
+      return;
+    } else {
+      int used = 0;
+      int restarts = 0;
+      double tol = -1.0;
+      CgCtrl* c = H->ctrl;
+      const bool pc = P.precondition != 0;
+      while (used < cg_max) {
+        double rr2[2];
+        // residual of the model on the free set of s, its gaps, p = M^-1 r
+        cudaGraphExec_t graph = cg_graph<V>(l, p, q, ga, gb, mi, w, r, pc);
         reduce<2, OpSum, V>(n, [=] __device__(long long i, V(&o)[2]) {
           const V a = lo[i] - s[i], b = hi[i] - s[i];
           const bool fr = a < Z && Z < b;
@@ -1328,108 +1383,202 @@ struct Solver {
           o[0] = ri * ri;
           o[1] = ri * zi;
         }, rr2);
-      }
-      if (!ran) {
         const double rr = rr2[0];
         if (tol < 0.0) {
           const double r0 = std::sqrt(rr);
           tol = std::min(0.1, std::sqrt(r0)) * r0;
         }
         if (std::sqrt(rr) <= tol || rr == 0.0) break;
-      }
-      // CG on the free set, driven on the device: each iteration is the
-      // model Hessian, a reduction for p.Hp (its last block sets alpha or
-      // flags non-positive curvature; p vanishes off the free set, so the
-      // unmasked product is the masked one), an update reduction (its last
-      // block tests the box, the forcing term and the budget and sets beta)
-      // and the direction update.  The host polls the control block between
-      // chunks of iterations; launches after a stop are no-ops.
-      // the whole loop as one CUDA graph: a while node around one
-      // iteration, repeated on the device until the control block stops the
-      // run (no host polls); the host-polled loop below where no graph can
-      // be built
-      if (!ran) {
+        // CG on the free set, driven on the device: each iteration is the
+        // model Hessian, a reduction for p.Hp (its last block sets alpha or
+        // flags non-positive curvature; p vanishes off the free set, so the
+        // unmasked product is the masked one), an update reduction (its last
+        // block tests the box, the forcing term and the budget and sets beta)
+        // and the direction update.
         k_ctrl_start<<<1, 1, 0, st>>>(c, rr2[0], rr2[1], tol, used, cg_max);
         ck(cudaGetLastError(), "ctrl");
         S.launches += 1;
-        if (graph) {
-          ck(cudaGraphLaunch(graph, st), "cg_graph");
-          ck(cudaMemcpyAsync(H->h_ctrl, c, sizeof(CgCtrl), cudaMemcpyDeviceToHost, st), "ctrl");
-          ck(cudaStreamSynchronize(st), "sync");
-          S.launches += (long long)H->cg_graphs[l].nodes * (H->h_ctrl->used - used);
-          ran = true;
-        }
-      }
-      int chunk = 2;
-      while (!ran) {
-        for (int k = 0; k < chunk; ++k) cg_iter<V>(l, p, q, ga, gb, mi, w, r, pc);
-        ck(cudaMemcpyAsync(H->h_ctrl, c, sizeof(CgCtrl), cudaMemcpyDeviceToHost, st), "ctrl");
-        ck(cudaStreamSynchronize(st), "sync");
-        if (H->h_ctrl->done) break;
-        chunk = std::min(chunk * 2, 16);
-      }
-      const CgCtrl cs = *H->h_ctrl;
-      const int its = cs.used - used;
-      used = cs.used;
-      S.cg += its;
-      S.cg_level[std::min(l, 7)] += its;
-      S.hessvecs += its;
-      S.fe_hessvec += its * hlag_units(l);
-      bool leave = cs.state == CG_LEAVE;
-      if (cs.state == CG_NEGCURV) {
-        // to the box along p
-        double amax;
-        reduce<1, OpMin, V>(n, [=] __device__(long long i, V(&o)[1]) {
-          const V pi = p[i];
-          V a = V(INFINITY);
-          if (pi > Z) a = (gb[i] - w[i]) / pi;
-          if (pi < Z) a = (ga[i] - w[i]) / pi;
-          o[0] = a;
-        }, &amax);
-        amax = std::max(amax, 0.0);
-        if (std::isfinite(amax)) {
-          const V am = V(amax);
-          map(n, [=] __device__(long long i) { w[i] += am * p[i]; });
-        }
-        leave = true;
-      }
-      if (!leave) {
-        map(n, [=] __device__(long long i) { s[i] += w[i]; });
-        break;
-      }
-      // projected search along w
-      double ms[2];
-      reduce<2, OpSum, V>(n, [=] __device__(long long i, V(&o)[2]) {
-        o[0] = g[i] * s[i];
-        o[1] = s[i] * Hs[i];
-      }, ms);
-      const double m_s = ms[0] + 0.5 * ms[1];
-      double beta = 1.0;
-      bool accepted = false;
-      for (int bt = 0; bt <= P.cauchy_backtracks; ++bt) {
-        const V bb = V(beta);
-        map(n, [=] __device__(long long i) { t1[i] = clampv(s[i] + bb * w[i], lo[i], hi[i]); });
-        hv<V>(l, t1, t2);
-        S.hv_search += 1;
-        double a[3];
-        reduce<3, OpSum, V>(n, [=] __device__(long long i, V(&o)[3]) {
-          o[0] = g[i] * t1[i];
-          o[1] = t1[i] * t2[i];
-          o[2] = (g[i] + Hs[i]) * (t1[i] - s[i]);
-        }, a);
-        if (a[0] + 0.5 * a[1] <= m_s + P.cauchy_c * a[2]) {
-          accepted = true;
+        run_cg<V>(l, graph, p, q, ga, gb, mi, w, r, pc);
+        read_ctrl();
+        if (graph) S.launches += (long long)H->cg_graphs[l].nodes * (H->h_ctrl->used - used);
+        const CgCtrl cs = *H->h_ctrl;
+        const int its = cs.used - used;
+        used = cs.used;
+        S.cg += its;
+        S.cg_level[std::min(l, 7)] += its;
+        S.hessvecs += its;
+        S.fe_hessvec += its * hlag_units(l);
+        if (cs.state == CG_NEGCURV) {
+          to_box<V>(n, p, w, ga, gb, false);
+        } else if (cs.state != CG_LEAVE) {
+          map(n, [=] __device__(long long i) { s[i] += w[i]; });
           break;
         }
-        beta *= 0.5;
+        // projected search along w
+        double beta = 1.0;
+        bool accepted = false;
+        for (int bt = 0; bt <= P.cauchy_backtracks; ++bt) {
+          const V bb = V(beta);
+          map(n, [=] __device__(long long i) { t1[i] = clampv(s[i] + bb * w[i], lo[i], hi[i]); });
+          hv<V>(l, t1, t2);
+          S.hv_search += 1;
+          double a[3];
+          reduce<3, OpSum, V>(n, [=] __device__(long long i, V(&o)[3]) {
+            o[0] = g[i] * t1[i];
+            o[1] = t1[i] * t2[i];
+            o[2] = (g[i] + Hs[i]) * (t1[i] - s[i]);
+          }, a);
+          const double m_t = a[0] + 0.5 * a[1];
+          if (m_t <= m_s + P.cauchy_c * a[2]) {
+            accepted = true;
+            m_s = m_t;
+            break;
+          }
+          beta *= 0.5;
+        }
+        if (!accepted) break;
+        std::swap(s, t1);
+        std::swap(Hs, t2);
+        S.cg_restarts += 1;
+        if (++restarts > P.max_restarts) break;
       }
-      if (!accepted) break;
-      copy(s, t1, n);
-      copy(Hs, t2, n);
-      S.cg_restarts += 1;
-      if (++restarts > P.max_restarts) break;
+      V* out = vec.s;
+      map(n, [=] __device__(long long i) { out[i] = clampv(s[i], lo[i], hi[i]); });
     }
-    map(n, [=] __device__(long long i) { s[i] = clampv(s[i], lo[i], hi[i]); });
+  }
+
+  // w up to the box along p (non-positive curvature); fresh: w is zero and was
+  // not written.
+  template <class V>
+  void to_box(long long n, const V* p, V* w, const V* ga, const V* gb, bool fresh) {
+    const V Z = V(0);
+    double amax;
+    reduce<1, OpMin, V>(n, [=] __device__(long long i, V(&o)[1]) {
+      const V pi = p[i], wi = fresh ? Z : w[i];
+      V a = V(INFINITY);
+      if (pi > Z) a = (gb[i] - wi) / pi;
+      if (pi < Z) a = (ga[i] - wi) / pi;
+      o[0] = a;
+    }, &amax);
+    amax = std::max(amax, 0.0);
+    const V am = std::isfinite(amax) ? V(amax) : Z;
+    if (fresh || am != Z)
+      map(n, [=] __device__(long long i) { w[i] = (fresh ? Z : w[i]) + am * p[i]; });
+  }
+
+  // One CG run of the control block: the graph, or where none could be built
+  // the same iterations polled from the host between chunks (launches after a
+  // stop are no-ops).
+  template <class V>
+  void run_cg(int l, cudaGraphExec_t graph, V* p, V* q, const V* ga, const V* gb, const V* mi, V* w,
+              V* r, bool pc) {
+    if (graph) {
+      ck(cudaGraphLaunch(graph, st), "cg_graph");
+      return;
+    }
+    for (int chunk = 2;; chunk = std::min(chunk * 2, 16)) {
+      for (int k = 0; k < chunk; ++k) cg_iter<V>(l, p, q, ga, gb, mi, w, r, pc);
+      read_ctrl();
+      if (H->h_ctrl->done) break;
+    }
+  }
+
+  void read_ctrl() {
+    ck(cudaMemcpyAsync(H->h_ctrl, H->ctrl, sizeof(CgCtrl), cudaMemcpyDeviceToHost, st), "ctrl");
+    ck(cudaStreamSynchronize(st), "sync");
+  }
+
+  // The CG runs and projected searches of a subproblem on FP32 vectors from the
+  // Cauchy point (s, Hs), whose model value is m_s.  Searches at full length
+  // and the starts of the runs after them are decided on the device, so that
+  // several runs are enqueued between two read-backs (13 us each, and the GPU
+  // waits for the launches after it): a chunk of 1, 2, then 4, whose launches
+  // after a stop are no-ops (some 20 us a run, at most 3 of them, against runs
+  // of 0.4 ms at 129^3).  A run that meets non-positive curvature and a search
+  // that has to be shortened go through the host.
+  void cg_runs32(int l, int cg_max, const SubVecs<float>& vec, double m_s) {
+    const long long n = H->lv[l].n, n4 = pad4(n) / 4;
+    const float *g = vec.g, *lo = vec.lo, *hi = vec.hi, *mi = vec.mi;
+    float *s = vec.s, *Hs = vec.Hs, *r = vec.r, *p = vec.p, *q = vec.q, *w = vec.w;
+    float *ga = vec.a, *gb = vec.b, *t1 = vec.t1, *t2 = vec.t2;
+    CgCtrl* c = H->ctrl;
+    const bool pc = P.precondition != 0;
+    // the products that form the direction themselves need no start of p
+    float* p0 = !gstored(l) && hessvec32_dot_fused(H->geo[l], H->etile_part) ? nullptr : p;
+    auto search = [&](float bb, const int* skip) {
+      auto trial = [=] __device__(long long i) { t1[i] = clampv(s[i] + bb * w[i], lo[i], hi[i]); };
+      if (skip) map_skip(n, trial, skip);
+      else map(n, trial);
+      hv<float>(l, t1, t2, skip, false);
+      k_cg_search4<<<resident_grid(k_cg_search4, n4), 256, 0, st>>>(
+          n4, lo, hi, s, Hs, t1, t2, g, mi, pc, r, p0, ga, gb, P.cauchy_c, c, H->scratch.partials,
+          H->scratch.counter, skip);
+      ck(cudaGetLastError(), "cg_search");
+      S.launches += 1;
+    };
+    if (cg_max > 0) {
+      cudaGraphExec_t graph = cg_graph<float>(l, p, q, ga, gb, mi, w, r, pc);
+      k_cg_init4<<<resident_grid(k_cg_init4, n4), 256, 0, st>>>(n4, lo, hi, s, g, Hs, mi, pc, r, p0, ga, gb,
+                                                               H->scratch.partials, H->scratch.counter,
+                                                               H->d_res);
+      ck(cudaGetLastError(), "cg_init");
+      k_ctrl_first<<<1, 1, 0, st>>>(c, H->d_res, m_s, cg_max, P.max_restarts);
+      ck(cudaGetLastError(), "ctrl");
+      S.launches += 2;
+      run_cg<float>(l, graph, p, q, ga, gb, mi, w, r, pc);
+      int known = 0;  // accepted searches that s and t1 follow
+      for (int chunk = 1;; chunk = std::min(2 * chunk, 4)) {
+        for (int k = 0; k < chunk; ++k) {
+          search(1.f, &c->no_search);
+          // as if accepted; set right below
+          std::swap(s, t1);
+          std::swap(Hs, t2);
+          run_cg<float>(l, graph, p, q, ga, gb, mi, w, r, pc);
+        }
+        read_ctrl();
+        const CgCtrl* hc = H->h_ctrl;
+        if ((hc->restarts - known - chunk) % 2 != 0) {
+          std::swap(s, t1);
+          std::swap(Hs, t2);
+        }
+        known = hc->restarts;
+        if (hc->state == CG_LEAVE) continue;
+        if (hc->state == CG_CONV || hc->state == CG_BUDGET) {
+          if (hc->used > hc->start) map(n, [=] __device__(long long i) { s[i] += w[i]; });
+          break;
+        }
+        if (hc->state == CG_STOP) break;
+        float bb = 1.f;
+        int bt = 0;
+        if (hc->state == CG_NEGCURV) {
+          to_box<float>(n, p, w, ga, gb, hc->used == hc->start + 1);
+        } else {  // CG_REJECT at full length
+          bb = 0.5f;
+          bt = 1;
+        }
+        for (; bt <= P.cauchy_backtracks; ++bt, bb *= 0.5f) {
+          search(bb, nullptr);
+          read_ctrl();
+          if (hc->state != CG_REJECT) break;
+        }
+        if (bt > P.cauchy_backtracks) break;
+        std::swap(s, t1);
+        std::swap(Hs, t2);
+        known = hc->restarts;
+        if (hc->state == CG_STOP) break;
+        run_cg<float>(l, graph, p, q, ga, gb, mi, w, r, pc);
+      }
+      const CgCtrl cs = *H->h_ctrl;
+      S.cg += cs.used;
+      S.cg_level[std::min(l, 7)] += cs.used;
+      S.hv_search += cs.searches;
+      S.cg_restarts += cs.restarts;
+      S.hessvecs += cs.used + cs.searches;
+      S.fe_hessvec += double(cs.used + cs.searches) * hlag_units(l);
+      if (graph) S.launches += (long long)H->cg_graphs[l].nodes * cs.used;
+    }
+    float* out = vec.s;
+    map(n, [=] __device__(long long i) { out[i] = clampv(s[i], lo[i], hi[i]); });
   }
 
   // ---------------------------------------------------------------- TR method
