@@ -24,6 +24,7 @@ struct Mat {
   T inv_h;                  // 1/h
   T w;                      // Gauss weight times det J = h^d / 2^d
   T gcl;                    // Gc / ls
+  T lmu, hmu;               // lam / mu, h / mu
 };
 
 // ---------------------------------------------------------------- 3D passes

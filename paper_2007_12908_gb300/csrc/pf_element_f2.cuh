@@ -1,9 +1,6 @@
-// Packed FP32 variant of the 3D Q1 Hessian-vector element operation.  The
-// two Gauss points of an element along x form one float2 (lane qx), so the
-// sum-factorised interpolation, the Gauss-point algebra and the adjoint
-// contraction run on the paired FP32 FMA/ADD/MUL instructions of sm_100+
-// (__ffma2_rn etc.).  Pairs are indexed pp = qy + 2 qz; Gauss point
-// q = qx + 2 qy + 4 qz of the scalar code is lane qx of pair pp.
+// Packed FP32 variant of the 3D Q1 Hessian-vector element operation on the
+// paired FP32 FMA/ADD/MUL instructions of sm_100+ (__ffma2_rn etc.): the two
+// Gauss points of a pair along z are the lanes of a float2.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -19,211 +16,198 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 // a - b, exact: b * (-1) + a rounds once
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, bc(-1.f), a); }
 
-// Values and raw-difference gradients of one field at the 8 Gauss points,
-// as 4 pairs.  The x-derivative is constant along x and returned scalar.
-struct Interp {
-  float2 val[4], gy[4], gz[4];
-  float gx[4];
+__device__ __forceinline__ float2 pair(float b, float a) {  // a + xi b at the two points of an axis
+  return make_float2(fmaf(float(PF_XI0), b, a), fmaf(float(PF_XI1), b, a));
+}
+
+// The two Gauss points between a and b, each from its nearer end: the rounding
+// of b - a enters with weight 0.21 at both.
+__device__ __forceinline__ float2 lerp2(float a, float b) {
+  const float x0 = float(PF_XI0), t = b - a;
+  return make_float2(fmaf(x0, t, a), fmaf(-x0, t, b));
+}
+__device__ __forceinline__ void lerp2(float2 a, float2 b, float2 (&o)[2]) {
+  const float2 t = sub2(b, a);
+  o[0] = fma2(bc(float(PF_XI0)), t, a);
+  o[1] = fma2(bc(-float(PF_XI0)), t, b);
+}
+__device__ __forceinline__ float at(float2 v, int q) { return q ? v.y : v.x; }
+
+// Raw-difference derivatives of one field: x by qy and y by qx (lanes qz), z by
+// qy (lanes qx).
+struct Grad {
+  float2 x[2], y[2], z[2];
+  // of a rough field (the direction: any nodal noise), differences along an
+  // axis first and then the other two axes; smooth fields lose nothing
+  __device__ __forceinline__ void rough(const float f[8]) {
+    lerp2(lerp2(f[1] - f[0], f[5] - f[4]), lerp2(f[3] - f[2], f[7] - f[6]), x);
+    lerp2(lerp2(f[2] - f[0], f[6] - f[4]), lerp2(f[3] - f[1], f[7] - f[5]), y);
+    lerp2(lerp2(f[4] - f[0], f[5] - f[1]), lerp2(f[6] - f[2], f[7] - f[3]), z);
+  }
+  // of a smooth one, through its monomials
+  __device__ __forceinline__ void smooth(const float f[8]) {
+    const float2 x0 = bc(float(PF_XI0)), x1 = bc(float(PF_XI1));
+    Mono3<float> m;
+    m.set(f);
+    const float2 a = pair(m.xz, m.x), a2 = pair(m.yz, m.y), b = pair(m.xyz, m.xy);
+    x[0] = fma2(x0, b, a);
+    x[1] = fma2(x1, b, a);
+    y[0] = fma2(x0, b, a2);
+    y[1] = fma2(x1, b, a2);
+    const float2 c = pair(m.yz, m.z), d = pair(m.xyz, m.xz);  // by qy
+    z[0] = pair(d.x, c.x);
+    z[1] = pair(d.y, c.y);
+  }
 };
 
-__device__ __forceinline__ void interp(const float f[8], Interp& o) {
+// N_0 and N_1 weighted sums along an axis
+__device__ __forceinline__ void n_sums2(float2 a, float2 b, float2& n0, float2& n1) {
+  const float2 x0 = bc(float(PF_XI0)), x1 = bc(float(PF_XI1));
+  n0 = fma2(x1, a, mul2(x0, b));
+  n1 = fma2(x0, a, mul2(x1, b));
+}
+
+// Test-function sums of one field: an x-derivative row by qy (summed over qx)
+// and a y-derivative row by qx (summed over qy), lanes qz, and a z-derivative
+// row by qy, lanes qx (summed over qz); with VALUE a value row [qx][qy], lanes
+// qz.
+template <bool VALUE>
+__device__ __forceinline__ void corners(const float2 (&sx)[2], const float2 (&sy)[2], const float2 (&sz)[2],
+                                        const float2 (&s0)[2][2], float (&r)[8]) {
   const float x0 = float(PF_XI0), x1 = float(PF_XI1);
-  const float2 xi = make_float2(x0, x1);
-  float2 X[2][2];  // [ay][az], lanes qx
-  float DX[2][2];
-#pragma unroll
-  for (int az = 0; az < 2; ++az)
-#pragma unroll
-    for (int ay = 0; ay < 2; ++ay) {
-      const float v0 = f[2 * ay + 4 * az], d = f[1 + 2 * ay + 4 * az] - v0;
-      DX[ay][az] = d;
-      X[ay][az] = fma2(bc(d), xi, bc(v0));
-    }
-  float2 XY[2][2];  // [qy][az]
-  float2 DY[2];     // [az]
-  float DXY[2][2];  // [qy][az]
-#pragma unroll
-  for (int az = 0; az < 2; ++az) {
-    const float2 d = sub2(X[1][az], X[0][az]);
-    DY[az] = d;
-    XY[0][az] = fma2(d, bc(x0), X[0][az]);
-    XY[1][az] = fma2(d, bc(x1), X[0][az]);
-    const float dd = DX[1][az] - DX[0][az];
-    DXY[0][az] = fmaf(x0, dd, DX[0][az]);
-    DXY[1][az] = fmaf(x1, dd, DX[0][az]);
+  float2 t0, t1, u0, u1, l[4];  // l: corners of a layer, lanes qz (0: negative)
+  n_sums2(sx[0], sx[1], t0, t1);
+  n_sums2(sy[0], sy[1], u0, u1);
+  l[0] = add2(t0, u0);
+  l[1] = sub2(t0, u1);
+  l[2] = sub2(u0, t1);
+  l[3] = add2(t1, u1);
+  if constexpr (VALUE) {
+    float2 n[2][2], v[2];
+    n_sums2(s0[0][0], s0[1][0], n[0][0], n[1][0]);
+    n_sums2(s0[0][1], s0[1][1], n[0][1], n[1][1]);
+    n_sums2(n[0][0], n[0][1], v[0], v[1]);
+    l[0] = sub2(l[0], v[0]);
+    l[2] = add2(l[2], v[1]);
+    n_sums2(n[1][0], n[1][1], v[0], v[1]);
+    l[1] = add2(l[1], v[0]);
+    l[3] = add2(l[3], v[1]);
   }
+  float2 n[2];
+  n_sums2(sz[0], sz[1], n[0], n[1]);
 #pragma unroll
-  for (int qy = 0; qy < 2; ++qy) {
-    const float2 d = sub2(XY[qy][1], XY[qy][0]);
-    o.val[qy] = fma2(d, bc(x0), XY[qy][0]);
-    o.val[qy + 2] = fma2(d, bc(x1), XY[qy][0]);
-    o.gz[qy] = d;
-    o.gz[qy + 2] = d;
-    const float dd = DXY[qy][1] - DXY[qy][0];
-    o.gx[qy] = fmaf(x0, dd, DXY[qy][0]);
-    o.gx[qy + 2] = fmaf(x1, dd, DXY[qy][0]);
-  }
-  const float2 d = sub2(DY[1], DY[0]);
-  const float2 a = fma2(d, bc(x0), DY[0]), b = fma2(d, bc(x1), DY[0]);
-  o.gy[0] = a; o.gy[1] = a;
-  o.gy[2] = b; o.gy[3] = b;
-}
-
-// Adjoint of interp: r[a] = sum over Gauss points of s0 N_a + sx Dx_a +
-// sy Dy_a + sz Dz_a (raw derivatives).  WITH_S0 = false skips the value term.
-template <bool WITH_S0>
-__device__ __forceinline__ void test(const float2 s0[4], const float2 sx[4], const float2 sy[4],
-                                     const float2 sz[4], float r[8]) {
-  const float x0 = float(PF_XI0), x1 = float(PF_XI1);
-  // z pass: XYb[qy][az] (pairs), DXYb[qy][az] (scalar), DYb[az] (pairs)
-  float2 XYb[2][2];
-  float DXYb[2][2];
-  float2 DYb[2];
-#pragma unroll
-  for (int qy = 0; qy < 2; ++qy) {
-    const float2 zs = add2(sz[qy], sz[qy + 2]);
-    if (WITH_S0) {
-      XYb[qy][0] = sub2(fma2(bc(x1), s0[qy], mul2(bc(x0), s0[qy + 2])), zs);
-      XYb[qy][1] = add2(fma2(bc(x0), s0[qy], mul2(bc(x1), s0[qy + 2])), zs);
-    } else {
-      XYb[qy][0] = sub2(make_float2(0.f, 0.f), zs);
-      XYb[qy][1] = zs;
-    }
-    const float a = sx[qy].x + sx[qy].y, b = sx[qy + 2].x + sx[qy + 2].y;
-    DXYb[qy][0] = fmaf(x1, a, x0 * b);
-    DXYb[qy][1] = fmaf(x0, a, x1 * b);
-  }
-  {
-    const float2 a = add2(sy[0], sy[1]), b = add2(sy[2], sy[3]);
-    DYb[0] = fma2(bc(x1), a, mul2(bc(x0), b));
-    DYb[1] = fma2(bc(x0), a, mul2(bc(x1), b));
-  }
-  // y pass: Xb[ay][az] (pairs), DXb[ay][az] (scalar)
-  float2 Xb[2][2];
-  float DXb[2][2];
-#pragma unroll
-  for (int az = 0; az < 2; ++az) {
-    Xb[0][az] = sub2(fma2(bc(x1), XYb[0][az], mul2(bc(x0), XYb[1][az])), DYb[az]);
-    Xb[1][az] = add2(fma2(bc(x0), XYb[0][az], mul2(bc(x1), XYb[1][az])), DYb[az]);
-    DXb[0][az] = fmaf(x1, DXYb[0][az], x0 * DXYb[1][az]);
-    DXb[1][az] = fmaf(x0, DXYb[0][az], x1 * DXYb[1][az]);
-  }
-  // x pass: lanes qx combine into the two corners along x
-#pragma unroll
-  for (int az = 0; az < 2; ++az)
-#pragma unroll
-    for (int ay = 0; ay < 2; ++ay) {
-      const float2 v = Xb[ay][az];
-      r[2 * ay + 4 * az] = fmaf(x1, v.x, fmaf(x0, v.y, -DXb[ay][az]));
-      r[1 + 2 * ay + 4 * az] = fmaf(x0, v.x, fmaf(x1, v.y, DXb[ay][az]));
-    }
-}
-
-// The lagged Gauss-point coefficients (see hess_coef) for the 4 pairs:
-// A, M and the symmetric B in sym order 00, 11, 22, 01, 02, 12.
-struct Coef {
-  float2 A, M, B[6];
-};
-
-__device__ __forceinline__ void coef(const float (*xe)[8], const Mat<float>& m, Coef cf[4]) {
-  Interp u[3], c;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) interp(xe[i], u[i]);
-  interp(xe[3], c);
-  const float omk = 1.f - m.k;
-  const float wh2 = m.w * m.inv_h * m.inv_h, wh = m.w * m.inv_h;
-#pragma unroll
-  for (int pp = 0; pp < 4; ++pp) {
-    // G[i][k] = d u_i / d x_k (physical)
-    float2 G[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      G[i][0] = mul2(bc(u[i].gx[pp]), bc(m.inv_h));
-      G[i][1] = mul2(u[i].gy[pp], bc(m.inv_h));
-      G[i][2] = mul2(u[i].gz[pp], bc(m.inv_h));
-    }
-    const float2 tr = add2(add2(G[0][0], G[1][1]), G[2][2]);
-    const float2 s01 = add2(G[0][1], G[1][0]), s02 = add2(G[0][2], G[2][0]), s12 = add2(G[1][2], G[2][1]);
-    float2 ee = mul2(G[0][0], G[0][0]);
-    ee = fma2(G[1][1], G[1][1], ee);
-    ee = fma2(G[2][2], G[2][2], ee);
-    const float2 half = bc(0.5f);
-    ee = fma2(mul2(half, s01), s01, ee);
-    ee = fma2(mul2(half, s02), s02, ee);
-    ee = fma2(mul2(half, s12), s12, ee);
-    const float2 psi = fma2(mul2(bc(0.5f * m.lam), tr), tr, mul2(bc(m.mu), ee));
-    const float2 omc = sub2(bc(1.f), c.val[pp]);
-    const float2 g = fma2(mul2(bc(omk), omc), omc, bc(m.k));
-    const float2 dgw = mul2(bc(-2.f * omk * wh), omc);
-    cf[pp].A = mul2(bc(wh2), g);
-    cf[pp].M = mul2(bc(m.w), fma2(bc(2.f * omk), fma2(bc(m.p), tr, psi), bc(m.gcl)));
-    const float2 diag = fma2(bc(m.lam), tr, bc(m.p));
-    const float2 tmu = bc(2.f * m.mu);
-    cf[pp].B[0] = mul2(dgw, fma2(tmu, G[0][0], diag));
-    cf[pp].B[1] = mul2(dgw, fma2(tmu, G[1][1], diag));
-    cf[pp].B[2] = mul2(dgw, fma2(tmu, G[2][2], diag));
-    const float2 dgm = mul2(dgw, bc(m.mu));
-    cf[pp].B[3] = mul2(dgm, s01);
-    cf[pp].B[4] = mul2(dgm, s02);
-    cf[pp].B[5] = mul2(dgm, s12);
+  for (int k = 0; k < 4; ++k) {
+    float a, b;
+    n_sums(n[k >> 1].x, n[k >> 1].y, a, b);
+    const float t = k & 1 ? b : a, s = k ? 1.f : -1.f;
+    r[k] = fmaf(s * x1, l[k].x, fmaf(s * x0, l[k].y, -t));
+    r[k + 4] = fmaf(s * x0, l[k].x, fmaf(s * x1, l[k].y, t));
   }
 }
 
-__device__ __forceinline__ void apply(const float (*ve)[8], const Coef cf[4], const Mat<float>& m,
-                                      float (*out)[8]) {
-  float2 su[3][3][4], s0[4], sc[3][4];
-  {
-    Interp v[3], vc;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) interp(ve[i], v[i]);
-    interp(ve[3], vc);
-    const float kc = m.w * m.Gc * m.ls * m.inv_h * m.inv_h;
-#pragma unroll
-    for (int pp = 0; pp < 4; ++pp) {
-      float2 G[3][3];  // raw differences of v_u
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        G[i][0] = bc(v[i].gx[pp]);
-        G[i][1] = v[i].gy[pp];
-        G[i][2] = v[i].gz[pp];
-      }
-      const float2 A = cf[pp].A, M = cf[pp].M, w = vc.val[pp];
-      const float2 trr = add2(add2(G[0][0], G[1][1]), G[2][2]);
-      const float2 lt = mul2(bc(m.lam), trr), am = mul2(A, bc(m.mu));
-      const float2 tmu = bc(2.f * m.mu);
-      float2 c0 = mul2(M, w);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const float2 Bii = cf[pp].B[i];
-        su[i][i][pp] = fma2(w, Bii, mul2(A, fma2(tmu, G[i][i], lt)));
-        c0 = fma2(Bii, G[i][i], c0);
-      }
-      const int ii[3] = {0, 0, 1}, kk[3] = {1, 2, 2};
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const float2 Bik = cf[pp].B[3 + j];
-        const float2 sik = add2(G[ii[j]][kk[j]], G[kk[j]][ii[j]]);
-        const float2 val = fma2(am, sik, mul2(w, Bik));
-        su[ii[j]][kk[j]][pp] = val;
-        su[kk[j]][ii[j]][pp] = val;
-        c0 = fma2(Bik, sik, c0);
-      }
-      s0[pp] = c0;
-      sc[0][pp] = bc(kc * vc.gx[pp]);
-      sc[1][pp] = mul2(bc(kc), vc.gy[pp]);
-      sc[2][pp] = mul2(bc(kc), vc.gz[pp]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 3; ++i) test<false>(nullptr, su[i][0], su[i][1], su[i][2], out[i]);
-  test<true>(s0, sc[0], sc[1], sc[2], out[3]);
-}
-
+// The 3D FP32 Hessian product of one element, bound by the FP32 pipe and the
+// issue slots: 1,050 operations (an FFMA2 counts as two), by
+// - the state in monomials (Mono3), the direction and the adjoint axis by axis;
+// - raw differences and stresses in units of mu / h, t_ik = (sigma + p I)_ik
+//   h / mu, so that shear stresses are the sums G_ik + G_ki themselves;
+// - the cross terms through t instead of the coefficient tensor B = g' t:
+//   q = g' w, su = A sigma(v) + q t, s0 = M w + g' t : grad v;
+// in pairs of Gauss points along z, whose lanes the z passes fill and take
+// apart by themselves (only the z-derivatives, the same at both, are copied).
+// With pairs along x, interpolation passes and the coefficient tensor it was
+// 1,310, and the element pass at 129^3 took 100 us, now 88.  In
+// monomials throughout, both ways, it would be 930, but the rounding of a
+// rough direction then grows twofold.
 __device__ __forceinline__ void elem_hessvec(const float (*xe)[8], const float (*ve)[8],
                                              const Mat<float>& m, float (*out)[8]) {
-  Coef cf[4];
-  coef(xe, m, cf);
-  apply(ve, cf, m, out);
+  Grad u[3], v[3], w;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    u[i].smooth(xe[i]);
+    v[i].rough(ve[i]);
+  }
+  w.rough(ve[3]);
+  float2 ov[2][2], wv[2][2];  // 1 - c and w at [qx][qy]
+  {
+    float2 o[4], e0[2], e1[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o[k] = lerp2(1.f - xe[3][k], 1.f - xe[3][k + 4]);
+    lerp2(o[0], o[1], e0);
+    lerp2(o[2], o[3], e1);
+    lerp2(e0[0], e1[0], ov[0]);
+    lerp2(e0[1], e1[1], ov[1]);
+    lerp2(lerp2(ve[3][0], ve[3][4]), lerp2(ve[3][1], ve[3][5]), e0);
+#pragma unroll
+    for (int qx = 0; qx < 2; ++qx) {
+      wv[qx][0] = fma2(w.y[qx], bc(float(PF_XI0)), e0[qx]);
+      wv[qx][1] = fma2(w.y[qx], bc(float(PF_XI1)), e0[qx]);
+    }
+  }
+  const float omk = 1.f - m.k;
+  const float kap = m.w * m.mu * m.inv_h * m.inv_h, ko = kap * omk, kk = kap * m.k;
+  const float pm = m.p * m.hmu, wg = m.w * m.gcl;
+  // a derivative of w stands for two Gauss points
+  const float kc = 2.f * m.w * m.Gc * m.ls * m.inv_h * m.inv_h;
+  const float2 lmu = bc(m.lmu), two = bc(2.f);
+  float2 sx[3][2], sy[3][2], sz[3][2], s0[2][2];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int qx = q & 1, qy = q >> 1;
+    float2 G[3][3], V[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      G[i][0] = u[i].x[qy];
+      G[i][1] = u[i].y[qx];
+      G[i][2] = bc(at(u[i].z[qy], qx));
+      V[i][0] = v[i].x[qy];
+      V[i][1] = v[i].y[qx];
+      V[i][2] = bc(at(v[i].z[qy], qx));
+    }
+    const float2 tr = add2(add2(G[0][0], G[1][1]), G[2][2]);
+    const float2 trv = add2(add2(V[0][0], V[1][1]), V[2][2]);
+    const float2 dia = fma2(lmu, tr, bc(pm)), lt = mul2(lmu, trv);
+    const float2 q1 = mul2(bc(ko), ov[qx][qy]);
+    const float2 A = fma2(q1, ov[qx][qy], bc(kk));
+    const float2 dg = mul2(bc(-2.f), q1), qw = mul2(dg, wv[qx][qy]);
+    float2 S[3][3];
+    float2 W = mul2(bc(pm), tr), dot;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const float2 t = fma2(two, G[i][i], dia);
+      W = fma2(t, G[i][i], W);
+      dot = i ? fma2(t, V[i][i], dot) : mul2(t, V[i][i]);
+      S[i][i] = fma2(A, fma2(two, V[i][i], lt), mul2(qw, t));
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = i + 1; k < 3; ++k) {
+        const float2 t = add2(G[i][k], G[k][i]), tv = add2(V[i][k], V[k][i]);
+        W = fma2(t, t, W);
+        dot = fma2(t, tv, dot);
+        S[i][k] = S[k][i] = fma2(A, tv, mul2(qw, t));
+      }
+    // Gauss weight times 2 (1 - k) (psi + p tr) + Gc / ls
+    const float2 M = fma2(bc(ko), W, bc(wg));
+    s0[qx][qy] = fma2(dg, dot, mul2(M, wv[qx][qy]));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      sx[i][qy] = qx ? add2(sx[i][qy], S[i][0]) : S[i][0];
+      sy[i][qx] = qy ? add2(sy[i][qx], S[i][1]) : S[i][1];
+      const float z = S[i][2].x + S[i][2].y;
+      if (qx) sz[i][qy].y = z;
+      else sz[i][qy].x = z;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) corners<false>(sx[i], sy[i], sz[i], s0, out[i]);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    w.x[k] = mul2(bc(kc), w.x[k]);
+    w.y[k] = mul2(bc(kc), w.y[k]);
+    w.z[k] = mul2(bc(kc), w.z[k]);
+  }
+  corners<true>(w.x, w.y, w.z, s0, out[3]);
 }
 
 }  // namespace p2

@@ -249,6 +249,7 @@ Mat<T> to_mat(const Mat<double>& m) {
   Mat<T> r;
   r.lam = T(m.lam); r.mu = T(m.mu); r.Gc = T(m.Gc); r.ls = T(m.ls); r.k = T(m.k);
   r.p = T(m.p); r.inv_h = T(m.inv_h); r.w = T(m.w); r.gcl = T(m.gcl);
+  r.lmu = T(m.lmu); r.hmu = T(m.hmu);
   return r;
 }
 

@@ -48,6 +48,8 @@ Mat<double> make_mat(const Geom& g, double E, double nu, double Gc, double ls, d
   m.inv_h = 1.0 / g.h;
   m.w = std::pow(g.h, g.dim) / double(1 << g.dim);
   m.gcl = Gc / ls;
+  m.lmu = m.lam / m.mu;
+  m.hmu = g.h / m.mu;
   return m;
 }
 
@@ -56,6 +58,7 @@ static Mat<T> cast_mat(const Mat<double>& m) {
   Mat<T> r;
   r.lam = T(m.lam); r.mu = T(m.mu); r.Gc = T(m.Gc); r.ls = T(m.ls); r.k = T(m.k);
   r.p = T(m.p); r.inv_h = T(m.inv_h); r.w = T(m.w); r.gcl = T(m.gcl);
+  r.lmu = T(m.lmu); r.hmu = T(m.hmu);
   return r;
 }
 
@@ -349,6 +352,17 @@ struct HessTile {
   static constexpr int THREADS = 128;  // four CTAs per SM at 128 registers (8^3 tiles)
 };
 
+// Asynchronous copy of a node's four fields (planes of N) to shared memory;
+// zero where !ok.
+__device__ __forceinline__ void copy4(float4* dst, const float* src, long long N, bool ok) {
+  const unsigned d = unsigned(__cvta_generic_to_shared(dst));
+  const int n = ok ? 4 : 0;
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d + 4 * f), "l"(src + f * N), "r"(n) : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // OP: OP_HESS (y = H(x) v, paired FP32 algebra) or OP_GDIFF (y += grad E(x)
 // - grad E(x - v), scalar FP32 algebra); TX: type of x in memory.
 // p_dev: when non-null, the pressure is read from it (a CUDA graph that
@@ -369,8 +383,15 @@ __global__ void __launch_bounds__(HessTile<T>::THREADS, 4)
   for (int j = threadIdx.x; j < NH; j += NT) {
     const int i = j % NN, jj = (j / NN) % NN, k = j / (NN * NN);
     const int gx = ox - 1 + i, gy = oy - 1 + jj, gz = oz - 1 + k;
+    const bool ok = gx >= 0 && gx < nx0 && gy >= 0 && gy < ny0 && gz >= 0 && gz < nz0;
+    if constexpr (OP == OP_HESS && sizeof(TV) == 4 && sizeof(TX) == 4) {
+      const long long idx = ok ? gx + (long long)nx0 * (gy + (long long)ny0 * gz) : 0;
+      copy4(&xs[j], x + idx, N, ok);
+      copy4(&vs[j], v + idx, N, ok);
+      continue;
+    }
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (gx >= 0 && gx < nx0 && gy >= 0 && gy < ny0 && gz >= 0 && gz < nz0) {
+    if (ok) {
       const long long idx = gx + (long long)nx0 * (gy + (long long)ny0 * gz);
       a = make_float4(float(x[idx]), float(x[N + idx]), float(x[2 * N + idx]), float(x[3 * N + idx]));
       b = make_float4(float(v[idx]), float(v[N + idx]), float(v[2 * N + idx]), float(v[3 * N + idx]));
@@ -380,6 +401,7 @@ __global__ void __launch_bounds__(HessTile<T>::THREADS, 4)
     vs[j] = b;
   }
   for (int i = threadIdx.x; i < T * T * T; i += NT) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  copy_wait();
   __syncthreads();
   constexpr int NEL = E * E * E;
   for (int base = 0; base < NEL; base += NT) {
@@ -495,9 +517,15 @@ cudaError_t elem_gradient(const Geom& g, const Mat<double>& m, const void* x, vo
 
 // Element-owned 3D FP32 Hessian product, pass 1: a CTA owns 8^3 elements
 // and evaluates each once (no halo re-evaluation).  It stages their 9^3
-// corner nodes of x_lag and v, sums the corner contributions into those
-// nodes in the colour phases of k_hess_tile3, and writes the 9^3 node sums
-// to part (one block of 729 float4 per tile).
+// corner nodes of x_lag and v and writes the 9^3 node sums to part (one block
+// of 729 float4 per tile).  Bound by the FP32 pipe (71% busy over the kernel,
+// 88 us at 129^3, of 4 x 4 warps an SM).  A warp owns two element layers and
+// sums their corner contributions, one corner of all lanes at a time, into node
+// planes of its own, so that the eight phases of 32 elements need no CTA barrier
+// (with the 9^3 sums shared by the CTA: 93 us); the planes of two warps meet in
+// the last pass.  One barrier per 32 elements stays: warps that drift apart miss
+// the instruction cache (98 us).  A persistent CTA that stages its next tile
+// beside the last elements of this one was slower (106 us).
 // With dir.r set (FP32 CG), v is the previous direction and the staged
 // operand is M^-1 r + beta v, beta = *beta; a run's first iteration (beta = 0)
 // does not read v.
@@ -510,48 +538,68 @@ __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
   if (skip && *skip) return;
   if (p_dev) m.p = *p_dev;
   const float be = dir.r ? float(*beta) : 0.f;
-  const bool use_v = !dir.r || be != 0.f;
-  constexpr int T = 8, NN = T + 1, NH = NN * NN * NN, NT = kEtileThreads;
-  __shared__ float4 xs[NH], vs[NH], acc[NH];
+  constexpr int T = 8, NN = T + 1, NP = NN * NN, NH = NP * NN, NT = kEtileThreads;
+  constexpr int NW = NT / 32, LZ = T / NW;        // warps, element layers of each
+  constexpr int NA = NW * (LZ + 1) * NP;          // node planes of all warps
+  constexpr bool F32 = sizeof(TV) == 4;
+  __shared__ float4 xs[NH], vs[NH], acc[NA];
   const int ox = blockIdx.x * T, oy = blockIdx.y * T, oz = blockIdx.z * T;
   const int nx0 = g.n[0], ny0 = g.n[1], nz0 = g.n[2];
   const long long N = g.N;
+  auto node = [&](int j, bool& ok) {
+    const int gx = ox + j % NN, gy = oy + (j / NN) % NN, gz = oz + j / NP;
+    ok = gx < nx0 && gy < ny0 && gz < nz0;
+    return ok ? gx + (long long)nx0 * (gy + (long long)ny0 * gz) : 0;
+  };
+  // x, and v or r and mi (the latter into acc, cleared below), without a
+  // register between: all copies of a thread are in flight at once
   for (int j = threadIdx.x; j < NH; j += NT) {
-    const int i = j % NN, jj = (j / NN) % NN, k = j / (NN * NN);
-    const int gx = ox + i, gy = oy + jj, gz = oz + k;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (gx < nx0 && gy < ny0 && gz < nz0) {
-      const long long idx = gx + (long long)nx0 * (gy + (long long)ny0 * gz);
-      a = make_float4(x[idx], x[N + idx], x[2 * N + idx], x[3 * N + idx]);
-      if (use_v)
-        b = make_float4(float(v[idx]), float(v[N + idx]), float(v[2 * N + idx]), float(v[3 * N + idx]));
-      if (dir.r) {
-        const float* r = dir.r;
-        const float4 m4 = dir.mi ? make_float4(dir.mi[idx], dir.mi[N + idx], dir.mi[2 * N + idx],
-                                               dir.mi[3 * N + idx])
-                                 : make_float4(1.f, 1.f, 1.f, 1.f);
-        b = make_float4(cg_direction(m4.x, r[idx], be, b.x),
-                        cg_direction(m4.y, r[N + idx], be, b.y),
-                        cg_direction(m4.z, r[2 * N + idx], be, b.z),
-                        cg_direction(m4.w, r[3 * N + idx], be, b.w));
-      }
+    bool ok;
+    const long long idx = node(j, ok);
+    copy4(&xs[j], x + idx, N, ok);
+    if constexpr (F32) {
+      copy4(&vs[j], (dir.r ? dir.r : v) + idx, N, ok);
+      if (dir.mi) copy4(&acc[j], dir.mi + idx, N, ok);
     }
-    xs[j] = a;
-    vs[j] = b;
-    acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
+  if (!F32 || dir.r) {
+    if (F32) copy_wait();
+    for (int j = threadIdx.x; j < NH; j += NT) {
+      bool ok;
+      const long long idx = node(j, ok);
+      float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (ok) {
+        if (!dir.r || be != 0.f)
+          b = make_float4(float(v[idx]), float(v[N + idx]), float(v[2 * N + idx]), float(v[3 * N + idx]));
+        if (dir.r) {
+          const float4 r4 = vs[j], m4 = dir.mi ? acc[j] : make_float4(1.f, 1.f, 1.f, 1.f);
+          b = make_float4(cg_direction(m4.x, r4.x, be, b.x), cg_direction(m4.y, r4.y, be, b.y),
+                          cg_direction(m4.z, r4.z, be, b.z), cg_direction(m4.w, r4.w, be, b.w));
+        }
+      }
+      vs[j] = b;
+    }
+    __syncthreads();  // acc is read above by other threads than clear it
+  }
+  for (int j = threadIdx.x; j < NA; j += NT) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+  copy_wait();
   __syncthreads();
-  for (int base = 0; base < T * T * T; base += NT) {
-    const int e = base + threadIdx.x;
-    const int lx = e % T, ly = (e / T) % T, lz = e / (T * T);
-    const bool valid = ox + lx < g.ne[0] && oy + ly < g.ne[1] && oz + lz < g.ne[2];
-    const int c0 = lx + NN * (ly + NN * lz);
+  const int ex = g.ne[0] - ox, ey = g.ne[1] - oy, ez = g.ne[2] - oz;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  float4* wa = acc + warp * (LZ + 1) * NP;
+#pragma unroll 1
+  for (int e = lane; e < T * T * LZ; e += 32) {
+    // in step: the warps of the four schedulers fetch the same code (16 KB)
+    __syncthreads();
+    const int lx = e % T, ly = (e / T) % T, lz = e / (T * T), gz = warp * LZ + lz;
+    const bool valid = lx < ex && ly < ey && gz < ez;
+    const int c0 = lx + NN * ly + NP * lz, cg = c0 + NP * LZ * warp;
     float out[4][8];
     if (valid) {
       float xe[4][8], ve[4][8];
 #pragma unroll
       for (int a = 0; a < 8; ++a) {
-        const int c = c0 + (a & 1) + NN * ((a >> 1) & 1) + NN * NN * ((a >> 2) & 1);
+        const int c = cg + (a & 1) + NN * ((a >> 1) & 1) + NP * ((a >> 2) & 1);
         const float4 xa = xs[c], va = vs[c];
         xe[0][a] = xa.x; xe[1][a] = xa.y; xe[2][a] = xa.z; xe[3][a] = xa.w;
         ve[0][a] = va.x; ve[1][a] = va.y; ve[2][a] = va.z; ve[3][a] = va.w;
@@ -561,20 +609,31 @@ __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
       if (valid) {
-        const int c = c0 + (a & 1) + NN * ((a >> 1) & 1) + NN * NN * ((a >> 2) & 1);
-        float4 t = acc[c];
+        const int c = c0 + (a & 1) + NN * ((a >> 1) & 1) + NP * ((a >> 2) & 1);
+        float4 t = wa[c];
         t.x += out[0][a];
         t.y += out[1][a];
         t.z += out[2][a];
         t.w += out[3][a];
-        acc[c] = t;
+        wa[c] = t;
       }
-      __syncthreads();
+      __syncwarp();
     }
   }
+  __syncthreads();
   const long long tile = blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
   float4* o = part + tile * NH;
-  for (int j = threadIdx.x; j < NH; j += NT) o[j] = acc[j];
+  for (int j = threadIdx.x; j < NH; j += NT) {
+    // plane k of the tile: the first of warp k / LZ, and where k > 0 divides
+    // LZ also the last of the warp before
+    const int k = j / NP, w = min(k / LZ, NW - 1), i = j - k * NP;
+    float4 t = acc[(w * (LZ + 1) + (k - w * LZ)) * NP + i];
+    if (k % LZ == 0 && k > 0 && k < T) {
+      const float4 b = acc[((w - 1) * (LZ + 1) + LZ) * NP + i];
+      t = make_float4(b.x + t.x, b.y + t.y, b.z + t.z, b.w + t.w);
+    }
+    o[j] = t;
+  }
 }
 
 // Sum at node n of the blocks of the up to 8 element tiles that contain
@@ -713,10 +772,14 @@ __global__ void __launch_bounds__(256, 4) k_etile_gather3_dot(Geom g,
   grid_finish_fn<1, OpSum>(acc, partials, counter, fin);
 }
 
+static dim3 etile_grid(const Geom& g) {
+  return dim3((g.ne[0] + 7) / 8, (g.ne[1] + 7) / 8, (g.ne[2] + 7) / 8);
+}
+
 long long etile_part_count(const Geom& g) {
   if (g.dim != 3) return 0;
-  const long long t = (long long)((g.ne[0] + 7) / 8) * ((g.ne[1] + 7) / 8) * ((g.ne[2] + 7) / 8);
-  return t * 729;
+  const dim3 t = etile_grid(g);
+  return (long long)t.x * t.y * t.z * 729;
 }
 
 static bool etile_eligible(const Geom& g) {
@@ -741,9 +804,8 @@ cudaError_t elem_hessvec32_dot(const Geom& g, const Mat<double>& m, const float*
                                float* q, CgCtrl* c, double* partials, unsigned* counter,
                                void* part, const float* p_dev, CgDirIn dir, cudaStream_t st) {
   if (!hessvec32_dot_fused(g, part)) return cudaErrorNotSupported;
-  const dim3 be((g.ne[0] + 7) / 8, (g.ne[1] + 7) / 8, (g.ne[2] + 7) / 8);
   float4* pp = static_cast<float4*>(part);
-  k_hess_etile3<float><<<be, kEtileThreads, 0, st>>>(g, cast_mat<float>(m), x, p, pp, &c->done, p_dev, dir,
+  k_hess_etile3<float><<<etile_grid(g), kEtileThreads, 0, st>>>(g, cast_mat<float>(m), x, p, pp, &c->done, p_dev, dir,
                                            &c->beta);
   // kMaxBlocks = two waves of 4 blocks per SM
   const int nb = int(std::min<long long>((g.N + 255) / 256, kMaxBlocks));
@@ -759,9 +821,8 @@ static cudaError_t launch_hess_tile3(const Geom& g, const Mat<double>& m, const 
     return dim3((g.n[0] + t - 1) / t, (g.n[1] + t - 1) / t, (g.n[2] + t - 1) / t);
   };
   if (etile_used(g, part)) {
-    const dim3 be((g.ne[0] + 7) / 8, (g.ne[1] + 7) / 8, (g.ne[2] + 7) / 8);
     float4* pp = static_cast<float4*>(part);
-    k_hess_etile3<TV><<<be, kEtileThreads, 0, st>>>(g, cast_mat<float>(m), x, v, pp, skip, p_dev,
+    k_hess_etile3<TV><<<etile_grid(g), kEtileThreads, 0, st>>>(g, cast_mat<float>(m), x, v, pp, skip, p_dev,
                                           CgDirIn{nullptr, nullptr}, nullptr);
     const int nb = int(std::min<long long>((g.N + 255) / 256, 8LL * 1216));
     k_etile_gather3<TV><<<nb, 256, 0, st>>>(g, pp, y, skip);
