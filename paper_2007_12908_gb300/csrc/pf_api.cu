@@ -292,11 +292,22 @@ pf_status pf_mesh_hierarchy_create(const pf_mesh_desc* d, pf_hierarchy** out) {
         return rc;
       }
     // the FP64 stencil (27 x 16 doubles per node in 3D) is allocated on a
-    // level's first FP64 lag (ensure_stencil): mixed-precision runs never
-    // hold it on their FIRST_ORDER levels
+    // level's first FP64 lag (ensure_stencil): mixed-precision runs do not
+    // hold it
     if ((rc = alloc(h, (void**)&B.coef, sizeof(double) * coef_count(h->geo[l])))) {
       pf_mesh_hierarchy_destroy(h);
       return rc;
+    }
+    // the FP64 stencil of the mixed mode's small 2D levels (8.4 MB at most);
+    // where there is no room for it they stay FP32
+    if (d->dim == 2 && subproblem_small(h->geo[l])) {
+      void* p = nullptr;
+      if (cudaMalloc(&p, sizeof(double) * stencil_count(h->geo[l])) == cudaSuccess) {
+        h->allocations.push_back(p);
+        B.small = static_cast<double*>(p);
+      } else {
+        cudaGetLastError();
+      }
     }
   }
   if (cudaStreamSynchronize(h->st) != cudaSuccess) {

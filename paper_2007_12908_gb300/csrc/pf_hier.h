@@ -25,6 +25,7 @@ struct LevelBuf {
   double* coef = nullptr;   // lagged Gauss-point coefficients (FP64 Hessian)
   double* stencil = nullptr;  // assembled lagged FP64 Hessian (3^d block stencil)
   float* gk = nullptr;        // FP32 Galerkin coefficient moments (mixed GALERKIN coarse levels)
+  double* small = nullptr;    // FP64 stencil of a small 2D level in the mixed mode
   float* gs = nullptr;        // FP32 Galerkin operator as a 3^d block stencil
 };
 

@@ -178,9 +178,9 @@ cudaError_t stencil_apply(const Geom& g, const double* S, const double* v, doubl
 cudaError_t pgs_sweep(const Geom& g, const double* S, const double* gv, const double* lo,
                       const double* hi, double* s, bool reverse, cudaStream_t st);
 cudaError_t scaled_rowsum(const Geom& g, const double* S, double* out, cudaStream_t st);
-// Diagonal of the Hessian at x (precision prec), written as FP64.
-cudaError_t elem_hessdiag(const Geom& g, const Mat<double>& m, const void* x, int prec,
-                          double* y, cudaStream_t st);
+// Diagonal of the FP32 Hessian at x, written as FP64.
+cudaError_t elem_hessdiag(const Geom& g, const Mat<double>& m, const float* x, double* y,
+                          cudaStream_t st);
 // FP32 Hessian at an FP32 copy of x applied to an FP64 v, written as FP64
 // (the mixed-precision solver's operator; conversions happen in registers).
 cudaError_t elem_hessvec_mixed(const Geom& g, const Mat<double>& m, const float* x32,

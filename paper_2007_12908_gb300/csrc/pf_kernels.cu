@@ -1257,13 +1257,10 @@ cudaError_t stencil_apply(const Geom& g, const double* S, const double* v, doubl
   return cudaGetLastError();
 }
 
-cudaError_t elem_hessdiag(const Geom& g, const Mat<double>& m, const void* x, int prec,
-                          double* y, cudaStream_t st) {
-  if (g.dim == 3)
-    return prec ? launch_scatter<3, float, double, OP_DIAG>(g, m, x, nullptr, y, nullptr, st)
-                : launch_scatter<3, double, double, OP_DIAG>(g, m, x, nullptr, y, nullptr, st);
-  return prec ? launch_scatter<2, float, double, OP_DIAG>(g, m, x, nullptr, y, nullptr, st)
-              : launch_scatter<2, double, double, OP_DIAG>(g, m, x, nullptr, y, nullptr, st);
+cudaError_t elem_hessdiag(const Geom& g, const Mat<double>& m, const float* x, double* y,
+                          cudaStream_t st) {
+  return g.dim == 3 ? launch_scatter<3, float, double, OP_DIAG>(g, m, x, nullptr, y, nullptr, st)
+                    : launch_scatter<2, float, double, OP_DIAG>(g, m, x, nullptr, y, nullptr, st);
 }
 
 cudaError_t elem_hessvec_mixed(const Geom& g, const Mat<double>& m, const float* x32,

@@ -492,10 +492,24 @@ struct Solver {
   // (grad h at B.x - B.s: an accepted step not yet applied to the gradient)
   enum { G_NONE = 0, G_AT_X = 1, G_STEP = 2 };
   std::vector<int> gstate;
+  // 2D levels of the mixed mode whose Hessian and subproblem are FP64: those the
+  // one-launch subproblem takes.  Its CG iteration costs 11 us there in FP64, where
+  // an FP32 iteration of separate launches takes 25 to 30 us; so the levels'
+  // products, gradients and energies are as in the FP64 mode (load steps of three
+  // levels: 129^2 92 and 101 -> 59 and 54 ms, 225 x 193 206 and 182 -> 113 and
+  // 82 ms).  In 3D an FP64 iteration reads its 27-point rows from L2 and takes
+  // 22 us at 17^3, no less than 27 us in FP32 with the FP64 assembly of each lag:
+  // 129^3 load steps came out equal over ten seeds, so 3D levels stay FP32.
+  std::vector<char> small64;
 
   Solver(pf_hierarchy* h, const pf_rmtr_params& p, pf_rmtr_stats& s)
       : H(h), P(p), S(s), st(h->st), L(h->L), F(h->dim + 1), mixed(p.precision == PF_FP32),
-        gstate(h->L, G_NONE) {}
+        gstate(h->L, G_NONE), small64(h->L, 0) {
+    for (int l = 0; l < L; ++l) small64[l] = mixed && H->sub_ok && !galerkin(l) && H->lv[l].small;
+  }
+
+  // The FP64 stencil of a level with an FP64 Hessian.
+  double* stencil(int l) const { return mixed ? H->lv[l].small : H->lv[l].stencil; }
 
   // ---------------------------------------------------------------- helpers
   template <class Fn>
@@ -598,19 +612,31 @@ struct Solver {
     return e;
   }
 
+  // The diagonal of a stored operator (its centre blocks).
+  template <class T>
+  void diagonal(int l, const T* op, double* d) {
+    const long long N = H->geo[l].N;
+    const int Fd = F, c = H->dim == 3 ? 13 : 4;
+    map(H->lv[l].n, [=] __device__(long long i) {
+      const int f = int(i / N);
+      const long long k = i - f * N;
+      d[i] = double(op[((long long)(c * Fd + f) * Fd + f) * N + k]);
+    });
+  }
+
   void set_lag(int l, const double* x) {
     LevelBuf& B = H->lv[l];
     copy(B.xlag, x, B.n);
-    if (mixed32(l)) {
+    if (mixed) {
       float* d = B.xlag32;
       const double* src = B.xlag;
       map(B.n, [=] __device__(long long i) { d[i] = float(src[i]); });
     }
     if (!mixed32(l)) {
       // FP64 Hessian of this level: Gauss-point coefficients, once per lag
-      ck(ensure_stencil(H, l), "FP64 stencil allocation");
+      if (!mixed) ck(ensure_stencil(H, l), "FP64 stencil allocation");
       ck(elem_hess_coef(H->geo[l], H->mat[l], B.xlag, B.coef, st), "hess_coef");
-      ck(stencil_assemble(H->geo[l], H->mat[l], B.coef, B.stencil, st), "assemble");
+      ck(stencil_assemble(H->geo[l], H->mat[l], B.coef, stencil(l), st), "assemble");
       S.launches += 2;
       S.fe_gradient += frac(l);
     }
@@ -619,22 +645,13 @@ struct Solver {
       // (the level's own Hessian at x0 for GALERKIN levels); FP32 on levels
       // whose subproblem runs on FP32 vectors (the diagonal goes through B.Hw,
       // free outside the subproblem)
-      const bool m32 = mixed32(l);
       double* d = sub32(l) ? B.Hw : B.minv;
       if (gstored(l)) {
-        // the stored Galerkin operator's own diagonal (its centre blocks)
-        const float* gsv = B.gs;
-        const long long N = H->geo[l].N;
-        const int Fd = F, c = H->dim == 3 ? 13 : 4;
-        map(B.n, [=] __device__(long long i) {
-          const int f = int(i / N);
-          const long long k = i - f * N;
-          d[i] = double(gsv[((long long)(c * Fd + f) * Fd + f) * N + k]);
-        });
+        diagonal(l, B.gs, d);
+      } else if (!mixed32(l)) {
+        diagonal(l, stencil(l), d);
       } else {
-        ck(elem_hessdiag(H->geo[l], H->mat[l], m32 ? (const void*)B.xlag32 : (const void*)B.xlag,
-                         m32 ? 1 : 0, d, st),
-           "hessdiag");
+        ck(elem_hessdiag(H->geo[l], H->mat[l], B.xlag32, d, st), "hessdiag");
         S.launches += 1;
       }
       if (sub32(l)) {
@@ -656,8 +673,9 @@ struct Solver {
   // ---------------------------------------------------------------- level model h^l
   bool finest(int l) const { return l == L - 1; }
   bool galerkin(int l) const { return !finest(l) && P.coarse_model == PF_GALERKIN; }
-  // mixed precision: FP32 Hessian (and FP32 subproblem) on every level
-  bool mixed32(int l) const { return mixed; }
+  // mixed precision: FP32 Hessian (and FP32 subproblem) on every level that is
+  // not small
+  bool mixed32(int l) const { return mixed && !small64[l]; }
 
   // GALERKIN levels of the mixed mode apply their model Hessian R G^{l+1} I
   // as a stored FP32 stencil built once per finest lag (galerkin_build)
@@ -688,7 +706,7 @@ struct Solver {
                               H->p_dev),
            "hessvec32");
       else
-        ck(stencil_apply(H->geo[l], B.stencil, v, out, st, skip), "hessvec");
+        ck(stencil_apply(H->geo[l], stencil(l), v, out, st, skip), "hessvec");
       S.launches += mixed32(l) ? hessvec32_launches(H->geo[l], H->etile_part) : 1;
       if (count) {
         S.hessvecs += 1;
@@ -716,7 +734,7 @@ struct Solver {
          "hessvec32");
       S.launches += hessvec32_launches(H->geo[l], H->etile_part);
     } else {
-      ck(stencil_apply(H->geo[l], B.stencil, v, B.dh, st), "hessvec");
+      ck(stencil_apply(H->geo[l], stencil(l), v, B.dh, st), "hessvec");
       S.launches += 1;
     }
     S.hessvecs += 1;
@@ -1239,8 +1257,8 @@ struct Solver {
     if (gstored(l)) {
       in.stencil = B.gs;
       in.fp32 = true;
-    } else if (!mixed && !galerkin(l)) {
-      in.stencil = B.stencil;
+    } else if (!mixed32(l) && !galerkin(l)) {
+      in.stencil = stencil(l);
     } else {
       return false;
     }
@@ -1624,8 +1642,8 @@ struct Solver {
         v[1] = s[i] * hs[i];
       };
       double pred, dh = 0.0;
-      const bool merged = mixed32(l) && !galerkin(l);
-      if (merged) {
+      const bool merged = !galerkin(l);
+      if (merged && mixed32(l)) {
         // the prediction's terms and the energy difference in one read-back
         reduce_dev<2, OpSum>(B.n, pred_terms, H->d_res + 4);
         ck(elem_energy_diff_hi(H->geo[l], H->mat[l], B.x, B.s, B.g, H->scratch, H->d_res, st),
@@ -1636,6 +1654,21 @@ struct Solver {
         fetch(6, r6);
         pred = -(r6[4] + 0.5 * r6[5]);
         dh = r6[0] + r6[1] + r6[2] + r6[3];
+      } else if (!galerkin(l)) {
+        // likewise with the FP64 energy difference and dg . s
+        const double* dg = finest(l) ? nullptr : B.dg;
+        reduce_dev<3, OpSum>(B.n, [=] __device__(long long i, double(&v)[3]) {
+          v[0] = g[i] * s[i];
+          v[1] = s[i] * hs[i];
+          v[2] = dg ? dg[i] * s[i] : 0.0;
+        }, H->d_res + 4);
+        ck(elem_energy_diff(H->geo[l], H->mat[l], B.x, B.s, 0, H->scratch, H->d_res, st), "ediff");
+        S.fe_energy += frac(l);
+        S.launches += 1;
+        double r7[7];
+        fetch(7, r7);
+        pred = -(r7[4] + 0.5 * r7[5]);
+        dh = (r7[0] + r7[1] + r7[2] + r7[3]) + r7[6];
       } else {
         double a[2];
         reduce<2, OpSum>(B.n, pred_terms, a);

@@ -41,3 +41,19 @@ def test_one_cycle_matches_oracle(dim, n, cg, restarts, pre):
     st = pf.rmtr_load_step(H, x, pf.default_params(precondition=pre, **kw), check=False)
     assert st["cg"] == ro.stats["cg"]
     assert relinf(host(x), ro.x) <= TOL
+
+
+@pytest.mark.parametrize("nc", [(57, 57), (58, 57)])
+def test_mixed_2d_with_small_levels(nc):
+    """Mixed 2D load steps whose levels are all small (113 x 113), and whose
+    finest is not (115 x 113), against the FP64 step."""
+    torch = require_cuda()
+    import paper_2007_12908_gb300 as pf
+    H, Ho = pair(2, nc, 2, 1 / 56, p=1e-3)
+    x = torch.zeros(H.ndof(), dtype=torch.float64, device="cuda")
+    pf.fractures_set(H, pf.PF_LINE2D, PI.centred_crack_2d(), Ho.fine.h, x)
+    x64 = x.clone()
+    s64 = pf.rmtr_load_step(H, x64, pf.default_params(rtol=1e-12))
+    s32 = pf.rmtr_load_step(H, x, pf.default_params(rtol=1e-12, precision=pf.PF_FP32))
+    assert s64["converged"] == 1 and s32["converged"] == 1
+    assert abs(s32["energy"] - s64["energy"]) <= 1e-8 * abs(s64["energy"])
