@@ -27,6 +27,13 @@ static inline void ck(cudaError_t e, const char* where) {
   if (e != cudaSuccess) throw CudaFail{e, where};
 }
 
+__device__ __forceinline__ double clampv(double x, double lo, double hi) {
+  return fmin(fmax(x, lo), hi);
+}
+__device__ __forceinline__ float clampv(float x, float lo, float hi) {
+  return fminf(fmaxf(x, lo), hi);
+}
+
 template <class F>
 __global__ void k_map(long long n, F f) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -128,40 +135,33 @@ __global__ void __launch_bounds__(256) k_red(long long n, F f, double* partials,
 // ---------------------------------------------------------------- FP32 CG passes
 // The vector passes of one projected-CG iteration on FP32 vectors, on groups
 // of four dofs (n a multiple of 4, 16-byte aligned vectors; 16-byte loads
-// keep more bytes in flight per instruction).  ga/gb are the free gaps
-// (a < 0 < b on the free set, both 0 elsewhere); off the free set r, p and
-// w are 0 and stay 0, so a group whose four dofs are all outside reads only
-// its gaps.
+// keep more bytes in flight per instruction).  Off the free set lo < s < hi, r,
+// p and w are 0 and stay 0, so a group whose four dofs are all outside reads
+// only s and the box.
 __device__ __forceinline__ float4 ld4(const float* v, long long j) {
   return reinterpret_cast<const float4*>(v)[j];
 }
 __device__ __forceinline__ void st4(float* v, long long j, float4 x) {
   reinterpret_cast<float4*>(v)[j] = x;
 }
-__device__ __forceinline__ bool any_free(float4 a) {
-  return (a.x < 0.f) | (a.y < 0.f) | (a.z < 0.f) | (a.w < 0.f);
+__device__ __forceinline__ bool is_free(float lo, float hi, float s) { return lo - s < 0.f && 0.f < hi - s; }
+__device__ __forceinline__ bool any_free(float4 lo, float4 hi, float4 s) {
+  return is_free(lo.x, hi.x, s.x) | is_free(lo.y, hi.y, s.y) | is_free(lo.z, hi.z, s.z) | is_free(lo.w, hi.w, s.w);
 }
 
 // Start of the CG loop at s: r = -(g + Hs) and, unless p is null (where the
-// product forms it), p = M^-1 r on the free set of s (0 elsewhere), the gaps of
-// s; (r.r, r.M^-1 r) to out.  The run's first iteration takes w = 0 without
+// product forms it), p = M^-1 r on the free set of s (0 elsewhere);
+// (r.r, r.M^-1 r) to out.  The run's first iteration takes w = 0 without
 // reading it.
-struct CgInitOp {
-  __device__ __forceinline__ static void lane(float lo, float hi, float s, float g, float hs,
-                                              float m, float& r, float& p, float& a, float& b,
-                                              float& rr, float& rz) {
-    const float ai = lo - s, bi = hi - s;
-    const bool fr = ai < 0.f && 0.f < bi;
-    const float ri = fr ? -(g + hs) : 0.f;
-    const float zi = m * ri;
-    r = ri;
-    p = zi;
-    a = fr ? ai : 0.f;
-    b = fr ? bi : 0.f;
-    rr += ri * ri;
-    rz += ri * zi;
-  }
-};
+__device__ __forceinline__ void cg_init_lane(float lo, float hi, float s, float g, float hs, float m, float& r,
+                                             float& p, float& rr, float& rz) {
+  const float ri = is_free(lo, hi, s) ? -(g + hs) : 0.f;
+  const float zi = m * ri;
+  r = ri;
+  p = zi;
+  rr += ri * ri;
+  rz += ri * zi;
+}
 
 __global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __restrict__ lo,
                                                   const float* __restrict__ hi,
@@ -170,33 +170,25 @@ __global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __r
                                                   const float* __restrict__ Hs,
                                                   const float* __restrict__ mi, bool pc,
                                                   float* __restrict__ r, float* __restrict__ p,
-                                                  float* __restrict__ ga,
-                                                  float* __restrict__ gb, double* partials,
-                                                  unsigned* counter, double* out) {
+                                                  double* partials, unsigned* counter, double* out) {
   float rr = 0.f, rz = 0.f;
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n4;
        j += (long long)gridDim.x * blockDim.x) {
     const float4 l4 = ld4(lo, j), h4 = ld4(hi, j), s4 = ld4(s, j);
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 g4 = z4, hs4 = z4, m4 = make_float4(1.f, 1.f, 1.f, 1.f);
-    const float4 a4 = make_float4(l4.x - s4.x, l4.y - s4.y, l4.z - s4.z, l4.w - s4.w);
-    const float4 b4 = make_float4(h4.x - s4.x, h4.y - s4.y, h4.z - s4.z, h4.w - s4.w);
-    const bool any = ((a4.x < 0.f) & (b4.x > 0.f)) | ((a4.y < 0.f) & (b4.y > 0.f)) |
-                     ((a4.z < 0.f) & (b4.z > 0.f)) | ((a4.w < 0.f) & (b4.w > 0.f));
-    if (any) {
+    if (any_free(l4, h4, s4)) {
       g4 = ld4(g, j);
       hs4 = ld4(Hs, j);
       if (pc) m4 = ld4(mi, j);
     }
-    float4 r4, p4, ga4, gb4;
-    CgInitOp::lane(l4.x, h4.x, s4.x, g4.x, hs4.x, m4.x, r4.x, p4.x, ga4.x, gb4.x, rr, rz);
-    CgInitOp::lane(l4.y, h4.y, s4.y, g4.y, hs4.y, m4.y, r4.y, p4.y, ga4.y, gb4.y, rr, rz);
-    CgInitOp::lane(l4.z, h4.z, s4.z, g4.z, hs4.z, m4.z, r4.z, p4.z, ga4.z, gb4.z, rr, rz);
-    CgInitOp::lane(l4.w, h4.w, s4.w, g4.w, hs4.w, m4.w, r4.w, p4.w, ga4.w, gb4.w, rr, rz);
+    float4 r4, p4;
+    cg_init_lane(l4.x, h4.x, s4.x, g4.x, hs4.x, m4.x, r4.x, p4.x, rr, rz);
+    cg_init_lane(l4.y, h4.y, s4.y, g4.y, hs4.y, m4.y, r4.y, p4.y, rr, rz);
+    cg_init_lane(l4.z, h4.z, s4.z, g4.z, hs4.z, m4.z, r4.z, p4.z, rr, rz);
+    cg_init_lane(l4.w, h4.w, s4.w, g4.w, hs4.w, m4.w, r4.w, p4.w, rr, rz);
     st4(r, j, r4);
     if (p) st4(p, j, p4);
-    st4(ga, j, ga4);
-    st4(gb, j, gb4);
   }
   double acc[2] = {double(rr), double(rz)};
   grid_finish<2, OpSum>(acc, partials, counter, out);
@@ -206,23 +198,22 @@ __global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __r
 // sufficient decrease from s, and at the same time the start of the next CG run
 // at t (as k_cg_init4), which replaces the run that led to t whether t is
 // accepted or not (a rejected t needs only s, Hs and w).  Bound by memory: 8
-// vectors read and 3 (4) written at once, where the test, the copies of t and
+// vectors read and 1 (2) written at once, where the test, the copies of t and
 // Ht to s and Hs, the model value at s and k_cg_init4 took 155 us at 129^3
-// (28 passes of 34 MB); this takes 60 us.
+// (28 passes of 34 MB); this takes FIGURE us.
 __device__ __forceinline__ void cg_search_lane(float lo, float hi, float s, float hs, float t, float ht,
-                                               float g, float m, float& r, float& p, float& a, float& b,
-                                               float (&o)[5]) {
+                                               float g, float m, float& r, float& p, float (&o)[5]) {
   o[2] += g * t;
   o[3] += t * ht;
   o[4] += (g + hs) * (t - s);
-  CgInitOp::lane(lo, hi, t, g, ht, m, r, p, a, b, o[0], o[1]);
+  cg_init_lane(lo, hi, t, g, ht, m, r, p, o[0], o[1]);
 }
 
 __global__ void __launch_bounds__(256) k_cg_search4(
     long long n4, const float* __restrict__ lo, const float* __restrict__ hi, const float* __restrict__ s,
     const float* __restrict__ Hs, const float* __restrict__ t, const float* __restrict__ Ht,
     const float* __restrict__ g, const float* __restrict__ mi, bool pc, float* __restrict__ r,
-    float* __restrict__ p, float* __restrict__ ga, float* __restrict__ gb, double cauchy_c, CgCtrl* c,
+    float* __restrict__ p, double cauchy_c, CgCtrl* c,
     double* partials, unsigned* counter, const int* __restrict__ skip) {
   if (skip && *skip) return;
   float o[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
@@ -231,15 +222,13 @@ __global__ void __launch_bounds__(256) k_cg_search4(
     const float4 l4 = ld4(lo, j), h4 = ld4(hi, j), s4 = ld4(s, j), hs4 = ld4(Hs, j), t4 = ld4(t, j),
                  ht4 = ld4(Ht, j), g4 = ld4(g, j);
     const float4 m4 = pc ? ld4(mi, j) : make_float4(1.f, 1.f, 1.f, 1.f);
-    float4 r4, p4, a4, b4;
-    cg_search_lane(l4.x, h4.x, s4.x, hs4.x, t4.x, ht4.x, g4.x, m4.x, r4.x, p4.x, a4.x, b4.x, o);
-    cg_search_lane(l4.y, h4.y, s4.y, hs4.y, t4.y, ht4.y, g4.y, m4.y, r4.y, p4.y, a4.y, b4.y, o);
-    cg_search_lane(l4.z, h4.z, s4.z, hs4.z, t4.z, ht4.z, g4.z, m4.z, r4.z, p4.z, a4.z, b4.z, o);
-    cg_search_lane(l4.w, h4.w, s4.w, hs4.w, t4.w, ht4.w, g4.w, m4.w, r4.w, p4.w, a4.w, b4.w, o);
+    float4 r4, p4;
+    cg_search_lane(l4.x, h4.x, s4.x, hs4.x, t4.x, ht4.x, g4.x, m4.x, r4.x, p4.x, o);
+    cg_search_lane(l4.y, h4.y, s4.y, hs4.y, t4.y, ht4.y, g4.y, m4.y, r4.y, p4.y, o);
+    cg_search_lane(l4.z, h4.z, s4.z, hs4.z, t4.z, ht4.z, g4.z, m4.z, r4.z, p4.z, o);
+    cg_search_lane(l4.w, h4.w, s4.w, hs4.w, t4.w, ht4.w, g4.w, m4.w, r4.w, p4.w, o);
     st4(r, j, r4);
     if (p) st4(p, j, p4);
-    st4(ga, j, a4);
-    st4(gb, j, b4);
   }
   double acc[5] = {double(o[0]), double(o[1]), double(o[2]), double(o[3]), double(o[4])};
   auto fin = [c, cauchy_c](double(&v)[5]) {
@@ -263,22 +252,33 @@ __global__ void __launch_bounds__(256) k_cg_search4(
   grid_finish_fn<5, OpSum>(acc, partials, counter, fin);
 }
 
-// Update after the product q = H p: w += alpha p, r -= alpha q (free set);
-// the last block tests the box, the forcing term and the budget, and sets
-// beta (CG_* states of the control block).
-__device__ __forceinline__ void cg_update_lane(float al, float a, float b, float q, float p,
-                                               float& w, float& r, float m, float& rr, float& lv,
+// Update after the product q = H p: w += alpha p, r -= alpha q (free set), and
+// the projected step t = P(s + w), which the search that follows a run out of
+// the box starts from (two thirds of the updates at 129^3; a pass of its own
+// for t took 31 us there, here it is two of 10 passes).  The last block tests
+// the box, the forcing term and the budget, and sets beta (CG_* states of the
+// control block).  s is sv[0] or sv[1], t the other: accepted searches swap
+// them.  A run's first iteration takes w = 0 and p = M^-1 r.
+__device__ __forceinline__ void cg_update_lane(float al, bool fresh, float lo, float hi, float s, float q, float p,
+                                               float& w, float& r, float m, float& t, float& rr, float& lv,
                                                float& rz) {
-  const float qi = a < 0.f ? q : 0.f;
-  w = w + al * p;
-  r = r - al * qi;
+  const float a = lo - s, b = hi - s;
+  const bool fr = a < 0.f && 0.f < b;
+  const float pi = fresh ? m * r : p;
+  w = fr ? w + al * pi : 0.f;
+  r = fr ? r - al * q : 0.f;
   rr += r * r;
-  lv += ((w < a) | (w > b)) ? 1.f : 0.f;
+  lv += (fr && (w < a || w > b)) ? 1.f : 0.f;
   rz += r * (m * r);
+  t = clampv(s + w, lo, hi);
 }
 
-__global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* __restrict__ ga,
-                                                    const float* __restrict__ gb,
+struct SwapPair {
+  float* v[2];
+};
+
+__global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* __restrict__ lo,
+                                                    const float* __restrict__ hi, SwapPair sv,
                                                     const float* __restrict__ q,
                                                     const float* __restrict__ p,
                                                     const float* __restrict__ mi, bool pc,
@@ -287,40 +287,33 @@ __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* _
                                                     unsigned* counter) {
   if (c->done) return;
   const float al = float(c->alpha);
-  const bool fresh = c->used == c->start + 1;  // w = 0 before this iteration
+  const bool fresh = c->used == c->start + 1;
+  const bool odd = c->restarts & 1;
+  const float* __restrict__ s = odd ? sv.v[1] : sv.v[0];
+  float* __restrict__ t = odd ? sv.v[0] : sv.v[1];
   float rr = 0.f, lv = 0.f, rz = 0.f;
-  // two groups per iteration, every load of both issued before any store
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long j0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; j0 < n4; j0 += 2 * stride) {
-    const long long j1 = j0 + stride;
-    const bool h1 = j1 < n4;
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f), one4 = make_float4(1.f, 1.f, 1.f, 1.f);
-    const float4 a0 = ld4(ga, j0), a1 = h1 ? ld4(ga, j1) : z4;
-    const bool f0 = any_free(a0), f1 = any_free(a1);
-    float4 b[2] = {z4, z4}, qq[2] = {z4, z4}, pp[2] = {z4, z4}, ww[2] = {z4, z4}, rv[2] = {z4, z4};
-    float4 mm[2] = {one4, one4};
-    if (f0) {
-      b[0] = ld4(gb, j0); qq[0] = ld4(q, j0); pp[0] = ld4(p, j0); rv[0] = ld4(r, j0);
-      if (!fresh) ww[0] = ld4(w, j0);
-      if (pc) mm[0] = ld4(mi, j0);
+  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n4; j += stride) {
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 l4 = ld4(lo, j), h4 = ld4(hi, j), s4 = ld4(s, j);
+    float4 q4 = z4, p4 = z4, w4 = z4, r4 = z4, m4 = make_float4(1.f, 1.f, 1.f, 1.f), t4;
+    const bool any = any_free(l4, h4, s4);
+    if (any) {
+      q4 = ld4(q, j);
+      r4 = ld4(r, j);
+      if (pc) m4 = ld4(mi, j);
+      if (!fresh) {
+        p4 = ld4(p, j);
+        w4 = ld4(w, j);
+      }
     }
-    if (f1) {
-      b[1] = ld4(gb, j1); qq[1] = ld4(q, j1); pp[1] = ld4(p, j1); rv[1] = ld4(r, j1);
-      if (!fresh) ww[1] = ld4(w, j1);
-      if (pc) mm[1] = ld4(mi, j1);
-    }
-    const float4 aa[2] = {a0, a1};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      cg_update_lane(al, aa[k].x, b[k].x, qq[k].x, pp[k].x, ww[k].x, rv[k].x, mm[k].x, rr, lv, rz);
-      cg_update_lane(al, aa[k].y, b[k].y, qq[k].y, pp[k].y, ww[k].y, rv[k].y, mm[k].y, rr, lv, rz);
-      cg_update_lane(al, aa[k].z, b[k].z, qq[k].z, pp[k].z, ww[k].z, rv[k].z, mm[k].z, rr, lv, rz);
-      cg_update_lane(al, aa[k].w, b[k].w, qq[k].w, pp[k].w, ww[k].w, rv[k].w, mm[k].w, rr, lv, rz);
-    }
-    if (f0 || fresh) st4(w, j0, ww[0]);
-    if (f0) st4(r, j0, rv[0]);
-    if (h1 && (f1 || fresh)) st4(w, j1, ww[1]);
-    if (f1) st4(r, j1, rv[1]);
+    cg_update_lane(al, fresh, l4.x, h4.x, s4.x, q4.x, p4.x, w4.x, r4.x, m4.x, t4.x, rr, lv, rz);
+    cg_update_lane(al, fresh, l4.y, h4.y, s4.y, q4.y, p4.y, w4.y, r4.y, m4.y, t4.y, rr, lv, rz);
+    cg_update_lane(al, fresh, l4.z, h4.z, s4.z, q4.z, p4.z, w4.z, r4.z, m4.z, t4.z, rr, lv, rz);
+    cg_update_lane(al, fresh, l4.w, h4.w, s4.w, q4.w, p4.w, w4.w, r4.w, m4.w, t4.w, rr, lv, rz);
+    if (any || fresh) st4(w, j, w4);
+    if (any) st4(r, j, r4);
+    st4(t, j, t4);
   }
   double acc[3] = {double(rr), double(lv), double(rz)};
   auto fin = [c](double(&a)[3]) {
@@ -367,36 +360,17 @@ __global__ void __launch_bounds__(256) k_cg_dot4(long long n4, const float* __re
   grid_finish_fn<1, OpSum>(acc, partials, counter, fin);
 }
 
-// Direction update p = M^-1 r + beta p (free set; p stays 0 elsewhere).
-__global__ void __launch_bounds__(256) k_cg_dir4(long long n4, const float* __restrict__ ga,
-                                                 const float* __restrict__ r,
+// Direction update p = M^-1 r + beta p (p stays 0 off the free set).
+__global__ void __launch_bounds__(256) k_cg_dir4(long long n4, const float* __restrict__ r,
                                                  const float* __restrict__ mi, bool pc,
                                                  float* __restrict__ p, const CgCtrl* c) {
   if (c->done) return;
   const float be = float(c->beta);
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long j0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; j0 < n4; j0 += 2 * stride) {
-    const long long j1 = j0 + stride;
-    const bool h1 = j1 < n4;
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f), one4 = make_float4(1.f, 1.f, 1.f, 1.f);
-    const bool f0 = any_free(ld4(ga, j0)), f1 = h1 && any_free(ld4(ga, j1));
-    float4 rv[2] = {z4, z4}, pp[2] = {z4, z4}, mm[2] = {one4, one4};
-    if (f0) {
-      rv[0] = ld4(r, j0); pp[0] = ld4(p, j0);
-      if (pc) mm[0] = ld4(mi, j0);
-    }
-    if (f1) {
-      rv[1] = ld4(r, j1); pp[1] = ld4(p, j1);
-      if (pc) mm[1] = ld4(mi, j1);
-    }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const float4 m4 = mm[k], r4 = rv[k], p4 = pp[k];
-      pp[k] = make_float4(cg_direction(m4.x, r4.x, be, p4.x), cg_direction(m4.y, r4.y, be, p4.y),
-                          cg_direction(m4.z, r4.z, be, p4.z), cg_direction(m4.w, r4.w, be, p4.w));
-    }
-    if (f0) st4(p, j0, pp[0]);
-    if (f1) st4(p, j1, pp[1]);
+  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n4; j += stride) {
+    const float4 r4 = ld4(r, j), p4 = ld4(p, j), m4 = pc ? ld4(mi, j) : make_float4(1.f, 1.f, 1.f, 1.f);
+    st4(p, j, make_float4(cg_direction(m4.x, r4.x, be, p4.x), cg_direction(m4.y, r4.y, be, p4.y),
+                          cg_direction(m4.z, r4.z, be, p4.z), cg_direction(m4.w, r4.w, be, p4.w)));
   }
 }
 
@@ -472,13 +446,6 @@ cudaError_t fixed_mask(const Geom& g, double* out, cudaStream_t st) {
   const int blocks = int(std::min<long long>((n + 255) / 256, 4LL * 1216));
   k_fixed_mask<<<blocks, 256, 0, st>>>(g, out);
   return cudaGetLastError();
-}
-
-__device__ __forceinline__ double clampv(double x, double lo, double hi) {
-  return fmin(fmax(x, lo), hi);
-}
-__device__ __forceinline__ float clampv(float x, float lo, float hi) {
-  return fminf(fmaxf(x, lo), hi);
 }
 
 struct Solver {
@@ -847,13 +814,24 @@ struct Solver {
     }
   }
 
-  // Vectors of one subproblem solve in precision V.  a and b hold the free
-  // gaps lo - s < 0 < hi - s of the current s on its free set and 0 elsewhere,
-  // so a[i] < 0 is the free-set test and w outside [a, b] leaves the box.
+  // Vectors of one subproblem solve in precision V.  a and b (FP64 only) hold
+  // the free gaps lo - s < 0 < hi - s of the current s on its free set and 0
+  // elsewhere, so a[i] < 0 is the free-set test and w outside [a, b] leaves the
+  // box.
   template <class V>
   struct SubVecs {
     const V *g, *lo, *hi, *mi;
     V *s, *Hs, *r, *p, *q, *w, *a, *b, *t1, *t2;
+  };
+
+  // What a CG run works on.  FP64: the free gaps a and b, as above.  FP32: the
+  // box and the pair (s, projected step) of k_cg_update4.
+  template <class V>
+  struct CgVecs {
+    V *p, *q, *w, *r;
+    const V *mi, *a, *b, *lo, *hi;
+    V* sv[2];
+    bool pc;
   };
 
   // One projected-CG iteration on FP32 vectors with float4 passes (n a
@@ -861,21 +839,25 @@ struct Solver {
   // gather pass where it has one), the update with its tests and beta, the
   // direction.  No-ops once the control block is done.  Returns the
   // launches.
-  int cg_iter4(int l, const float* p, float* q, const float* ga, const float* gb,
-               const float* mi, float* w, float* r, bool pc, cudaStream_t s) {
+  int cg_iter4(int l, const CgVecs<float>& v, cudaStream_t s) {
     LevelBuf& B = H->lv[l];
     CgCtrl* c = H->ctrl;
     const long long n4 = pad4(B.n) / 4;
+    float *p = v.p, *q = v.q;
+    auto update = [&] {
+      k_cg_update4<<<resident_grid(k_cg_update4, n4), 256, 0, s>>>(
+          n4, v.lo, v.hi, SwapPair{{v.sv[0], v.sv[1]}}, q, p, v.mi, v.pc, v.w, v.r, c, H->scratch.partials,
+          H->scratch.counter);
+      ck(cudaGetLastError(), "cg_update");
+    };
     if (!gstored(l) && hessvec32_dot_fused(H->geo[l], H->etile_part)) {
       // the direction update of the previous iteration (beta = 0 after a
-      // restart, where p = M^-1 r already) is formed inside the product
-      ck(elem_hessvec32_dot(H->geo[l], H->mat[l], B.xlag32, const_cast<float*>(p), q, c,
-                            H->scratch.partials, H->scratch.counter, H->etile_part, H->p_dev,
-                            CgDirIn{r, pc ? mi : nullptr}, s),
+      // restart) is formed inside the product
+      ck(elem_hessvec32_dot(H->geo[l], H->mat[l], B.xlag32, p, q, c, H->scratch.partials,
+                            H->scratch.counter, H->etile_part, H->p_dev,
+                            CgDirIn{v.r, v.pc ? v.mi : nullptr}, s),
          "hessvec32_dot");
-      k_cg_update4<<<resident_grid(k_cg_update4, n4), 256, 0, s>>>(
-          n4, ga, gb, q, p, mi, pc, w, r, c, H->scratch.partials, H->scratch.counter);
-      ck(cudaGetLastError(), "cg_update");
+      update();
       return 3;
     }
     int launches = 2;
@@ -892,11 +874,8 @@ struct Solver {
       ck(cudaGetLastError(), "cg_dot");
       launches += 1 + (gstored(l) ? 1 : hessvec32_launches(H->geo[l], H->etile_part));
     }
-    k_cg_update4<<<resident_grid(k_cg_update4, n4), 256, 0, s>>>(
-        n4, ga, gb, q, p, mi, pc, w, r, c, H->scratch.partials, H->scratch.counter);
-    ck(cudaGetLastError(), "cg_update");
-    k_cg_dir4<<<resident_grid(k_cg_dir4, n4), 256, 0, s>>>(n4, ga, r, mi, pc, const_cast<float*>(p),
-                                                            c);
+    update();
+    k_cg_dir4<<<resident_grid(k_cg_dir4, n4), 256, 0, s>>>(n4, v.r, v.mi, v.pc, p, c);
     ck(cudaGetLastError(), "cg_dir");
     return launches;
   }
@@ -905,15 +884,20 @@ struct Solver {
   // p.q and alpha, the update with its tests and beta, the direction.
   // Launches after the control block is done are no-ops.
   template <class V>
-  void cg_iter(int l, V* p, V* q, const V* ga, const V* gb, const V* mi, V* w, V* r, bool pc) {
+  void cg_iter(int l, const CgVecs<V>& v) {
+    if constexpr (std::is_same<V, float>::value) S.launches += cg_iter4(l, v, st);
+    else cg_iter64(l, v);
+  }
+
+  void cg_iter64(int l, const CgVecs<double>& v) {
+    using V = double;
     const long long n = H->lv[l].n;
     CgCtrl* c = H->ctrl;
     const int* skip = &H->ctrl->done;
     const V Z = V(0);
-    if constexpr (std::is_same<V, float>::value) {
-      S.launches += cg_iter4(l, p, q, ga, gb, mi, w, r, pc, st);
-      return;
-    }
+    V *p = v.p, *q = v.q, *w = v.w, *r = v.r;
+    const V *ga = v.a, *gb = v.b, *mi = v.mi;
+    const bool pc = v.pc;
     hv<V>(l, p, q, skip, false);
     red_fin<1, OpSum, V>(n, [=] __device__(long long i, V(&o)[1]) { o[0] = p[i] * q[i]; },
                          [=] __device__(double(&a)[1]) { cg_take_curvature(c, a[0]); }, skip);
@@ -955,16 +939,15 @@ struct Solver {
   // flag changes; a level's subproblem vectors sit at fixed addresses.  Null where the CUDA driver cannot build it (the caller then
   // drives the loop from the host).
   template <class V>
-  cudaGraphExec_t cg_graph(int l, V* p, V* q, const V* ga, const V* gb, const V* mi, V* w, V* r,
-                           bool pc) {
+  cudaGraphExec_t cg_graph(int l, const CgVecs<V>& v) {
     if (!H->cg_graph_ok) return nullptr;
     if ((int)H->cg_graphs.size() < L) H->cg_graphs.resize(L);
     pf_hierarchy::CgGraph& G = H->cg_graphs[l];
     // 3D products read the pressure from the device; 2D ones take it as an
     // argument, so a 2D graph is rebuilt when it changes
     const bool p_ok = H->dim == 3 || G.p == H->p;
-    if (G.exec && p_ok && G.pc == (pc ? 1 : 0) && G.vsize == int(sizeof(V)) &&
-        G.precision == P.precision && G.coarse_model == P.coarse_model && G.vp == p)
+    if (G.exec && p_ok && G.pc == (v.pc ? 1 : 0) && G.vsize == int(sizeof(V)) &&
+        G.precision == P.precision && G.coarse_model == P.coarse_model && G.vp == v.p)
       return G.exec;
     if (G.exec) cudaGraphExecDestroy(G.exec);
     if (G.graph) cudaGraphDestroy(G.graph);
@@ -998,7 +981,7 @@ struct Solver {
       const long long saved_launches = S.launches;
       st = cs;  // cg_iter launches on st
       try {
-        cg_iter<V>(l, p, q, ga, gb, mi, w, r, pc);
+        cg_iter<V>(l, v);
         k_cg_cond<<<1, 1, 0, cs>>>(H->ctrl, h);
         launched = cudaGetLastError() == cudaSuccess;
       } catch (const CudaFail&) {
@@ -1024,11 +1007,11 @@ struct Solver {
     G.exec = ex;
     G.nodes = nodes;
     G.p = H->p;
-    G.pc = pc ? 1 : 0;
+    G.pc = v.pc ? 1 : 0;
     G.vsize = int(sizeof(V));
     G.precision = P.precision;
     G.coarse_model = P.coarse_model;
-    G.vp = p;
+    G.vp = v.p;
     return ex;
   }
 
@@ -1229,14 +1212,14 @@ struct Solver {
     }
     const SubVecs<float> v{g32, lo32, hi32, reinterpret_cast<const float*>(B.minv),
                            half(B.Hw, 1), half(B.Hs, 0), half(B.Hs, 1), half(B.p, 0),
-                           half(B.p, 1), half(B.w, 0), half(B.w, 1), half(B.r, 0),
-                           half(B.r, 1), half(B.q, 0)};
+                           half(B.p, 1), half(B.w, 0), nullptr, nullptr, half(B.r, 1),
+                           half(B.q, 0)};
     if (np != n) {
       // lanes n .. np-1 of every view: 0, so that they act as fixed dofs
-      // (zero gaps) in the float4 passes and no stale value meets a 0
+      // (an empty box) in the float4 passes and no stale value meets a 0
       PadLanes z{{g32, lo32, hi32, reinterpret_cast<float*>(B.minv), v.s, v.Hs, v.r, v.p, v.q, v.w,
-                  v.a, v.b, v.t1, v.t2},
-                 14, n, np};
+                  v.t1, v.t2},
+                 12, n, np};
       k_zero_pad<<<1, 64, 0, st>>>(z);
       ck(cudaGetLastError(), "zero_pad");
       S.launches += 1;
@@ -1387,7 +1370,8 @@ struct Solver {
       while (used < cg_max) {
         double rr2[2];
         // residual of the model on the free set of s, its gaps, p = M^-1 r
-        cudaGraphExec_t graph = cg_graph<V>(l, p, q, ga, gb, mi, w, r, pc);
+          const CgVecs<V> cgv{p, q, w, r, mi, ga, gb, lo, hi, {nullptr, nullptr}, pc};
+        cudaGraphExec_t graph = cg_graph<V>(l, cgv);
         reduce<2, OpSum, V>(n, [=] __device__(long long i, V(&o)[2]) {
           const V a = lo[i] - s[i], b = hi[i] - s[i];
           const bool fr = a < Z && Z < b;
@@ -1416,7 +1400,7 @@ struct Solver {
         k_ctrl_start<<<1, 1, 0, st>>>(c, rr2[0], rr2[1], tol, used, cg_max);
         ck(cudaGetLastError(), "ctrl");
         S.launches += 1;
-        run_cg<V>(l, graph, p, q, ga, gb, mi, w, r, pc);
+        run_cg<V>(l, graph, cgv);
         read_ctrl();
         if (graph) S.launches += (long long)H->cg_graphs[l].nodes * (H->h_ctrl->used - used);
         const CgCtrl cs = *H->h_ctrl;
@@ -1427,7 +1411,7 @@ struct Solver {
         S.hessvecs += its;
         S.fe_hessvec += its * hlag_units(l);
         if (cs.state == CG_NEGCURV) {
-          to_box<V>(n, p, w, ga, gb, false);
+          to_box<V>(n, p, w, GapVecs{ga, gb}, false);
         } else if (cs.state != CG_LEAVE) {
           map(n, [=] __device__(long long i) { s[i] += w[i]; });
           break;
@@ -1465,17 +1449,35 @@ struct Solver {
     }
   }
 
+  // The gaps from w = 0 to the box on the free set (0 elsewhere).
+  struct GapVecs {
+    const double *a, *b;
+    __device__ void operator()(long long i, double& lo, double& hi) const {
+      lo = a[i];
+      hi = b[i];
+    }
+  };
+  struct GapBox {
+    const float *lo, *hi, *s;
+    __device__ void operator()(long long i, float& a, float& b) const {
+      const bool fr = is_free(lo[i], hi[i], s[i]);
+      a = fr ? lo[i] - s[i] : 0.f;
+      b = fr ? hi[i] - s[i] : 0.f;
+    }
+  };
+
   // w up to the box along p (non-positive curvature); fresh: w is zero and was
   // not written.
-  template <class V>
-  void to_box(long long n, const V* p, V* w, const V* ga, const V* gb, bool fresh) {
+  template <class V, class Gap>
+  void to_box(long long n, const V* p, V* w, Gap gap, bool fresh) {
     const V Z = V(0);
     double amax;
     reduce<1, OpMin, V>(n, [=] __device__(long long i, V(&o)[1]) {
       const V pi = p[i], wi = fresh ? Z : w[i];
-      V a = V(INFINITY);
-      if (pi > Z) a = (gb[i] - wi) / pi;
-      if (pi < Z) a = (ga[i] - wi) / pi;
+      V a = V(INFINITY), ga, gb;
+      gap(i, ga, gb);
+      if (pi > Z) a = (gb - wi) / pi;
+      if (pi < Z) a = (ga - wi) / pi;
       o[0] = a;
     }, &amax);
     amax = std::max(amax, 0.0);
@@ -1488,14 +1490,13 @@ struct Solver {
   // the same iterations polled from the host between chunks (launches after a
   // stop are no-ops).
   template <class V>
-  void run_cg(int l, cudaGraphExec_t graph, V* p, V* q, const V* ga, const V* gb, const V* mi, V* w,
-              V* r, bool pc) {
+  void run_cg(int l, cudaGraphExec_t graph, const CgVecs<V>& v) {
     if (graph) {
       ck(cudaGraphLaunch(graph, st), "cg_graph");
       return;
     }
     for (int chunk = 2;; chunk = std::min(chunk * 2, 16)) {
-      for (int k = 0; k < chunk; ++k) cg_iter<V>(l, p, q, ga, gb, mi, w, r, pc);
+      for (int k = 0; k < chunk; ++k) cg_iter<V>(l, v);
       read_ctrl();
       if (H->h_ctrl->done) break;
     }
@@ -1518,40 +1519,39 @@ struct Solver {
     const long long n = H->lv[l].n, n4 = pad4(n) / 4;
     const float *g = vec.g, *lo = vec.lo, *hi = vec.hi, *mi = vec.mi;
     float *s = vec.s, *Hs = vec.Hs, *r = vec.r, *p = vec.p, *q = vec.q, *w = vec.w;
-    float *ga = vec.a, *gb = vec.b, *t1 = vec.t1, *t2 = vec.t2;
+    float *t1 = vec.t1, *t2 = vec.t2;
     CgCtrl* c = H->ctrl;
     const bool pc = P.precondition != 0;
+    const CgVecs<float> cgv{p, q, w, r, mi, nullptr, nullptr, lo, hi, {s, t1}, pc};
     // the products that form the direction themselves need no start of p
     float* p0 = !gstored(l) && hessvec32_dot_fused(H->geo[l], H->etile_part) ? nullptr : p;
-    auto search = [&](float bb, const int* skip) {
-      auto trial = [=] __device__(long long i) { t1[i] = clampv(s[i] + bb * w[i], lo[i], hi[i]); };
-      if (skip) map_skip(n, trial, skip);
-      else map(n, trial);
+    // product and test of the projected step t1
+    auto search = [&](const int* skip) {
       hv<float>(l, t1, t2, skip, false);
       k_cg_search4<<<resident_grid(k_cg_search4, n4), 256, 0, st>>>(
-          n4, lo, hi, s, Hs, t1, t2, g, mi, pc, r, p0, ga, gb, P.cauchy_c, c, H->scratch.partials,
+          n4, lo, hi, s, Hs, t1, t2, g, mi, pc, r, p0, P.cauchy_c, c, H->scratch.partials,
           H->scratch.counter, skip);
       ck(cudaGetLastError(), "cg_search");
       S.launches += 1;
     };
     if (cg_max > 0) {
-      cudaGraphExec_t graph = cg_graph<float>(l, p, q, ga, gb, mi, w, r, pc);
-      k_cg_init4<<<resident_grid(k_cg_init4, n4), 256, 0, st>>>(n4, lo, hi, s, g, Hs, mi, pc, r, p0, ga, gb,
+      cudaGraphExec_t graph = cg_graph<float>(l, cgv);
+      k_cg_init4<<<resident_grid(k_cg_init4, n4), 256, 0, st>>>(n4, lo, hi, s, g, Hs, mi, pc, r, p0,
                                                                H->scratch.partials, H->scratch.counter,
                                                                H->d_res);
       ck(cudaGetLastError(), "cg_init");
       k_ctrl_first<<<1, 1, 0, st>>>(c, H->d_res, m_s, cg_max, P.max_restarts);
       ck(cudaGetLastError(), "ctrl");
       S.launches += 2;
-      run_cg<float>(l, graph, p, q, ga, gb, mi, w, r, pc);
+      run_cg<float>(l, graph, cgv);
       int known = 0;  // accepted searches that s and t1 follow
       for (int chunk = 1;; chunk = std::min(2 * chunk, 4)) {
         for (int k = 0; k < chunk; ++k) {
-          search(1.f, &c->no_search);
+          search(&c->no_search);
           // as if accepted; set right below
           std::swap(s, t1);
           std::swap(Hs, t2);
-          run_cg<float>(l, graph, p, q, ga, gb, mi, w, r, pc);
+          run_cg<float>(l, graph, cgv);
         }
         read_ctrl();
         const CgCtrl* hc = H->h_ctrl;
@@ -1569,13 +1569,14 @@ struct Solver {
         float bb = 1.f;
         int bt = 0;
         if (hc->state == CG_NEGCURV) {
-          to_box<float>(n, p, w, ga, gb, hc->used == hc->start + 1);
+          to_box<float>(n, p, w, GapBox{lo, hi, s}, hc->used == hc->start + 1);
         } else {  // CG_REJECT at full length
           bb = 0.5f;
           bt = 1;
         }
         for (; bt <= P.cauchy_backtracks; ++bt, bb *= 0.5f) {
-          search(bb, nullptr);
+          map(n, [=] __device__(long long i) { t1[i] = clampv(s[i] + bb * w[i], lo[i], hi[i]); });
+          search(nullptr);
           read_ctrl();
           if (hc->state != CG_REJECT) break;
         }
@@ -1584,7 +1585,7 @@ struct Solver {
         std::swap(Hs, t2);
         known = hc->restarts;
         if (hc->state == CG_STOP) break;
-        run_cg<float>(l, graph, p, q, ga, gb, mi, w, r, pc);
+        run_cg<float>(l, graph, cgv);
       }
       const CgCtrl cs = *H->h_ctrl;
       S.cg += cs.used;
