@@ -149,6 +149,8 @@ pf_status pf_mesh_hierarchy_destroy(pf_hierarchy* h) {
   for (void* p : h->allocations) cudaFree(p);
   if (h->h_res) cudaFreeHost(h->h_res);
   if (h->h_ctrl) cudaFreeHost(h->h_ctrl);
+  for (cudaEvent_t e : h->cg_ev)
+    if (e) cudaEventDestroy(e);
   delete h;
   return PF_OK;
 }
@@ -261,12 +263,19 @@ pf_status pf_mesh_hierarchy_create(const pf_mesh_desc* d, pf_hierarchy** out) {
   h->sub_ctl = reinterpret_cast<SubCtrl*>(h->sub_bar + 32);
   cudaMemsetAsync(h->sub_bar, 0, 256, h->st);
   if (cudaMallocHost((void**)&h->h_res, sizeof(double) * kMaxSlots) != cudaSuccess ||
-      cudaMallocHost((void**)&h->h_ctrl, sizeof(CgCtrl) + sizeof(SubCtrl)) != cudaSuccess) {
+      cudaMallocHost((void**)&h->h_ctrl, 3 * sizeof(CgCtrl) + sizeof(SubCtrl)) != cudaSuccess) {
     pf_mesh_hierarchy_destroy(h);
     set_error("cudaMallocHost failed");
     return PF_ENOMEM;
   }
-  h->h_sub_ctl = reinterpret_cast<SubCtrl*>(h->h_ctrl + 1);
+  h->h_chain = h->h_ctrl + 1;
+  h->h_sub_ctl = reinterpret_cast<SubCtrl*>(h->h_ctrl + 3);
+  for (cudaEvent_t& e : h->cg_ev)
+    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+      pf_mesh_hierarchy_destroy(h);
+      set_error("cudaEventCreate failed");
+      return PF_ECUDA;
+    }
   cudaMemsetAsync(h->scratch.counter, 0, sizeof(unsigned), h->st);
   cudaMemsetAsync(h->p_dev, 0, sizeof(float), h->st);  // the material starts at p = 0
   cudaMemsetAsync(h->c_prev, 0, sizeof(double) * h->geo.back().N, h->st);

@@ -48,6 +48,8 @@ struct pf_hierarchy {
   double* c_prev_save = nullptr;  // c_prev at the start of a load step (restored on failure)
   pf::CgCtrl* ctrl = nullptr;    // device CG control block
   pf::CgCtrl* h_ctrl = nullptr;  // pinned host mirror
+  pf::CgCtrl* h_chain = nullptr; // pinned, two mirrors read behind cg_ev
+  cudaEvent_t cg_ev[2] = {nullptr, nullptr};
   // one-launch subproblems of small levels (pf_subproblem.cu)
   double* sub_partials = nullptr;
   void* sub_work = nullptr;          // 5 vectors of the largest small level

@@ -147,13 +147,25 @@ int hessvec32_launches(const Geom& g, const void* part);
 // cg_take_curvature on c.  Returns cudaErrorNotSupported, launching
 // nothing, where that path does not apply (the caller then takes p.q in a
 // pass of its own).  partials needs kMaxBlocks doubles.
-// With dir.r set, p is first replaced by M^-1 r + beta p (beta =
-// c->beta), the direction update of the previous iteration; the product and
-// p.q use the new p.
+// With dir.r set and beta = c->beta not 0, p is first replaced by
+// M^-1 r + beta p, the direction update of the previous iteration; the product
+// and p.q use the new p.
 cudaError_t elem_hessvec32_dot(const Geom& g, const Mat<double>& m, const float* x, float* p,
                                float* q, CgCtrl* c, double* partials, unsigned* counter,
                                void* part, const float* p_dev, CgDirIn dir, cudaStream_t st);
 bool hessvec32_dot_fused(const Geom& g, const void* part);
+
+// Two vectors of which a parity (of CgCtrl::restarts) picks one.
+struct SwapPair {
+  float* v[2];
+};
+
+// The element-owned FP32 product of the v of a pair into the same y of another,
+// picked by *odd (hessvec32_dot_fused levels).  A no-op once *skip is set (skip
+// may be null).
+cudaError_t elem_hessvec32_pair(const Geom& g, const Mat<double>& m, const float* x, SwapPair v, SwapPair y,
+                                const int* odd, void* part, const float* p_dev, const int* skip,
+                                cudaStream_t st);
 // FP64 lagged Hessian: Gauss-point coefficients of x (coef holds
 // NE * 2^d * (2 + d(d+1)/2) doubles), the input of the stencil assembly.
 cudaError_t elem_hess_coef(const Geom& g, const Mat<double>& m, const double* x, double* coef,

@@ -528,16 +528,20 @@ cudaError_t elem_gradient(const Geom& g, const Mat<double>& m, const void* x, vo
 // beside the last elements of this one was slower (106 us).
 // With dir.r set (FP32 CG), v is the previous direction and the staged
 // operand is M^-1 r + beta v, beta = *beta; a run's first iteration (beta = 0)
-// does not read v.
+// takes v, which its start wrote: staging r and M^-1 instead costs 25 us more
+// than the 5 us of that write.
 constexpr int kEtileThreads = 128;  // 4 CTAs per SM at 128 registers
 template <class TV>
 __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
     k_hess_etile3(Geom g, Mat<float> m, const float* __restrict__ x, const TV* __restrict__ v,
                   float4* __restrict__ part, const int* __restrict__ skip,
-                  const float* __restrict__ p_dev, CgDirIn dir, const double* beta) {
+                  const float* __restrict__ p_dev, CgDirIn dir, const double* beta,
+                  const TV* __restrict__ v_odd = nullptr, const int* __restrict__ odd = nullptr) {
   if (skip && *skip) return;
   if (p_dev) m.p = *p_dev;
+  if (odd && (*odd & 1)) v = v_odd;
   const float be = dir.r ? float(*beta) : 0.f;
+  if (be == 0.f) dir.r = dir.mi = nullptr;
   constexpr int T = 8, NN = T + 1, NP = NN * NN, NH = NP * NN, NT = kEtileThreads;
   constexpr int NW = NT / 32, LZ = T / NW;        // warps, element layers of each
   constexpr int NA = NW * (LZ + 1) * NP;          // node planes of all warps
@@ -569,8 +573,7 @@ __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
       const long long idx = node(j, ok);
       float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
       if (ok) {
-        if (!dir.r || be != 0.f)
-          b = make_float4(float(v[idx]), float(v[N + idx]), float(v[2 * N + idx]), float(v[3 * N + idx]));
+        b = make_float4(float(v[idx]), float(v[N + idx]), float(v[2 * N + idx]), float(v[3 * N + idx]));
         if (dir.r) {
           const float4 r4 = vs[j], m4 = dir.mi ? acc[j] : make_float4(1.f, 1.f, 1.f, 1.f);
           b = make_float4(cg_direction(m4.x, r4.x, be, b.x), cg_direction(m4.y, r4.y, be, b.y),
@@ -704,8 +707,11 @@ __device__ __forceinline__ float4 etile_node_sum(const Geom& g, const float4* __
 template <class TV>
 __global__ void __launch_bounds__(256) k_etile_gather3(Geom g, const float4* __restrict__ part,
                                                        TV* __restrict__ y,
-                                                       const int* __restrict__ skip) {
+                                                       const int* __restrict__ skip,
+                                                       TV* __restrict__ y_odd = nullptr,
+                                                       const int* __restrict__ odd = nullptr) {
   if (skip && *skip) return;
+  if (odd && (*odd & 1)) y = y_odd;
   constexpr int T = 8;
   const int tx = (g.ne[0] + T - 1) / T, ty = (g.ne[1] + T - 1) / T, tz = (g.ne[2] + T - 1) / T;
   const long long N = g.N;
@@ -736,16 +742,11 @@ __global__ void __launch_bounds__(256, 4) k_etile_gather3_dot(Geom g,
   const int tx = (g.ne[0] + T - 1) / T, ty = (g.ne[1] + T - 1) / T, tz = (g.ne[2] + T - 1) / T;
   const long long N = g.N;
   const float be = dir.r ? float(c->beta) : 0.f;
+  if (be == 0.f) dir.r = nullptr;
   float pq = 0.f;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
-    float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
-    if (!dir.r || be != 0.f) {
-      p0 = p[n];
-      p1 = p[N + n];
-      p2 = p[2 * N + n];
-      p3 = p[3 * N + n];
-    }
+    float p0 = p[n], p1 = p[N + n], p2 = p[2 * N + n], p3 = p[3 * N + n];
     if (dir.r) {
       const float* r = dir.r;
       const float4 m4 = dir.mi ? make_float4(dir.mi[n], dir.mi[N + n], dir.mi[2 * N + n],
@@ -810,6 +811,18 @@ cudaError_t elem_hessvec32_dot(const Geom& g, const Mat<double>& m, const float*
   // kMaxBlocks = two waves of 4 blocks per SM
   const int nb = int(std::min<long long>((g.N + 255) / 256, kMaxBlocks));
   k_etile_gather3_dot<<<nb, 256, 0, st>>>(g, pp, p, q, c, partials, counter, dir);
+  return cudaGetLastError();
+}
+
+cudaError_t elem_hessvec32_pair(const Geom& g, const Mat<double>& m, const float* x, SwapPair v, SwapPair y,
+                                const int* odd, void* part, const float* p_dev, const int* skip,
+                                cudaStream_t st) {
+  if (!hessvec32_dot_fused(g, part)) return cudaErrorNotSupported;
+  float4* pp = static_cast<float4*>(part);
+  k_hess_etile3<float><<<etile_grid(g), kEtileThreads, 0, st>>>(
+      g, cast_mat<float>(m), x, v.v[0], pp, skip, p_dev, CgDirIn{nullptr, nullptr}, nullptr, v.v[1], odd);
+  const int nb = int(std::min<long long>((g.N + 255) / 256, 8LL * 1216));
+  k_etile_gather3<float><<<nb, 256, 0, st>>>(g, pp, y.v[0], skip, y.v[1], odd);
   return cudaGetLastError();
 }
 

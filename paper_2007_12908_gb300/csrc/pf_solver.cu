@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "pf_hier.h"
+#include "pf_cg.cuh"
 #include "pf_reduce.cuh"
 
 namespace pf {
@@ -25,13 +26,6 @@ struct CudaFail {
 
 static inline void ck(cudaError_t e, const char* where) {
   if (e != cudaSuccess) throw CudaFail{e, where};
-}
-
-__device__ __forceinline__ double clampv(double x, double lo, double hi) {
-  return fmin(fmax(x, lo), hi);
-}
-__device__ __forceinline__ float clampv(float x, float lo, float hi) {
-  return fminf(fmaxf(x, lo), hi);
 }
 
 template <class F>
@@ -94,22 +88,6 @@ __global__ void k_ctrl_start(CgCtrl* c, double rr, double rz, double tol, int us
   c->no_search = 1;
 }
 
-// Start of a CG run from a restart's (r.r, r.M^-1 r) on the device; a run that
-// starts already converged is stopped before its first iteration (CG_CONV), so
-// the host needs no read-back before it.
-__device__ __forceinline__ void ctrl_start(CgCtrl* c, double rr, double rz) {
-  c->rr = rr;
-  c->rz = rz;
-  c->alpha = 0.0;
-  c->beta = 0.0;
-  c->kappa = 0.0;
-  c->start = c->used;
-  c->no_search = 1;
-  const bool stop = sqrt(rr) <= c->tol || rr == 0.0;
-  c->done = stop ? 1 : 0;
-  c->state = stop ? CG_CONV : CG_RUNNING;
-}
-
 // The first run of a subproblem: with the forcing tolerance
 // min(0.1, sqrt||r0||) ||r0||.
 __global__ void k_ctrl_first(CgCtrl* c, const double* rrz, double m_s, int cg_max, int max_restarts) {
@@ -121,7 +99,7 @@ __global__ void k_ctrl_first(CgCtrl* c, const double* rrz, double m_s, int cg_ma
   c->searches = 0;
   c->restarts = 0;
   c->max_restarts = max_restarts;
-  ctrl_start(c, rrz[0], rrz[1]);
+  cg_start(c, rrz[0], rrz[1]);
 }
 
 template <int K, class Op, class A, class F>
@@ -144,25 +122,13 @@ __device__ __forceinline__ float4 ld4(const float* v, long long j) {
 __device__ __forceinline__ void st4(float* v, long long j, float4 x) {
   reinterpret_cast<float4*>(v)[j] = x;
 }
-__device__ __forceinline__ bool is_free(float lo, float hi, float s) { return lo - s < 0.f && 0.f < hi - s; }
 __device__ __forceinline__ bool any_free(float4 lo, float4 hi, float4 s) {
   return is_free(lo.x, hi.x, s.x) | is_free(lo.y, hi.y, s.y) | is_free(lo.z, hi.z, s.z) | is_free(lo.w, hi.w, s.w);
 }
 
-// Start of the CG loop at s: r = -(g + Hs) and, unless p is null (where the
-// product forms it), p = M^-1 r on the free set of s (0 elsewhere);
-// (r.r, r.M^-1 r) to out.  The run's first iteration takes w = 0 without
+// Start of the CG loop at s: r = -(g + Hs) and p = M^-1 r on the free set of s
+// (0 elsewhere); (r.r, r.M^-1 r) to out.  The run's first iteration takes w = 0 without
 // reading it.
-__device__ __forceinline__ void cg_init_lane(float lo, float hi, float s, float g, float hs, float m, float& r,
-                                             float& p, float& rr, float& rz) {
-  const float ri = is_free(lo, hi, s) ? -(g + hs) : 0.f;
-  const float zi = m * ri;
-  r = ri;
-  p = zi;
-  rr += ri * ri;
-  rz += ri * zi;
-}
-
 __global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __restrict__ lo,
                                                   const float* __restrict__ hi,
                                                   const float* __restrict__ s,
@@ -188,7 +154,7 @@ __global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __r
     cg_init_lane(l4.z, h4.z, s4.z, g4.z, hs4.z, m4.z, r4.z, p4.z, rr, rz);
     cg_init_lane(l4.w, h4.w, s4.w, g4.w, hs4.w, m4.w, r4.w, p4.w, rr, rz);
     st4(r, j, r4);
-    if (p) st4(p, j, p4);
+    st4(p, j, p4);
   }
   double acc[2] = {double(rr), double(rz)};
   grid_finish<2, OpSum>(acc, partials, counter, out);
@@ -198,24 +164,20 @@ __global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __r
 // sufficient decrease from s, and at the same time the start of the next CG run
 // at t (as k_cg_init4), which replaces the run that led to t whether t is
 // accepted or not (a rejected t needs only s, Hs and w).  Bound by memory: 8
-// vectors read and 1 (2) written at once, where the test, the copies of t and
+// vectors read and 2 written at once, where the test, the copies of t and
 // Ht to s and Hs, the model value at s and k_cg_init4 took 155 us at 129^3
 // (28 passes of 34 MB); this takes FIGURE us.
-__device__ __forceinline__ void cg_search_lane(float lo, float hi, float s, float hs, float t, float ht,
-                                               float g, float m, float& r, float& p, float (&o)[5]) {
-  o[2] += g * t;
-  o[3] += t * ht;
-  o[4] += (g + hs) * (t - s);
-  cg_init_lane(lo, hi, t, g, ht, m, r, p, o[0], o[1]);
-}
-
 __global__ void __launch_bounds__(256) k_cg_search4(
-    long long n4, const float* __restrict__ lo, const float* __restrict__ hi, const float* __restrict__ s,
-    const float* __restrict__ Hs, const float* __restrict__ t, const float* __restrict__ Ht,
+    long long n4, const float* __restrict__ lo, const float* __restrict__ hi, SwapPair sv, SwapPair hv,
     const float* __restrict__ g, const float* __restrict__ mi, bool pc, float* __restrict__ r,
-    float* __restrict__ p, double cauchy_c, CgCtrl* c,
-    double* partials, unsigned* counter, const int* __restrict__ skip) {
+    float* __restrict__ p, double cauchy_c, CgCtrl* c, double* partials, unsigned* counter,
+    const int* __restrict__ skip) {
   if (skip && *skip) return;
+  const bool odd = c->restarts & 1;
+  const float* __restrict__ s = odd ? sv.v[1] : sv.v[0];
+  const float* __restrict__ t = odd ? sv.v[0] : sv.v[1];
+  const float* __restrict__ Hs = odd ? hv.v[1] : hv.v[0];
+  const float* __restrict__ Ht = odd ? hv.v[0] : hv.v[1];
   float o[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n4;
        j += (long long)gridDim.x * blockDim.x) {
@@ -228,27 +190,10 @@ __global__ void __launch_bounds__(256) k_cg_search4(
     cg_search_lane(l4.z, h4.z, s4.z, hs4.z, t4.z, ht4.z, g4.z, m4.z, r4.z, p4.z, o);
     cg_search_lane(l4.w, h4.w, s4.w, hs4.w, t4.w, ht4.w, g4.w, m4.w, r4.w, p4.w, o);
     st4(r, j, r4);
-    if (p) st4(p, j, p4);
+    st4(p, j, p4);
   }
   double acc[5] = {double(o[0]), double(o[1]), double(o[2]), double(o[3]), double(o[4])};
-  auto fin = [c, cauchy_c](double(&v)[5]) {
-    c->searches += 1;
-    c->no_search = 1;
-    const double m_t = v[2] + 0.5 * v[3];
-    if (!(m_t <= c->m_s + cauchy_c * v[4])) {
-      c->done = 1;
-      c->state = CG_REJECT;
-      return;
-    }
-    c->m_s = m_t;
-    c->restarts += 1;
-    if (c->restarts > c->max_restarts || c->used >= c->cg_max) {
-      c->done = 1;
-      c->state = CG_STOP;
-      return;
-    }
-    ctrl_start(c, v[0], v[1]);
-  };
+  auto fin = [c, cauchy_c](double(&v)[5]) { cg_search_done(c, v, cauchy_c); };
   grid_finish_fn<5, OpSum>(acc, partials, counter, fin);
 }
 
@@ -272,10 +217,6 @@ __device__ __forceinline__ void cg_update_lane(float al, bool fresh, float lo, f
   rz += r * (m * r);
   t = clampv(s + w, lo, hi);
 }
-
-struct SwapPair {
-  float* v[2];
-};
 
 __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* __restrict__ lo,
                                                     const float* __restrict__ hi, SwapPair sv,
@@ -1359,7 +1300,8 @@ struct Solver {
       return;
     }
     if constexpr (std::is_same<V, float>::value) {
-      cg_runs32(l, cg_max, vec, m_s);
+      if (!gstored(l) && hessvec32_dot_fused(H->geo[l], H->etile_part)) cg_chain32(l, cg_max, vec, m_s);
+      else cg_runs32(l, cg_max, vec, m_s);
       return;
     } else {
       int used = 0;
@@ -1508,13 +1450,102 @@ struct Solver {
   }
 
   // The CG runs and projected searches of a subproblem on FP32 vectors from the
-  // Cauchy point (s, Hs), whose model value is m_s.  Searches at full length
-  // and the starts of the runs after them are decided on the device, so that
-  // several runs are enqueued between two read-backs (13 us each, and the GPU
-  // waits for the launches after it): a chunk of 1, 2, then 4, whose launches
-  // after a stop are no-ops (some 20 us a run, at most 3 of them, against runs
-  // of 0.4 ms at 129^3).  A run that meets non-positive curvature and a search
-  // that has to be shortened go through the host.
+  // Cauchy point (s, Hs) with model value m_s, on levels whose product is
+  // element-owned.  A step is one CG iteration and the search due if it left
+  // the box (no-ops once the run or the subproblem has stopped; the device
+  // decides).  Steps go out in pairs, one pair ahead of the one whose control
+  // block the host waits for, so the GPU does not idle.  At 129^3 two runs in
+  // three are one iteration long: with a graph launch per run, its while node
+  // (5.5 us a turn) and a read-back per 4 runs the load step took FIGURE.
+  // A run that meets non-positive curvature and a search that has to be
+  // shortened go through the host.
+  void cg_chain32(int l, int cg_max, const SubVecs<float>& vec, double m_s) {
+    LevelBuf& B = H->lv[l];
+    const long long n = B.n, n4 = pad4(n) / 4;
+    const float *lo = vec.lo, *hi = vec.hi;
+    float *w = vec.w, *out = vec.s;
+    float *sv[2] = {vec.s, vec.t1};
+    CgCtrl* c = H->ctrl;
+    CgCtrl hc{};
+    if (cg_max > 0) {
+      const bool pc = P.precondition != 0;
+      const CgVecs<float> cgv{vec.p, vec.q, w, vec.r, vec.mi, nullptr, nullptr, lo, hi, {sv[0], sv[1]}, pc};
+      const SwapPair sp{{sv[0], sv[1]}}, hp{{vec.Hs, vec.t2}};
+      auto search = [&](const int* skip) {
+        // Ht = H t, t and Ht the other of their pairs
+        ck(elem_hessvec32_pair(H->geo[l], H->mat[l], B.xlag32, SwapPair{{sv[1], sv[0]}},
+                               SwapPair{{vec.t2, vec.Hs}}, &c->restarts, H->etile_part, H->p_dev, skip, st),
+           "hessvec32");
+        k_cg_search4<<<resident_grid(k_cg_search4, n4), 256, 0, st>>>(
+            n4, lo, hi, sp, hp, vec.g, vec.mi, pc, vec.r, vec.p, P.cauchy_c, c, H->scratch.partials,
+            H->scratch.counter, skip);
+        ck(cudaGetLastError(), "cg_search");
+        S.launches += 3;
+      };
+      k_cg_init4<<<resident_grid(k_cg_init4, n4), 256, 0, st>>>(n4, lo, hi, vec.s, vec.g, vec.Hs, vec.mi, pc,
+                                                               vec.r, vec.p, H->scratch.partials,
+                                                               H->scratch.counter, H->d_res);
+      ck(cudaGetLastError(), "cg_init");
+      k_ctrl_first<<<1, 1, 0, st>>>(c, H->d_res, m_s, cg_max, P.max_restarts);
+      ck(cudaGetLastError(), "ctrl");
+      S.launches += 2;
+      for (;;) {
+        for (int k = 0;; ++k) {
+          for (int j = 0; j < 2; ++j) {
+            S.launches += cg_iter4(l, cgv, st);
+            search(&c->no_search);
+          }
+          ck(cudaMemcpyAsync(H->h_chain + (k & 1), c, sizeof(CgCtrl), cudaMemcpyDeviceToHost, st), "ctrl");
+          ck(cudaEventRecord(H->cg_ev[k & 1], st), "event");
+          if (k == 0) continue;
+          ck(cudaEventSynchronize(H->cg_ev[(k - 1) & 1]), "sync");
+          hc = H->h_chain[(k - 1) & 1];
+          if (hc.done && hc.no_search) break;  // the pair in flight changes nothing
+        }
+        const int odd = hc.restarts & 1;
+        float *s = sv[odd], *t = sv[1 - odd];
+        if (hc.state == CG_CONV || hc.state == CG_BUDGET) {
+          if (hc.used > hc.start) map(n, [=] __device__(long long i) { s[i] += w[i]; });
+          break;
+        }
+        if (hc.state == CG_STOP) break;
+        float bb = 1.f;
+        int bt = 0;
+        if (hc.state == CG_NEGCURV) {
+          to_box<float>(n, vec.p, w, GapBox{lo, hi, s}, hc.used == hc.start + 1);
+        } else {  // CG_REJECT at full length
+          bb = 0.5f;
+          bt = 1;
+        }
+        for (; bt <= P.cauchy_backtracks; ++bt, bb *= 0.5f) {
+          map(n, [=] __device__(long long i) { t[i] = clampv(s[i] + bb * w[i], lo[i], hi[i]); });
+          search(nullptr);
+          read_ctrl();
+          hc = *H->h_ctrl;
+          if (hc.state != CG_REJECT) break;
+        }
+        if (bt > P.cauchy_backtracks || hc.state == CG_STOP) break;
+      }
+      count_cg(l, hc);
+    }
+    const float* s = sv[hc.restarts & 1];
+    map(n, [=] __device__(long long i) { out[i] = clampv(s[i], lo[i], hi[i]); });
+  }
+
+  void count_cg(int l, const CgCtrl& c) {
+    S.cg += c.used;
+    S.cg_level[std::min(l, 7)] += c.used;
+    S.hv_search += c.searches;
+    S.cg_restarts += c.restarts;
+    S.hessvecs += c.used + c.searches;
+    S.fe_hessvec += double(c.used + c.searches) * hlag_units(l);
+  }
+
+  // The same on the other FP32 levels, whose runs are longer and whose
+  // iterations are short (25 to 30 us as a graph): several runs are enqueued
+  // between two read-backs (13 us each, and the GPU waits for the launches after
+  // it), a chunk of 1, 2, then 4, whose launches after a stop are no-ops (some
+  // 20 us a run, at most 3 of them).
   void cg_runs32(int l, int cg_max, const SubVecs<float>& vec, double m_s) {
     const long long n = H->lv[l].n, n4 = pad4(n) / 4;
     const float *g = vec.g, *lo = vec.lo, *hi = vec.hi, *mi = vec.mi;
@@ -1523,20 +1554,18 @@ struct Solver {
     CgCtrl* c = H->ctrl;
     const bool pc = P.precondition != 0;
     const CgVecs<float> cgv{p, q, w, r, mi, nullptr, nullptr, lo, hi, {s, t1}, pc};
-    // the products that form the direction themselves need no start of p
-    float* p0 = !gstored(l) && hessvec32_dot_fused(H->geo[l], H->etile_part) ? nullptr : p;
     // product and test of the projected step t1
     auto search = [&](const int* skip) {
       hv<float>(l, t1, t2, skip, false);
       k_cg_search4<<<resident_grid(k_cg_search4, n4), 256, 0, st>>>(
-          n4, lo, hi, s, Hs, t1, t2, g, mi, pc, r, p0, P.cauchy_c, c, H->scratch.partials,
+          n4, lo, hi, SwapPair{{vec.s, vec.t1}}, SwapPair{{vec.Hs, vec.t2}}, g, mi, pc, r, p, P.cauchy_c, c, H->scratch.partials,
           H->scratch.counter, skip);
       ck(cudaGetLastError(), "cg_search");
       S.launches += 1;
     };
     if (cg_max > 0) {
       cudaGraphExec_t graph = cg_graph<float>(l, cgv);
-      k_cg_init4<<<resident_grid(k_cg_init4, n4), 256, 0, st>>>(n4, lo, hi, s, g, Hs, mi, pc, r, p0,
+      k_cg_init4<<<resident_grid(k_cg_init4, n4), 256, 0, st>>>(n4, lo, hi, s, g, Hs, mi, pc, r, p,
                                                                H->scratch.partials, H->scratch.counter,
                                                                H->d_res);
       ck(cudaGetLastError(), "cg_init");
@@ -1587,14 +1616,8 @@ struct Solver {
         if (hc->state == CG_STOP) break;
         run_cg<float>(l, graph, cgv);
       }
-      const CgCtrl cs = *H->h_ctrl;
-      S.cg += cs.used;
-      S.cg_level[std::min(l, 7)] += cs.used;
-      S.hv_search += cs.searches;
-      S.cg_restarts += cs.restarts;
-      S.hessvecs += cs.used + cs.searches;
-      S.fe_hessvec += double(cs.used + cs.searches) * hlag_units(l);
-      if (graph) S.launches += (long long)H->cg_graphs[l].nodes * cs.used;
+      count_cg(l, *H->h_ctrl);
+      if (graph) S.launches += (long long)H->cg_graphs[l].nodes * H->h_ctrl->used;
     }
     float* out = vec.s;
     map(n, [=] __device__(long long i) { out[i] = clampv(s[i], lo[i], hi[i]); });
