@@ -7,10 +7,10 @@
 // read-back of 13 us per scalar.  A 65^2 FP64 load step took 34 to 37 ms for
 // about 1,030 iterations, some 30 us each.  Here the whole solve -- Cauchy
 // point, CG runs, projected searches, restarts -- is one kernel whose CTAs
-// meet at a grid barrier: two per CG iteration, which takes 11 us (3.5 of them
+// meet at a grid barrier: two per CG iteration, which takes 9.5 us (3.5 of them
 // the barriers' latency, the rest FP64 chains: the product's 27 multiply-adds
 // in 9 warps of an SM at 16 cycles each, the trees of the sums, a division),
-// and the load step 14 ms.
+// and the load step 13 ms.
 //
 // A row (node and field) belongs to one lane for the whole solve: its vectors
 // stay in registers, and where they fit (all but FP64 in 3D) so do its stencil
@@ -206,11 +206,17 @@ struct Sub {
     }
     if (!barrier()) return false;
     if (w < K) {
-      double x = w == 0 ? Op0::id() : 0.0;
-#pragma unroll 4
-      for (int b = wl; b < nb; b += 32) {
-        const double y = __ldcg(p + w * kMaxCoopBlocks + b);
-        x = w == 0 ? Op0::op(x, y) : x + y;
+      const double id = w == 0 ? Op0::id() : 0.0;
+      double x = id;
+      for (int b0 = wl; b0 < nb; b0 += 32 * 5) {  // one round of loads for 160 CTAs
+        double y[5];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+          const int b = b0 + 32 * i;
+          y[i] = b < nb ? __ldcg(p + w * kMaxCoopBlocks + b) : id;
+        }
+#pragma unroll
+        for (int i = 0; i < 5; ++i) x = w == 0 ? Op0::op(x, y[i]) : x + y[i];
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
