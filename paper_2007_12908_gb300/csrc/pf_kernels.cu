@@ -15,6 +15,7 @@
 #include "pf_df.cuh"
 #include "pf_element_f2.cuh"
 #include "pf_internal.h"
+#include "pf_launch.cuh"
 #include "pf_reduce.cuh"
 #include "pf_stencil.cuh"
 
@@ -255,8 +256,8 @@ __global__ void __launch_bounds__(256) k_hess_coef(Geom g, Mat<T> m, const T* __
 // share an SM and hide the gather and barrier latency.
 template <int D, class TC, class TIO, int OP, class TM = TC, class TS = Tile<D>>
 __global__ void __launch_bounds__(TS::THREADS, sizeof(TC) == 4 ? 2 : 1)
-    k_elem_scatter(Geom g, Mat<TC> m, const TM* __restrict__ x, const TIO* __restrict__ v,
-                   TIO* __restrict__ y, const int* __restrict__ skip) {
+    k_elem_scatter(Geom g, Mat<TC> m, const TM* x, const TIO* v, TIO* y, const int* skip) {
+  launch_wait();
   if (skip && *skip) return;
   constexpr int F = D + 1, NC = 1 << D;
   constexpr int TX = TS::X, TY = TS::Y, TZ = TS::Z;
@@ -369,9 +370,9 @@ __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" 
 // captured the launch then follows pf_pressure_set).
 template <class TV, int T = 8, int OP = OP_HESS, class TX = float>
 __global__ void __launch_bounds__(HessTile<T>::THREADS, 4)
-    k_hess_tile3(Geom g, Mat<float> m, const TX* __restrict__ x, const TV* __restrict__ v,
-                 TV* __restrict__ y, const int* __restrict__ skip,
-                 const float* __restrict__ p_dev = nullptr) {
+    k_hess_tile3(Geom g, Mat<float> m, const TX* x, const TV* v, TV* y, const int* skip,
+                 const float* p_dev = nullptr) {
+  launch_wait();
   if (skip && *skip) return;
   if (p_dev) m.p = *p_dev;
   constexpr int E = T + 1, NN = T + 2, NH = NN * NN * NN, NT = HessTile<T>::THREADS;
@@ -468,10 +469,9 @@ static dim3 scatter_grid(const Geom& g) {
 template <int D, class TC, class TIO, int OP, class TM = TC, class TS = Tile<D>>
 static cudaError_t launch_scatter(const Geom& g, const Mat<double>& m, const void* x,
                                   const void* v, void* y, const int* skip, cudaStream_t st) {
-  k_elem_scatter<D, TC, TIO, OP, TM, TS><<<scatter_grid<D, TS>(g), TS::THREADS, 0, st>>>(
-      g, cast_mat<TC>(m), static_cast<const TM*>(x), static_cast<const TIO*>(v),
-      static_cast<TIO*>(y), skip);
-  return cudaGetLastError();
+  return launch_dependent(k_elem_scatter<D, TC, TIO, OP, TM, TS>, scatter_grid<D, TS>(g), dim3(TS::THREADS), st, g,
+                          cast_mat<TC>(m), static_cast<const TM*>(x), static_cast<const TIO*>(v),
+                          static_cast<TIO*>(y), skip);
 }
 
 // The 2D FP32 Hessian product on the node tile of the grid's variant.
@@ -844,12 +844,10 @@ static cudaError_t launch_hess_tile3(const Geom& g, const Mat<double>& m, const 
   const dim3 b8 = tiles(8);
   const bool t8 = g.hv_variant ? g.hv_variant != 3 : (long long)b8.x * b8.y * b8.z >= 2 * 152;
   if (t8)
-    k_hess_tile3<TV, 8><<<b8, HessTile<8>::THREADS, 0, st>>>(g, cast_mat<float>(m), x, v, y, skip,
-                                                              p_dev);
-  else
-    k_hess_tile3<TV, 4><<<tiles(4), HessTile<4>::THREADS, 0, st>>>(g, cast_mat<float>(m), x, v, y,
-                                                                  skip, p_dev);
-  return cudaGetLastError();
+    return launch_dependent(k_hess_tile3<TV, 8>, b8, dim3(HessTile<8>::THREADS), st, g, cast_mat<float>(m), x,
+                            v, y, skip, p_dev);
+  return launch_dependent(k_hess_tile3<TV, 4>, tiles(4), dim3(HessTile<4>::THREADS), st, g, cast_mat<float>(m),
+                          x, v, y, skip, p_dev);
 }
 
 cudaError_t elem_hessvec(const Geom& g, const Mat<double>& m, const void* x, const void* v,

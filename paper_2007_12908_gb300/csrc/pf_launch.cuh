@@ -1,0 +1,44 @@
+// Programmatic dependent launch of short kernels: the CTAs start while the
+// launch before them drains, and wait for it (launch_wait) before they first
+// touch global memory, so that back-to-back launches of a few microseconds do
+// not pay the launch latency each.  3D FP32 product on 33 x 25 x 29 nodes, one
+// after another: 8.2 -> 5.7 us; FP64 energy, gradient, lag and eight products
+// on 69 x 45: 100 -> 86 us.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <utility>
+
+namespace pf {
+
+// Every earlier launch of the stream has ended and its writes are visible
+// after this; the launch after this one may then start.  Pointers whose first
+// read follows it are not __restrict__: a load known to be invariant could be
+// moved before it.
+__device__ __forceinline__ void launch_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch of a kernel whose threads call launch_wait() before any global memory
+// access.  An ordinary launch under stream capture (the CG graphs' bodies).
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, A&&... a) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    cap = cudaStreamCaptureStatusActive;
+  }
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, std::forward<A>(a)...);
+}
+
+}  // namespace pf

@@ -8,10 +8,12 @@
 // as 0, so no load waits for a branch.  One thread per row walking its 27 or
 // 108 entries took 9.5 us for the 9,315 FP64 rows of 69 x 45 nodes and 74 us
 // for the 143,748 FP32 rows of 33^3 (ncu, cold cache); now 6.5 and 17.6 us.
+// A launch starts while the one before it drains (launch_dependent).
 #pragma once
 #include <cuda_runtime.h>
 
 #include "pf_internal.h"
+#include "pf_launch.cuh"
 
 namespace pf {
 
@@ -23,8 +25,8 @@ struct StencilRows {
 
 template <int D, class TS, class TV>
 __global__ void __launch_bounds__(StencilRows<D>::THREADS)
-    k_stencil_rows(Geom g, const TS* __restrict__ S, const TV* __restrict__ v, TV* __restrict__ y,
-                   const int* __restrict__ skip) {
+    k_stencil_rows(Geom g, const TS* S, const TV* v, TV* y, const int* skip) {
+  launch_wait();
   if (skip && *skip) return;
   constexpr int F = D + 1, LINES = StencilRows<D>::LINES, LANES = StencilRows<D>::LANES;
   __shared__ TV part[LINES][LANES];
@@ -87,8 +89,7 @@ inline cudaError_t stencil_rows(const Geom& g, const TS* S, const TV* v, TV* y, 
   using R = StencilRows<D>;
   const long long nb = ((D + 1) * g.N + R::LANES - 1) / R::LANES;
   if (nb > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  k_stencil_rows<D, TS, TV><<<unsigned(nb), R::THREADS, 0, st>>>(g, S, v, y, skip);
-  return cudaGetLastError();
+  return launch_dependent(k_stencil_rows<D, TS, TV>, dim3(unsigned(nb)), dim3(R::THREADS), st, g, S, v, y, skip);
 }
 
 }  // namespace pf
