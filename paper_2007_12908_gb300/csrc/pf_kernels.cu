@@ -533,10 +533,10 @@ cudaError_t elem_gradient(const Geom& g, const Mat<double>& m, const void* x, vo
 constexpr int kEtileThreads = 128;  // 4 CTAs per SM at 128 registers
 template <class TV>
 __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
-    k_hess_etile3(Geom g, Mat<float> m, const float* __restrict__ x, const TV* __restrict__ v,
-                  float4* __restrict__ part, const int* __restrict__ skip,
-                  const float* __restrict__ p_dev, CgDirIn dir, const double* beta,
-                  const TV* __restrict__ v_odd = nullptr, const int* __restrict__ odd = nullptr) {
+    k_hess_etile3(Geom g, Mat<float> m, const float* x, const TV* v, float4* part, const int* skip,
+                  const float* p_dev, CgDirIn dir, const double* beta, const TV* v_odd = nullptr,
+                  const int* odd = nullptr) {
+  launch_wait();
   if (skip && *skip) return;
   if (p_dev) m.p = *p_dev;
   if (odd && (*odd & 1)) v = v_odd;
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
 // hold the node are loaded and added; the loads of each z layer of
 // candidates are issued together, so a node costs one memory latency (two
 // on a z boundary), not one per tile.
-__device__ __forceinline__ float4 etile_node_sum(const Geom& g, const float4* __restrict__ part,
+__device__ __forceinline__ float4 etile_node_sum(const Geom& g, const float4* part,
                                                  long long n, int tx, int ty, int tz) {
   constexpr int T = 8, NN = T + 1, NH = NN * NN * NN;
   int i, j, k;
@@ -705,11 +705,9 @@ __device__ __forceinline__ float4 etile_node_sum(const Geom& g, const float4* __
 // Pass 2: each node sums the blocks of the tiles that contain it and
 // writes y.
 template <class TV>
-__global__ void __launch_bounds__(256) k_etile_gather3(Geom g, const float4* __restrict__ part,
-                                                       TV* __restrict__ y,
-                                                       const int* __restrict__ skip,
-                                                       TV* __restrict__ y_odd = nullptr,
-                                                       const int* __restrict__ odd = nullptr) {
+__global__ void __launch_bounds__(256) k_etile_gather3(Geom g, const float4* part, TV* y, const int* skip,
+                                                       TV* y_odd = nullptr, const int* odd = nullptr) {
+  launch_wait();
   if (skip && *skip) return;
   if (odd && (*odd & 1)) y = y_odd;
   constexpr int T = 8;
@@ -737,6 +735,7 @@ __global__ void __launch_bounds__(256, 4) k_etile_gather3_dot(Geom g,
                                                               float* __restrict__ y, CgCtrl* c,
                                                               double* partials,
                                                               unsigned* counter, CgDirIn dir) {
+  launch_wait();
   if (c->done) return;
   constexpr int T = 8;
   const int tx = (g.ne[0] + T - 1) / T, ty = (g.ne[1] + T - 1) / T, tz = (g.ne[2] + T - 1) / T;
@@ -806,12 +805,13 @@ cudaError_t elem_hessvec32_dot(const Geom& g, const Mat<double>& m, const float*
                                void* part, const float* p_dev, CgDirIn dir, cudaStream_t st) {
   if (!hessvec32_dot_fused(g, part)) return cudaErrorNotSupported;
   float4* pp = static_cast<float4*>(part);
-  k_hess_etile3<float><<<etile_grid(g), kEtileThreads, 0, st>>>(g, cast_mat<float>(m), x, p, pp, &c->done, p_dev, dir,
-                                           &c->beta);
+  const cudaError_t e = launch_dependent(k_hess_etile3<float>, etile_grid(g), dim3(kEtileThreads), st, g,
+                                         cast_mat<float>(m), x, p, pp, &c->done, p_dev, dir, &c->beta,
+                                         nullptr, nullptr);
+  if (e != cudaSuccess) return e;
   // kMaxBlocks = two waves of 4 blocks per SM
   const int nb = int(std::min<long long>((g.N + 255) / 256, kMaxBlocks));
-  k_etile_gather3_dot<<<nb, 256, 0, st>>>(g, pp, p, q, c, partials, counter, dir);
-  return cudaGetLastError();
+  return launch_dependent(k_etile_gather3_dot, dim3(nb), dim3(256), st, g, pp, p, q, c, partials, counter, dir);
 }
 
 cudaError_t elem_hessvec32_pair(const Geom& g, const Mat<double>& m, const float* x, SwapPair v, SwapPair y,
@@ -819,11 +819,12 @@ cudaError_t elem_hessvec32_pair(const Geom& g, const Mat<double>& m, const float
                                 cudaStream_t st) {
   if (!hessvec32_dot_fused(g, part)) return cudaErrorNotSupported;
   float4* pp = static_cast<float4*>(part);
-  k_hess_etile3<float><<<etile_grid(g), kEtileThreads, 0, st>>>(
-      g, cast_mat<float>(m), x, v.v[0], pp, skip, p_dev, CgDirIn{nullptr, nullptr}, nullptr, v.v[1], odd);
+  const cudaError_t e = launch_dependent(k_hess_etile3<float>, etile_grid(g), dim3(kEtileThreads), st, g,
+                                         cast_mat<float>(m), x, v.v[0], pp, skip, p_dev,
+                                         CgDirIn{nullptr, nullptr}, nullptr, v.v[1], odd);
+  if (e != cudaSuccess) return e;
   const int nb = int(std::min<long long>((g.N + 255) / 256, 8LL * 1216));
-  k_etile_gather3<float><<<nb, 256, 0, st>>>(g, pp, y.v[0], skip, y.v[1], odd);
-  return cudaGetLastError();
+  return launch_dependent(k_etile_gather3<float>, dim3(nb), dim3(256), st, g, pp, y.v[0], skip, y.v[1], odd);
 }
 
 template <class TV>
@@ -835,11 +836,12 @@ static cudaError_t launch_hess_tile3(const Geom& g, const Mat<double>& m, const 
   };
   if (etile_used(g, part)) {
     float4* pp = static_cast<float4*>(part);
-    k_hess_etile3<TV><<<etile_grid(g), kEtileThreads, 0, st>>>(g, cast_mat<float>(m), x, v, pp, skip, p_dev,
-                                          CgDirIn{nullptr, nullptr}, nullptr);
+    const cudaError_t e = launch_dependent(k_hess_etile3<TV>, etile_grid(g), dim3(kEtileThreads), st, g,
+                                           cast_mat<float>(m), x, v, pp, skip, p_dev,
+                                           CgDirIn{nullptr, nullptr}, nullptr, nullptr, nullptr);
+    if (e != cudaSuccess) return e;
     const int nb = int(std::min<long long>((g.N + 255) / 256, 8LL * 1216));
-    k_etile_gather3<TV><<<nb, 256, 0, st>>>(g, pp, y, skip);
-    return cudaGetLastError();
+    return launch_dependent(k_etile_gather3<TV>, dim3(nb), dim3(256), st, g, pp, y, skip, nullptr, nullptr);
   }
   const dim3 b8 = tiles(8);
   const bool t8 = g.hv_variant ? g.hv_variant != 3 : (long long)b8.x * b8.y * b8.z >= 2 * 152;

@@ -15,6 +15,7 @@
 
 #include "pf_hier.h"
 #include "pf_cg.cuh"
+#include "pf_launch.cuh"
 #include "pf_reduce.cuh"
 
 namespace pf {
@@ -30,13 +31,15 @@ static inline void ck(cudaError_t e, const char* where) {
 
 template <class F>
 __global__ void k_map(long long n, F f) {
+  launch_wait();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     f(i);
 }
 
 template <class F>
-__global__ void k_map_skip(long long n, F f, const int* __restrict__ skip) {
+__global__ void k_map_skip(long long n, F f, const int* skip) {
+  launch_wait();
   if (*skip) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
@@ -66,7 +69,8 @@ __device__ __forceinline__ void thread_part(long long n, F& f, double (&out)[K])
 // device; a no-op launch when *skip is set.
 template <int K, class Op, class A, class F, class Fin>
 __global__ void __launch_bounds__(256) k_red_fin(long long n, F f, Fin fin, double* partials,
-                                                 unsigned* counter, const int* __restrict__ skip) {
+                                                 unsigned* counter, const int* skip) {
+  launch_wait();
   if (*skip) return;
   double acc[K];
   thread_part<K, Op, A>(n, f, acc);
@@ -74,6 +78,7 @@ __global__ void __launch_bounds__(256) k_red_fin(long long n, F f, Fin fin, doub
 }
 
 __global__ void k_ctrl_start(CgCtrl* c, double rr, double rz, double tol, int used, int cg_max) {
+  launch_wait();
   c->rr = rr;
   c->rz = rz;
   c->tol = tol;
@@ -91,6 +96,7 @@ __global__ void k_ctrl_start(CgCtrl* c, double rr, double rz, double tol, int us
 // The first run of a subproblem: with the forcing tolerance
 // min(0.1, sqrt||r0||) ||r0||.
 __global__ void k_ctrl_first(CgCtrl* c, const double* rrz, double m_s, int cg_max, int max_restarts) {
+  launch_wait();
   const double r0 = sqrt(rrz[0]);
   c->tol = fmin(0.1, sqrt(r0)) * r0;
   c->m_s = m_s;
@@ -105,6 +111,7 @@ __global__ void k_ctrl_first(CgCtrl* c, const double* rrz, double m_s, int cg_ma
 template <int K, class Op, class A, class F>
 __global__ void __launch_bounds__(256) k_red(long long n, F f, double* partials, unsigned* counter,
                                              double* out) {
+  launch_wait();
   double acc[K];
   thread_part<K, Op, A>(n, f, acc);
   grid_finish<K, Op>(acc, partials, counter, out);
@@ -129,14 +136,11 @@ __device__ __forceinline__ bool any_free(float4 lo, float4 hi, float4 s) {
 // Start of the CG loop at s: r = -(g + Hs) and p = M^-1 r on the free set of s
 // (0 elsewhere); (r.r, r.M^-1 r) to out.  The run's first iteration takes w = 0 without
 // reading it.
-__global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* __restrict__ lo,
-                                                  const float* __restrict__ hi,
-                                                  const float* __restrict__ s,
-                                                  const float* __restrict__ g,
-                                                  const float* __restrict__ Hs,
-                                                  const float* __restrict__ mi, bool pc,
-                                                  float* __restrict__ r, float* __restrict__ p,
-                                                  double* partials, unsigned* counter, double* out) {
+__global__ void __launch_bounds__(256) k_cg_init4(long long n4, const float* lo, const float* hi, const float* s,
+                                                  const float* g, const float* Hs, const float* mi,
+                                                  bool pc, float* r, float* p, double* partials,
+                                                  unsigned* counter, double* out) {
+  launch_wait();
   float rr = 0.f, rz = 0.f;
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n4;
        j += (long long)gridDim.x * blockDim.x) {
@@ -171,7 +175,8 @@ __global__ void __launch_bounds__(256) k_cg_search4(
     long long n4, const float* __restrict__ lo, const float* __restrict__ hi, SwapPair sv, SwapPair hv,
     const float* __restrict__ g, const float* __restrict__ mi, bool pc, float* __restrict__ r,
     float* __restrict__ p, double cauchy_c, CgCtrl* c, double* partials, unsigned* counter,
-    const int* __restrict__ skip) {
+    const int* skip) {
+  launch_wait();
   if (skip && *skip) return;
   const bool odd = c->restarts & 1;
   const float* __restrict__ s = odd ? sv.v[1] : sv.v[0];
@@ -226,6 +231,7 @@ __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* _
                                                     float* __restrict__ w, float* __restrict__ r,
                                                     CgCtrl* c, double* partials,
                                                     unsigned* counter) {
+  launch_wait();
   if (c->done) return;
   const float al = float(c->alpha);
   const bool fresh = c->used == c->start + 1;
@@ -283,6 +289,7 @@ __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* _
 __global__ void __launch_bounds__(256) k_cg_dot4(long long n4, const float* __restrict__ p,
                                                  const float* __restrict__ q, CgCtrl* c,
                                                  double* partials, unsigned* counter) {
+  launch_wait();
   if (c->done) return;
   float pq = 0.f;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -305,6 +312,7 @@ __global__ void __launch_bounds__(256) k_cg_dot4(long long n4, const float* __re
 __global__ void __launch_bounds__(256) k_cg_dir4(long long n4, const float* __restrict__ r,
                                                  const float* __restrict__ mi, bool pc,
                                                  float* __restrict__ p, const CgCtrl* c) {
+  launch_wait();
   if (c->done) return;
   const float be = float(c->beta);
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -422,31 +430,29 @@ struct Solver {
   // ---------------------------------------------------------------- helpers
   template <class Fn>
   void map(long long n, Fn f) {
-    k_map<<<resident_grid(k_map<Fn>, n), 256, 0, st>>>(n, f);
-    ck(cudaGetLastError(), "map");
+    ck(launch_dependent(k_map<Fn>, dim3(resident_grid(k_map<Fn>, n)), dim3(256), st, n, f), "map");
     S.launches += 1;
   }
 
   template <class Fn>
   void map_skip(long long n, Fn f, const int* skip) {
-    k_map_skip<<<map_grid(n), 256, 0, st>>>(n, f, skip);
-    ck(cudaGetLastError(), "map_skip");
+    ck(launch_dependent(k_map_skip<Fn>, dim3(map_grid(n)), dim3(256), st, n, f, skip), "map_skip");
     S.launches += 1;
   }
 
   template <int K, class Op, class A = double, class Fn, class Fin>
   void red_fin(long long n, Fn f, Fin fin, const int* skip) {
-    k_red_fin<K, Op, A><<<reduce_grid(n), 256, 0, st>>>(n, f, fin, H->scratch.partials,
-                                                         H->scratch.counter, skip);
-    ck(cudaGetLastError(), "red_fin");
+    ck(launch_dependent(k_red_fin<K, Op, A, Fn, Fin>, dim3(reduce_grid(n)), dim3(256), st, n, f, fin,
+                        H->scratch.partials, H->scratch.counter, skip),
+       "red_fin");
     S.launches += 1;
   }
 
   template <int K, class Op, class A = double, class Fn>
   void reduce(long long n, Fn f, double* out) {
-    k_red<K, Op, A><<<resident_grid(k_red<K, Op, A, Fn>, n), 256, 0, st>>>(
-        n, f, H->scratch.partials, H->scratch.counter, H->d_res);
-    ck(cudaGetLastError(), "reduce");
+    ck(launch_dependent(k_red<K, Op, A, Fn>, dim3(resident_grid(k_red<K, Op, A, Fn>, n)), dim3(256), st, n, f,
+                        H->scratch.partials, H->scratch.counter, H->d_res),
+       "reduce");
     S.launches += 1;
     fetch(K, out);
   }
@@ -454,9 +460,9 @@ struct Solver {
   // reduce() without the read-back: results stay at out_dev
   template <int K, class Op, class A = double, class Fn>
   void reduce_dev(long long n, Fn f, double* out_dev) {
-    k_red<K, Op, A><<<resident_grid(k_red<K, Op, A, Fn>, n), 256, 0, st>>>(
-        n, f, H->scratch.partials, H->scratch.counter, out_dev);
-    ck(cudaGetLastError(), "reduce");
+    ck(launch_dependent(k_red<K, Op, A, Fn>, dim3(resident_grid(k_red<K, Op, A, Fn>, n)), dim3(256), st, n, f,
+                        H->scratch.partials, H->scratch.counter, out_dev),
+       "reduce");
     S.launches += 1;
   }
 
@@ -786,10 +792,10 @@ struct Solver {
     const long long n4 = pad4(B.n) / 4;
     float *p = v.p, *q = v.q;
     auto update = [&] {
-      k_cg_update4<<<resident_grid(k_cg_update4, n4), 256, 0, s>>>(
-          n4, v.lo, v.hi, SwapPair{{v.sv[0], v.sv[1]}}, q, p, v.mi, v.pc, v.w, v.r, c, H->scratch.partials,
-          H->scratch.counter);
-      ck(cudaGetLastError(), "cg_update");
+      ck(launch_dependent(k_cg_update4, dim3(resident_grid(k_cg_update4, n4)), dim3(256), s, n4, v.lo, v.hi,
+                          SwapPair{{v.sv[0], v.sv[1]}}, q, p, v.mi, v.pc, v.w, v.r, c, H->scratch.partials,
+                          H->scratch.counter),
+         "cg_update");
     };
     if (!gstored(l) && hessvec32_dot_fused(H->geo[l], H->etile_part)) {
       // the direction update of the previous iteration (beta = 0 after a
@@ -810,14 +816,14 @@ struct Solver {
                         H->p_dev),
            "hessvec32");
       }
-      k_cg_dot4<<<resident_grid(k_cg_dot4, n4), 256, 0, s>>>(n4, p, q, c, H->scratch.partials,
-                                                              H->scratch.counter);
-      ck(cudaGetLastError(), "cg_dot");
+      ck(launch_dependent(k_cg_dot4, dim3(resident_grid(k_cg_dot4, n4)), dim3(256), s, n4, p, q, c,
+                          H->scratch.partials, H->scratch.counter),
+         "cg_dot");
       launches += 1 + (gstored(l) ? 1 : hessvec32_launches(H->geo[l], H->etile_part));
     }
     update();
-    k_cg_dir4<<<resident_grid(k_cg_dir4, n4), 256, 0, s>>>(n4, v.r, v.mi, v.pc, p, c);
-    ck(cudaGetLastError(), "cg_dir");
+    ck(launch_dependent(k_cg_dir4, dim3(resident_grid(k_cg_dir4, n4)), dim3(256), s, n4, v.r, v.mi, v.pc, p, c),
+       "cg_dir");
     return launches;
   }
 
@@ -1339,8 +1345,8 @@ struct Solver {
         // unmasked product is the masked one), an update reduction (its last
         // block tests the box, the forcing term and the budget and sets beta)
         // and the direction update.
-        k_ctrl_start<<<1, 1, 0, st>>>(c, rr2[0], rr2[1], tol, used, cg_max);
-        ck(cudaGetLastError(), "ctrl");
+        ck(launch_dependent(k_ctrl_start, dim3(1), dim3(1), st, c, rr2[0], rr2[1], tol, used, cg_max),
+           "ctrl");
         S.launches += 1;
         run_cg<V>(l, graph, cgv);
         read_ctrl();
@@ -1476,18 +1482,18 @@ struct Solver {
         ck(elem_hessvec32_pair(H->geo[l], H->mat[l], B.xlag32, SwapPair{{sv[1], sv[0]}},
                                SwapPair{{vec.t2, vec.Hs}}, &c->restarts, H->etile_part, H->p_dev, skip, st),
            "hessvec32");
-        k_cg_search4<<<resident_grid(k_cg_search4, n4), 256, 0, st>>>(
-            n4, lo, hi, sp, hp, vec.g, vec.mi, pc, vec.r, vec.p, P.cauchy_c, c, H->scratch.partials,
-            H->scratch.counter, skip);
-        ck(cudaGetLastError(), "cg_search");
+        ck(launch_dependent(k_cg_search4, dim3(resident_grid(k_cg_search4, n4)), dim3(256), st, n4, lo, hi,
+                            sp, hp, vec.g, vec.mi, pc, vec.r, vec.p, P.cauchy_c, c, H->scratch.partials,
+                            H->scratch.counter, skip),
+           "cg_search");
         S.launches += 3;
       };
-      k_cg_init4<<<resident_grid(k_cg_init4, n4), 256, 0, st>>>(n4, lo, hi, vec.s, vec.g, vec.Hs, vec.mi, pc,
-                                                               vec.r, vec.p, H->scratch.partials,
-                                                               H->scratch.counter, H->d_res);
-      ck(cudaGetLastError(), "cg_init");
-      k_ctrl_first<<<1, 1, 0, st>>>(c, H->d_res, m_s, cg_max, P.max_restarts);
-      ck(cudaGetLastError(), "ctrl");
+      ck(launch_dependent(k_cg_init4, dim3(resident_grid(k_cg_init4, n4)), dim3(256), st, n4, lo, hi, vec.s,
+                          vec.g, vec.Hs, vec.mi, pc, vec.r, vec.p, H->scratch.partials, H->scratch.counter,
+                          H->d_res),
+         "cg_init");
+      ck(launch_dependent(k_ctrl_first, dim3(1), dim3(1), st, c, H->d_res, m_s, cg_max, P.max_restarts),
+         "ctrl");
       S.launches += 2;
       for (;;) {
         for (int k = 0;; ++k) {
@@ -1557,20 +1563,19 @@ struct Solver {
     // product and test of the projected step t1
     auto search = [&](const int* skip) {
       hv<float>(l, t1, t2, skip, false);
-      k_cg_search4<<<resident_grid(k_cg_search4, n4), 256, 0, st>>>(
-          n4, lo, hi, SwapPair{{vec.s, vec.t1}}, SwapPair{{vec.Hs, vec.t2}}, g, mi, pc, r, p, P.cauchy_c, c, H->scratch.partials,
-          H->scratch.counter, skip);
-      ck(cudaGetLastError(), "cg_search");
+      ck(launch_dependent(k_cg_search4, dim3(resident_grid(k_cg_search4, n4)), dim3(256), st, n4, lo, hi,
+                          SwapPair{{vec.s, vec.t1}}, SwapPair{{vec.Hs, vec.t2}}, g, mi, pc, r, p,
+                          P.cauchy_c, c, H->scratch.partials, H->scratch.counter, skip),
+         "cg_search");
       S.launches += 1;
     };
     if (cg_max > 0) {
       cudaGraphExec_t graph = cg_graph<float>(l, cgv);
-      k_cg_init4<<<resident_grid(k_cg_init4, n4), 256, 0, st>>>(n4, lo, hi, s, g, Hs, mi, pc, r, p,
-                                                               H->scratch.partials, H->scratch.counter,
-                                                               H->d_res);
-      ck(cudaGetLastError(), "cg_init");
-      k_ctrl_first<<<1, 1, 0, st>>>(c, H->d_res, m_s, cg_max, P.max_restarts);
-      ck(cudaGetLastError(), "ctrl");
+      ck(launch_dependent(k_cg_init4, dim3(resident_grid(k_cg_init4, n4)), dim3(256), st, n4, lo, hi, s, g,
+                          Hs, mi, pc, r, p, H->scratch.partials, H->scratch.counter, H->d_res),
+         "cg_init");
+      ck(launch_dependent(k_ctrl_first, dim3(1), dim3(1), st, c, H->d_res, m_s, cg_max, P.max_restarts),
+         "ctrl");
       S.launches += 2;
       run_cg<float>(l, graph, cgv);
       int known = 0;  // accepted searches that s and t1 follow
