@@ -33,6 +33,7 @@
 #include "../../include/pf.h"
 #include "pf_element.cuh"
 #include "pf_internal.h"
+#include "pf_launch.cuh"
 #include "pf_stencil.cuh"
 
 namespace pf {
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(GalDims<D>::THREADS)
   using G = GalDims<D>;
   constexpr int NC = G::NC, F = G::F, EL = G::EL;
   extern __shared__ float cf_s[];  // [coefficient][point][element]
-  const long long e0 = blockIdx.x * (long long)EL;
+  const long long e0 = launch_wait_block() * (long long)EL;
   {
     // thread -> element and child, neighbouring threads along x
     const int cx = threadIdx.x & 1, el = (threadIdx.x >> 1) % EL, cyz = threadIdx.x / (2 * EL);
@@ -173,10 +174,11 @@ __device__ __forceinline__ void to_parent(int c, const float (&w)[3], float (&o)
 template <int D>
 __global__ void __launch_bounds__(128) k_gal_coarsen(Geom gc, Geom gf, const float* __restrict__ mf,
                                                      float* __restrict__ mc) {
+  const unsigned blk = launch_wait_block();
   using G = GalDims<D>;
   constexpr int NL = D == 3 ? 3 : 1;
   const long long total = gc.NE * G::NCF;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
+  for (long long t = blk * (long long)blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
     const int k = int(t / gc.NE);
     const long long e = t - k * gc.NE;
@@ -276,7 +278,7 @@ static cudaError_t launch_gal_fine(const Geom& gc, const Geom& gf, const Mat<flo
                                        int(G::smem));
   if (e != cudaSuccess) return e;
   const long long nb = (gc.NE + G::EL - 1) / G::EL;
-  k_gal_fine<D><<<unsigned(nb), G::THREADS, G::smem, st>>>(gc, gf, m, x, mom);
+  launch_dependent(k_gal_fine<D>, dim3(unsigned(nb)), dim3(G::THREADS), size_t(G::smem), st, gc, gf, m, x, mom);
   return cudaGetLastError();
 }
 
@@ -290,8 +292,8 @@ cudaError_t galerkin_coarsen(const Geom& gc, const Geom& gf, const float* mom_f,
                              cudaStream_t st) {
   const int ncf = gc.dim == 3 ? GalDims<3>::NCF : GalDims<2>::NCF;
   const int nb = blocks_for(gc.NE * ncf, 128, 32LL * 1216);
-  if (gc.dim == 3) k_gal_coarsen<3><<<nb, 128, 0, st>>>(gc, gf, mom_f, mom_c);
-  else k_gal_coarsen<2><<<nb, 128, 0, st>>>(gc, gf, mom_f, mom_c);
+  if (gc.dim == 3) launch_dependent(k_gal_coarsen<3>, dim3(nb), dim3(128), st, gc, gf, mom_f, mom_c);
+  else launch_dependent(k_gal_coarsen<2>, dim3(nb), dim3(128), st, gc, gf, mom_f, mom_c);
   return cudaGetLastError();
 }
 

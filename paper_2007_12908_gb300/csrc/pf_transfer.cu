@@ -26,6 +26,7 @@
 #include <cmath>
 
 #include "pf_internal.h"
+#include "pf_launch.cuh"
 
 namespace pf {
 
@@ -61,15 +62,14 @@ __device__ __forceinline__ double add_half(double a, double b) { return __fma_rn
 __device__ __forceinline__ float add_half(float a, float b) { return __fmaf_rn(0.5f, b, a); }
 
 // A thread's column, plane and range of coarse layers from the block's linear
-// index (a plain 1D grid: axes of up to 2^20 nodes exceed grid.y and .z).
+// index b (a plain 1D grid: axes of up to 2^20 nodes exceed grid.y and .z).
 // Columns off the x and y faces come first, in rows, then those on them.
 struct Column {
   int x, y, f, z0, z1;  // z1 exclusive
   bool live;
 };
 __device__ __forceinline__ Column my_column(const Geom& gc, unsigned blocks_xy, unsigned chunks,
-                                            int chunk) {
-  unsigned b = blockIdx.x;
+                                            int chunk, unsigned b) {
   Column c;
   long long t = (long long)(b % blocks_xy) * kThreads + threadIdx.x;
   b /= blocks_xy;
@@ -107,9 +107,10 @@ __device__ __forceinline__ Column my_column(const Geom& gc, unsigned blocks_xy, 
 template <class T>
 __global__ void __launch_bounds__(kThreads)
     k_prolong(Geom gc, Geom gf, unsigned blocks_xy, unsigned chunks, int chunk,
-              const T* __restrict__ in, T* __restrict__ out, const int* __restrict__ skip) {
+              const T* __restrict__ in, T* __restrict__ out, const int* skip) {
+  const unsigned blk = launch_wait_block();
   if (skip && *skip) return;
-  const Column c = my_column(gc, blocks_xy, chunks, chunk);
+  const Column c = my_column(gc, blocks_xy, chunks, chunk, blk);
   if (!c.live) return;
   const bool hx = c.x + 1 < gc.n[0], hy = c.y + 1 < gc.n[1];
   const long long cl = (long long)gc.n[0] * gc.n[1], fl = (long long)gf.n[0] * gf.n[1];
@@ -215,9 +216,10 @@ template <int D, class T>
 __global__ void __launch_bounds__(kThreads)
     k_restrict(Geom gc, Geom gf, unsigned blocks_xy, unsigned chunks, int chunk,
                const T* __restrict__ in, T* __restrict__ out, bool normalise,
-               const int* __restrict__ skip) {
+               const int* skip) {
+  const unsigned blk = launch_wait_block();
   if (skip && *skip) return;
-  const Column c = my_column(gc, blocks_xy, chunks, chunk);
+  const Column c = my_column(gc, blocks_xy, chunks, chunk, blk);
   if (!c.live) return;
   const auto g = gather_of<T, OpHalf<T>>(c, gf, in, OpHalf<T>());
   const long long cl = (long long)gc.n[0] * gc.n[1];
@@ -318,8 +320,9 @@ __global__ void __launch_bounds__(kThreads)
     k_bounds(Geom gc, Geom gf, unsigned blocks_xy, unsigned chunks, int chunk, int nf,
              const long long* __restrict__ lo_f, const long long* __restrict__ hi_f,
              long long* __restrict__ lo_c, long long* __restrict__ hi_c) {
+  const unsigned blk = launch_wait_block();
   // planes 0 .. nf-1: lo, nf .. 2 nf - 1: hi
-  Column c = my_column(gc, blocks_xy, chunks, chunk);
+  Column c = my_column(gc, blocks_xy, chunks, chunk, blk);
   if (!c.live) return;
   if (c.f < nf) {
     bound_column<D, OpKeyMax>(c, gc, gf, lo_f, lo_c);
@@ -361,7 +364,8 @@ cudaError_t prolong_t(const Geom& gc, const Geom& gf, int nf, const void* in, vo
   if (!s.ok) return cudaErrorInvalidConfiguration;
   const T* i = static_cast<const T*>(in);
   T* o = static_cast<T*>(out);
-  k_prolong<T><<<s.blocks, kThreads, 0, st>>>(gc, gf, s.blocks_xy, s.chunks, s.chunk, i, o, skip);
+  launch_dependent(k_prolong<T>, dim3(s.blocks), dim3(kThreads), st, gc, gf, s.blocks_xy, s.chunks, s.chunk,
+                   i, o, skip);
   return cudaGetLastError();
 }
 
@@ -373,9 +377,11 @@ cudaError_t restrict_t(const Geom& gc, const Geom& gf, int nf, const void* in, v
   const T* i = static_cast<const T*>(in);
   T* o = static_cast<T*>(out);
   if (gc.dim == 3)
-    k_restrict<3, T><<<s.blocks, kThreads, 0, st>>>(gc, gf, s.blocks_xy, s.chunks, s.chunk, i, o, normalise, skip);
+    launch_dependent(k_restrict<3, T>, dim3(s.blocks), dim3(kThreads), st, gc, gf, s.blocks_xy, s.chunks,
+                     s.chunk, i, o, normalise, skip);
   else
-    k_restrict<2, T><<<s.blocks, kThreads, 0, st>>>(gc, gf, s.blocks_xy, s.chunks, s.chunk, i, o, normalise, skip);
+    launch_dependent(k_restrict<2, T>, dim3(s.blocks), dim3(kThreads), st, gc, gf, s.blocks_xy, s.chunks,
+                     s.chunk, i, o, normalise, skip);
   return cudaGetLastError();
 }
 
@@ -402,9 +408,11 @@ cudaError_t xfer_bounds(const Geom& gc, const Geom& gf, int nf, const double* lo
   auto* lc = reinterpret_cast<long long*>(lo_c);
   auto* hc = reinterpret_cast<long long*>(hi_c);
   if (gc.dim == 3)
-    k_bounds<3><<<s.blocks, kThreads, 0, st>>>(gc, gf, s.blocks_xy, s.chunks, s.chunk, nf, lf, hf, lc, hc);
+    launch_dependent(k_bounds<3>, dim3(s.blocks), dim3(kThreads), st, gc, gf, s.blocks_xy, s.chunks,
+                     s.chunk, nf, lf, hf, lc, hc);
   else
-    k_bounds<2><<<s.blocks, kThreads, 0, st>>>(gc, gf, s.blocks_xy, s.chunks, s.chunk, nf, lf, hf, lc, hc);
+    launch_dependent(k_bounds<2>, dim3(s.blocks), dim3(kThreads), st, gc, gf, s.blocks_xy, s.chunks,
+                     s.chunk, nf, lf, hf, lc, hc);
   return cudaGetLastError();
 }
 
