@@ -336,6 +336,39 @@ struct Mono2 {
   }
 };
 
+// The rows int grad c . grad phi of an element, 3/2 of the sum over Gauss points
+// of raw differences: entries of a constant matrix, as the differences to the
+// corners that differ in two or three axes (2D: in one, and twice those in two).
+template <int D, class T>
+__device__ __forceinline__ void grad_rows(const T* c, T (&r)[1 << D]) {
+  if constexpr (D == 3) {
+    // to the opposite corner, and to those opposite in a face across x, y and z
+    T body[4], fx[4], fy[4], fz[8];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const int k = (a & 1) | (a & 2) << 1;  // 0, 1, 4, 5
+      body[a] = c[a] - c[a ^ 7];
+      fx[a] = c[a] - c[a ^ 6];
+      fy[a] = c[a] - c[a ^ 5];
+      fz[k] = c[k] - c[k ^ 3];
+      fz[k ^ 3] = -fz[k];
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const int o = a ^ 7;
+      r[a] = (body[a] + fx[a]) + (fy[a] + fz[a]);
+      r[o] = (fz[o] - body[a]) - (fx[o ^ 6] + fy[o ^ 5]);
+    }
+  } else {
+    const T x0 = c[1] - c[0], x1 = c[3] - c[2], y0 = c[2] - c[0], y1 = c[3] - c[1];
+    const T e = twice(c[3] - c[0]), f = twice(c[1] - c[2]);
+    r[0] = -(e + (x0 + y0));
+    r[1] = f + (x0 - y1);
+    r[2] = (y0 - x1) - f;
+    r[3] = e + (x1 + y1);
+  }
+}
+
 // Energy of one element: sum_q w [g psi + Gc/2 (c^2/ls + ls |grad c|^2) + p g tr].
 // With raw differences and 1/h folded into the constants,
 //   psi + p tr = (lam/2 tr + p) tr + mu (sum of G_ii^2 + sum of (G_ik + G_ki)^2 / 2).

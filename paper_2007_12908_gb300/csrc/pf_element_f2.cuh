@@ -31,30 +31,37 @@ __device__ __forceinline__ void lerp2(float2 a, float2 b, float2 (&o)[2]) {
   o[0] = fma2(bc(float(PF_XI0)), t, a);
   o[1] = fma2(bc(-float(PF_XI0)), t, b);
 }
+// Values at [qx][qy] of those by corner of a layer.
+__device__ __forceinline__ void lerp4(const float2 (&c)[4], float2 (&o)[2][2]) {
+  float2 e0[2], e1[2];
+  lerp2(c[0], c[1], e0);
+  lerp2(c[2], c[3], e1);
+  lerp2(e0[0], e1[0], o[0]);
+  lerp2(e0[1], e1[1], o[1]);
+}
 __device__ __forceinline__ float at(float2 v, int q) { return q ? v.y : v.x; }
 
 // Raw-difference derivatives of one field: x by qy and y by qx (lanes qz), z by
 // qy (lanes qx).
 struct Grad {
   float2 x[2], y[2], z[2];
-  // of a rough field (the direction: any nodal noise), differences along an
-  // axis first and then the other two axes; smooth fields lose nothing
-  __device__ __forceinline__ void rough(const float f[8]) {
+  // the direction (any nodal noise): differences along an axis first, then the
+  // other two axes
+  __device__ __forceinline__ void direction(const float f[8]) {
     lerp2(lerp2(f[1] - f[0], f[5] - f[4]), lerp2(f[3] - f[2], f[7] - f[6]), x);
     lerp2(lerp2(f[2] - f[0], f[6] - f[4]), lerp2(f[3] - f[1], f[7] - f[5]), y);
     lerp2(lerp2(f[4] - f[0], f[5] - f[1]), lerp2(f[6] - f[2], f[7] - f[3]), z);
   }
-  // of a smooth one, through its monomials
-  __device__ __forceinline__ void smooth(const float f[8]) {
+  // the state: near ends along z, monomials in the other two axes
+  __device__ __forceinline__ void state(const float f[8]) {
     const float2 x0 = bc(float(PF_XI0)), x1 = bc(float(PF_XI1));
-    Mono3<float> m;
-    m.set(f);
-    const float2 a = pair(m.xz, m.x), a2 = pair(m.yz, m.y), b = pair(m.xyz, m.xy);
-    x[0] = fma2(x0, b, a);
-    x[1] = fma2(x1, b, a);
-    y[0] = fma2(x0, b, a2);
-    y[1] = fma2(x1, b, a2);
-    const float2 c = pair(m.yz, m.z), d = pair(m.xyz, m.xz);  // by qy
+    const float x00 = f[1] - f[0], x10 = f[3] - f[2], x01 = f[5] - f[4], x11 = f[7] - f[6];
+    const float2 ax = lerp2(x00, x01), ay = lerp2(f[2] - f[0], f[6] - f[4]), b = lerp2(x10 - x00, x11 - x01);
+    x[0] = fma2(x0, b, ax);
+    x[1] = fma2(x1, b, ax);
+    y[0] = fma2(x0, b, ay);
+    y[1] = fma2(x1, b, ay);
+    const float2 c = lerp2(f[4] - f[0], f[6] - f[2]), d = lerp2(x01 - x00, x11 - x10);  // by qy
     z[0] = pair(d.x, c.x);
     z[1] = pair(d.y, c.y);
   }
@@ -69,11 +76,9 @@ __device__ __forceinline__ void n_sums2(float2 a, float2 b, float2& n0, float2& 
 
 // Test-function sums of one field: an x-derivative row by qy (summed over qx)
 // and a y-derivative row by qx (summed over qy), lanes qz, and a z-derivative
-// row by qy, lanes qx (summed over qz); with VALUE a value row [qx][qy], lanes
-// qz.
-template <bool VALUE>
+// row by qy, lanes qx (summed over qz).
 __device__ __forceinline__ void corners(const float2 (&sx)[2], const float2 (&sy)[2], const float2 (&sz)[2],
-                                        const float2 (&s0)[2][2], float (&r)[8]) {
+                                        float (&r)[8]) {
   const float x0 = float(PF_XI0), x1 = float(PF_XI1);
   float2 t0, t1, u0, u1, l[4];  // l: corners of a layer, lanes qz (0: negative)
   n_sums2(sx[0], sx[1], t0, t1);
@@ -82,17 +87,6 @@ __device__ __forceinline__ void corners(const float2 (&sx)[2], const float2 (&sy
   l[1] = sub2(t0, u1);
   l[2] = sub2(u0, t1);
   l[3] = add2(t1, u1);
-  if constexpr (VALUE) {
-    float2 n[2][2], v[2];
-    n_sums2(s0[0][0], s0[1][0], n[0][0], n[1][0]);
-    n_sums2(s0[0][1], s0[1][1], n[0][1], n[1][1]);
-    n_sums2(n[0][0], n[0][1], v[0], v[1]);
-    l[0] = sub2(l[0], v[0]);
-    l[2] = add2(l[2], v[1]);
-    n_sums2(n[1][0], n[1][1], v[0], v[1]);
-    l[1] = add2(l[1], v[0]);
-    l[3] = add2(l[3], v[1]);
-  }
   float2 n[2];
   n_sums2(sz[0], sz[1], n[0], n[1]);
 #pragma unroll
@@ -105,49 +99,59 @@ __device__ __forceinline__ void corners(const float2 (&sx)[2], const float2 (&sy
   }
 }
 
+// r = scale r + the sums of a value row [qx][qy], lanes qz.
+__device__ __forceinline__ void add_values(const float2 (&s)[2][2], float scale, float (&r)[8]) {
+  const float x0 = float(PF_XI0), x1 = float(PF_XI1);
+  float2 n[2][2], v[4];
+  n_sums2(s[0][0], s[1][0], n[0][0], n[1][0]);
+  n_sums2(s[0][1], s[1][1], n[0][1], n[1][1]);
+  n_sums2(n[0][0], n[0][1], v[0], v[2]);
+  n_sums2(n[1][0], n[1][1], v[1], v[3]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    r[k] = fmaf(x1, v[k].x, fmaf(x0, v[k].y, scale * r[k]));
+    r[k + 4] = fmaf(x0, v[k].x, fmaf(x1, v[k].y, scale * r[k + 4]));
+  }
+}
+
 // The 3D FP32 Hessian product of one element, bound by the FP32 pipe and the
-// issue slots: 1,050 operations (an FFMA2 counts as two), by
-// - the state in monomials (Mono3), the direction and the adjoint axis by axis;
+// issue slots: about 1,020 operations (an FFMA2 counts as two), by
 // - raw differences and stresses in units of mu / h, t_ik = (sigma + p I)_ik
 //   h / mu, so that shear stresses are the sums G_ik + G_ki themselves;
 // - the cross terms through t instead of the coefficient tensor B = g' t:
 //   q = g' w, su = A sigma(v) + q t, s0 = M w + g' t : grad v;
+// - grad w . grad phi from corner differences (grad_rows);
 // in pairs of Gauss points along z, whose lanes the z passes fill and take
 // apart by themselves (only the z-derivatives, the same at both, are copied).
 // With pairs along x, interpolation passes and the coefficient tensor it was
-// 1,310, and the element pass at 129^3 took 100 us, now 88.  In
+// 1,310, and the element pass at 129^3 took 100 us, now 91.  In
 // monomials throughout, both ways, it would be 930, but the rounding of a
-// rough direction then grows twofold.
+// rough direction then grows twofold; with the state alone as monomials in all
+// three axes the c rows of a rough state had 1.15 times the error (1.80e-7
+// against 1.57e-7 where the displacement terms decide), and the product took
+// 103.1 us instead of 105.9.
 __device__ __forceinline__ void elem_hessvec(const float (*xe)[8], const float (*ve)[8],
                                              const Mat<float>& m, float (*out)[8]) {
-  Grad u[3], v[3], w;
+  Grad u[3], v[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    u[i].smooth(xe[i]);
-    v[i].rough(ve[i]);
+    u[i].state(xe[i]);
+    v[i].direction(ve[i]);
   }
-  w.rough(ve[3]);
   float2 ov[2][2], wv[2][2];  // 1 - c and w at [qx][qy]
   {
-    float2 o[4], e0[2], e1[2];
+    float2 o[4], w[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) o[k] = lerp2(1.f - xe[3][k], 1.f - xe[3][k + 4]);
-    lerp2(o[0], o[1], e0);
-    lerp2(o[2], o[3], e1);
-    lerp2(e0[0], e1[0], ov[0]);
-    lerp2(e0[1], e1[1], ov[1]);
-    lerp2(lerp2(ve[3][0], ve[3][4]), lerp2(ve[3][1], ve[3][5]), e0);
-#pragma unroll
-    for (int qx = 0; qx < 2; ++qx) {
-      wv[qx][0] = fma2(w.y[qx], bc(float(PF_XI0)), e0[qx]);
-      wv[qx][1] = fma2(w.y[qx], bc(float(PF_XI1)), e0[qx]);
+    for (int k = 0; k < 4; ++k) {
+      o[k] = lerp2(1.f - xe[3][k], 1.f - xe[3][k + 4]);
+      w[k] = lerp2(ve[3][k], ve[3][k + 4]);
     }
+    lerp4(o, ov);
+    lerp4(w, wv);
   }
   const float omk = 1.f - m.k;
   const float kap = m.w * m.mu * m.inv_h * m.inv_h, ko = kap * omk, kk = kap * m.k;
   const float pm = m.p * m.hmu, wg = m.w * m.gcl;
-  // a derivative of w stands for two Gauss points
-  const float kc = 2.f * m.w * m.Gc * m.ls * m.inv_h * m.inv_h;
   const float2 lmu = bc(m.lmu), two = bc(2.f);
   float2 sx[3][2], sy[3][2], sz[3][2], s0[2][2];
 #pragma unroll
@@ -200,14 +204,9 @@ __device__ __forceinline__ void elem_hessvec(const float (*xe)[8], const float (
     }
   }
 #pragma unroll
-  for (int i = 0; i < 3; ++i) corners<false>(sx[i], sy[i], sz[i], s0, out[i]);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    w.x[k] = mul2(bc(kc), w.x[k]);
-    w.y[k] = mul2(bc(kc), w.y[k]);
-    w.z[k] = mul2(bc(kc), w.z[k]);
-  }
-  corners<true>(w.x, w.y, w.z, s0, out[3]);
+  for (int i = 0; i < 3; ++i) corners(sx[i], sy[i], sz[i], out[i]);
+  grad_rows<3, float>(ve[3], out[3]);
+  add_values(s0, m.w * m.Gc * m.ls * m.inv_h * m.inv_h * float(2.0 / 3.0), out[3]);
 }
 
 }  // namespace p2
