@@ -250,14 +250,19 @@ __device__ __forceinline__ constexpr int sym_index(int i, int k) {
 // Every op takes the element's nodal values xe[f][a] (f = field plane,
 // a = corner) and, for hessvec / energy_diff, a second vector ve[f][a].
 
-// ---------------------------------------------------------------- monomials
-// An element field as c + x X + y Y + ... in its reference coordinates: 12
-// (4 in 2D) differences, after which values and derivatives at the Gauss
-// points are nested FMAs that share their inner terms (at fixed z, the
-// x-derivative is a + y b and the y-derivative a2 + x b with the same b).
-// Energy, gradient and Hessian coefficients are written this way because
-// FP64 and double-float instructions are what bounds them (in 3D 2 lanes of
-// FP64 per SM and clock; some 13 instructions per double-float operation).
+// ---------------------------------------------------------------- Gauss values
+// Values and derivatives at the Gauss points from differences of corner values,
+// taken before anything is interpolated (a translation of the field does not
+// enter them), each point from its nearest corner: XI0 (0.21) is the weight of
+// every difference and of its rounding.  As monomials in coordinates from one
+// corner (weights up to XI1 = 0.79, errors of the far points in common) the
+// energy and the gradient of a rough element had 1.4 to 1.6 times this rounding,
+// for less arithmetic: FP64 operators on 65 x 49 x 57 3,214 us, now 3,245, double-float
+// energy and gradient of 97 x 105 x 89 nodes 557, now 596, the batched 2D case
+// 1,167, now 1,229.  A mixed difference serves both of its axes.
+// FP64 and double-float instructions are what bounds energy, gradient and
+// Hessian coefficients (in 3D 2 lanes of FP64 per SM and clock; some 13
+// instructions per double-float operation).
 
 // a b + c
 template <class T>
@@ -266,79 +271,132 @@ __device__ __forceinline__ T madd(T a, T b, T c) { return a * b + c; }
 template <class T>
 __device__ __forceinline__ T twice(T x) { return x + x; }
 
+// the two Gauss points between p and q
 template <class T>
-struct Mono3 {
-  T c, x, y, z, xy, xz, yz, xyz;
-  __device__ __forceinline__ void set(const T f[8]) {
-    c = f[0];
-    x = f[1] - f[0];
-    y = f[2] - f[0];
-    z = f[4] - f[0];
-    const T x10 = f[3] - f[2], x01 = f[5] - f[4], x11 = f[7] - f[6], y01 = f[6] - f[4];
-    xy = x10 - x;
-    xz = x01 - x;
-    yz = y01 - y;
-    xyz = (x11 - x01) - xy;
+__device__ __forceinline__ void lerp(T p, T q, T& o0, T& o1) {
+  const T d = q - p;
+  o0 = madd(T(PF_XI0), d, p);
+  o1 = madd(T(-PF_XI0), d, q);
+}
+
+// KEEP holds the differences along z, which are otherwise formed again in each
+// layer of Gauss points (8 values of a field in registers instead of 16).
+template <class T, bool KEEP>
+struct Corners3 {
+  T f[8], z[4], xz[2], yz[2];  // z by corner, mixed differences by ay and ax
+  __device__ __forceinline__ void set(const T g[8]) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) f[k] = g[k];
+    differences(f, f + 4, z, xz, yz);
   }
   // z-derivative at Gauss point (qx, qy), independent of z
   __device__ __forceinline__ void dz(T (&o)[2][2]) const {
+    const T t = T(PF_XI0);
+    lerp(madd(t, xz[0], z[0]), madd(t, xz[1], z[2]), o[0][0], o[0][1]);
+    lerp(madd(-t, xz[0], z[1]), madd(-t, xz[1], z[3]), o[1][0], o[1][1]);
+  }
+  // in Gauss layer qz: x-derivative by qy, y-derivative by qx
+  __device__ __forceinline__ void dxy(int qz, T (&gx)[2], T (&gy)[2]) const {
+    T n[4], d[4], dxz[2], dyz[2];
+    const T t = T(PF_XI0), tz = layer(qz, n, d, dxz, dyz);
+    // x-derivative by ay and y-derivative by ax at the layer's height
+    const T a0 = madd(tz, dxz[0], n[1] - n[0]), a1 = madd(tz, dxz[1], n[3] - n[2]);
+    const T b0 = madd(tz, dyz[0], n[2] - n[0]), b1 = madd(tz, dyz[1], n[3] - n[1]);
+    const T m = a1 - a0;
+    gx[0] = madd(t, m, a0);
+    gx[1] = madd(-t, m, a1);
+    gy[0] = madd(t, m, b0);
+    gy[1] = madd(-t, m, b1);
+  }
+  // the values v[qx][qy] of the layer
+  __device__ __forceinline__ void values(int qz, T (&v)[2][2]) const {
+    T n[4], d[4], dxz[2], dyz[2], e[2][2];  // e[qx][ay]
+    const T tz = layer(qz, n, d, dxz, dyz);
 #pragma unroll
-    for (int qy = 0; qy < 2; ++qy) {
-      const T t = qy ? T(PF_XI1) : T(PF_XI0), a = madd(t, yz, z), b = madd(t, xyz, xz);
-      o[0][qy] = madd(T(PF_XI0), b, a);
-      o[1][qy] = madd(T(PF_XI1), b, a);
+    for (int ay = 0; ay < 2; ++ay)
+      lerp(madd(tz, d[2 * ay], n[2 * ay]), madd(tz, d[2 * ay + 1], n[2 * ay + 1]), e[0][ay], e[1][ay]);
+#pragma unroll
+    for (int qx = 0; qx < 2; ++qx) lerp(e[qx][0], e[qx][1], v[qx][0], v[qx][1]);
+  }
+
+ private:
+  static __device__ __forceinline__ void differences(const T* n, const T* m, T (&d)[4], T (&dxz)[2], T (&dyz)[2]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) d[k] = m[k] - n[k];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      dxz[k] = d[2 * k + 1] - d[2 * k];
+      dyz[k] = d[k + 2] - d[k];
     }
   }
-  // at height zq: x-derivative by qy, y-derivative by qx
-  __device__ __forceinline__ void dxy(T zq, T (&gx)[2], T (&gy)[2]) const {
-    const T a = madd(zq, xz, x), a2 = madd(zq, yz, y), b = madd(zq, xyz, xy);
-    gx[0] = madd(T(PF_XI0), b, a);
-    gx[1] = madd(T(PF_XI1), b, a);
-    gy[0] = madd(T(PF_XI0), b, a2);
-    gy[1] = madd(T(PF_XI1), b, a2);
-  }
-  // the same and the values v[qx][qy]
-  __device__ __forceinline__ void all(T zq, T (&v)[2][2], T (&gx)[2], T (&gy)[2]) const {
-    const T v0 = madd(zq, z, c), a = madd(zq, xz, x);
-    dxy(zq, gx, gy);
+  // the layer's nearer corners n, the differences and their weight
+  __device__ __forceinline__ T layer(int qz, T (&n)[4], T (&d)[4], T (&dxz)[2], T (&dyz)[2]) const {
 #pragma unroll
-    for (int qx = 0; qx < 2; ++qx) {
-      const T s = madd(qx ? T(PF_XI1) : T(PF_XI0), a, v0);
-      v[qx][0] = madd(T(PF_XI0), gy[qx], s);
-      v[qx][1] = madd(T(PF_XI1), gy[qx], s);
+    for (int k = 0; k < 4; ++k) n[k] = qz ? f[k + 4] : f[k];
+    if constexpr (KEEP) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) d[k] = z[k];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        dxz[k] = xz[k];
+        dyz[k] = yz[k];
+      }
+      return qz ? T(-PF_XI0) : T(PF_XI0);
+    } else {
+      T m[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) m[k] = qz ? f[k] : f[k + 4];
+      differences(n, m, d, dxz, dyz);
+      return T(PF_XI0);
     }
   }
 };
 
 template <class T>
-struct Mono2 {
-  T c, x, y, xy;
-  __device__ __forceinline__ void set(const T f[4]) {
-    c = f[0];
-    x = f[1] - f[0];
-    y = f[2] - f[0];
-    xy = (f[3] - f[2]) - x;
+struct Corners2 {
+  T f[4], x[2], y[2], xy;
+  __device__ __forceinline__ void set(const T g[4]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f[k] = g[k];
+    x[0] = f[1] - f[0];
+    x[1] = f[3] - f[2];
+    y[0] = f[2] - f[0];
+    y[1] = f[3] - f[1];
+    xy = x[1] - x[0];
   }
   __device__ __forceinline__ void dxy(T (&gx)[2], T (&gy)[2]) const {
-    gx[0] = madd(T(PF_XI0), xy, x);
-    gx[1] = madd(T(PF_XI1), xy, x);
-    gy[0] = madd(T(PF_XI0), xy, y);
-    gy[1] = madd(T(PF_XI1), xy, y);
+    const T t = T(PF_XI0);
+    gx[0] = madd(t, xy, x[0]);
+    gx[1] = madd(-t, xy, x[1]);
+    gy[0] = madd(t, xy, y[0]);
+    gy[1] = madd(-t, xy, y[1]);
   }
-  __device__ __forceinline__ void all(T (&v)[2][2], T (&gx)[2], T (&gy)[2]) const {
-    dxy(gx, gy);
-#pragma unroll
-    for (int qx = 0; qx < 2; ++qx) {
-      const T s = madd(qx ? T(PF_XI1) : T(PF_XI0), x, c);
-      v[qx][0] = madd(T(PF_XI0), gy[qx], s);
-      v[qx][1] = madd(T(PF_XI1), gy[qx], s);
-    }
+  __device__ __forceinline__ void values(T (&v)[2][2]) const {
+    const T t = T(PF_XI0);
+    lerp(madd(t, x[0], f[0]), madd(t, x[1], f[2]), v[0][0], v[0][1]);
+    lerp(madd(-t, x[0], f[1]), madd(-t, x[1], f[3]), v[1][0], v[1][1]);
   }
 };
 
-// The rows int grad c . grad phi of an element, 3/2 of the sum over Gauss points
-// of raw differences: entries of a constant matrix, as the differences to the
+// Three times the sum over Gauss points of grad c . grad c (raw differences), a
+// quadratic form with constant entries: the squared differences of the pairs of
 // corners that differ in two or three axes (2D: in one, and twice those in two).
+template <int D, class T>
+__device__ __forceinline__ T grad_squares(const T* c) {
+  T s = T(0);
+#pragma unroll
+  for (int a = 0; a < (1 << D); ++a)
+#pragma unroll
+    for (int b = a + 1; b < (1 << D); ++b) {
+      const int n = ((a ^ b) & 1) + (((a ^ b) >> 1) & 1) + ((a ^ b) >> 2);
+      if (D == 3 && n == 1) continue;
+      const T d = c[b] - c[a];
+      s = D == 2 && n == 2 ? madd(twice(d), d, s) : madd(d, d, s);
+    }
+  return s;
+}
+// Half the derivative of grad_squares: for each corner the differences to its
+// partners (3/2 of the rows int grad c . grad phi in the same units).
 template <int D, class T>
 __device__ __forceinline__ void grad_rows(const T* c, T (&r)[1 << D]) {
   if constexpr (D == 3) {
@@ -375,45 +433,38 @@ __device__ __forceinline__ void grad_rows(const T* c, T (&r)[1 << D]) {
 // tr and the symmetric sums are formed before they are squared: a quadratic in
 // the single derivatives (lam/2 + mu) G_ii^2 + lam G_ii G_kk + ... cancels, its
 // error grown by lam / mu where tr is small against them (1e-12 at nu =
-// 0.499999) and by |rotation|^2 / |strain|^2.  The squares G_ii^2 depend on two
-// axes only and are shared by two Gauss points; it costs no more (double-float
-// energy and gradient of 97 x 105 x 89 nodes 567 -> 557 us).  ROLL keeps the two z layers of
-// Gauss points a loop (see the double-float kernels).
+// 0.499999) and by |rotation|^2 / |strain|^2.  A square G_ii^2 is shared by two
+// Gauss points.  ROLL keeps the two z layers of Gauss points a loop (see the
+// double-float kernels).
 template <int D, class T, bool ROLL = false>
 __device__ __forceinline__ T elem_energy(const T (*xe)[1 << D], const Mat<T>& m) {
-  const T x0 = T(PF_XI0), x1 = T(PF_XI1);
   const T omk = T(1) - m.k, ih2 = m.inv_h * m.inv_h;
   const T hl = T(0.5) * m.lam * ih2, cm = m.mu * ih2, hcm = T(0.5) * cm;
   const T cp = m.p * m.inv_h;
-  T acc = T(0), c2 = T(0), gr = T(0);
+  T acc = T(0), c2 = T(0);
+  auto weighted = [&](T W, T cq, T sum) {
+    const T o = T(1) - cq;
+    c2 = madd(cq, cq, c2);
+    return madd(madd(omk * o, o, m.k), W, sum);
+  };
   if constexpr (D == 3) {
-    Mono3<T> u[3], c;
+    Corners3<T, true> u[3], c;
 #pragma unroll
     for (int i = 0; i < 3; ++i) u[i].set(xe[i]);
     c.set(xe[3]);
     T uz[3][2][2], C[2][2];
 #pragma unroll
     for (int i = 0; i < 3; ++i) u[i].dz(uz[i]);
-    {
-      T cz[2][2];
-      c.dz(cz);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const T t = cz[k & 1][k >> 1], zz = uz[2][k & 1][k >> 1];
-        gr = madd(t, t, gr);
-        C[k & 1][k >> 1] = zz * zz;
-      }
-    }
+    for (int k = 0; k < 4; ++k) C[k & 1][k >> 1] = uz[2][k & 1][k >> 1] * uz[2][k & 1][k >> 1];
 #pragma unroll (ROLL ? 1 : 2)
     for (int qz = 0; qz < 2; ++qz) {
-      const T zq = qz ? x1 : x0;
-      T ux[3][2], uy[3][2], v[2][2], cx[2], cy[2], A[2], B[2];
+      T ux[3][2], uy[3][2], v[2][2], A[2], B[2], sum = T(0);
 #pragma unroll
-      for (int i = 0; i < 3; ++i) u[i].dxy(zq, ux[i], uy[i]);
-      c.all(zq, v, cx, cy);
+      for (int i = 0; i < 3; ++i) u[i].dxy(qz, ux[i], uy[i]);
+      c.values(qz, v);
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        gr = madd(cx[k], cx[k], madd(cy[k], cy[k], gr));
         A[k] = ux[0][k] * ux[0][k];
         B[k] = uy[1][k] * uy[1][k];
       }
@@ -425,23 +476,21 @@ __device__ __forceinline__ T elem_energy(const T (*xe)[1 << D], const Mat<T>& m)
           const T s01 = ux[1][qy] + uy[0][qx], s02 = ux[2][qy] + uz[0][qx][qy], s12 = uy[2][qx] + uz[1][qx][qy];
           const T off = madd(s01, s01, madd(s02, s02, s12 * s12));
           const T W = madd(madd(hl, tr, cp), tr, madd(hcm, off, cm * ((A[qy] + B[qx]) + C[qx][qy])));
-          const T cq = v[qx][qy], o = T(1) - cq;
-          acc = madd(madd(omk * o, o, m.k), W, acc);
-          c2 = madd(cq, cq, c2);
+          sum = weighted(W, v[qx][qy], sum);
         }
+      acc = acc + sum;
     }
   } else {
-    Mono2<T> u[2], c;
+    Corners2<T> u[2], c;
     u[0].set(xe[0]);
     u[1].set(xe[1]);
     c.set(xe[2]);
-    T ux[2][2], uy[2][2], v[2][2], cx[2], cy[2], A[2], B[2];
+    T ux[2][2], uy[2][2], v[2][2], A[2], B[2];
     u[0].dxy(ux[0], uy[0]);
     u[1].dxy(ux[1], uy[1]);
-    c.all(v, cx, cy);
+    c.values(v);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      gr = madd(cx[k], cx[k], madd(cy[k], cy[k], gr));
       A[k] = ux[0][k] * ux[0][k];
       B[k] = uy[1][k] * uy[1][k];
     }
@@ -450,14 +499,12 @@ __device__ __forceinline__ T elem_energy(const T (*xe)[1 << D], const Mat<T>& m)
 #pragma unroll
       for (int qy = 0; qy < 2; ++qy) {
         const T tr = ux[0][qy] + uy[1][qx], s01 = ux[1][qy] + uy[0][qx];
-        const T W = madd(madd(hl, tr, cp), tr, madd(hcm, s01 * s01, cm * (A[qy] + B[qx])));
-        const T cq = v[qx][qy], o = T(1) - cq;
-        acc = madd(madd(omk * o, o, m.k), W, acc);
-        c2 = madd(cq, cq, c2);
+        const T W = madd(madd(hl, tr, cp), tr, madd(hcm * s01, s01, cm * (A[qy] + B[qx])));
+        acc = weighted(W, v[qx][qy], acc);
       }
   }
-  // each derivative of c was squared once for its two Gauss points
-  return m.w * madd(T(0.5) * m.gcl, c2, madd(m.Gc * m.ls * ih2, gr, acc));
+  const T gr = (m.Gc * m.ls) * ih2 * T(1.0 / 3.0);
+  return m.w * madd(T(0.5) * m.gcl, c2, madd(gr, grad_squares<D, T>(xe[D]), acc));
 }
 
 // What the gradient and the Hessian coefficients share at one Gauss point,
@@ -635,34 +682,30 @@ __device__ __forceinline__ void elem_gradient(const T (*xe)[1 << D], const Mat<T
   const T x0 = T(PF_XI0), x1 = T(PF_XI1);
   const T wh = m.w * m.inv_h, wo = wh * (T(1) - m.k), wk = wh * m.k, wc = m.w * m.gcl;
   const T lh = m.lam * m.inv_h, mh = m.mu * m.inv_h, mh2 = twice(mh);
-  const T kc2 = twice(wh * m.Gc * m.ls * m.inv_h);  // a derivative of c stands for two Gauss points
+  const T kc = wh * m.Gc * m.ls * m.inv_h * T(2.0 / 3.0);  // of grad_rows
   if constexpr (D == 3) {
-    Mono3<T> u[3], c;
+    Corners3<T, !ROLL> u[3], c;
 #pragma unroll
     for (int i = 0; i < 3; ++i) u[i].set(xe[i]);
     c.set(xe[3]);
     T uz[3][2][2];
 #pragma unroll
     for (int i = 0; i < 3; ++i) u[i].dz(uz[i]);
-    Rows3<T> r[3], rc;
-    T s[2][2][2];  // value row of c: [ax][ay][az]
+    Rows3<T> r[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) r[i].zero();
-    rc.zero();
+    T s[8];  // row of c
+    grad_rows<3, T>(xe[3], s);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) s[i & 1][(i >> 1) & 1][i >> 2] = T(0);
+    for (int i = 0; i < 8; ++i) s[i] = kc * s[i];
 #pragma unroll (ROLL ? 1 : 2)
     for (int qz = 0; qz < 2; ++qz) {
-      const T zq = qz ? x1 : x0, w0 = qz ? x0 : x1, w1 = zq;
+      const T w0 = qz ? x0 : x1, w1 = qz ? x1 : x0;
       T ux[3][2], uy[3][2], v[2][2], s0[2][2];
       T sx[3][2], sy[3][2];  // by qy, by qx
 #pragma unroll
-      for (int i = 0; i < 3; ++i) u[i].dxy(zq, ux[i], uy[i]);
-      {
-        T cx[2], cy[2];
-        c.all(zq, v, cx, cy);
-        rc.add_xy(cx[0], cx[1], cy[0], cy[1], w0, w1);
-      }
+      for (int i = 0; i < 3; ++i) u[i].dxy(qz, ux[i], uy[i]);
+      c.values(qz, v);
 #pragma unroll
       for (int qx = 0; qx < 2; ++qx)
 #pragma unroll
@@ -696,26 +739,23 @@ __device__ __forceinline__ void elem_gradient(const T (*xe)[1 << D], const Mat<T
       n_sums(n[1][0], n[1][1], nn[1][0], nn[1][1]);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        s[i & 1][i >> 1][0] = madd(w0, nn[i & 1][i >> 1], s[i & 1][i >> 1][0]);
-        s[i & 1][i >> 1][1] = madd(w1, nn[i & 1][i >> 1], s[i & 1][i >> 1][1]);
+        s[i] = madd(w0, nn[i & 1][i >> 1], s[i]);
+        s[i + 4] = madd(w1, nn[i & 1][i >> 1], s[i + 4]);
       }
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) r[i].corners(out[i]);
-    c.dz(rc.zs);
-    T rr[8];
-    rc.corners(rr);
 #pragma unroll
-    for (int a = 0; a < 8; ++a) out[3][a] = madd(kc2, rr[a], s[a & 1][(a >> 1) & 1][a >> 2]);
+    for (int a = 0; a < 8; ++a) out[3][a] = s[a];
   } else {
-    Mono2<T> u[2], c;
+    Corners2<T> u[2], c;
     u[0].set(xe[0]);
     u[1].set(xe[1]);
     c.set(xe[2]);
-    T ux[2][2], uy[2][2], v[2][2], cx[2], cy[2], s0[2][2], sx[2][2], sy[2][2];
+    T ux[2][2], uy[2][2], v[2][2], s0[2][2], sx[2][2], sy[2][2];
     u[0].dxy(ux[0], uy[0]);
     u[1].dxy(ux[1], uy[1]);
-    c.all(v, cx, cy);
+    c.values(v);
 #pragma unroll
     for (int qx = 0; qx < 2; ++qx)
 #pragma unroll
@@ -734,24 +774,23 @@ __device__ __forceinline__ void elem_gradient(const T (*xe)[1 << D], const Mat<T
         }
       }
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < 2; ++i) {
       T a, b, e, f;
-      n_sums(i < 2 ? sx[i & 1][0] : cx[0], i < 2 ? sx[i & 1][1] : cx[1], a, b);  // by ay
-      n_sums(i < 2 ? sy[i & 1][0] : cy[0], i < 2 ? sy[i & 1][1] : cy[1], e, f);  // by ax
-      const T d[4] = {-a - e, a - f, e - b, b + f};
-      if (i < 2) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) out[i][k] = d[k];
-      } else {
-        T n[2][2], nn[2][2];
-        n_sums(s0[0][0], s0[1][0], n[0][0], n[1][0]);
-        n_sums(s0[0][1], s0[1][1], n[0][1], n[1][1]);
-        n_sums(n[0][0], n[0][1], nn[0][0], nn[0][1]);
-        n_sums(n[1][0], n[1][1], nn[1][0], nn[1][1]);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) out[2][k] = madd(kc2, d[k], nn[k & 1][k >> 1]);
-      }
+      n_sums(sx[i][0], sx[i][1], a, b);  // by ay
+      n_sums(sy[i][0], sy[i][1], e, f);  // by ax
+      out[i][0] = -a - e;
+      out[i][1] = a - f;
+      out[i][2] = e - b;
+      out[i][3] = b + f;
     }
+    T n[2][2], nn[2][2], d[4];
+    n_sums(s0[0][0], s0[1][0], n[0][0], n[1][0]);
+    n_sums(s0[0][1], s0[1][1], n[0][1], n[1][1]);
+    n_sums(n[0][0], n[0][1], nn[0][0], nn[0][1]);
+    n_sums(n[1][0], n[1][1], nn[1][0], nn[1][1]);
+    grad_rows<2, T>(xe[2], d);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) out[2][k] = madd(kc, d[k], nn[k & 1][k >> 1]);
   }
 }
 
@@ -864,7 +903,7 @@ __device__ __forceinline__ void hess_coef(const T (*xe)[1 << D], const Mat<T>& m
     }
   };
   if constexpr (D == 3) {
-    Mono3<T> u[3], c;
+    Corners3<T, true> u[3], c;
 #pragma unroll
     for (int i = 0; i < 3; ++i) u[i].set(xe[i]);
     c.set(xe[3]);
@@ -873,11 +912,10 @@ __device__ __forceinline__ void hess_coef(const T (*xe)[1 << D], const Mat<T>& m
     for (int i = 0; i < 3; ++i) u[i].dz(uz[i]);
 #pragma unroll
     for (int qz = 0; qz < 2; ++qz) {
-      const T zq = qz ? T(PF_XI1) : T(PF_XI0);
-      T ux[3][2], uy[3][2], v[2][2], cx[2], cy[2];
+      T ux[3][2], uy[3][2], v[2][2];
 #pragma unroll
-      for (int i = 0; i < 3; ++i) u[i].dxy(zq, ux[i], uy[i]);
-      c.all(zq, v, cx, cy);
+      for (int i = 0; i < 3; ++i) u[i].dxy(qz, ux[i], uy[i]);
+      c.values(qz, v);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int qx = q & 1, qy = q >> 1;
@@ -892,14 +930,14 @@ __device__ __forceinline__ void hess_coef(const T (*xe)[1 << D], const Mat<T>& m
       }
     }
   } else {
-    Mono2<T> u[2], c;
+    Corners2<T> u[2], c;
     u[0].set(xe[0]);
     u[1].set(xe[1]);
     c.set(xe[2]);
-    T ux[2][2], uy[2][2], v[2][2], cx[2], cy[2];
+    T ux[2][2], uy[2][2], v[2][2];
     u[0].dxy(ux[0], uy[0]);
     u[1].dxy(ux[1], uy[1]);
-    c.all(v, cx, cy);
+    c.values(v);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int qx = q & 1, qy = q >> 1;

@@ -14,7 +14,9 @@ from tests.gpu_common import require_cuda
 pytestmark = pytest.mark.gpu
 
 E, NU, GC, H1, N = 2.5, 0.25, 2.0**-40, 1.0 / 16.0, 2000
-LIMIT = {"product u": 1.06e-7, "product c": 1.57e-7}
+LIMIT = {"energy": 1.52e-16, "gradient u": 2.08e-16, "gradient c": 1.93e-16,
+         "energy df": 3.87e-15, "gradient df u": 5.45e-15, "gradient df c": 4.37e-15,
+         "product u": 1.06e-7, "product c": 1.57e-7}
 
 
 def _states(seed, n):
@@ -32,6 +34,25 @@ def _element(pf):
     H = pf.mesh_hierarchy_create(3, (2, 2, 2), 1, H1, E=E, nu=NU, Gc=GC)
     pf.pressure_set(H, 0.0)
     return H
+
+
+def test_energy_and_gradient():
+    torch = require_cuda()
+    import paper_2007_12908_gb300 as pf
+    H = _element(pf)
+    x = _states(51, N)
+    xd = torch.from_numpy(x.reshape(N, -1)).cuda()
+    energy, _ = X.energy_terms(3, x, NU, GC, H1, E=E)
+    grad = X.gradient(3, x, NU, GC, H1, E=E)
+    got = {}
+    for name, ef, gf in (("", pf.energy, pf.gradient), (" df", pf.energy_df, pf.gradient_df)):
+        e = np.array([ef(H, 0, v) for v in xd])
+        g = torch.stack([gf(H, 0, v) for v in xd]).cpu().numpy().reshape(x.shape)
+        got["energy" + name] = _rms(e[:, None], energy[:, None], slice(None))
+        got["gradient" + name + " u"] = _rms(g, grad, slice(0, 3))
+        got["gradient" + name + " c"] = _rms(g, grad, slice(3, 4))
+    H.close()
+    assert all(got[k] <= 1.07 * LIMIT[k] for k in got), got
 
 
 def test_fp32_product():
