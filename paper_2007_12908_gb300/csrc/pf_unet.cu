@@ -714,13 +714,26 @@ __global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __re
   }
 }
 
+// float(double(d) * inv) for inv = hi + lo + less than 2^-48 inv, in FP32: the
+// product's leading part q and the rest r with an error below 2^-46 |q|.  Where
+// that could change the rounding (one value in 2^20), and below 2^-100, where
+// the parts leave FP32's range, the product is taken in FP64, in a call: as a
+// selected value it would be computed for every d.
+__device__ __noinline__ float scale_fp64(float d, double inv) { return float(double(d) * inv); }
+__device__ __forceinline__ float scale_exact(float d, double inv, float hi, float lo) {
+  const float q = __fmul_rn(d, hi);  // not fused with the additions below
+  const float r = fmaf(d, lo, fmaf(d, hi, -q)), tol = fabsf(q) * 0x1p-45f;
+  const float a = q + (r - tol), b = q + (r + tol);
+  if ((fabsf(q) >= 0x1p-100f && a == b) || d == 0.f) return d == 0.f ? q : a;
+  return scale_fp64(d, inv);
+}
+
 // masked MSE: loss partials per block, dy = (y - t) mask / n.  One FP64
-// conversion and FMA per value: dy's quotient is formed in FP32 with 1/n as
-// inv + inv_lo and the product's rounding error (26 -> 7 us at 528 x 520;
-// with FP64 products and back-conversions that pipe was 81 % busy).
+// conversion and FMA per value (26 -> 12 us at 528 x 520, cold; with FP64 products and
+// back-conversions that pipe was 81 % busy).
 __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, const float* __restrict__ t,
                                              const float* __restrict__ mask, int C, long long HW,
-                                             float inv, float inv_lo, float* __restrict__ dy,
+                                             double inv, float inv_hi, float inv_lo, float* __restrict__ dy,
                                              double* __restrict__ part) {
   double acc = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HW;
@@ -729,8 +742,7 @@ __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, const 
     for (int c = 0; c < C; ++c) {
       const long long j = c * HW + i;
       const float d = (y[j] - t[j]) * mk;
-      const float q = d * inv, r = fmaf(d, inv_lo, fmaf(d, inv, -q));
-      dy[j] = isfinite(r) ? q + r : q;
+      dy[j] = scale_exact(d, inv, inv_hi, inv_lo);
       acc += double(d) * double(d);
     }
   }
@@ -1161,7 +1173,7 @@ pf_status pf_unet_mse(pf_unet* u, const float* y, const float* t, const float* m
   const double n = double(u->nout) * (mask ? n_valid : double(HW));
   const int nb = grid1(HW);
   const double inv = 1.0 / n;
-  k_mse<<<nb, 256, 0, u->st>>>(y, t, mask, u->nout, HW, float(inv), float(inv - double(float(inv))), dy,
+  k_mse<<<nb, 256, 0, u->st>>>(y, t, mask, u->nout, HW, inv, float(inv), float(inv - double(float(inv))), dy,
                                u->lpart);
   cudaError_t e = cudaMemcpyAsync(u->h_loss, u->lpart, sizeof(double) * nb, cudaMemcpyDeviceToHost, u->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(u->st);
