@@ -66,10 +66,19 @@ __device__ __forceinline__ float cg_direction(float mi, float r, float beta, flo
 // Inputs of the direction update fused into the FP32 CG product: the
 // product's operand becomes p = M^-1 r + beta p (beta from the control
 // block), formed where the operand is read and stored back by the gather
-// pass.  mi null: no preconditioner.
+// pass.  mi null: no preconditioner.  r null: no update; neither is there one
+// in a run's first iteration, whose p its start wrote.
 struct CgDirIn {
   const float* r;
   const float* mi;
+  const CgCtrl* c;
+  // beta, or 0 and r and mi null where there is no update (a beta of 0 does
+  // not say that: r.M^-1 r may become 0 in mid-run)
+  __device__ __forceinline__ float take_beta() {
+    if (r && c->used != c->start) return float(c->beta);
+    r = mi = nullptr;
+    return 0.f;
+  }
 };
 
 // The curvature step of a CG iteration from kappa = p.Hp: counts the
@@ -147,9 +156,9 @@ int hessvec32_launches(const Geom& g, const void* part);
 // cg_take_curvature on c.  Returns cudaErrorNotSupported, launching
 // nothing, where that path does not apply (the caller then takes p.q in a
 // pass of its own).  partials needs kMaxBlocks doubles.
-// With dir.r set and beta = c->beta not 0, p is first replaced by
-// M^-1 r + beta p, the direction update of the previous iteration; the product
-// and p.q use the new p.
+// With dir.r set, p is first replaced by M^-1 r + beta p, the direction update
+// of the previous iteration (but in a run's first); the product and p.q use the
+// new p.
 cudaError_t elem_hessvec32_dot(const Geom& g, const Mat<double>& m, const float* x, float* p,
                                float* q, CgCtrl* c, double* partials, unsigned* counter,
                                void* part, const float* p_dev, CgDirIn dir, cudaStream_t st);

@@ -527,21 +527,18 @@ cudaError_t elem_gradient(const Geom& g, const Mat<double>& m, const void* x, vo
 // the instruction cache (98 us).  A persistent CTA that stages its next tile
 // beside the last elements of this one was slower (106 us).
 // With dir.r set (FP32 CG), v is the previous direction and the staged
-// operand is M^-1 r + beta v, beta = *beta; a run's first iteration (beta = 0)
-// takes v, which its start wrote: staging r and M^-1 instead costs 25 us more
-// than the 5 us of that write.
+// operand is M^-1 r + beta v; a run's first iteration takes v, which its start
+// wrote: staging r and M^-1 instead costs 25 us more than the 5 us of that write.
 constexpr int kEtileThreads = 128;  // 4 CTAs per SM at 128 registers
 template <class TV>
 __global__ void __launch_bounds__(kEtileThreads, 512 / kEtileThreads)
     k_hess_etile3(Geom g, Mat<float> m, const float* x, const TV* v, float4* part, const int* skip,
-                  const float* p_dev, CgDirIn dir, const double* beta, const TV* v_odd = nullptr,
-                  const int* odd = nullptr) {
+                  const float* p_dev, CgDirIn dir, const TV* v_odd = nullptr, const int* odd = nullptr) {
   launch_wait();
   if (skip && *skip) return;
   if (p_dev) m.p = *p_dev;
   if (odd && (*odd & 1)) v = v_odd;
-  const float be = dir.r ? float(*beta) : 0.f;
-  if (be == 0.f) dir.r = dir.mi = nullptr;
+  const float be = dir.take_beta();
   constexpr int T = 8, NN = T + 1, NP = NN * NN, NH = NP * NN, NT = kEtileThreads;
   constexpr int NW = NT / 32, LZ = T / NW;        // warps, element layers of each
   constexpr int NA = NW * (LZ + 1) * NP;          // node planes of all warps
@@ -740,8 +737,7 @@ __global__ void __launch_bounds__(256, 4) k_etile_gather3_dot(Geom g,
   constexpr int T = 8;
   const int tx = (g.ne[0] + T - 1) / T, ty = (g.ne[1] + T - 1) / T, tz = (g.ne[2] + T - 1) / T;
   const long long N = g.N;
-  const float be = dir.r ? float(c->beta) : 0.f;
-  if (be == 0.f) dir.r = nullptr;
+  const float be = dir.take_beta();
   float pq = 0.f;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -806,8 +802,7 @@ cudaError_t elem_hessvec32_dot(const Geom& g, const Mat<double>& m, const float*
   if (!hessvec32_dot_fused(g, part)) return cudaErrorNotSupported;
   float4* pp = static_cast<float4*>(part);
   const cudaError_t e = launch_dependent(k_hess_etile3<float>, etile_grid(g), dim3(kEtileThreads), st, g,
-                                         cast_mat<float>(m), x, p, pp, &c->done, p_dev, dir, &c->beta,
-                                         nullptr, nullptr);
+                                         cast_mat<float>(m), x, p, pp, &c->done, p_dev, dir, nullptr, nullptr);
   if (e != cudaSuccess) return e;
   // kMaxBlocks = two waves of 4 blocks per SM
   const int nb = int(std::min<long long>((g.N + 255) / 256, kMaxBlocks));
@@ -821,7 +816,7 @@ cudaError_t elem_hessvec32_pair(const Geom& g, const Mat<double>& m, const float
   float4* pp = static_cast<float4*>(part);
   const cudaError_t e = launch_dependent(k_hess_etile3<float>, etile_grid(g), dim3(kEtileThreads), st, g,
                                          cast_mat<float>(m), x, v.v[0], pp, skip, p_dev,
-                                         CgDirIn{nullptr, nullptr}, nullptr, v.v[1], odd);
+                                         CgDirIn{}, v.v[1], odd);
   if (e != cudaSuccess) return e;
   const int nb = int(std::min<long long>((g.N + 255) / 256, 8LL * 1216));
   return launch_dependent(k_etile_gather3<float>, dim3(nb), dim3(256), st, g, pp, y.v[0], skip, y.v[1], odd);
@@ -838,7 +833,7 @@ static cudaError_t launch_hess_tile3(const Geom& g, const Mat<double>& m, const 
     float4* pp = static_cast<float4*>(part);
     const cudaError_t e = launch_dependent(k_hess_etile3<TV>, etile_grid(g), dim3(kEtileThreads), st, g,
                                            cast_mat<float>(m), x, v, pp, skip, p_dev,
-                                           CgDirIn{nullptr, nullptr}, nullptr, nullptr, nullptr);
+                                           CgDirIn{}, nullptr, nullptr);
     if (e != cudaSuccess) return e;
     const int nb = int(std::min<long long>((g.N + 255) / 256, 8LL * 1216));
     return launch_dependent(k_etile_gather3<TV>, dim3(nb), dim3(256), st, g, pp, y, skip, nullptr, nullptr);

@@ -798,11 +798,11 @@ struct Solver {
          "cg_update");
     };
     if (!gstored(l) && hessvec32_dot_fused(H->geo[l], H->etile_part)) {
-      // the direction update of the previous iteration (beta = 0 after a
-      // restart) is formed inside the product
+      // the direction update of the previous iteration is formed inside the
+      // product
       ck(elem_hessvec32_dot(H->geo[l], H->mat[l], B.xlag32, p, q, c, H->scratch.partials,
                             H->scratch.counter, H->etile_part, H->p_dev,
-                            CgDirIn{v.r, v.pc ? v.mi : nullptr}, s),
+                            CgDirIn{v.r, v.pc ? v.mi : nullptr, c}, s),
          "hessvec32_dot");
       update();
       return 3;

@@ -1,0 +1,27 @@
+// C entries to internal pieces of libpf.so for tests: kernels whose special
+// cases no load step can be made to reach.
+#include "pf_hier.h"
+
+using namespace pf;
+
+extern "C" {
+
+// The fused FP32 CG product at the given point of a run (started at `start`
+// products, `used` by now): p and q as it leaves them.
+int probe_cg_product(pf_hierarchy* h, int level, const float* x, float* p, float* q, const float* r, const float* mi,
+                     double beta, int start, int used) {
+  CgCtrl c{};
+  c.rz = 1.0;
+  c.beta = beta;
+  c.start = start;
+  c.used = used;
+  c.cg_max = 1000;
+  if (cudaMemcpyAsync(h->ctrl, &c, sizeof c, cudaMemcpyHostToDevice, h->st) != cudaSuccess) return 1;
+  const CgDirIn dir{r, mi, h->ctrl};
+  if (elem_hessvec32_dot(h->geo[level], h->mat[level], x, p, q, h->ctrl, h->scratch.partials, h->scratch.counter,
+                         h->etile_part, h->p_dev, dir, h->st) != cudaSuccess)
+    return 2;
+  return cudaStreamSynchronize(h->st) != cudaSuccess ? 3 : 0;
+}
+
+}  // extern "C"
