@@ -57,6 +57,7 @@ struct pf_hierarchy {
   pf::SubCtrl* sub_ctl = nullptr;
   pf::SubCtrl* h_sub_ctl = nullptr;  // pinned host mirror
   bool sub_ok = true;                // false once a wait ran out or the launch was refused
+  long long sub_spin_limit = pf::kSubSpinLimit;
   void* etile_part = nullptr;  // node sums of the element-owned FP32 Hessian tiles (3D)
   float* p_dev = nullptr;      // the pressure in FP32 on the device (kept by pf_pressure_set)
   // executable graphs of the FP32 CG loop per level (built by the solver)

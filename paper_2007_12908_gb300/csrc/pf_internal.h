@@ -235,7 +235,7 @@ cudaError_t hess2_march(const Geom& g, const Mat<double>& m, const float* x, con
 // The trust-region subproblem of a small level in one cooperative launch
 // (pf_subproblem.cu): min gr.s + s.H s / 2 over lo <= s <= hi with H a stencil
 // (FP64, or FP32 with FP32 arithmetic), the step to s.  Fields of SubCtrl are
-// written when it is done; failed: a wait ran out and s is not written.
+// written when it is done; failed: a wait ran out and s is undefined.
 struct SubCtrl {
   int failed;     // cleared by the caller
   unsigned base;  // arrivals at the barrier when the last launch had ended
@@ -252,8 +252,10 @@ struct SubIn {
   unsigned* bar;      // zero, as ctl, before the first launch
   SubCtrl* ctl;
   double delta, cauchy_c;
+  long long spin_limit;  // polls of a barrier after which the wait has run out
   int backtracks, cg_max, max_restarts;
 };
+constexpr long long kSubSpinLimit = 2000000;  // about a second
 constexpr int kSubPartials = 2 * 4 * 1216;
 // Whether the level is small enough; cudaErrorNotSupported from the launch
 // where it is not, or where the device cannot hold the CTAs at once.

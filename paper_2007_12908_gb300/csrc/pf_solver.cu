@@ -408,8 +408,9 @@ struct Solver {
   // (grad h at B.x - B.s: an accepted step not yet applied to the gradient)
   enum { G_NONE = 0, G_AT_X = 1, G_STEP = 2 };
   std::vector<int> gstate;
-  // 2D levels of the mixed mode whose Hessian and subproblem are FP64: those the
-  // one-launch subproblem takes.  Its CG iteration costs 11 us there in FP64, where
+  // 2D levels of the mixed mode whose Hessian and subproblem are FP64: those of
+  // the one-launch subproblem's size, also where this hierarchy's subproblems
+  // have gone to separate launches (the same arithmetic, more slowly).  Its CG iteration costs 11 us there in FP64, where
   // an FP32 iteration of separate launches takes 25 to 30 us; so the levels'
   // products, gradients and energies are as in the FP64 mode (load steps of three
   // levels: 129^2 92 and 101 -> 59 and 54 ms, 225 x 193 206 and 182 -> 113 and
@@ -421,7 +422,7 @@ struct Solver {
   Solver(pf_hierarchy* h, const pf_rmtr_params& p, pf_rmtr_stats& s)
       : H(h), P(p), S(s), st(h->st), L(h->L), F(h->dim + 1), mixed(p.precision == PF_FP32),
         gstate(h->L, G_NONE), small64(h->L, 0) {
-    for (int l = 0; l < L; ++l) small64[l] = mixed && H->sub_ok && !galerkin(l) && H->lv[l].small;
+    for (int l = 0; l < L; ++l) small64[l] = mixed && !galerkin(l) && H->lv[l].small;
   }
 
   // The FP64 stencil of a level with an FP64 Hessian.
@@ -1203,6 +1204,7 @@ struct Solver {
     in.ctl = H->sub_ctl;
     in.delta = delta;
     in.cauchy_c = P.cauchy_c;
+    in.spin_limit = H->sub_spin_limit;
     in.backtracks = P.cauchy_backtracks;
     in.cg_max = cg_max;
     in.max_restarts = P.max_restarts;

@@ -38,7 +38,6 @@ namespace {
 
 constexpr int kLanes = 128, kLines = 3, kThreads = kLanes * kLines;
 constexpr int kMaxCoopBlocks = 1216;       // partials hold this many
-constexpr long long kSpinLimit = 2000000;  // about a second of polling
 
 template <int D, class TS, class V>
 struct SubArgs {
@@ -53,6 +52,7 @@ struct SubArgs {
   unsigned* bar;               // arrivals so far
   SubCtrl* ctl;
   double delta, cauchy_c;
+  long long spin_limit;
   int backtracks, cg_max, max_restarts;
 };
 
@@ -169,7 +169,7 @@ struct Sub {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(A.bar) : "memory");
         if (int(c - target) >= 0) break;
         ++spin;
-        if ((spin & 255) == 0 && (spin > kSpinLimit || *(volatile int*)&A.ctl->failed)) {
+        if ((spin & 255) == 0 && (spin > A.spin_limit || *(volatile int*)&A.ctl->failed)) {
           atomicExch(&A.ctl->failed, 1);
           sh.go = 0;
           break;
@@ -455,6 +455,7 @@ SubArgs<D, TS, V> make_args(const Geom& g, const SubIn& in) {
   a.ctl = in.ctl;
   a.delta = in.delta;
   a.cauchy_c = in.cauchy_c;
+  a.spin_limit = in.spin_limit;
   a.backtracks = in.backtracks;
   a.cg_max = in.cg_max;
   a.max_restarts = in.max_restarts;

@@ -24,4 +24,20 @@ int probe_cg_product(pf_hierarchy* h, int level, const float* x, float* p, float
   return cudaStreamSynchronize(h->st) != cudaSuccess ? 3 : 0;
 }
 
+// Sends the hierarchy's subproblems of small levels to separate launches.
+void probe_separate_launches(pf_hierarchy* h) { h->sub_ok = false; }
+int probe_one_launch(pf_hierarchy* h) { return h->sub_ok ? 1 : 0; }
+
+// Lets the grid barrier of the next one-launch subproblem wait for an arrival
+// that no CTA makes, for at most `polls` polls.
+int probe_stuck_barrier(pf_hierarchy* h, long long polls) {
+  h->sub_spin_limit = polls;
+  SubCtrl c{};
+  if (cudaMemcpyAsync(&c, h->sub_ctl, sizeof c, cudaMemcpyDeviceToHost, h->st) != cudaSuccess) return 1;
+  if (cudaStreamSynchronize(h->st) != cudaSuccess) return 2;
+  c.base += 1;
+  if (cudaMemcpyAsync(h->sub_ctl, &c, sizeof c, cudaMemcpyHostToDevice, h->st) != cudaSuccess) return 3;
+  return cudaStreamSynchronize(h->st) != cudaSuccess ? 4 : 0;
+}
+
 }  // extern "C"
