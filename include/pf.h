@@ -93,7 +93,10 @@ typedef struct {
                             terms of rho's energy difference; double-float
                             (pf_gradient_df) stopping-test gradients and
                             energy; FP64 first-order term of rho, radius and
-                            norms                                            */
+                            norms.  2D levels of up to 38,912 values (12,970
+                            nodes) that are not GALERKIN coarse levels are
+                            as in PF_FP64 (Hessian, subproblem, gradient,
+                            energy difference): faster there, in one launch  */
   int precondition;      /* 1: Jacobi (Hessian-diagonal) preconditioned CG (1) */
   double level_rtol;     /* a non-finest level stops its TR steps once its
                             projected gradient fell by this factor (1e-3;
@@ -173,8 +176,9 @@ const char* pf_last_error(void);
  * Not counted there: a level's assembled FP64 Hessian stencil (27 x 16
  * doubles per node in 3D), allocated on the level's first FP64 lag (an
  * FP64-precision load step, a GALERKIN coarse level, or
- * pf_hessvec_lag_set with PF_FP64); if it does not fit, that call returns
- * PF_ENOMEM.
+ * pf_hessvec_lag_set with PF_FP64), and in 2D another one (8.4 MB at most) of
+ * each level that the mixed mode takes in FP64, allocated by the first mixed
+ * load step; if it does not fit, that call returns PF_ENOMEM.
  * Errors: PF_EINVAL for a bad descriptor, PF_ENOMEM, PF_ECUDA. */
 pf_status pf_mesh_hierarchy_create(const pf_mesh_desc* desc, pf_hierarchy** out);
 pf_status pf_mesh_hierarchy_destroy(pf_hierarchy* h);

@@ -37,16 +37,20 @@ static pf_status bad(const char* msg) {
 }
 
 namespace pf {
-cudaError_t ensure_stencil(pf_hierarchy* h, int l) {
-  LevelBuf& B = h->lv[l];
-  if (B.stencil) return cudaSuccess;
+static cudaError_t alloc_stencil(pf_hierarchy* h, int l, double*& S) {
+  if (S) return cudaSuccess;
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, sizeof(double) * stencil_count(h->geo[l]));
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return e;
+  }
   h->allocations.push_back(p);
-  B.stencil = static_cast<double*>(p);
+  S = static_cast<double*>(p);
   return cudaSuccess;
 }
+cudaError_t ensure_stencil(pf_hierarchy* h, int l) { return alloc_stencil(h, l, h->lv[l].stencil); }
+cudaError_t ensure_small(pf_hierarchy* h, int l) { return alloc_stencil(h, l, h->lv[l].small); }
 cudaError_t ensure_galerkin(pf_hierarchy* h, int l) {
   LevelBuf& B = h->lv[l];
   if (B.gs) return cudaSuccess;
@@ -301,22 +305,11 @@ pf_status pf_mesh_hierarchy_create(const pf_mesh_desc* d, pf_hierarchy** out) {
         return rc;
       }
     // the FP64 stencil (27 x 16 doubles per node in 3D) is allocated on a
-    // level's first FP64 lag (ensure_stencil): mixed-precision runs do not
-    // hold it
+    // level's first FP64 lag (ensure_stencil), a small 2D level's own of the
+    // mixed mode on the first mixed load step (ensure_small)
     if ((rc = alloc(h, (void**)&B.coef, sizeof(double) * coef_count(h->geo[l])))) {
       pf_mesh_hierarchy_destroy(h);
       return rc;
-    }
-    // the FP64 stencil of the mixed mode's small 2D levels (8.4 MB at most);
-    // where there is no room for it they stay FP32
-    if (d->dim == 2 && subproblem_small(h->geo[l])) {
-      void* p = nullptr;
-      if (cudaMalloc(&p, sizeof(double) * stencil_count(h->geo[l])) == cudaSuccess) {
-        h->allocations.push_back(p);
-        B.small = static_cast<double*>(p);
-      } else {
-        cudaGetLastError();
-      }
     }
   }
   if (cudaStreamSynchronize(h->st) != cudaSuccess) {

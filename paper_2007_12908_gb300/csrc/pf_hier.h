@@ -89,8 +89,10 @@ pf_status projected_gradient_impl(pf_hierarchy* H, const double* x_dev, double* 
 pf_status qp_impl(pf_hierarchy* H, int level, const double* g, const double* lo, const double* hi,
                   double* s, int sweeps, double tol, int maxit, int* products);
 void refresh_pressure(pf_hierarchy* H);
-// Allocates level l's FP64 stencil on first use (held until destroy).
+// Allocates level l's FP64 stencil on first use (held until destroy), and that
+// of a small level in the mixed mode.
 cudaError_t ensure_stencil(pf_hierarchy* H, int l);
+cudaError_t ensure_small(pf_hierarchy* H, int l);
 // Allocates level l's Galerkin element matrices and FP32 stencil on first
 // use, and builds the FP32 Galerkin operators of every coarse level from
 // the finest level's FP32 lag x (R G I chain, see pf_galerkin.cu).

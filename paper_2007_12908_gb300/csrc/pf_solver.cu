@@ -422,7 +422,7 @@ struct Solver {
   Solver(pf_hierarchy* h, const pf_rmtr_params& p, pf_rmtr_stats& s)
       : H(h), P(p), S(s), st(h->st), L(h->L), F(h->dim + 1), mixed(p.precision == PF_FP32),
         gstate(h->L, G_NONE), small64(h->L, 0) {
-    for (int l = 0; l < L; ++l) small64[l] = mixed && !galerkin(l) && H->lv[l].small;
+    for (int l = 0; l < L; ++l) small64[l] = mixed && !galerkin(l) && H->dim == 2 && subproblem_small(H->geo[l]);
   }
 
   // The FP64 stencil of a level with an FP64 Hessian.
@@ -1851,6 +1851,8 @@ struct Solver {
       }, &bad_count);
       if (bad_count != 0.0) return PF_ENONFINITE;
     }
+    for (int l = 0; l < L; ++l)
+      if (small64[l]) ck(ensure_small(H, l), "FP64 stencil allocation");
     // c_prev of the caller's last step, restored if this step fails
     copy(H->c_prev_save, H->c_prev, N);
     bool g_at_t3 = false;  // B.g holds the FP64 gradient at B.t3 = the plain start

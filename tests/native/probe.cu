@@ -40,4 +40,7 @@ int probe_stuck_barrier(pf_hierarchy* h, long long polls) {
   return cudaStreamSynchronize(h->st) != cudaSuccess ? 4 : 0;
 }
 
+// Whether the level holds the FP64 stencil of the mixed mode's small levels.
+int probe_small_stencil(pf_hierarchy* h, int level) { return h->lv[level].small ? 1 : 0; }
+
 }  // extern "C"
