@@ -732,14 +732,14 @@ __global__ void __launch_bounds__(256, 4) k_etile_gather3_dot(Geom g,
                                                               float* __restrict__ y, CgCtrl* c,
                                                               double* partials,
                                                               unsigned* counter, CgDirIn dir) {
-  launch_wait();
+  const unsigned blk = launch_wait_block();
   if (c->done) return;
   constexpr int T = 8;
   const int tx = (g.ne[0] + T - 1) / T, ty = (g.ne[1] + T - 1) / T, tz = (g.ne[2] + T - 1) / T;
   const long long N = g.N;
   const float be = dir.take_beta();
   float pq = 0.f;
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
+  for (long long n = blk * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
     float p0 = p[n], p1 = p[N + n], p2 = p[2 * N + n], p3 = p[3 * N + n];
     if (dir.r) {

@@ -19,9 +19,9 @@
 namespace pf {
 
 // Every earlier launch of the stream has ended and its writes are visible
-// after this; the launch after this one may then start.  Pointers whose first
-// read follows it are not __restrict__ (a load known to be invariant could be
-// moved before it), except where that read depends on a value loaded after it.
+// after this; the launch after this one may then start.  A kernel that calls it
+// has no __restrict__ pointers: a load through one could be moved before it,
+// also past a branch on a value loaded after it.
 __device__ __forceinline__ void launch_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(256) k_cg_search4(
     const float* __restrict__ g, const float* __restrict__ mi, bool pc, float* __restrict__ r,
     float* __restrict__ p, double cauchy_c, CgCtrl* c, double* partials, unsigned* counter,
     const int* skip) {
-  launch_wait();
+  const unsigned blk = launch_wait_block();
   if (skip && *skip) return;
   const bool odd = c->restarts & 1;
   const float* __restrict__ s = odd ? sv.v[1] : sv.v[0];
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(256) k_cg_search4(
   const float* __restrict__ Hs = odd ? hv.v[1] : hv.v[0];
   const float* __restrict__ Ht = odd ? hv.v[0] : hv.v[1];
   float o[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n4;
+  for (long long j = blk * (long long)blockDim.x + threadIdx.x; j < n4;
        j += (long long)gridDim.x * blockDim.x) {
     const float4 l4 = ld4(lo, j), h4 = ld4(hi, j), s4 = ld4(s, j), hs4 = ld4(Hs, j), t4 = ld4(t, j),
                  ht4 = ld4(Ht, j), g4 = ld4(g, j);
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* _
                                                     float* __restrict__ w, float* __restrict__ r,
                                                     CgCtrl* c, double* partials,
                                                     unsigned* counter) {
-  launch_wait();
+  const unsigned blk = launch_wait_block();
   if (c->done) return;
   const float al = float(c->alpha);
   const bool fresh = c->used == c->start + 1;
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* _
   float* __restrict__ t = odd ? sv.v[0] : sv.v[1];
   float rr = 0.f, lv = 0.f, rz = 0.f;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n4; j += stride) {
+  for (long long j = blk * (long long)blockDim.x + threadIdx.x; j < n4; j += stride) {
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
     const float4 l4 = ld4(lo, j), h4 = ld4(hi, j), s4 = ld4(s, j);
     float4 q4 = z4, p4 = z4, w4 = z4, r4 = z4, m4 = make_float4(1.f, 1.f, 1.f, 1.f), t4;
@@ -289,11 +289,11 @@ __global__ void __launch_bounds__(256) k_cg_update4(long long n4, const float* _
 __global__ void __launch_bounds__(256) k_cg_dot4(long long n4, const float* __restrict__ p,
                                                  const float* __restrict__ q, CgCtrl* c,
                                                  double* partials, unsigned* counter) {
-  launch_wait();
+  const unsigned blk = launch_wait_block();
   if (c->done) return;
   float pq = 0.f;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long j0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; j0 < n4; j0 += 2 * stride) {
+  for (long long j0 = blk * (long long)blockDim.x + threadIdx.x; j0 < n4; j0 += 2 * stride) {
     const long long j1 = j0 + stride;
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
     const float4 p0 = ld4(p, j0), p1 = j1 < n4 ? ld4(p, j1) : z4;
@@ -312,11 +312,11 @@ __global__ void __launch_bounds__(256) k_cg_dot4(long long n4, const float* __re
 __global__ void __launch_bounds__(256) k_cg_dir4(long long n4, const float* __restrict__ r,
                                                  const float* __restrict__ mi, bool pc,
                                                  float* __restrict__ p, const CgCtrl* c) {
-  launch_wait();
+  const unsigned blk = launch_wait_block();
   if (c->done) return;
   const float be = float(c->beta);
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n4; j += stride) {
+  for (long long j = blk * (long long)blockDim.x + threadIdx.x; j < n4; j += stride) {
     const float4 r4 = ld4(r, j), p4 = ld4(p, j), m4 = pc ? ld4(mi, j) : make_float4(1.f, 1.f, 1.f, 1.f);
     st4(p, j, make_float4(cg_direction(m4.x, r4.x, be, p4.x), cg_direction(m4.y, r4.y, be, p4.y),
                           cg_direction(m4.z, r4.z, be, p4.z), cg_direction(m4.w, r4.w, be, p4.w)));
