@@ -40,6 +40,45 @@ int probe_stuck_barrier(pf_hierarchy* h, long long polls) {
   return cudaStreamSynchronize(h->st) != cudaSuccess ? 4 : 0;
 }
 
+// A copy of the level's stored Galerkin operator.
+int probe_galerkin_stencil(pf_hierarchy* h, int level, float* out) {
+  const size_t n = size_t(galerkin_stencil_count(h->geo[level]));
+  if (!h->lv[level].gs) return 1;
+  if (cudaMemcpyAsync(out, h->lv[level].gs, sizeof(float) * n, cudaMemcpyDeviceToDevice, h->st) != cudaSuccess) return 2;
+  return cudaStreamSynchronize(h->st) != cudaSuccess ? 3 : 0;
+}
+
+// The one-launch subproblem of a level: min g.s + s.S s / 2 over lo <= s <= hi
+// (S and mi FP32 or FP64); stats: CG products, restarts.
+int probe_subproblem(pf_hierarchy* h, int level, int fp32, const void* S, const void* mi, const double* g,
+                     const double* lo, const double* hi, double* s, int cg_max, int max_restarts, int* stats) {
+  SubIn in{};
+  in.stencil = S;
+  in.fp32 = fp32 != 0;
+  in.gr = g;
+  in.lo = lo;
+  in.hi = hi;
+  in.mi = mi;
+  in.s = s;
+  in.work = h->sub_work;
+  in.partials = h->sub_partials;
+  in.bar = h->sub_bar;
+  in.ctl = h->sub_ctl;
+  in.delta = 1.0;
+  in.cauchy_c = 0.01;
+  in.spin_limit = h->sub_spin_limit;
+  in.backtracks = 30;
+  in.cg_max = cg_max;
+  in.max_restarts = max_restarts;
+  if (subproblem_coop(h->geo[level], in, h->st) != cudaSuccess) return 1;
+  SubCtrl c{};
+  if (cudaMemcpyAsync(&c, h->sub_ctl, sizeof c, cudaMemcpyDeviceToHost, h->st) != cudaSuccess) return 2;
+  if (cudaStreamSynchronize(h->st) != cudaSuccess) return 3;
+  stats[0] = c.used;
+  stats[1] = c.restarts;
+  return c.failed ? 4 : 0;
+}
+
 // Whether the level holds the FP64 stencil of the mixed mode's small levels.
 int probe_small_stencil(pf_hierarchy* h, int level) { return h->lv[level].small ? 1 : 0; }
 
