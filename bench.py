@@ -72,14 +72,15 @@ METRIC = "RMTR s/load-step & hessvec GDoF/s: mixed+learned vs FP64 plain, same G
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
 # roofline kernels on this workload, from one ncu capture of
 # `bench.py --kernels-only`; to be re-captured whenever those kernels change.
-TRAFFIC_HESSVEC_FP32 = (69.044e6 + 17.576e6) + (47.787e6 + 1.250e6)  # element pass + gather
+TRAFFIC_HESSVEC_FP32 = (69.043e6 + 14.898e6) + (47.789e6 + 0.850e6)  # element pass + gather
 TRAFFIC_HESSVEC_FP64 = 7595.291e6 + 86.475e6
 UNIT = "s/load-step"
 # FP32 flops of one element of the 3D FP32 Hessian product (the paired-FMA
 # element algebra and its corner sums), from the FP32 instruction counts of
-# one ncu capture (FFMA2 x4, FFMA x2, FADD2/FMUL2 x2, FADD/FMUL x1): 6,135 M
-# flop over the 144^3 element evaluations of an owner-computes launch.
-FLOP32_PER_ELEMENT = 2055
+# one ncu capture of its element pass (FFMA2 x4, FFMA x2, FADD2/FMUL2 x2,
+# FADD/FMUL x1): 3,464 M flop over 128^3 elements, the work that is done (an
+# earlier algebra took 2,055 per element for the same product).
+FLOP32_PER_ELEMENT = 1652
 # FP32 lanes per SM (Blackwell): the ALU roofline is SMs x lanes x 2 flop
 # (one FMA) x the SM clock sampled while the kernels ran.
 FP32_LANES_PER_SM = 128

@@ -325,9 +325,11 @@ pf_status pf_coarse_bounds(pf_hierarchy* h, int coarse, const double* lo_f_dev,
  * V-cycles (Algorithm 1, mu1 = mu2 = 1, Hessian lagging of Sec. 4.2.1) until
  * the projected gradient meets rtol/atol or max_cycles.  x_dev: finest FP64
  * state, updated in place.  params NULL = defaults.  stats may be NULL.
- * Each level's CG loop runs as one CUDA graph (a conditional while node
- * around one CG iteration), built on first use, rebuilt when the pressure,
- * precision or coarse model change, and held by the hierarchy until
+ * A small level's subproblem is one cooperative launch; on element-owned FP32
+ * levels CG iterations are enqueued ahead of their read-back; elsewhere the CG
+ * loop runs as one CUDA graph (a conditional while node around one CG
+ * iteration), built on first use, rebuilt when the pressure, precision or
+ * coarse model change, and held by the hierarchy until
  * pf_mesh_hierarchy_destroy.  The call synchronises the hierarchy's stream
  * (it reads scalars back) and cannot itself be captured into a graph.
  * Errors: PF_ENOTCONV (x still updated), PF_ENONFINITE (a NaN/Inf in x on

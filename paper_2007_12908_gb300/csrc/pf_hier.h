@@ -93,7 +93,7 @@ void refresh_pressure(pf_hierarchy* H);
 // of a small level in the mixed mode.
 cudaError_t ensure_stencil(pf_hierarchy* H, int l);
 cudaError_t ensure_small(pf_hierarchy* H, int l);
-// Allocates level l's Galerkin element matrices and FP32 stencil on first
+// Allocates level l's Galerkin coefficient moments and FP32 stencil on first
 // use, and builds the FP32 Galerkin operators of every coarse level from
 // the finest level's FP32 lag x (R G I chain, see pf_galerkin.cu).
 cudaError_t ensure_galerkin(pf_hierarchy* H, int l);

@@ -518,8 +518,9 @@ cudaError_t elem_gradient(const Geom& g, const Mat<double>& m, const void* x, vo
 // Element-owned 3D FP32 Hessian product, pass 1: a CTA owns 8^3 elements
 // and evaluates each once (no halo re-evaluation).  It stages their 9^3
 // corner nodes of x_lag and v and writes the 9^3 node sums to part (one block
-// of 729 float4 per tile).  Bound by the FP32 pipe (71% busy over the kernel,
-// 88 us at 129^3, of 4 x 4 warps an SM).  A warp owns two element layers and
+// of 729 float4 per tile).  Bound by FP32 issue (2.4 of 4 warp instructions per
+// cycle, 46 % of them FMA-pipe slots by count, 4 x 4 warps an SM; 91 us at 129^3,
+// 103 with the next pass).  A warp owns two element layers and
 // sums their corner contributions, one corner of all lanes at a time, into node
 // planes of its own, so that the eight phases of 32 elements need no CTA barrier
 // (with the 9^3 sums shared by the CTA: 93 us); the planes of two warps meet in
@@ -950,9 +951,9 @@ cudaError_t elem_gradient_fp64(const Geom& g, const Mat<double>& m, const double
 // A double-float operation is 7 to 15 instructions, so an element's code is
 // what bounds these passes: the fully unrolled gradient (11,400 instructions,
 // 183 KB) was fetched from L2 by every warp and issued 31 % of the time.  The
-// two z layers of Gauss points are a loop now (9,400 instructions executed,
-// well under the instruction cache's size in memory): issue 70 %, 828 ->
-// 305 us on 97 x 105 x 89 nodes; the energy 268 -> 167 us.
+// two z layers of Gauss points are a loop now, well under the instruction
+// cache's size in memory: issue 66 %, 828 -> 330 us on 97 x 105 x 89 nodes (305
+// with more rounding, see Corners3); the energy 268 -> 170 us.
 __global__ void k_to_df(long long n, const double* __restrict__ x, float2* __restrict__ xd) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {

@@ -3,7 +3,9 @@
 // touch global memory, so that back-to-back launches of a few microseconds do
 // not pay the launch latency each.  3D FP32 product on 33 x 25 x 29 nodes, one
 // after another: 8.2 -> 5.7 us; FP64 energy, gradient, lag and eight products
-// on 69 x 45: 100 -> 86 us.  Between larger kernels the last wave of one and
+// on 69 x 45: 100 -> 86 us.  That is the overlap of one launch with the launch
+// before it: a single product after other work takes what it did.  Between
+// larger kernels the last wave of one and
 // the start of the next overlap: the two launches of the 129^3 product 108.6 ->
 // 102.9 us, a mixed 129^3 load step (some 3,000 launches) 210 -> 202 ms, the
 // five transfers at 129^3 177 -> 168 us, the Galerkin operators of a 65^3

@@ -12,8 +12,9 @@
 // cp.async pieces and an ldmatrix row is 8 channels of any pixel: a tap is a
 // shift of row addresses.  With channel planes every operand word was two
 // scalar loads with the pooling, upsampling or concatenation worked out per
-// value, and the tensor pipe was 4-9 % busy; now it is 40-60 % busy on the
-// large layers (of what mma.sync can issue).  Forward and backward:
+// value, and the tensor pipe was 4-9 % busy; now it is 34-70 % busy (of what
+// mma.sync can issue) in the 3 x 3 products of 1032^2, but for those whose
+// epilogue spreads a pooled gradient (15-19 %), and 6-11 % in the 1 x 1 head.  Forward and backward:
 //   1032^2  1.92 -> 0.44 ms and  9.19 -> 1.61 ms
 //    136^2   604 ->   66 us and  1183 ->  271 us (latency of 16 and 45
 //                                                launches in sequence)
@@ -1100,6 +1101,9 @@ pf_status pf_unet_backward(pf_unet* u, const float* dy) {
     e = c.k == 3 ? launch_wgrad<3>(dh, dl, c.coP, in, c.ca, c.cb, H, W, c.co, P, u->wpart, u->side)
                  : launch_wgrad<1>(dh, dl, c.coP, in, c.ca, c.cb, H, W, c.co, P, u->wpart, u->side);
     if (e != cudaSuccess) break;
+    // narrow blocks where there are many partials: backward at 136^2 274 us
+    // against 280 with 32 columns throughout (and 338 with 8), 394 against 393 at
+    // 264^2, 714 against 698 at 528 x 520
     const int cols = P >= 64 ? 8 : 32;
     k_sum_parts<<<unsigned((nw + cols - 1) / cols + (c.co + kBiasCols - 1) / kBiasCols), 256, 0, u->side>>>(
         u->wpart, P, nw, cols, u->g + c.off_w, u->bpart[l], Pb, c.co, c.coP, u->g + c.off_b);
